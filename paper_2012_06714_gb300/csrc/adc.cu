@@ -57,6 +57,7 @@ struct adc_handle {
     int* pair_idx = nullptr;  // [3][npairs] (i, a, b) for EA, (i, j, a) for IP
     LadderTC* tc = nullptr;  // tensor-core ladder state (BF16x3 operands of B^Q_vv; open shells: the alpha block)
     LadderTC* tc_b = nullptr;  // open shells: the beta virtual block's ladder state
+    size_t pairs_limit = 0;    // device bytes the ladder's pair integrals may take (0: not held)
     int nva = 0;               // open shells: alpha virtual spin orbitals (the first nva of the v)
     // tensor-core ladder arithmetic: Davidson sigma, the setup ladder of t, and
     // the final refinement of converged roots
@@ -966,6 +967,16 @@ static void make_t1_third_order(adc_handle* h) {
 
 static void transition_parts(adc_handle* h, bool third, double* Tpp, double* t1x);
 
+// the timeout flag of the handle's tensor-core kernels (waits for the work issued so far)
+static void check_flag(adc_handle* h, const char* where) {
+    Ctx& c = h->ctx;
+    if (!c.d_err) return;
+    int e = 0;
+    ADC_CUDA(cudaMemcpyAsync(&e, c.d_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+    ADC_CUDA(cudaStreamSynchronize(c.stream));
+    if (e) throw Error(ADC_ERR_TIMEOUT, std::string(where) + ": a bounded device wait of the tensor-core GEMM timed out");
+}
+
 static void setup(adc_handle* h, const double* eps_in, const double* B_in, int on_device) {
     Ctx& c = h->ctx;
     // phase timer: 0 inputs and the ladder's operand planes, 1 integrals, 2 amplitudes and E(2),
@@ -1019,6 +1030,8 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
     if (h->opt.tune_cache && h->opt.tune_cache[0]) c.tuner = tune_cache_open(h->opt.tune_cache);
     h->opt.tune_cache = nullptr;  // the caller's string is not kept
     if (h->opt.precision != ADC_PREC_FP64) {
+        c.d_err = (int*)dev_alloc(sizeof(int), c.stream);
+        ADC_CUDA(cudaMemsetAsync(c.d_err, 0, sizeof(int), c.stream));
         h->tc = ladder_tc_create(c, h->Bvv, (int)Q, (int)v, h->opt.aux_chunk);
         noalloc_prepare();  // the allocation-free ladder's scratch address on this device, resolved up front
     }
@@ -1080,21 +1093,32 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
     }
     tick(2);
     Scope setup_scope(c.arena);
+    PairsPin setup_pin(h->tc, c, true);
     double* XL = nullptr;  // EA: the ladder term of the 1p-1p block, formed while the ladder of t is alive
     if (h->order >= 3) {
         const T T4 = op_t(h, false);
+        // The ladder's pair integrals: for the setup ladder, and for sigma on a plain EA handle.  Forming
+        // them is naux v^4 flops, the two passes of the setup ladder o^2 v^4 each with them and
+        // 4 naux o^2 v^3 each without: they are made when that does not cost the setup more.
+        const bool pairs = h->tc && (double)v * (Q + 2.0 * o * o) < 8.0 * Q * o * o &&
+                           ladder_pairs_bytes((int)v) <= h->pairs_limit && ladder_pairs_prepare(*h->tc, c, h->Bvv);
+        // three-plane pairs: partial sums promoted every K block, where the small products come first
+        // and only four MMAs truncate at full size; no extrapolation
+        const bool three = pairs && ladder_pairs_third(h->tc);
+        const LadderMode lm = three ? LadderMode{3, 1, 1} : h->lm_setup;
+        const bool extrapolate = h->opt.precision != ADC_PREC_FP64 && h->tc && !three;
         const bool keep_Lt = h->opt.m11_on_the_fly && h->kind == ADC_EA;  // sigma applies the block from it
         double* Lt = h->dmalloc(o2v2);
         if (!lean) {
             fill(c, o2v2, 0.0, Lt);
-            ladder(h, h->t, o * o, Lt, h->lm_setup);  // sum_cd (ac|bd) t_ij^cd (it feeds M_11 directly)
-            if (h->opt.precision != ADC_PREC_FP64 && h->tc) {
+            ladder(h, h->t, o * o, Lt, lm);  // sum_cd (ac|bd) t_ij^cd (it feeds M_11 directly)
+            if (extrapolate) {
                 // The tensor core's truncating FP32 accumulation biases each promoted partial sum
                 // toward zero, about linearly in the accumulation length.  With L(E) the ladder
                 // accumulated in epochs of E K blocks, 2 L(E) - L(2E) removes the linear part of
                 // that bias (Richardson extrapolation in E): measured on t2(2), bias -1.8e-7 ->
                 // -6e-8 relative at E = 1.  Formed in place: Lt <- -2 L(E), then += L(2E), negated.
-                const LadderMode twice{h->lm_setup.planes, 2 * h->lm_setup.epoch1, 2 * h->lm_setup.epoch2};
+                const LadderMode twice{lm.planes, 2 * lm.epoch1, 2 * lm.epoch2};
                 axpby(c, o2v2, 0.0, Lt, -2.0, Lt);
                 ladder(h, h->t, o * o, Lt, twice);
                 axpby(c, o2v2, 0.0, Lt, -1.0, Lt);
@@ -1121,14 +1145,14 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
             k_pairs_gather<<<grid_for(np * vv), 256, 0, c.stream>>>(np, vv, (int)o, dpi, dpj, h->t, P);
             launch_check(c);
             fill(c, np * vv, 0.0, Lp);
-            ladder(h, P, np, Lp, h->lm_setup);
-            if (h->opt.precision != ADC_PREC_FP64 && h->tc) {
+            ladder(h, P, np, Lp, lm);
+            if (extrapolate) {
                 // The tensor core's truncating FP32 accumulation biases each promoted partial sum
                 // toward zero, about linearly in the accumulation length.  With L(E) the ladder
                 // accumulated in epochs of E K blocks, 2 L(E) - L(2E) removes the linear part of
                 // that bias (Richardson extrapolation in E): measured on t2(2), bias -1.8e-7 ->
                 // -6e-8 relative at E = 1.  Formed in place: Lp <- -2 L(E), then += L(2E), negated.
-                const LadderMode twice{h->lm_setup.planes, 2 * h->lm_setup.epoch1, 2 * h->lm_setup.epoch2};
+                const LadderMode twice{lm.planes, 2 * lm.epoch1, 2 * lm.epoch2};
                 axpby(c, np * vv, 0.0, Lp, -2.0, Lp);
                 ladder(h, P, np, Lp, twice);
                 axpby(c, np * vv, 0.0, Lp, -1.0, Lp);
@@ -1137,6 +1161,14 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
             k_pairs_scatter<<<(unsigned)std::min<long long>(np * nt * nt, 152LL * 16), dim3(32, 8), 0, c.stream>>>(
                 np, (int)v, (int)o, dpi, dpj, Lp, Lt);
             launch_check(c);
+        }
+        if (pairs) {
+            check_flag(h, "setup");
+            // the IP sigma has no ladder, and a lean handle keeps its memory small
+            if (h->kind != ADC_EA || lean)
+                ladder_pairs_drop(*h->tc, c);
+            else
+                ladder_pairs_drop_third(*h->tc, c);
         }
         tick(3);
         double* N = Lt;  // t2(2) numerator, formed in the ladder's buffer unless the ladder is kept
@@ -1439,14 +1471,8 @@ static void sigma_launch(adc_handle* h, const double* X, double* S, long long nv
 }
 
 static void sigma_device(adc_handle* h, const double* X, double* S, long long nvec) {
-    Ctx& c = h->ctx;
     sigma_launch(h, X, S, nvec);
-    if (c.d_err) {
-        int e = 0;
-        ADC_CUDA(cudaMemcpyAsync(&e, c.d_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
-        ADC_CUDA(cudaStreamSynchronize(c.stream));
-        if (e) throw Error(ADC_ERR_TIMEOUT, "sigma: a bounded device wait of the tensor-core GEMM timed out");
-    }
+    check_flag(h, "sigma");
 }
 
 // sigma through a CUDA graph (cuda_graphs, mixed-precision handles): the launches of one sigma
@@ -1505,12 +1531,7 @@ static void sigma_run(adc_handle* h, const double* X, double* S, long long n) {
     ADC_CUDA(cudaMemcpyAsync(g->X, X, (size_t)n * dim * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
     ADC_CUDA(cudaGraphLaunch(g->exec, c.stream));
     ADC_CUDA(cudaMemcpyAsync(S, g->S, (size_t)n * dim * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
-    if (c.d_err) {
-        int e = 0;
-        ADC_CUDA(cudaMemcpyAsync(&e, c.d_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
-        ADC_CUDA(cudaStreamSynchronize(c.stream));
-        if (e) throw Error(ADC_ERR_TIMEOUT, "sigma: a bounded device wait of the tensor-core GEMM timed out");
-    }
+    check_flag(h, "sigma");
     if (h->tc) ladder_tc_check(*h->tc, c);
     if (h->tc_b) ladder_tc_check(*h->tc_b, c);
 }
@@ -3005,6 +3026,7 @@ int adc_mlp_samples(adc_handle* h, int nroots, const int* iters, int n_iters, lo
             return ADC_ERR_ARG;
         }
     GUARD(h, {
+        PairsPin pin(h->tc, h->ctx, true);
         mlp_samples(h, nroots, iters, n_iters, per_vector, seed, exact_tol, d, blk, r, t);
         return ADC_OK;
     })
@@ -3074,16 +3096,25 @@ static int setup_one(const double* eps, const double* Bq, int nocc, int nvir, in
             ADC_CUDA(cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking));
             h->ctx.set_stream(h->own_stream);
         }
+        // the plain layout's setup peak: B^Q blocks and input, the ladder's BF16 planes, ~9 o^2 v^2
+        // FP64 tensors at once
+        const double od = nocc, vd = nvir, Qd = naux, nmo = od + vd;
+        const double plain_bytes = 8.0 * (Qd * nmo * nmo * (on_device ? 2.0 : 1.0) + 9.0 * od * od * vd * vd) +
+                                   8.0 * Qd * vd * (vd + 31.0);
         bool lean = h->opt.lean > 0;
         if (h->opt.lean < 0 && lean_ok) {
             // automatic: lean when the plain layout's setup peak would not fit the free memory
-            // (B^Q blocks and input, the ladder's BF16 planes, ~9 o^2 v^2 FP64 tensors at once)
             size_t fr = 0, tot = 0;
             ADC_CUDA(cudaMemGetInfo(&fr, &tot));
-            const double o = nocc, v = nvir, Q = naux, nmo = o + v;
-            const double plain = 8.0 * (Q * nmo * nmo * (on_device ? 2.0 : 1.0) + 9.0 * o * o * v * v) +
-                                 8.0 * Q * v * (v + 31.0);
-            lean = plain > 0.9 * (double)fr;
+            lean = plain_bytes > 0.9 * (double)fr;
+        }
+        if (h->opt.precision != ADC_PREC_FP64) {
+            // the pair integrals of the ladder: at most a third of the free memory, and what the
+            // plain layout's setup leaves (plain_bytes)
+            size_t fr = 0, tot = 0;
+            ADC_CUDA(cudaMemGetInfo(&fr, &tot));
+            const double left = 0.9 * (double)fr - plain_bytes;
+            h->pairs_limit = (size_t)std::max(0.0, std::min((double)fr / 3.0, left));
         }
         if (lean) {
             h->lean = true;
@@ -3258,6 +3289,7 @@ int adc_sigma(adc_handle* h, const double* X, double* S, int nvec, int on_device
     }
     GUARD(h, {
         Ctx& c = h->ctx;
+        PairsPin pin(h->tc, c, true);
         const long long dim = h->dim();
         if (on_device) {
             sigma_device(h, X, S, nvec);
@@ -3282,6 +3314,7 @@ int adc_davidson(adc_handle* h, int nroots, double tol, const double* guess, dou
         return ADC_ERR_ARG;
     }
     GUARD(h, {
+        PairsPin pin(h->tc, h->ctx, !h->opt.cuda_graphs);  // (captured sigmas hold the integrals' address)
         int st = davidson(h, nroots, tol, guess, energies, specfac, vectors, stats);
         if (st == ADC_ERR_NOT_CONVERGED) h->err = "adc_davidson: not converged within max_iter";
         // the solver's scratch (subspace, residuals, sigma intermediates) goes back to the device:

@@ -20,11 +20,27 @@ struct PermArgs {
     long long sin[kMaxDim];  // input stride for each output axis
 };
 
+// the inputs of the permutes: an array, or the FP64 sum of S FP32 arrays `stride` apart
+template <typename Tin>
+struct Plain {
+    const Tin* p;
+    __device__ double operator()(long long i) const { return (double)p[i]; }
+};
+struct SumOf {
+    const float* p;
+    int S;
+    long long stride;
+    __device__ double operator()(long long i) const {
+        double x = (double)p[i];
+        for (int s = 1; s < S; ++s) x += (double)p[s * stride + i];
+        return x;
+    }
+};
+
 // I: the index type of the coordinate arithmetic (32-bit when every offset fits: integer
 // division by a runtime divisor is several times cheaper than in 64 bits)
-template <typename I>
-__global__ void permute_kernel(const double* __restrict__ in, double* __restrict__ out, PermArgs a, long long total,
-                               double alpha, double beta) {
+template <typename I, typename In, typename Tout>
+__global__ void permute_kernel(In in, Tout* __restrict__ out, PermArgs a, long long total, double alpha, double beta) {
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
         I r = (I)idx, off = 0;
@@ -34,24 +50,7 @@ __global__ void permute_kernel(const double* __restrict__ in, double* __restrict
             off += (r - q * d) * (I)a.sin[j];
             r = q;
         }
-        double v = alpha * in[off];
-        out[idx] = (beta == 0.0) ? v : v + beta * out[idx];
-    }
-}
-
-template <typename I, typename Tin, typename Tout>
-__global__ void permute_cvt_kernel(const Tin* __restrict__ in, Tout* __restrict__ out, PermArgs a, long long total,
-                                   double alpha, double beta) {
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        I r = (I)idx, off = 0;
-        for (int j = a.nd - 1; j >= 0; --j) {
-            const I d = (I)a.dout[j];
-            const I q = r / d;
-            off += (r - q * d) * (I)a.sin[j];
-            r = q;
-        }
-        double v = alpha * (double)in[off];
+        const double v = alpha * in(off);
         out[idx] = (Tout)((beta == 0.0) ? v : v + beta * (double)out[idx]);
     }
 }
@@ -66,10 +65,21 @@ __global__ void fill_kernel(long long n, double v, double* __restrict__ y) {
         y[i] = v;
 }
 
-// out[p][r*Kp + k] (two BF16 planes) from the permuted input, zero for k >= K
+// x as BF16 planes: o0 + o1 (+ o2 where there is a third), each the rounded remainder of those before
+__device__ __forceinline__ void put_planes(double x, long long ad, __nv_bfloat16* o0, __nv_bfloat16* o1, __nv_bfloat16* o2) {
+    const __nv_bfloat16 h = __double2bfloat16(x);
+    o0[ad] = h;
+    x -= (double)__bfloat162float(h);
+    const __nv_bfloat16 m = __double2bfloat16(x);
+    o1[ad] = m;
+    if (o2) o2[ad] = __double2bfloat16(x - (double)__bfloat162float(m));
+}
+
+// out[p][r*Kp + k] (two or three BF16 planes) from the permuted input, zero for k >= K
 template <typename I, typename Tin>
 __global__ void permute_split_kernel(const Tin* __restrict__ in, __nv_bfloat16* __restrict__ o0,
-                                     __nv_bfloat16* __restrict__ o1, PermArgs a, long long rows, long long K, long long Kp) {
+                                     __nv_bfloat16* __restrict__ o1, __nv_bfloat16* __restrict__ o2, PermArgs a,
+                                     long long rows, long long K, long long Kp) {
     const long long total = rows * Kp;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -85,9 +95,7 @@ __global__ void permute_split_kernel(const Tin* __restrict__ in, __nv_bfloat16* 
             }
             x = (double)in[off];
         }
-        const __nv_bfloat16 h = __double2bfloat16(x);
-        o0[idx] = h;
-        o1[idx] = __double2bfloat16(x - (double)__bfloat162float(h));
+        put_planes(x, idx, o0, o1, o2);
     }
 }
 
@@ -103,19 +111,15 @@ struct TileArgs {
     long long ntx, nty, nblocks;
 };
 
-// output of two split BF16 planes [rows][Kp] (the linear output index counts [rows][K])
+// output of split BF16 planes [rows][Kp] (the linear output index counts [rows][K])
 struct OpPlanes {
-    __nv_bfloat16 *o0, *o1;
+    __nv_bfloat16 *o0, *o1, *o2;
     long long K, Kp;
     __device__ long long addr(long long lin) const {
         const long long r = lin / K;
         return r * Kp + (lin - r * K);
     }
-    __device__ void put(long long ad, double x) const {
-        const __nv_bfloat16 h = __double2bfloat16(x);
-        o0[ad] = h;
-        o1[ad] = __double2bfloat16(x - (double)__bfloat162float(h));
-    }
+    __device__ void put(long long ad, double x) const { put_planes(x, ad, o0, o1, o2); }
 };
 // out = alpha x + beta out
 template <typename Tout>
@@ -129,8 +133,8 @@ struct OpAxpby {
     }
 };
 
-template <typename Tin, typename Op>
-__global__ void __launch_bounds__(256) k_permute_tiled(const Tin* __restrict__ in, TileArgs a, Op op) {
+template <typename In, typename Op>
+__global__ void __launch_bounds__(256) k_permute_tiled(In in, TileArgs a, Op op) {
     __shared__ double tile[32][33];
     for (long long b = blockIdx.x; b < a.nblocks; b += gridDim.x) {
         long long t = b;
@@ -148,7 +152,7 @@ __global__ void __launch_bounds__(256) k_permute_tiled(const Tin* __restrict__ i
         const long long x0 = tx * 32, y0 = ty * 32;
         for (int i = threadIdx.y; i < 32; i += 8) {
             const long long x = x0 + i, y = y0 + threadIdx.x;
-            if (x < a.nx && y < a.ny) tile[threadIdx.x][i] = (double)in[in_off + x * a.sx_in + y];
+            if (x < a.nx && y < a.ny) tile[threadIdx.x][i] = in(in_off + x * a.sx_in + y);
         }
         __syncthreads();
         for (int i = threadIdx.y; i < 32; i += 8) {
@@ -164,21 +168,14 @@ __global__ void __launch_bounds__(256) k_permute_tiled(const Tin* __restrict__ i
 }
 
 // zero the K padding columns of split planes [rows][Kp]
-__global__ void k_zero_pad(__nv_bfloat16* __restrict__ o0, __nv_bfloat16* __restrict__ o1, long long rows, long long K,
-                           long long Kp) {
+__global__ void k_zero_pad(__nv_bfloat16* __restrict__ o0, __nv_bfloat16* __restrict__ o1, __nv_bfloat16* __restrict__ o2,
+                           long long rows, long long K, long long Kp) {
     const long long w = Kp - K, n = rows * w;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const long long r = i / w, k = K + (i - r * w);
         o0[r * Kp + k] = __double2bfloat16(0.0);
         o1[r * Kp + k] = __double2bfloat16(0.0);
-    }
-}
-
-__global__ void sum_slices_kernel(int S, long long n, const double* __restrict__ T, double* __restrict__ C) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        double a = 0.0;
-        for (int s = 0; s < S; ++s) a += T[s * n + i];
-        C[i] = a;
+        if (o2) o2[r * Kp + k] = __double2bfloat16(0.0);
     }
 }
 
@@ -524,38 +521,10 @@ static bool tiled_args(const PermArgs& p, TileArgs& t) {
     return true;
 }
 
-template <typename Tin, typename Op>
-static void launch_tiled(Ctx& c, const Tin* in, const TileArgs& t, const Op& op) {
+template <typename In, typename Op>
+static void launch_tiled(Ctx& c, const In& in, const TileArgs& t, const Op& op) {
     const long long g = std::min<long long>(t.nblocks, 152LL * 16);
-    k_permute_tiled<Tin, Op><<<(unsigned)g, dim3(32, 8), 0, c.stream>>>(in, t, op);
-    ++c.kernels;
-    ADC_CUDA(cudaGetLastError());
-}
-
-void permute(Ctx& c, const double* in, const Shape& s, const int* perm, double* out, double alpha, double beta) {
-    PermArgs a;
-    a.nd = s.nd;
-    long long st[kMaxDim];
-    long long acc = 1, total = 1;
-    for (int j = s.nd - 1; j >= 0; --j) {
-        st[j] = acc;
-        acc *= s.d[j];
-    }
-    for (int j = 0; j < s.nd; ++j) {
-        a.dout[j] = s.d[perm[j]];
-        a.sin[j] = st[perm[j]];
-        total *= a.dout[j];
-    }
-    if (total == 0) return;
-    TileArgs t;
-    if (tiled_args(a, t)) {
-        launch_tiled(c, in, t, OpAxpby<double>{out, alpha, beta});
-        return;
-    }
-    if (total <= 0xffffffffLL)  // every offset is below total
-        permute_kernel<unsigned><<<grid_for(total), 256, 0, c.stream>>>(in, out, a, total, alpha, beta);
-    else
-        permute_kernel<long long><<<grid_for(total), 256, 0, c.stream>>>(in, out, a, total, alpha, beta);
+    k_permute_tiled<In, Op><<<(unsigned)g, dim3(32, 8), 0, c.stream>>>(in, t, op);
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
 }
@@ -578,8 +547,8 @@ static PermArgs perm_args(const Shape& s, const int* perm, long long& total) {
     return a;
 }
 
-template <typename Tin, typename Tout>
-static void permute_cvt(Ctx& c, const Tin* in, const Shape& s, const int* perm, Tout* out, double alpha, double beta) {
+template <typename In, typename Tout>
+static void permute_in(Ctx& c, const In& in, const Shape& s, const int* perm, Tout* out, double alpha, double beta) {
     long long total;
     PermArgs a = perm_args(s, perm, total);
     if (total == 0) return;
@@ -588,23 +557,38 @@ static void permute_cvt(Ctx& c, const Tin* in, const Shape& s, const int* perm, 
         launch_tiled(c, in, t, OpAxpby<Tout>{out, alpha, beta});
         return;
     }
-    if (total <= 0xffffffffLL)
-        permute_cvt_kernel<unsigned, Tin, Tout><<<grid_for(total), 256, 0, c.stream>>>(in, out, a, total, alpha, beta);
+    if (total <= 0xffffffffLL)  // every offset is below total
+        permute_kernel<unsigned, In, Tout><<<grid_for(total), 256, 0, c.stream>>>(in, out, a, total, alpha, beta);
     else
-        permute_cvt_kernel<long long, Tin, Tout><<<grid_for(total), 256, 0, c.stream>>>(in, out, a, total, alpha, beta);
+        permute_kernel<long long, In, Tout><<<grid_for(total), 256, 0, c.stream>>>(in, out, a, total, alpha, beta);
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
 }
 
+void permute(Ctx& c, const double* in, const Shape& s, const int* perm, double* out, double alpha, double beta) {
+    permute_in(c, Plain<double>{in}, s, perm, out, alpha, beta);
+}
+
+void permute_sum(Ctx& c, const float* in, int S, const Shape& s, const int* perm, void* out, bool out32, double alpha,
+                 double beta) {
+    long long n = 1;
+    for (int j = 0; j < s.nd; ++j) n *= s.d[j];
+    if (out32)
+        permute_in(c, SumOf{in, S, n}, s, perm, (float*)out, alpha, beta);
+    else
+        permute_in(c, SumOf{in, S, n}, s, perm, (double*)out, alpha, beta);
+}
+
 template <typename Tin>
 static void split_planes_t(Ctx& c, const Tin* in, const PermArgs& a, long long rows, long long K, long long Kp,
-                           void* const* out) {
+                           void* const* out, int planes) {
     TileArgs t;
+    __nv_bfloat16 *o0 = (__nv_bfloat16*)out[0], *o1 = (__nv_bfloat16*)out[1];
+    __nv_bfloat16* o2 = planes == 3 ? (__nv_bfloat16*)out[2] : nullptr;
     if (tiled_args(a, t)) {
-        launch_tiled(c, in, t, OpPlanes{(__nv_bfloat16*)out[0], (__nv_bfloat16*)out[1], K, Kp});
+        launch_tiled(c, Plain<Tin>{in}, t, OpPlanes{o0, o1, o2, K, Kp});
         if (Kp > K) {
-            k_zero_pad<<<grid_for(rows * (Kp - K)), 256, 0, c.stream>>>((__nv_bfloat16*)out[0], (__nv_bfloat16*)out[1],
-                                                                         rows, K, Kp);
+            k_zero_pad<<<grid_for(rows * (Kp - K)), 256, 0, c.stream>>>(o0, o1, o2, rows, K, Kp);
             ++c.kernels;
             ADC_CUDA(cudaGetLastError());
         }
@@ -612,37 +596,37 @@ static void split_planes_t(Ctx& c, const Tin* in, const PermArgs& a, long long r
     }
     // 32-bit coordinates when the output index fits (every input offset is below rows * K)
     if (rows * Kp <= 0xffffffffLL)
-        permute_split_kernel<unsigned, Tin><<<grid_for(rows * Kp), 256, 0, c.stream>>>(
-            in, (__nv_bfloat16*)out[0], (__nv_bfloat16*)out[1], a, rows, K, Kp);
+        permute_split_kernel<unsigned, Tin><<<grid_for(rows * Kp), 256, 0, c.stream>>>(in, o0, o1, o2, a, rows, K, Kp);
     else
-        permute_split_kernel<long long, Tin><<<grid_for(rows * Kp), 256, 0, c.stream>>>(
-            in, (__nv_bfloat16*)out[0], (__nv_bfloat16*)out[1], a, rows, K, Kp);
+        permute_split_kernel<long long, Tin><<<grid_for(rows * Kp), 256, 0, c.stream>>>(in, o0, o1, o2, a, rows, K, Kp);
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
 }
 
 void split_planes(Ctx& c, const double* in, const Shape& s, const int* perm, long long rows, long long K, long long Kp,
-                  void* const* out, bool in32) {
+                  void* const* out, bool in32, int planes) {
     long long total;
     PermArgs a = perm_args(s, perm, total);
     if (total != rows * K) throw Error(-1, "split_planes: shape mismatch");
     if (rows * Kp == 0) return;
     if (in32)
-        split_planes_t(c, (const float*)in, a, rows, K, Kp, out);
+        split_planes_t(c, (const float*)in, a, rows, K, Kp, out, planes);
     else
-        split_planes_t(c, in, a, rows, K, Kp, out);
+        split_planes_t(c, in, a, rows, K, Kp, out, planes);
 }
 
 void permute_any(Ctx& c, const void* in, bool in32, const Shape& s, const int* perm, void* out, bool out32,
                  double alpha, double beta) {
+    const Plain<double> d{(const double*)in};
+    const Plain<float> f{(const float*)in};
     if (!in32 && !out32)
-        permute(c, (const double*)in, s, perm, (double*)out, alpha, beta);
+        permute_in(c, d, s, perm, (double*)out, alpha, beta);
     else if (in32 && out32)
-        permute_cvt(c, (const float*)in, s, perm, (float*)out, alpha, beta);
+        permute_in(c, f, s, perm, (float*)out, alpha, beta);
     else if (in32)
-        permute_cvt(c, (const float*)in, s, perm, (double*)out, alpha, beta);
+        permute_in(c, f, s, perm, (double*)out, alpha, beta);
     else
-        permute_cvt(c, (const double*)in, s, perm, (float*)out, alpha, beta);
+        permute_in(c, d, s, perm, (float*)out, alpha, beta);
 }
 
 void axpby(Ctx& c, long long n, double alpha, const double* x, double beta, double* y) {
@@ -650,27 +634,6 @@ void axpby(Ctx& c, long long n, double alpha, const double* x, double beta, doub
     axpby_kernel<<<grid_for(n), 256, 0, c.stream>>>(n, alpha, x, beta, y);
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
-}
-
-void sum_slices(Ctx& c, int S, long long n, const double* T, double* C) {
-    if (n <= 0) return;
-    sum_slices_kernel<<<grid_for(n), 256, 0, c.stream>>>(S, n, T, C);
-    ++c.kernels;
-    ADC_CUDA(cudaGetLastError());
-}
-
-void ensure_side_streams(Ctx& c, int count) {
-    if (c.capturing && (!c.side_fork || (int)c.side.size() < count))
-        throw Error(-3, "side stream creation during stream capture");
-    if (!c.side_fork) ADC_CUDA(cudaEventCreateWithFlags(&c.side_fork, cudaEventDisableTiming));
-    while ((int)c.side.size() < count) {
-        cudaStream_t s = nullptr;
-        cudaEvent_t e = nullptr;
-        ADC_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-        ADC_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        c.side.push_back(s);
-        c.side_join.push_back(e);
-    }
 }
 
 void fill(Ctx& c, long long n, double v, double* y) {
@@ -825,8 +788,8 @@ static void einsum_fp32(Ctx& c, const std::string& la, const std::string& lb, co
 
 // Tensor-core contraction (gemm_mode 2): operands permuted into K-major GEMM
 // order and split into two BF16 planes (constant operands once, cached), the
-// tcgen05 split-BF16 GEMM into an FP64 temporary, then permuted and
-// accumulated into the output.
+// tcgen05 split-BF16 GEMM into FP32 results (one per K slice), whose FP64 sum is permuted and
+// accumulated into the output in one pass.
 static void einsum_tc(Ctx& c, const std::string& la, const std::string& lb, const std::string& lc,
                       std::map<char, long long>& dim, const std::string& fa, const std::string& fb, const std::string& con,
                       double alpha, const T& A, const T& B, double beta, void* C, bool c32) {
@@ -871,17 +834,17 @@ static void einsum_tc(Ctx& c, const std::string& la, const std::string& lb, cons
         c.d_err = (int*)dev_alloc(sizeof(int), c.stream);
         ADC_CUDA(cudaMemsetAsync(c.d_err, 0, sizeof(int), c.stream));
     }
-    double* T = c.arena.dalloc((size_t)(M * N));
     const void* A2[2] = {pa, (const char*)pa + M * Kp * 2};
     const void* B2[2] = {pb, (const char*)pb + N * Kp * 2};
-    tc_gemm(c, A2, B2, M, N, Kp, 2.0 * M * N * K, T);
+    int S = 1;
+    const float* T = tc_gemm(c, A2, B2, M, N, Kp, 2.0 * M * N * K, S);
     std::string tord = fa + fb;
     Shape sh;
     sh.nd = (int)tord.size();
     for (int j = 0; j < sh.nd; ++j) sh.d[j] = dim[tord[j]];
     int perm[kMaxDim];
     for (int j = 0; j < sh.nd; ++j) perm[j] = (int)tord.find(lc[j]);
-    permute_any(c, T, false, sh, perm, C, c32, alpha, beta);
+    permute_sum(c, T, S, sh, perm, C, c32, alpha, beta);
 }
 
 static void einsum_core(Ctx& c, const char* specstr, double alpha, const T& A, const T& B, double beta, void* C, bool c32,

@@ -35,6 +35,20 @@ struct Error : std::runtime_error {
                                std::string(#x) + ": cublas status " + std::to_string((int)s_));       \
     } while (0)
 
+// Releases device memory that handles without a call in progress hold for speed only (pair
+// integrals of the ladder, ladder_tc.cu) on the current device; false if there was none.
+bool device_memory_reclaim();
+
+// cudaMallocAsync that reclaims such memory once before it gives up
+inline cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t s) {
+    cudaError_t e = cudaMallocAsync(p, bytes, s);
+    if (e == cudaErrorMemoryAllocation && device_memory_reclaim()) {
+        cudaGetLastError();
+        e = cudaMallocAsync(p, bytes, s);
+    }
+    return e;
+}
+
 // Device scratch: blocks are allocated on demand and kept; mark()/release()
 // give stack semantics so that repeated calls reuse the same memory.  Blocks
 // come from the stream-ordered allocator on `stream` (no device-wide
@@ -67,7 +81,7 @@ class Arena {
         if (big_bytes && bytes >= big_bytes) {
             if (frozen) throw Error(-3, "arena: growth during stream capture");
             void* p = nullptr;
-            ADC_CUDA(cudaMallocAsync(&p, bytes, stream));
+            ADC_CUDA(dev_malloc(&p, bytes, stream));
             big_.push_back(p);
             return p;
         }
@@ -86,7 +100,7 @@ class Arena {
         if (frozen) throw Error(-3, "arena: growth during stream capture");
         size_t cap = bytes > (size_t(256) << 20) ? bytes : (size_t(256) << 20);
         void* p = nullptr;
-        ADC_CUDA(cudaMallocAsync(&p, cap, stream));
+        ADC_CUDA(dev_malloc(&p, cap, stream));
         blocks_.push_back(p);
         caps_.push_back(cap);
         tops_.push_back(bytes);
@@ -124,7 +138,7 @@ class Arena {
 // Stream-ordered device allocation (memory from it is freed with cudaFree).
 inline void* dev_alloc(size_t bytes, cudaStream_t s) {
     void* p = nullptr;
-    ADC_CUDA(cudaMallocAsync(&p, bytes ? bytes : 1, s));
+    ADC_CUDA(dev_malloc(&p, bytes ? bytes : 1, s));
     return p;
 }
 
@@ -168,17 +182,10 @@ struct Ctx {
     // a CUDA-graph capture of sigma is recording on `stream`: no host synchronisation, no
     // allocation, no tuning; the timeout flags are read after the graph's replay instead
     bool capturing = false;
-    // side streams for concurrent K slices of a contraction, with their fork / join events
-    std::vector<cudaStream_t> side;
-    std::vector<cudaEvent_t> side_join;
-    cudaEvent_t side_fork = nullptr;
     ~Ctx() {
         for (auto& kv : f32cache) cudaFree(kv.second);
         for (auto& kv : bf16cache) cudaFree(kv.second);
         if (d_err) cudaFree(d_err);
-        for (auto s : side) cudaStreamDestroy(s);
-        for (auto e : side_join) cudaEventDestroy(e);
-        if (side_fork) cudaEventDestroy(side_fork);
         for (auto e : ev_start) cudaEventDestroy(e);
         for (auto e : ev_stop) cudaEventDestroy(e);
     }
@@ -194,10 +201,6 @@ struct Shape {
 void permute(Ctx& c, const double* in, const Shape& in_shape, const int* perm, double* out, double alpha, double beta);
 void axpby(Ctx& c, long long n, double alpha, const double* x, double beta, double* y);  // y = a x + b y
 void fill(Ctx& c, long long n, double v, double* y);
-// C[i] = sum_s T[s*n + i]
-void sum_slices(Ctx& c, int S, long long n, const double* T, double* C);
-// make at least `count` side streams (non-blocking) and their events
-void ensure_side_streams(Ctx& c, int count);
 
 // ---- contraction executor -------------------------------------------------
 struct T {
@@ -216,12 +219,15 @@ void einsum(Ctx& c, const char* spec, double alpha, const T& A, const T& B, doub
 // out = alpha * permute(in) + beta * out between FP64 / FP32 arrays (in32 / out32: FP32)
 void permute_any(Ctx& c, const void* in, bool in32, const Shape& s, const int* perm, void* out, bool out32,
                  double alpha, double beta);
+// the same for the FP64 sum of S FP32 arrays, one after another in `in` (the slices of tc_gemm)
+void permute_sum(Ctx& c, const float* in, int S, const Shape& s, const int* perm, void* out, bool out32, double alpha,
+                 double beta);
 
 // Permute `in` (shape s, output axis j = input axis perm[j]) into row-major
-// [rows][K] order and split each value x into BF16 planes x = p0 + p1 (two
-// planes), written K-major as out[p][r * Kp + k] with zeros for K <= k < Kp.
+// [rows][K] order and split each value x into BF16 planes x = p0 + p1 (+ p2: two
+// or three planes), written K-major as out[p][r * Kp + k] with zeros for K <= k < Kp.
 void split_planes(Ctx& c, const double* in, const Shape& s, const int* perm, long long rows, long long K, long long Kp,
-                  void* const* out, bool in32 = false);
+                  void* const* out, bool in32 = false, int planes = 2);
 
 // The library's own kernels for small and skinny contractions (row-major A [M][K],
 // B [K][N], C [M][N] with leading dimensions): C = alpha A B + beta C.  M <= 8 or

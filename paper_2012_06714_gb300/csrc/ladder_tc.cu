@@ -14,6 +14,9 @@
 // and laid out as GEMM2's K-major A operand; GEMM2 accumulates in FP32 over
 // one chunk and adds into the FP64 output, so FP64 carries the sum over chunks.
 //
+// Where the device memory allows it, the (ac|bd) themselves are kept, adapted to symmetric and
+// antisymmetric pairs, and the ladder is one contraction over pairs (ladder_pairs_*, below).
+//
 // Index padding: the virtual index on every K axis is padded to vp (multiple
 // of 32) with zeros so that TMA row strides and coordinates are 16-byte
 // aligned and 16-column epilogue chunks never straddle a matrix.
@@ -32,17 +35,13 @@
 #include <vector>
 
 #include "ladder_tc.cuh"
+#include "tcgen05.cuh"
 
 namespace adc {
 
 namespace {
 
 constexpr int BM = 128;
-// K block: 64 BF16 = 128-byte rows in the 128-byte swizzle (8-row atoms of
-// 1024 bytes).  (32-deep blocks with the 64-byte swizzle also work -- twice the
-// stages of half the size -- but measured slower.)
-constexpr int BK = 64;
-constexpr int ROW_BYTES = BK * 2;
 constexpr int KB_PER_EPOCH_UNIT = 64 / BK;  // LadderMode epochs count 64-deep K blocks
 constexpr int MAX_STAGES = 8;
 constexpr int EPI_WARPS = 8;
@@ -52,160 +51,48 @@ constexpr int A_BYTES = BM * BK * 2;
 // Always request (nearly) all of shared memory so that exactly one CTA, and one
 // 512-column TMEM allocation, lives on each SM.
 constexpr size_t SMEM_BYTES = 226 * 1024;
-constexpr unsigned long long WAIT_NS = 2000000000ull;  // bounded waits: 2 s
-
-__device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint64_t gtime() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t n) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(b)), "r"(n) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(su32(b)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// try_wait that lets the hardware suspend the thread (up to the hint, in ns)
-// until the phase completes, instead of spinning on issue slots.
-__device__ __forceinline__ bool mbar_try_sleep(uint64_t* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-        "selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(su32(b)), "r"(parity), "r"(20000u)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait: false on timeout (raises the CTA abort flag and the global
-// error flag) or when another role of the CTA has already aborted.  The abort
-// flag and the clock are checked every 16 tries only.
-__device__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag, int* err) {
-    if (mbar_try(b, parity)) return true;
-    const uint64_t t0 = gtime();
-    for (uint32_t n = 1;; ++n) {
-        if (mbar_try_sleep(b, parity)) return true;
-        if ((n & 15u) == 0) {
-            if (*abort_flag) return false;
-            if (gtime() - t0 > WAIT_NS) {
-                *abort_flag = 1;
-                atomicExch(err, 1);
-                return false;
-            }
-        }
-    }
-}
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* m, uint64_t* bar, int x, int y) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
-            su32(dst)),
-        "l"((uint64_t)m), "r"(su32(bar)), "r"(x), "r"(y)
-        : "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// tcgen05 shared-memory matrix descriptor: K-major, ROW_BYTES swizzle, 8-row
-// core groups 8 * ROW_BYTES apart.
-__device__ __forceinline__ uint64_t smem_desc(const void* p) {
-    uint64_t d = 0;
-    d |= (uint64_t)((su32(p) >> 4) & 0x3FFF);
-    d |= (uint64_t)1 << 16;                     // leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)((8 * ROW_BYTES) >> 4) << 32;  // stride byte offset
-    d |= (uint64_t)1 << 46;                     // descriptor version
-    d |= (uint64_t)(ROW_BYTES == 128 ? 2 : 4) << 61;  // layout: 128-byte (2) or 64-byte (4) swizzle
-    return d;
-}
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(bar)) : "memory");
-}
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tmem_ld32_add(uint32_t taddr, float* acc) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
-        "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) acc[i] += __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 struct Epi {
     int mode;  // 0: split store of Z (GEMM1, through shared memory and TMA), 1: FP64 accumulate (GEMM2),
-               // 2: FP64 store (generic contraction)
+               // 2: FP32 store (one result per part, see Parts)
     int M, N;
     // mode 0: row r = q*vpa + a (a padded to vpa, a multiple of 32), col j = n*vp + dp;
     // Z[((n*v + a)*qn + q)*vp + dp] per plane, written through the 4-D tensor maps Maps::z
     int vpa, vp;
-    // modes 1, 2: out[r*ldc + j] (+)= acc
+    // mode 1: out[r*ldc + j] += acc; mode 2: out32[z*zout + r*ldc + j] = acc for part z
     double* out;
     long long ldc;
     int vec;  // out rows 16-byte aligned (vector loads and stores)
     int* err;
+    float* out32;
+    long long zout;
 };
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(b)) : "memory");
-}
+// Several GEMMs of one shape, and K slices of each, as one launch (k_gemm_pair): part z is
+// matrix z / slices, K blocks [(z % slices) * kb, ...) of it; matrix m takes the A operand's rows
+// from m * a_step and the B operand's from m * b_step.  Every part is a set of output tiles of
+// its own (Epi mode 2), so a shape of few tiles still fills the chip from a single launch.
+struct Parts {
+    int n = 1, slices = 1, kb = 1 << 30;  // parts, K slices per matrix, K blocks (BK deep) per slice
+    int a_step = 0, b_step = 0;
+};
 
-// 16 consecutive FP32 results of one row into the FP64 output: accumulated
-// (mode 1, GEMM2 of the ladder) or stored (mode 2, generic contractions).
-__device__ __forceinline__ void store_out16(const Epi& ep, int row, int col0, const float* v) {
-    double* o = ep.out + (long long)row * ep.ldc + col0;
+// 16 consecutive FP32 results of one row into the output: FP64 accumulated
+// (mode 1, GEMM2 of the ladder), or stored as FP32 (mode 2, part z).
+__device__ __forceinline__ void store_out16(const Epi& ep, int row, int col0, const float* v, int z = 0) {
     if (ep.mode == 2) {
+        float* f = ep.out32 + z * ep.zout + (long long)row * ep.ldc + col0;
         if (ep.vec && col0 + 16 <= ep.N) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) ((double2*)o)[i] = make_double2((double)v[2 * i], (double)v[2 * i + 1]);
+            for (int i = 0; i < 4; ++i) ((float4*)f)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         } else {
 #pragma unroll
             for (int i = 0; i < 16; ++i)
-                if (col0 + i < ep.N) o[i] = (double)v[i];
+                if (col0 + i < ep.N) f[i] = v[i];
         }
         return;
     }
+    double* o = ep.out + (long long)row * ep.ldc + col0;
     if (ep.vec && col0 + 16 <= ep.N) {
         // 8 columns at a time: four 16-byte loads in flight before the stores
 #pragma unroll
@@ -294,345 +181,43 @@ __device__ __forceinline__ void store_z_drain(int lane) {
     __syncwarp();
 }
 
-// Persistent GEMM C = A B^T with split-BF16 operands.  Roles: warp 0 lane 0
-// issues TMA loads through a ring of `stages` shared-memory stages, running
-// ahead across tiles; warp 1 owns TMEM and its lane 0 issues the MMAs; warps
-// 2-9 are the epilogue.
+// Persistent GEMM C = A B^T with split-BF16 operands, each tile 256 rows high and computed by
+// a CTA pair (a cluster of two) through cta_group::2 MMAs: CTA r holds rows [128 r, 128 r + 128)
+// of the A tile and rows [BN/2 r, BN/2 (r+1)) of the B tile, so each SM receives A + B/2 per K
+// block.  Both CTAs' TMA loads complete on the leader's (rank 0) full barrier; the leader's MMA
+// thread issues every MMA and its commits arrive on the barriers of both CTAs; each CTA's
+// epilogue drains its own tensor memory (its 128 rows of the tile, all BN columns) and releases
+// the accumulator on the leader's barrier (2 x EPI_WARPS arrivals).  Roles: warp 0 lane 0 issues
+// TMA loads through a ring of `stages` shared-memory stages, running ahead across tiles; warp 1
+// owns TMEM and its lane 0 issues the MMAs; warps 2-9 are the epilogue.
 //
-// Accumulation.  The tensor core's FP32 accumulate truncates, so a long
-// accumulation in one TMEM accumulator drifts toward zero by about a quarter
-// ulp per MMA (measured: 2e-5 relative over a 4160-deep chunk).  The MMAs of a
-// tile are therefore issued in short epochs of `ekb` K blocks, alternating
-// between two TMEM accumulators; the epilogue warps add every epoch into FP32
-// registers with round-to-nearest (unbiased) while the next epoch runs, and
-// write the tile once after its last epoch.  Epilogue warp w covers TMEM lane
-// quarter (w % 4) and one half of the tile's columns.
-
-// kPromote = false (one epoch per tile) streams each tile from TMEM to global
-// memory without the register accumulator.
-// (ten warps: three share a sub-partition's 16K registers, so at most 168 per thread)
-template <bool kPromote>
-__global__ void __launch_bounds__(THREADS, 1)
-    k_gemm_bf16x3(const __grid_constant__ Maps maps, int planes, int a_row0, int b_x0, int K, int BN, int stages,
-                  int m_fastest, int mt, int nt, int ekb, int nbuf, Epi ep) {
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t full_bar[MAX_STAGES], empty_bar[MAX_STAGES], tfull[2], tempty[2], done_bar;
-    __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int num_k = (K + BK - 1) / BK;
-    const int epochs = (num_k + ekb - 1) / ekb;  // per tile
-    const int B_BYTES = BN * BK * 2;
-    const int STAGE = planes * (A_BYTES + B_BYTES);  // [A planes][B planes]
-    const int ntiles = mt * nt;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(&full_bar[s], 1);
-            mbar_init(&empty_bar[s], 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], EPI_WARPS);  // one arrival per epilogue warp
-        }
-        mbar_init(&done_bar, 1);
-        abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_slot)), "r"(TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    fence_before();
-    __syncthreads();
-    fence_after();
-    const uint32_t tmem = tmem_slot;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            long long g = 0;
-            for (int t = blockIdx.x; t < ntiles && !abort_flag; t += gridDim.x) {
-                const int m_tile = m_fastest ? t % mt : t / nt;
-                const int n_tile = m_fastest ? t / mt : t % nt;
-                for (int kb = 0; kb < num_k; ++kb, ++g) {
-                    const int s = (int)(g % stages);
-                    const uint32_t ph = (uint32_t)((g / stages) & 1);
-                    if (g >= stages && !mbar_wait(&empty_bar[s], ph ^ 1, &abort_flag, ep.err)) break;
-                    uint8_t* st = smem + (size_t)s * STAGE;
-                    mbar_expect_tx(&full_bar[s], STAGE);
-                    const int kx = kb * BK;
-                    // plane indices are compile-time constants so that the tensor maps stay in the parameter space
-                    uint8_t* sb = st + planes * A_BYTES;
-                    const int ya = a_row0 + m_tile * BM, yb = n_tile * BN;
-                    tma_load_2d(st, &maps.a[0], &full_bar[s], kx, ya);
-                    tma_load_2d(st + A_BYTES, &maps.a[1], &full_bar[s], kx, ya);
-                    if (planes == 3) tma_load_2d(st + 2 * A_BYTES, &maps.a[2], &full_bar[s], kx, ya);
-                    tma_load_2d(sb, &maps.b[0], &full_bar[s], b_x0 + kx, yb);
-                    tma_load_2d(sb + B_BYTES, &maps.b[1], &full_bar[s], b_x0 + kx, yb);
-                    if (planes == 3) tma_load_2d(sb + 2 * B_BYTES, &maps.b[2], &full_bar[s], b_x0 + kx, yb);
-                }
-            }
-            if (abort_flag) {
-                // let the copies of the last `stages` issues land before the CTA retires (bounded)
-                for (long long q = (g > stages ? g - stages : 0); q < g; ++q) {
-                    const uint64_t t0 = gtime();
-                    while (!mbar_try(&full_bar[q % stages], (uint32_t)((q / stages) & 1)) && gtime() - t0 < WAIT_NS) {
-                    }
-                }
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-            long long g = 0;   // stage uses
-            long long e = 0;   // epochs issued by this CTA (across tiles)
-            bool ok = true;
-            for (int t = blockIdx.x; t < ntiles && ok && !abort_flag; t += gridDim.x) {
-                int left = 0;  // K blocks left in the current epoch (epochs are whole K blocks)
-                uint32_t tacc = 0;
-                for (int kb = 0; kb < num_k; ++kb, ++g) {
-                    const int s = (int)(g % stages);
-                    if (!mbar_wait(&full_bar[s], (uint32_t)((g / stages) & 1), &abort_flag, ep.err)) {
-                        ok = false;
-                        break;
-                    }
-                    uint32_t first = 1u;
-                    if (left == 0) {
-                        // new epoch: wait until the epilogue has drained this buffer's previous epoch
-                        const int b = (int)(e & 1);
-                        if (e >= 2 && !mbar_wait(&tempty[b], (uint32_t)(((e >> 1) & 1) ^ 1), &abort_flag, ep.err)) {
-                            ok = false;
-                            break;
-                        }
-                        tacc = tmem + (uint32_t)(b * 256);
-                        left = ekb;
-                        first = 0u;
-                    }
-                    fence_after();
-                    uint8_t* st = smem + (size_t)s * STAGE;
-                    const uint64_t a0 = smem_desc(st), a1 = smem_desc(st + A_BYTES);
-                    const uint64_t b0 = smem_desc(st + planes * A_BYTES), b1 = smem_desc(st + planes * A_BYTES + B_BYTES);
-                    if (planes == 3) {
-                        const uint64_t a2 = smem_desc(st + 2 * A_BYTES), b2 = smem_desc(st + planes * A_BYTES + 2 * B_BYTES);
-#pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) {
-                            const uint64_t o = (uint64_t)(kk * 2);  // 16 BF16 = 32 bytes along K
-                            mma_bf16(tacc, a0 + o, b0 + o, idesc, kk == 0 ? first : 1u);
-                            mma_bf16(tacc, a0 + o, b1 + o, idesc, 1u);
-                            mma_bf16(tacc, a1 + o, b0 + o, idesc, 1u);
-                            mma_bf16(tacc, a0 + o, b2 + o, idesc, 1u);
-                            mma_bf16(tacc, a2 + o, b0 + o, idesc, 1u);
-                            mma_bf16(tacc, a1 + o, b1 + o, idesc, 1u);
-                        }
-                    } else {
-#pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) {
-                            const uint64_t o = (uint64_t)(kk * 2);
-                            mma_bf16(tacc, a0 + o, b0 + o, idesc, kk == 0 ? first : 1u);
-                            mma_bf16(tacc, a0 + o, b1 + o, idesc, 1u);
-                            mma_bf16(tacc, a1 + o, b0 + o, idesc, 1u);
-                        }
-                    }
-                    mma_commit(&empty_bar[s]);
-                    if (--left == 0 || kb == num_k - 1) {
-                        mma_commit(&tfull[e & 1]);
-                        ++e;
-                        left = 0;
-                    }
-                }
-            }
-            mma_commit(&done_bar);  // fires when every MMA issued above has completed
-        }
-    } else {
-        const int ew = warp - 2;
-        const int quarter = warp & 3;  // TMEM lanes 32*quarter .. +31
-        const int half = ew >> 2;      // column half of the tile
-        // The halves split on a 16-column boundary, [0, h0) and [h0, BN): both
-        // widths are multiples of 16 (BN is) and at most 128.
-        const int h0 = ((BN >> 1) + 15) & ~15;
-        const int cbeg = half ? h0 : 0, cw = half ? BN - h0 : h0;
-        // Z staging of this warp (mode 0) after the pipeline stages
-        uint8_t* stg = smem + (size_t)stages * STAGE + (size_t)ew * nbuf * planes * 1024;
-        int nchunk = 0;
-        long long e = 0;
-        bool ok = true;
-        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-            const int m_tile = m_fastest ? t % mt : t / nt;
-            const int n_tile = m_fastest ? t / mt : t % nt;
-            const int row = m_tile * BM + quarter * 32 + lane;
-            const int colt = n_tile * BN + cbeg;  // first output column of this warp
-            if constexpr (kPromote) {
-                float acc[128];
-#pragma unroll
-                for (int i = 0; i < 128; ++i) acc[i] = 0.0f;
-                for (int ep_i = 0; ep_i < epochs; ++ep_i, ++e) {
-                    if (ep.mode == 1 && ep_i == epochs - 1 && row < ep.M) {
-                        // pull this thread's FP64 output segment into L2 while the last epoch runs
-                        const double* o = ep.out + (long long)row * ep.ldc + colt;
-                        for (int c0 = 0; c0 < cw; c0 += 16)
-                            if (colt + c0 < ep.N) asm volatile("prefetch.global.L2 [%0];" ::"l"(o + c0));
-                    }
-                    const int b = (int)(e & 1);
-                    if (!mbar_wait(&tfull[b], (uint32_t)((e >> 1) & 1), &abort_flag, ep.err)) {
-                        ok = false;
-                        break;
-                    }
-                    fence_after();
-                    const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 256 + cbeg);
-                    // 32-column loads (one wait each), then a 16-column tail
-#pragma unroll
-                    for (int c0 = 0; c0 < 128; c0 += 32)
-                        if (c0 + 32 <= cw) tmem_ld32_add(tbase + (uint32_t)c0, acc + c0);
-#pragma unroll
-                    for (int c0 = 0; c0 < 128; c0 += 16) {
-                        if (c0 >= (cw & ~31) && c0 < cw) {
-                            float v[16];
-                            tmem_ld16(tbase + (uint32_t)c0, v);
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
-                        }
-                    }
-                    fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&tempty[b]);
-                }
-                if (!ok) break;
-#pragma unroll
-                for (int c0 = 0; c0 < 128; c0 += 16) {
-                    if (c0 >= cw || colt + c0 >= ep.N) continue;  // uniform across the warp
-                    if (ep.mode == 0)
-                        store_z16(maps, ep, planes, row - lane, colt + c0, acc + c0, stg, nbuf, nchunk, lane);
-                    else if (row < ep.M)
-                        store_out16(ep, row, colt + c0, acc + c0);
-                }
-            } else {
-                // one epoch per tile: stream TMEM -> global 16 columns at a time, then release the buffer
-                const int b = (int)(e & 1);
-                if (!mbar_wait(&tfull[b], (uint32_t)((e >> 1) & 1), &abort_flag, ep.err)) {
-                    ok = false;
-                    break;
-                }
-                ++e;
-                fence_after();
-                const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 256 + cbeg);
-                for (int c0 = 0; c0 < cw; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(tbase + (uint32_t)c0, v);  // warp-collective: every lane loads
-                    if (colt + c0 < ep.N) {  // uniform across the warp
-                        if (ep.mode == 0)
-                            store_z16(maps, ep, planes, row - lane, colt + c0, v, stg, nbuf, nchunk, lane);
-                        else if (row < ep.M)
-                            store_out16(ep, row, colt + c0, v);
-                    }
-                }
-                fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[b]);
-            }
-        }
-        if (ep.mode == 0) store_z_drain(lane);  // this warp's Z stores have completed
-    }
-    fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        const uint64_t t0 = gtime();
-        while (!mbar_try(&done_bar, 0) && gtime() - t0 < WAIT_NS) {
-        }
-        fence_after();
-    }
-    if (warp == 1)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
-}
-
-// ---- 2-SM variant: one MMA tile of 256 rows on a CTA pair (cta_group::2) -----
-__device__ __forceinline__ uint32_t mapa_rank(const void* p, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(su32(p)), "r"(rank));
-    return r;
-}
-// TMA load into this CTA's shared memory that completes its bytes on an
-// mbarrier of either CTA of the pair (shared::cluster address)
-__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m, uint32_t bar, int x, int y) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], "
-        "[%2];" ::"r"(su32(dst)),
-        "l"((uint64_t)m), "r"(bar), "r"(x), "r"(y)
-        : "memory");
-}
-__device__ __forceinline__ void mma_bf16_pair(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-// arrive on the mbarrier at `bar`'s offset in both CTAs once the pair's MMAs issued so far have completed
-__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            su32(bar)),
-        "h"((uint16_t)3)
-        : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_cluster(uint64_t* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(su32(b)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// bounded wait with cluster-scope acquire (for arrivals from the peer CTA)
-__device__ bool mbar_wait_cluster(uint64_t* b, uint32_t parity, volatile int* abort_flag, int* err) {
-    const uint64_t t0 = gtime();
-    for (uint32_t n = 0;; ++n) {
-        if (mbar_try_cluster(b, parity)) return true;
-        if ((n & 15u) == 15u) {
-            if (*abort_flag) return false;
-            if (gtime() - t0 > WAIT_NS) {
-                *abort_flag = 1;
-                atomicExch(err, 1);
-                return false;
-            }
-        }
-    }
-}
-
-// Persistent GEMM C = A B^T as k_gemm_bf16x3, with each tile 256 rows high and
-// computed by a CTA pair (a cluster of two) through cta_group::2 MMAs: CTA r
-// holds rows [128 r, 128 r + 128) of the A tile and rows [BN/2 r, BN/2 (r+1))
-// of the B tile, so each SM receives A + B/2 per K block instead of A + B and
-// a stage is a third smaller.  Both CTAs' TMA loads complete on the leader's
-// (rank 0) full barrier; the leader's MMA thread issues every MMA and its
-// commits arrive on the barriers of both CTAs; each CTA's epilogue drains its
-// own tensor memory (its 128 rows of the tile, all BN columns) and releases
-// the accumulator on the leader's barrier (2 x EPI_WARPS arrivals).
+// Accumulation.  The tensor core's FP32 accumulate truncates, so a long accumulation in one TMEM
+// accumulator drifts toward zero by about a quarter ulp per MMA (measured: 2e-5 relative over a
+// 4160-deep chunk).  The MMAs of a tile are therefore issued in short epochs of `ekb` K blocks,
+// alternating between two TMEM accumulators; the epilogue warps add every epoch into FP32
+// registers with round-to-nearest (unbiased) while the next epoch runs, and write the tile once
+// after its last epoch.  Epilogue warp w covers TMEM lane quarter (w % 4) and one half of the
+// tile's columns.  kPromote = false (one epoch per tile) streams each tile from TMEM to global
+// memory without the register accumulator.  (Ten warps: three share a sub-partition's 16K
+// registers, so at most 168 per thread.)
 template <bool kPromote>
 __global__ void __launch_bounds__(THREADS, 1)
     k_gemm_pair(const __grid_constant__ Maps maps, int planes, int a_row0, int b_x0, int K, int BN, int stages,
-                int m_fastest, int mt, int nt, int ekb, int nbuf, Epi ep) {
+                int m_fastest, int mt, int nt, int ekb, int nbuf, Parts parts, Epi ep) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ uint64_t full_bar[MAX_STAGES], empty_bar[MAX_STAGES], tfull[2], tempty[2], done_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int num_k = (K + BK - 1) / BK;
-    const int epochs = (num_k + ekb - 1) / ekb;  // per tile
+    const int all_k = (K + BK - 1) / BK;
     const int BH = BN / 2;                       // B rows held by each CTA
     const int BH_BYTES = BH * ROW_BYTES;
     const int STAGE = planes * (A_BYTES + BH_BYTES);  // per CTA: [A planes][B-half planes]
     const int rank = (int)cluster_rank();
     const bool leader = rank == 0;
     const int mt2 = (mt + 1) / 2;  // 256-row tiles
-    const int nunits = mt2 * nt;
+    const int per_part = mt2 * nt, nunits = per_part * parts.n;
     const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
 
     if (threadIdx.x == 0) {
@@ -664,10 +249,13 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (lane == 0) {
             long long g = 0;
             for (int u = cid; u < nunits && !abort_flag; u += ncl) {
-                const int m2 = m_fastest ? u % mt2 : u / nt;
-                const int n_tile = m_fastest ? u / mt2 : u % nt;
-                const int ya = a_row0 + m2 * 2 * BM + rank * BM, yb = n_tile * BN + rank * BH;
-                for (int kb = 0; kb < num_k; ++kb, ++g) {
+                const int z = u / per_part, t = u - z * per_part, zm = z / parts.slices;
+                const int m2 = m_fastest ? t % mt2 : t / nt;
+                const int n_tile = m_fastest ? t / mt2 : t % nt;
+                const int ya = a_row0 + zm * parts.a_step + m2 * 2 * BM + rank * BM;
+                const int yb = zm * parts.b_step + n_tile * BN + rank * BH;
+                const int kb0 = (z - zm * parts.slices) * parts.kb, kb1 = min(all_k, kb0 + parts.kb);
+                for (int kb = kb0; kb < kb1; ++kb, ++g) {
                     const int s = (int)(g % stages);
                     const uint32_t ph = (uint32_t)((g / stages) & 1);
                     if (g >= stages && !mbar_wait(&empty_bar[s], ph ^ 1, &abort_flag, ep.err)) break;
@@ -700,9 +288,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             long long e = 0;  // epochs issued (across tiles)
             bool ok = true;
             for (int u = cid; u < nunits && ok && !abort_flag; u += ncl) {
+                const int z = u / per_part, kb0 = (z % parts.slices) * parts.kb, kb1 = min(all_k, kb0 + parts.kb);
                 int left = 0;
                 uint32_t tacc = 0;
-                for (int kb = 0; kb < num_k; ++kb, ++g) {
+                for (int kb = kb0; kb < kb1; ++kb, ++g) {
                     const int s = (int)(g % stages);
                     if (!mbar_wait(&full_bar[s], (uint32_t)((g / stages) & 1), &abort_flag, ep.err)) {
                         ok = false;
@@ -723,29 +312,38 @@ __global__ void __launch_bounds__(THREADS, 1)
                     uint8_t* st = smem + (size_t)s * STAGE;
                     const uint64_t a0 = smem_desc(st), a1 = smem_desc(st + A_BYTES);
                     const uint64_t b0 = smem_desc(st + planes * A_BYTES), b1 = smem_desc(st + planes * A_BYTES + BH_BYTES);
+                    // small products first: every MMA truncates at the accumulator's size, so in short
+                    // epochs only the hi * hi ones (4 of 12 or 24 per K block) cost a full-size ulp
                     if (planes == 3) {
                         const uint64_t a2 = smem_desc(st + 2 * A_BYTES), b2 = smem_desc(st + planes * A_BYTES + 2 * BH_BYTES);
 #pragma unroll
                         for (int kk = 0; kk < BK / 16; ++kk) {
                             const uint64_t o = (uint64_t)(kk * 2);
-                            mma_bf16_pair(tacc, a0 + o, b0 + o, idesc, kk == 0 ? first : 1u);
-                            mma_bf16_pair(tacc, a0 + o, b1 + o, idesc, 1u);
-                            mma_bf16_pair(tacc, a1 + o, b0 + o, idesc, 1u);
-                            mma_bf16_pair(tacc, a0 + o, b2 + o, idesc, 1u);
+                            mma_bf16_pair(tacc, a0 + o, b2 + o, idesc, kk == 0 ? first : 1u);
                             mma_bf16_pair(tacc, a2 + o, b0 + o, idesc, 1u);
                             mma_bf16_pair(tacc, a1 + o, b1 + o, idesc, 1u);
+                        }
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            const uint64_t o = (uint64_t)(kk * 2);
+                            mma_bf16_pair(tacc, a0 + o, b1 + o, idesc, 1u);
+                            mma_bf16_pair(tacc, a1 + o, b0 + o, idesc, 1u);
                         }
                     } else {
 #pragma unroll
                         for (int kk = 0; kk < BK / 16; ++kk) {
                             const uint64_t o = (uint64_t)(kk * 2);
-                            mma_bf16_pair(tacc, a0 + o, b0 + o, idesc, kk == 0 ? first : 1u);
-                            mma_bf16_pair(tacc, a0 + o, b1 + o, idesc, 1u);
+                            mma_bf16_pair(tacc, a0 + o, b1 + o, idesc, kk == 0 ? first : 1u);
                             mma_bf16_pair(tacc, a1 + o, b0 + o, idesc, 1u);
                         }
                     }
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk) {
+                        const uint64_t o = (uint64_t)(kk * 2);
+                        mma_bf16_pair(tacc, a0 + o, b0 + o, idesc, 1u);
+                    }
                     mma_commit_pair(&empty_bar[s]);
-                    if (--left == 0 || kb == num_k - 1) {
+                    if (--left == 0 || kb == kb1 - 1) {
                         mma_commit_pair(&tfull[e & 1]);
                         ++e;
                         left = 0;
@@ -766,11 +364,14 @@ __global__ void __launch_bounds__(THREADS, 1)
         long long e = 0;
         bool ok = true;
         for (int u = cid; u < nunits && ok; u += ncl) {
-            const int m2 = m_fastest ? u % mt2 : u / nt;
-            const int n_tile = m_fastest ? u / mt2 : u % nt;
+            const int z = u / per_part, t = u - z * per_part;
+            const int m2 = m_fastest ? t % mt2 : t / nt;
+            const int n_tile = m_fastest ? t / mt2 : t % nt;
             const int row = m2 * 2 * BM + rank * BM + quarter * 32 + lane;  // rows past M are skipped
             const int colt = n_tile * BN + cbeg;
             if constexpr (kPromote) {
+                const int kb0 = (z % parts.slices) * parts.kb;
+                const int epochs = (min(all_k, kb0 + parts.kb) - kb0 + ekb - 1) / ekb;
                 float acc[128];
 #pragma unroll
                 for (int i = 0; i < 128; ++i) acc[i] = 0.0f;
@@ -810,7 +411,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (ep.mode == 0)
                         store_z16(maps, ep, planes, row - lane, colt + c0, acc + c0, stg, nbuf, nchunk, lane);
                     else if (row < ep.M)
-                        store_out16(ep, row, colt + c0, acc + c0);
+                        store_out16(ep, row, colt + c0, acc + c0, z);
                 }
             } else {
                 const int b = (int)(e & 1);
@@ -828,7 +429,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                         if (ep.mode == 0)
                             store_z16(maps, ep, planes, row - lane, colt + c0, v, stg, nbuf, nchunk, lane);
                         else if (row < ep.M)
-                            store_out16(ep, row, colt + c0, v);
+                            store_out16(ep, row, colt + c0, v, z);
                     }
                 }
                 fence_before();
@@ -909,6 +510,103 @@ __global__ void k_split_XT(const double* __restrict__ X, long long nmat, int va,
     }
 }
 
+// ---- pair-adapted ladder: operands and result ---------------------------------------
+// A v x v matrix x as its pairs c >= d, p = c (c + 1) / 2 + d: half 0 x_cd + x_dc, half 1
+// x_cd - x_dc, each split into two or three (o.p[2] not NULL) BF16 planes
+// o.p[plane][(half * rows + row) * Pk + p] (zeros for P <= p < Pk).  Matrix m of the input: element (r, s) at in[base(m) + r * rs + s].
+//   integrals (Tin float): m -> a = a0 + m / nb, b = m % nb (b <= a, others skipped), the matrix
+//     (ac|bd) over (c, d), row a (a + 1) / 2 + b of the planes; the diagonal c = d holds 2 (ac|bc)
+//   vectors (Tin double): matrix m is row m; the diagonal holds x_cc
+// Bound by HBM: every element is read once (32 x 32 tiles, the mirrored tile through shared
+// memory) and written as four or six 2-byte values.
+template <typename Tin>
+__global__ void __launch_bounds__(256) k_pair_planes(const Tin* __restrict__ in, int v, long long nmat, long long ms,
+                                                     long long rs, int integrals, int a0, int nb, long long rows,
+                                                     long long P, long long Pk, Planes o) {
+    __shared__ Tin t1[32][33], t2[32][33];
+    const int nt = (v + 31) / 32;
+    const long long ntri = (long long)nt * (nt + 1) / 2;
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    for (long long u = blockIdx.x; u < nmat * ntri; u += gridDim.x) {
+        const long long m = u / ntri;
+        int r = (int)(u - m * ntri), ct = (int)((sqrtf(8.0f * r + 1.0f) - 1.0f) * 0.5f);
+        while ((ct + 1) * (ct + 2) / 2 <= r) ++ct;
+        while (ct * (ct + 1) / 2 > r) --ct;
+        const int dt = r - ct * (ct + 1) / 2, c0 = ct * 32, d0 = dt * 32;
+        long long row = m, base = m * ms;
+        if (integrals) {
+            const long long a = m / nb, b = m - a * nb;
+            if (b > a0 + a) continue;  // uniform over the block
+            row = (a0 + a) * (a0 + a + 1) / 2 + b;
+            base = a * v * rs + b * v;
+        }
+        for (int i = ty; i < 32; i += 8) {
+            const int cc = c0 + i, dd = d0 + tx;
+            t1[i][tx] = cc < v && dd < v ? in[base + (long long)cc * rs + dd] : (Tin)0;
+            const int c2 = d0 + i, d2 = c0 + tx;  // the mirrored tile: rows d, columns c
+            t2[i][tx] = c2 < v && d2 < v ? in[base + (long long)c2 * rs + d2] : (Tin)0;
+        }
+        __syncthreads();
+        for (int i = ty; i < 32; i += 8) {
+            const int cc = c0 + i, dd = d0 + tx;
+            if (cc < v && dd <= cc) {
+                const double x = (double)t1[i][tx], y = (double)t2[tx][i];
+                const double ps = dd == cc && !integrals ? x : x + y, pa = x - y;
+                const long long p = (long long)cc * (cc + 1) / 2 + dd, o0 = row * Pk + p, o1 = (rows + row) * Pk + p;
+                const int planes = o.p[2] ? 3 : 2;
+                splitp(ps, planes, o.p[0] + o0, o.p[1] + o0, o.p[2] + o0);
+                splitp(pa, planes, o.p[0] + o1, o.p[1] + o1, o.p[2] + o1);
+            }
+        }
+        if (ct == nt - 1 && dt == nt - 1 && ty == 0 && tx < Pk - P) {
+            for (int p = 0; p < 3; ++p)
+                if (o.p[p]) o.p[p][row * Pk + P + tx] = o.p[p][(rows + row) * Pk + P + tx] = __float2bfloat16(0.0f);
+        }
+        __syncthreads();
+    }
+}
+
+// out[m][a][b] += (S + A) / 2 and out[m][b][a] += (S - A) / 2 for the pairs a >= b, with S and A
+// the FP64 sums over the K slices of T[half][slice][p][m] (p = a (a + 1) / 2 + b, halves 0 and 1).
+// 16 x 16 pair tiles x 8 matrices through shared memory: T is read in whole sectors along m, out
+// updated along its rows in both orientations.
+__global__ void __launch_bounds__(256) k_pair_unfold(const float* __restrict__ T, int slices, long long P, int nm, int v,
+                                                     double* __restrict__ out) {
+    __shared__ double u[8][16][17], w[8][16][17];
+    const int nt = (v + 15) / 16, nmt = (nm + 7) / 8;
+    const long long ntri = (long long)nt * (nt + 1) / 2, part = P * nm;
+    for (long long blk = blockIdx.x; blk < ntri * nmt; blk += gridDim.x) {
+        const int r = (int)(blk / nmt), m0 = (int)(blk % nmt) * 8;
+        int at = (int)((sqrtf(8.0f * r + 1.0f) - 1.0f) * 0.5f);
+        while ((at + 1) * (at + 2) / 2 <= r) ++at;
+        while (at * (at + 1) / 2 > r) --at;
+        const int bt = r - at * (at + 1) / 2, a0 = at * 16, b0 = bt * 16;
+        const int mi = threadIdx.x & 7, m = m0 + mi;
+        for (int e = threadIdx.x >> 3; e < 256; e += 32) {
+            const int a = a0 + e / 16, b = b0 + e % 16;
+            if (a < v && b <= a && m < nm) {
+                const float* t = T + ((long long)a * (a + 1) / 2 + b) * nm + m;
+                double S = 0.0, A = 0.0;
+                for (int k = 0; k < slices; ++k) {
+                    S += (double)t[k * part];
+                    A += (double)t[(slices + k) * part];
+                }
+                u[mi][e / 16][e % 16] = 0.5 * (S + A);
+                w[mi][e / 16][e % 16] = 0.5 * (S - A);
+            }
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < 8 * 256; e += 256) {
+            const int k = e / 256, i = (e / 16) % 16, j = e % 16, mm = m0 + k;
+            if (mm >= nm) continue;
+            if (a0 + i < v && b0 + j <= a0 + i) out[((long long)mm * v + a0 + i) * v + b0 + j] += u[k][i][j];
+            // the mirrored tile: rows b, columns a > b
+            if (b0 + i < v && a0 + j < v && b0 + i < a0 + j) out[((long long)mm * v + b0 + i) * v + a0 + j] += w[k][j][i];
+        }
+        __syncthreads();
+    }
+}
+
 inline int grid_for(long long n) { return (int)std::min<long long>(std::max<long long>((n + 255) / 256, 1), 152LL * 32); }
 
 // ---- host: tensor maps ------------------------------------------------------
@@ -969,23 +667,6 @@ CUtensorMap make_map_z(const void* base, int vp, int qn, int v, long long nm) {
     return m;
 }
 
-// 2-D BF16 tensor [rows][cols] with a row stride of `ld` elements (a column
-// slice of a wider matrix); box {BK, box_rows}, ROW_BYTES swizzle
-CUtensorMap make_map_ld(const void* base, long long rows, long long cols, long long ld, int box_rows) {
-    if (((uintptr_t)base & 15) || (ld * 2) % 16) throw Error(-1, "tensor map: misaligned operand slice");
-    CUtensorMap m;
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
-    cuuint32_t es[2] = {1, 1};
-    CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
-                             CU_TENSOR_MAP_INTERLEAVE_NONE,
-                             ROW_BYTES == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) throw Error(-3, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
-    return m;
-}
-
 int pick_bn(int n, int maxbn) {
     int best = maxbn;
     double best_cost = 1e300;
@@ -1017,8 +698,6 @@ const DevInfo& dev_info() {
         auto chk = [&d](cudaError_t e) {
             if (e != cudaSuccess && d.st == cudaSuccess) d.st = e;
         };
-        chk(cudaFuncSetAttribute(k_gemm_bf16x3<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-        chk(cudaFuncSetAttribute(k_gemm_bf16x3<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
         chk(cudaFuncSetAttribute(k_gemm_pair<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
         chk(cudaFuncSetAttribute(k_gemm_pair<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
         chk(cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1040,19 +719,19 @@ const DevInfo& dev_info() {
     return d;
 }
 
-// ekb: accumulation epoch in 64-deep K blocks (0 = one epoch per tile);
-// pair: 256-row tiles on CTA pairs (k_gemm_pair), else 128-row tiles per CTA
+// ekb: accumulation epoch in 64-deep K blocks (0 = one epoch per tile); ladder: the launch counts
+// as one of the DF ladder's in the live timing
 void launch_gemm(Ctx& c, const Maps& maps, int planes, int a_row0, int b_x0, int M, int N, int K, int BN, int m_fastest,
-                 int ekb, bool pair, const Epi& ep, double algo_flops, cudaStream_t stream_override = nullptr) {
-    const cudaStream_t st = stream_override ? stream_override : c.stream;
+                 int ekb, const Epi& ep, double algo_flops, const Parts& parts = Parts(), bool ladder = false) {
+    const cudaStream_t st = c.stream;
     if (BN % 16 || BN < 16 || BN > 256) throw Error(-1, "ladder: tile width must be a multiple of 16 in [16, 256]");
     const DevInfo& di = dev_info();
-    const int num_sms = di.num_sms, max_pairs = di.max_pairs;
+    const int max_pairs = di.max_pairs;
     const int mt = (M + BM - 1) / BM, nt = (N + BN - 1) / BN;
     const long long ntiles = (long long)mt * nt;
     if (ntiles <= 0) return;
     if (ntiles > (1LL << 31) - 1) throw Error(-1, "ladder: tile count too large");
-    const int stage_bytes = planes * (A_BYTES + (pair ? BN / 2 : BN) * ROW_BYTES);
+    const int stage_bytes = planes * (A_BYTES + BN / 2 * ROW_BYTES);
     // mode 0: per-warp Z staging of planes x 1 KB, double-buffered when two pipeline stages still fit
     const int stg = ep.mode == 0 ? EPI_WARPS * planes * 1024 : 0;
     int nbuf = ep.mode == 0 ? 2 : 0;
@@ -1073,13 +752,9 @@ void launch_gemm(Ctx& c, const Maps& maps, int planes, int a_row0, int b_x0, int
     cfg.stream = st;
     cfg.attrs = cl;
     cfg.numAttrs = 1;
-    int grid;
-    if (!pair) {
-        grid = (int)std::min<long long>(ntiles, num_sms);
-    } else {
-        const long long units = (long long)((mt + 1) / 2) * nt;  // 256-row tiles
-        grid = (int)std::min<long long>(units, max_pairs) * 2;
-    }
+    const long long units = (long long)((mt + 1) / 2) * nt * parts.n;  // 256-row tiles of every part
+    if (units > (1LL << 31) - 1) throw Error(-1, "ladder: tile count too large");
+    const int grid = (int)std::min<long long>(units, max_pairs) * 2;
     cfg.gridDim = dim3((unsigned)grid);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (c.timing) {
@@ -1088,25 +763,21 @@ void launch_gemm(Ctx& c, const Maps& maps, int planes, int a_row0, int b_x0, int
         ADC_CUDA(cudaEventRecord(e0, st));
     }
     // epoch length in the kernel's K blocks (MMAs per epoch = ekb * BK/16 * (3 or 6 products))
-    ekb = ekb <= 0 ? (K + BK - 1) / BK : ekb * KB_PER_EPOCH_UNIT;
+    const int tile_kb = std::min((K + BK - 1) / BK, parts.kb);  // K blocks of a tile
+    ekb = ekb <= 0 ? tile_kb : ekb * KB_PER_EPOCH_UNIT;
     // one accumulation epoch per tile: the streaming epilogue without register accumulation
-    const bool promote = ekb < (K + BK - 1) / BK;
-    if (pair) {
-        auto kp = promote ? k_gemm_pair<true> : k_gemm_pair<false>;
-        ADC_CUDA(cudaLaunchKernelEx(&cfg, kp, maps, planes, a_row0, b_x0, K, BN, stages, m_fastest, mt, nt, ekb, nbuf, ep));
-    } else {
-        auto kern = promote ? k_gemm_bf16x3<true> : k_gemm_bf16x3<false>;
-        kern<<<grid, THREADS, SMEM_BYTES, st>>>(maps, planes, a_row0, b_x0, K, BN, stages, m_fastest, mt, nt, ekb, nbuf,
-                                                      ep);
-    }
+    const bool promote = ekb < tile_kb;
+    auto kp = promote ? k_gemm_pair<true> : k_gemm_pair<false>;
+    ADC_CUDA(cudaLaunchKernelEx(&cfg, kp, maps, planes, a_row0, b_x0, K, BN, stages, m_fastest, mt, nt, ekb, nbuf, parts, ep));
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
     if (c.timing) {
         ADC_CUDA(cudaEventRecord(e1, st));
         c.ev_start.push_back(e0);
         c.ev_stop.push_back(e1);
-        const double mma = (planes == 3 ? 6.0 : 3.0) * 2.0 * (double)mt * BM * (double)nt * BN * (double)(((K + BK - 1) / BK) * BK);
-        c.ev_ladder.push_back(ep.mode != 2);  // the DF ladder's two GEMMs (mode 2: other contractions)
+        const double mma = (planes == 3 ? 6.0 : 3.0) * 2.0 * (double)mt * BM * (double)nt * BN *
+                           (double)(((K + BK - 1) / BK) * BK) * (parts.n / parts.slices);
+        c.ev_ladder.push_back(ladder);
         c.ev_algo.push_back(algo_flops);
         c.ev_mma.push_back(mma);
         for (double x : {(double)M, (double)N, (double)K, (double)BN}) c.ev_shape.push_back(x);
@@ -1117,16 +788,24 @@ void launch_gemm(Ctx& c, const Maps& maps, int planes, int a_row0, int b_x0, int
 
 }  // namespace
 
+static void ladder_pairs_forget(LadderTC* L);
+
 struct LadderTC {
     int naux = 0, v = 0, vp = 0, chunk = 0;
-    bool pair1 = true, pair2 = true;    // 2-SM tiles (cta_group::2 on CTA pairs) for GEMM1 / GEMM2
     int bn2[4] = {256, 256, 256, 256};  // GEMM2 tile width by plane count (2 or 3)
     const double* Bvv = nullptr;        // FP64 source (owned by the caller, outlives this object)
     int nplanes = 0;                    // BF16 planes held (2; 3 once a three-plane ladder was asked for)
     __nv_bfloat16 *Bs[3] = {}, *Bp[3] = {};  // BF16 planes of B^Q in the GEMM1-A and GEMM2-B layouts
     CUtensorMap mBs[3];                       // GEMM1-A maps
     int* d_err = nullptr;
+    // pair-adapted integrals (ladder_pairs_prepare): planes [2 halves][P][Pk], NULL when not held
+    __nv_bfloat16* pairs[3] = {};  // (the third plane has an allocation of its own, held during setup)
+    long long P = 0, Pk = 0;
+    int device = 0, pins = 0;  // pins: calls in progress that may read the pairs (g_pairs_mu)
     ~LadderTC() {
+        ladder_pairs_forget(this);
+        cudaFree(pairs[0]);
+        cudaFree(pairs[2]);
         for (int p = 0; p < 3; ++p) {
             cudaFree(Bs[p]);
             cudaFree(Bp[p]);
@@ -1196,7 +875,7 @@ void run_ladder(LadderTC& Ll, LadderTC& Lr, Ctx& c, const double* X, long long n
     const int va = Ll.v, vpa = Ll.vp, vb = Lr.v, vpb = Lr.vp, naux = Ll.naux, planes = md.planes;
     const int bn1 = BN1[planes];
     CUtensorMap mBp[3];  // GEMM2-B maps: one CTA's half of the tile in pair mode
-    for (int p = 0; p < planes; ++p) mBp[p] = make_map(Lr.Bp[p], vb, (long long)naux * vpb, Lr.pair2 ? bn2 / 2 : bn2);
+    for (int p = 0; p < planes; ++p) mBp[p] = make_map(Lr.Bp[p], vb, (long long)naux * vpb, bn2 / 2);
     for (long long m0 = 0; m0 < nmat; m0 += mg) {
         const long long nm = std::min(mg, nmat - m0);
         k_split_XT<<<grid_for(nm * vpb * vpa), 256, 0, c.stream>>>(X + m0 * va * vb, nm, va, vb, vpa, vpb, planes, xt);
@@ -1205,7 +884,7 @@ void run_ladder(LadderTC& Ll, LadderTC& Lr, Ctx& c, const double* X, long long n
         Maps m1;
         for (int p = 0; p < planes; ++p) {
             m1.a[p] = Ll.mBs[p];
-            m1.b[p] = make_map(xt.p[p], nm * vpb, vpa, Ll.pair1 ? bn1 / 2 : bn1);
+            m1.b[p] = make_map(xt.p[p], nm * vpb, vpa, bn1 / 2);
         }
         for (int q0 = 0; q0 < naux; q0 += qc) {
             const int qn = std::min(qc, naux - q0);
@@ -1218,8 +897,8 @@ void run_ladder(LadderTC& Ll, LadderTC& Lr, Ctx& c, const double* X, long long n
             e1.vp = vpb;
             e1.err = Ll.d_err;
             for (int p = 0; p < planes; ++p) m1.z[p] = make_map_z(zt.p[p], vpb, qn, va, nm);
-            launch_gemm(c, m1, planes, q0 * vpa, 0, e1.M, e1.N, vpa, bn1, 1, md.epoch1, Ll.pair1, e1,
-                        2.0 * (double)qn * va * (double)nm * vb * va);  // unpadded products
+            launch_gemm(c, m1, planes, q0 * vpa, 0, e1.M, e1.N, vpa, bn1, 1, md.epoch1, e1,
+                        2.0 * (double)qn * va * (double)nm * vb * va, Parts(), true);  // unpadded products
             // GEMM2: out[(n,a),b] += sum_(q,d) Z_n[a,(q,d)] B_r^q[d,b]
             Maps m2;
             for (int p = 0; p < planes; ++p) {
@@ -1234,8 +913,8 @@ void run_ladder(LadderTC& Ll, LadderTC& Lr, Ctx& c, const double* X, long long n
             e2.ldc = vb;
             e2.vec = ((uintptr_t)e2.out % 16 == 0) && (vb % 2 == 0);
             e2.err = Ll.d_err;
-            launch_gemm(c, m2, planes, 0, q0 * vpb, e2.M, e2.N, qn * vpb, bn2, 0, md.epoch2, Lr.pair2, e2,
-                        2.0 * (double)nm * va * (double)vb * qn * vb);
+            launch_gemm(c, m2, planes, 0, q0 * vpb, e2.M, e2.N, qn * vpb, bn2, 0, md.epoch2, e2,
+                        2.0 * (double)nm * va * (double)vb * qn * vb, Parts(), true);
         }
     }
 }
@@ -1334,8 +1013,276 @@ TuneCache* tune_cache_open(const char* path) {
     return slot.get();
 }
 
+// ---- the ladder over pair-adapted integrals ----------------------------------------
+// With x+-_cd = x_cd +- x_dc, the symmetric and antisymmetric parts of the ladder are
+//   out_ab +- out_ba = sum_{c>=d} V+-_{ab,cd} x+-_cd,  V+-_{ab,cd} = (ac|bd) +- (ad|bc)
+// (diagonal weights in k_pair_planes): nmat v^4 flops for nmat matrices instead of the
+// 4 naux v^3 nmat of the two-GEMM form over the auxiliary index, i.e. 4 naux / v times fewer (13
+// at 180 virtuals and 600 auxiliary functions, 14 at 400 / 1400).  The integrals cost naux v^4
+// flops once per handle and 4 v^4 bytes (two BF16 planes of both halves: 4.2 GB at v = 180, 51 GB
+// at 400), so they are held where that fits the device and the two-GEMM form stays for the rest.
+// Measured, a sigma of 4 vectors at 20/180/600: 7.9 -> 4.0 ms; at 40/400/1400: 159 -> 36 ms.
+//
+// The integrals are a convenience and go back to the device when an allocation of any handle
+// fails (device_memory_reclaim): those of handles with no call in progress (pins == 0), and those
+// of the call that fails itself, outside a ladder and outside a solve that replays CUDA graphs.
+namespace {
+std::mutex g_pairs_mu;
+std::vector<LadderTC*> g_pairs;  // holders of pair integrals
+// the handle whose call runs on this host thread, if that call may give its own integrals up
+thread_local LadderTC* tl_own = nullptr;
+thread_local cudaStream_t tl_own_stream = nullptr;
+
+constexpr long long kPairSliceK = 16384;  // FP32 register sums of at most this many terms, FP64 beyond
+}  // namespace
+
+static void ladder_pairs_forget(LadderTC* L) {
+    std::lock_guard<std::mutex> lk(g_pairs_mu);
+    g_pairs.erase(std::remove(g_pairs.begin(), g_pairs.end(), L), g_pairs.end());
+}
+
+PairsPin::PairsPin(LadderTC* l, Ctx& c, bool own) : L(l) {
+    if (!L) return;
+    std::lock_guard<std::mutex> lk(g_pairs_mu);
+    ++L->pins;
+    before = tl_own;
+    tl_own = own ? L : nullptr;
+    tl_own_stream = c.stream;
+}
+PairsPin::~PairsPin() {
+    if (!L) return;
+    std::lock_guard<std::mutex> lk(g_pairs_mu);
+    --L->pins;
+    tl_own = (LadderTC*)before;
+}
+
+void ladder_pairs_drop(LadderTC& L, Ctx& c) {
+    if (!L.pairs[0]) return;
+    ladder_pairs_forget(&L);
+    cudaFreeAsync(L.pairs[0], c.stream);
+    L.pairs[0] = L.pairs[1] = nullptr;
+    ladder_pairs_drop_third(L, c);
+}
+
+void ladder_pairs_drop_third(LadderTC& L, Ctx& c) {
+    if (L.pairs[2]) cudaFreeAsync(L.pairs[2], c.stream);
+    L.pairs[2] = nullptr;
+}
+
+bool device_memory_reclaim() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lk(g_pairs_mu);
+    bool any = false;
+    for (size_t i = 0; i < g_pairs.size();) {
+        LadderTC* L = g_pairs[i];
+        const bool own = L == tl_own && L->pins == 1;
+        if (L->device != dev || (L->pins > 0 && !own)) {
+            ++i;
+            continue;
+        }
+        // a handle with no call in progress has no work in flight (every call returns after its
+        // work has completed); this thread's own call waits for what it has issued so far
+        if (own && cudaStreamSynchronize(tl_own_stream) != cudaSuccess) return any;
+        cudaFree(L->pairs[0]);
+        cudaFree(L->pairs[2]);
+        L->pairs[0] = L->pairs[1] = L->pairs[2] = nullptr;
+        g_pairs.erase(g_pairs.begin() + i);
+        any = true;
+    }
+    return any;
+}
+
+size_t ladder_pairs_bytes(int v) {
+    const size_t P = (size_t)v * (v + 1) / 2, Pk = (P + 7) / 8 * 8;
+    return 2 * P * Pk * 2 * sizeof(__nv_bfloat16);
+}
+
+bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv) {
+    const long long v = L.v, Q = L.naux, Qp = (Q + 7) / 8 * 8, P = v * (v + 1) / 2, Pk = (P + 7) / 8 * 8;
+    if (2 * P >= (1LL << 30) || v * v >= (1LL << 30)) return false;  // 32-bit tile coordinates
+    void* base = nullptr;
+    if (cudaMallocAsync(&base, ladder_pairs_bytes((int)v), c.stream) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    void* third = nullptr;
+    if (cudaMallocAsync(&third, ladder_pairs_bytes((int)v) / 2, c.stream) != cudaSuccess) {
+        cudaGetLastError();
+        third = nullptr;
+    }
+    L.P = P;
+    L.Pk = Pk;
+    L.pairs[2] = (__nv_bfloat16*)third;
+    L.pairs[0] = (__nv_bfloat16*)base;
+    L.pairs[1] = L.pairs[0] + 2 * P * Pk;
+    ADC_CUDA(cudaGetDevice(&L.device));
+    {
+        std::lock_guard<std::mutex> lk(g_pairs_mu);
+        g_pairs.push_back(&L);
+    }
+    PairsPin pin(&L, c, false);  // its own allocations may not take them away again
+    Arena::Mark mk = c.arena.mark();
+    // K-major planes of B^Q as [(p, q)][Q]: both operands of (ac|bd) = sum_Q B^Q_ac B^Q_bd
+    // in three planes (the six products of order <= 2): with two, the dropped lo * lo products of the
+    // coherent integrals, sum_Q (B^Q_ac)^2, are a sum of squares -- a bias of -1.4e-6 of t2(2), against
+    // -8e-8 of the two-GEMM form, which this form then keeps
+    __nv_bfloat16* bt = (__nv_bfloat16*)c.arena.alloc(3 * v * v * Qp * 2);
+    void* planes[3] = {bt, bt + v * v * Qp, bt + 2 * v * v * Qp};
+    const int perm[2] = {1, 0};
+    split_planes(c, Bvv, Shape{2, {Q, v * v}}, perm, v * v, Q, Qp, planes, false, 3);
+    // rows (a, c) of a block of a's against the columns (b, d), b <= the block's last a: FP32 of at
+    // most 1 GB, then packed into pairs
+    for (long long a0 = 0; a0 < v;) {
+        long long na = 1;
+        while (a0 + na < v && (na + 1) * v * (a0 + na + 1) * v * 4 <= (1LL << 30)) ++na;
+        const long long nb = a0 + na;
+        Arena::Mark m2 = c.arena.mark();
+        float* G = (float*)c.arena.alloc((size_t)(na * v * nb * v) * sizeof(float));
+        Maps m{};
+        for (int p = 0; p < 3; ++p) {
+            m.a[p] = make_map(planes[p], v * v, Qp, BM);
+            m.b[p] = make_map(planes[p], nb * v, Qp, BN1[3] / 2);
+        }
+        Epi e{};
+        e.mode = 2;
+        e.M = (int)(na * v);
+        e.N = (int)(nb * v);
+        e.ldc = nb * v;
+        e.err = c.d_err;
+        e.out32 = G;
+        e.vec = (nb * v) % 4 == 0;
+        // partial sums promoted every K block: the integrals enter the setup ladder too
+        launch_gemm(c, m, 3, (int)(a0 * v), 0, e.M, e.N, (int)Qp, BN1[3], 1, 1, e, 2.0 * na * v * nb * v * Q);
+        const long long nt = (v + 31) / 32, tiles = na * nb * nt * (nt + 1) / 2;
+        k_pair_planes<float><<<(unsigned)std::min<long long>(tiles, 152LL * 16), dim3(32, 8), 0, c.stream>>>(
+            G, (int)v, na * nb, 0, nb * v, 1, (int)a0, (int)nb, P, P, Pk, Planes{{L.pairs[0], L.pairs[1], L.pairs[2]}});
+        ++c.kernels;
+        ADC_CUDA(cudaGetLastError());
+        c.arena.release(m2);
+        a0 += na;
+    }
+    c.arena.release(mk);
+    return true;
+}
+
+bool ladder_pairs_third(const LadderTC* L) { return L && L->pairs[2]; }
+
+namespace {
+
+// S+A products of one group of nm matrices (split vectors x, [2][nm][Pk] planes) at tile width bn:
+// FP32 results [2][S][P][nm] in c.arena.  The integrals are streamed once and both halves are
+// matrices of one launch, cut into S slices along K so that the rounds of tiles over the CTA pairs
+// are nearly full and no FP32 sum runs over more than kPairSliceK terms.
+float* pairs_gemm(LadderTC& L, Ctx& c, const Planes& x, int planes, long long nm, int bn, int ekb, int& S) {
+    const long long P = L.P, Pk = L.Pk;
+    const int nkb = (int)((Pk + BK - 1) / BK), smin = (int)((Pk + kPairSliceK - 1) / kPairSliceK);
+    const int pairs = dev_info().max_pairs;
+    const long long per = ((P + 255) / 256) * ((nm + bn - 1) / bn) * 2;
+    double best = 1e300;
+    S = smin;
+    for (int t = smin; t <= smin + 31 && t <= nkb; ++t) {
+        const int kb = (nkb + t - 1) / t;
+        if ((nkb + kb - 1) / kb != t) continue;  // the last slice would be empty
+        // rounds x (K blocks + pipeline fill and epilogue), and a slice's result written and read
+        const double cost = (double)((per * t + pairs - 1) / pairs) * (kb + 4) + 0.002 * per * t / pairs * bn;
+        if (cost < best * 0.999) best = cost, S = t;
+    }
+    const int kb = (nkb + S - 1) / S;
+    S = (nkb + kb - 1) / kb;
+    float* T = (float*)c.arena.alloc((size_t)(2 * S * P * nm) * sizeof(float));
+    Maps m{};
+    for (int p = 0; p < planes; ++p) {
+        m.a[p] = make_map(L.pairs[p], 2 * P, Pk, BM);
+        m.b[p] = make_map(x.p[p], 2 * nm, Pk, bn / 2);
+    }
+    Epi e{};
+    e.mode = 2;
+    e.M = (int)P;
+    e.N = (int)nm;
+    e.ldc = nm;
+    e.err = c.d_err;
+    e.out32 = T;
+    e.zout = P * nm;
+    e.vec = nm % 4 == 0;
+    Parts parts;
+    parts.n = 2 * S;
+    parts.slices = S;
+    parts.kb = kb;
+    parts.a_step = (int)P;
+    parts.b_step = (int)nm;
+    launch_gemm(c, m, planes, 0, 0, (int)P, (int)nm, (int)Pk, bn, 0, ekb, e, 4.0 * (double)P * nm * P, parts, true);
+    return T;
+}
+
+void pairs_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* out, const LadderMode& md) {
+    const long long v = L.v, P = L.P, Pk = L.Pk;
+    const int planes = md.planes, maxbn = planes == 3 ? BN1[3] : 256;
+    // groups of matrices whose split vectors (8 or 12 P bytes each) and FP32 results stay within ~4 GiB
+    const long long smin = (Pk + kPairSliceK - 1) / kPairSliceK;
+    const long long mg = std::max<long long>(1, std::min<long long>(nmat, (4LL << 30) / (4 * planes * Pk + 8 * P * (smin + 2))));
+    PairsPin pin(&L, c, false);  // its own allocations may not take the integrals away
+    for (long long m0 = 0; m0 < nmat; m0 += mg) {
+        const long long nm = std::min(mg, nmat - m0);
+        Arena::Mark mk = c.arena.mark();
+        Planes x{};
+        x.p[0] = (__nv_bfloat16*)c.arena.alloc(planes * 2 * nm * Pk * 2);
+        for (int p = 1; p < planes; ++p) x.p[p] = x.p[p - 1] + 2 * nm * Pk;
+        const long long nt = (v + 31) / 32, tiles = nm * nt * (nt + 1) / 2;
+        k_pair_planes<double><<<(unsigned)std::min<long long>(tiles, 152LL * 16), dim3(32, 8), 0, c.stream>>>(
+            X + m0 * v * v, (int)v, nm, v * v, v, 0, 0, 1, nm, P, Pk, x);
+        ++c.kernels;
+        ADC_CUDA(cudaGetLastError());
+        int bn = pick_bn((int)nm, maxbn), S = 1;
+        if (c.tuner && !c.timing && !c.capturing && md.epoch1 == 0) {
+            // tile width of the sigma ladder, measured once per shape (setup and refinement are one-off)
+            TuneCache* tc = (TuneCache*)c.tuner;
+            const std::string key = "ladder:sm" + std::to_string(dev_info().num_sms) + ":pairs:v" + std::to_string(v) +
+                                    ":n" + std::to_string(nm) + ":e" + std::to_string(md.epoch2);
+            std::vector<int> got;
+            if (tune_get(tc, key, got) && got.size() == 1) {
+                bn = got[0];
+            } else {
+                float least = 1e30f;
+                int bb = bn;
+                for (int b : bn_candidates((int)nm, maxbn, {256, 128, 64})) {
+                    Arena::Mark m2 = c.arena.mark();
+                    const float ms = time_on_stream(c, [&] { pairs_gemm(L, c, x, planes, nm, b, md.epoch2, S); });
+                    c.arena.release(m2);
+                    if (ms < least) least = ms, bb = b;
+                }
+                bn = bb;
+                tune_put(tc, key, {bn});
+            }
+        }
+        const float* T = pairs_gemm(L, c, x, planes, nm, bn, md.epoch2, S);
+        const long long ut = (v + 15) / 16, blocks = ut * (ut + 1) / 2 * ((nm + 7) / 8);
+        k_pair_unfold<<<(unsigned)std::min<long long>(blocks, 152LL * 32), 256, 0, c.stream>>>(T, S, P, (int)nm, (int)v,
+                                                                                           out + m0 * v * v);
+        ++c.kernels;
+        ADC_CUDA(cudaGetLastError());
+        c.arena.release(mk);
+    }
+}
+
+}  // namespace
+
 void ladder_tc_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* out, const LadderMode& md) {
-    ladder_tc_apply_pair(L, L, c, X, nmat, out, md);
+    if (nmat <= 0) return;
+    // Few matrices: the pair form streams 4 v^4 bytes whatever their number (6.5 TB/s), the
+    // two-GEMM form computes 4 naux v^3 flops for each (about 420 TF/s), which is faster below
+    // nmat = 65 v / naux (about 19 at naux = 3.5 v) -- unless the integrals stay in L2.
+    // Precision: a pair integral rounded to two planes (2^-18 relative at most) is not averaged over
+    // the auxiliary index as the two-GEMM form's factors are, so with two planes the pair form is
+    // sigma's only (its error there is no larger: 5.2e-7 against 6.0e-7 at 20/180/600); the setup
+    // ladder takes three (md.planes == 3) and the refinement the two-GEMM form.
+    const double v = L.v;
+    const bool accurate = md.planes == 3 && L.pairs[2];
+    const bool pairs = L.pairs[0] && (accurate || (md.planes == 2 && md.epoch1 == 0)) && (accurate || nmat * (double)L.naux >= 65.0 * v || 4.0 * v * v * v * v < 9e7);
+    if (pairs)
+        pairs_apply(L, c, X, nmat, out, md);
+    else
+        ladder_tc_apply_pair(L, L, c, X, nmat, out, md);
 }
 
 void ladder_tc_check(LadderTC& L, Ctx& c) {
@@ -1455,16 +1402,68 @@ bool tc_gemm_fits(long long M, long long N, long long K) {
     return M < (1LL << 30) && N < (1LL << 30) && K < (1LL << 30) && K >= 64;
 }
 
-static void tc_gemm_bn(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp,
-                       double algo_flops, double* C, int BN);
+namespace {
 
-void tc_gemm(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp, double algo_flops,
-             double* C) {
+// K slices of an M x N x K contraction at tile width bn.  A tile's time counts its K blocks plus
+// about 4 more (pipeline fill, epilogue), a launch takes as many rounds of tiles over the CTA
+// pairs as its tiles need, and every slice beyond the first writes and reads back an FP32 result
+// (8 bytes per element; a 64-deep K block of a 256-row tile takes about 0.8 us).  The slices are
+// parts of one launch: at 20/180/600 (IP, 5 vectors) the launches on side streams that this
+// replaced took 1.1 of the 2.7 ms of a sigma in launch and event calls alone.
+int pick_slices(long long M, long long N, long long Kp, int bn, int pairs) {
+    const long long tiles = ((M + 255) / 256) * ((N + bn - 1) / bn), nkb = (Kp + BK - 1) / BK;
+    const double kb_us = 0.8 * std::max(bn / 2.0, 32.0 + bn / 4.0) / 128.0;
+    int best = 1;
+    double best_cost = 1e300;
+    for (int S = 1; S <= 32 && S <= nkb; ++S) {
+        const long long kb = (nkb + S - 1) / S;
+        if ((nkb + kb - 1) / kb != S) continue;  // the last slice would be empty
+        const double rounds = (double)((tiles * S + pairs - 1) / pairs);
+        const double cost = rounds * (kb + 4) * kb_us + (S - 1) * (double)M * N * 8.0 / 4e6;
+        if (cost < best_cost * 0.999) {
+            best_cost = cost;
+            best = S;
+        }
+    }
+    return best;
+}
+
+float* tc_gemm_bn(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp,
+                  double algo_flops, int BN, int& S) {
+    S = pick_slices(M, N, Kp, BN, dev_info().max_pairs);
+    const long long nkb = (Kp + BK - 1) / BK, kb = (nkb + S - 1) / S;
+    float* T = (float*)c.arena.alloc((size_t)S * M * N * sizeof(float));
+    Epi e{};
+    e.mode = 2;
+    e.M = (int)M;
+    e.N = (int)N;
+    e.ldc = N;
+    e.err = c.d_err;
+    e.out32 = T;
+    e.zout = M * N;
+    e.vec = N % 4 == 0;  // (arena blocks are 256-byte aligned)
+    const int m_fastest = M <= N ? 1 : 0;  // consecutive tiles share the B tile when A is the smaller operand
+    Maps m{};
+    for (int p = 0; p < 2; ++p) {
+        m.a[p] = make_map(A[p], M, Kp, BM);
+        m.b[p] = make_map(B[p], N, Kp, BN / 2);
+    }
+    Parts parts;
+    parts.n = parts.slices = S;
+    parts.kb = (int)kb;
+    launch_gemm(c, m, 2, 0, 0, (int)M, (int)N, (int)Kp, BN, m_fastest, 16, e, algo_flops, parts);
+    return T;
+}
+
+}  // namespace
+
+float* tc_gemm(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp, double algo_flops,
+               int& S) {
     if (!c.d_err) throw Error(-1, "tc_gemm: no device error flag");
     const int n = (int)std::min<long long>(N, 1 << 20);
     int BN = pick_bn(n, 256);
     if (c.tuner && !c.timing && !c.capturing) {
-        // tile width measured once per shape (every run overwrites C, so the runs are interchangeable)
+        // tile width measured once per shape
         TuneCache* tc = (TuneCache*)c.tuner;
         const std::string key = "gemm:sm" + std::to_string(dev_info().num_sms) + ":M" + std::to_string(M) + ":N" +
                                 std::to_string(N) + ":K" + std::to_string(Kp);
@@ -1473,68 +1472,18 @@ void tc_gemm(Ctx& c, const void* const* A, const void* const* B, long long M, lo
             BN = got[0];
         } else {
             float best = 1e30f;
-            int bb = BN, last = BN;
+            int bb = BN;
             for (int b : bn_candidates(n, 256, {256, 128})) {
-                const float ms = time_on_stream(c, [&] { tc_gemm_bn(c, A, B, M, N, Kp, algo_flops, C, b); });
-                last = b;
+                Arena::Mark mk = c.arena.mark();
+                const float ms = time_on_stream(c, [&] { tc_gemm_bn(c, A, B, M, N, Kp, algo_flops, b, S); });
+                c.arena.release(mk);
                 if (ms < best) best = ms, bb = b;
             }
             tune_put(tc, key, {bb});
-            if (bb == last) return;  // C already holds the result of the chosen tile width
             BN = bb;
         }
     }
-    tc_gemm_bn(c, A, B, M, N, Kp, algo_flops, C, BN);
-}
-
-static void tc_gemm_bn(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp,
-                       double algo_flops, double* C, int BN) {
-    const bool pair = true;
-    const long long tiles = ((M + 255) / 256) * ((N + BN - 1) / BN);
-    // K slices, each its own launch on a side stream (the launches of few tiles run side by side)
-    int S = 1;
-    long long ks = Kp;
-    if (tiles < 64) {
-        S = (int)std::min<long long>(16, std::max<long long>(2, (64 + tiles - 1) / tiles));
-        ks = ((Kp + S - 1) / S + 63) / 64 * 64;
-        S = (int)((Kp + ks - 1) / ks);
-    }
-    Epi e{};
-    e.mode = 2;
-    e.M = (int)M;
-    e.N = (int)N;
-    e.ldc = N;
-    e.err = c.d_err;
-    const int m_fastest = M <= N ? 1 : 0;  // consecutive tiles share the B tile when A is the smaller operand
-    if (S == 1) {
-        Maps m{};
-        for (int p = 0; p < 2; ++p) {
-            m.a[p] = make_map(A[p], M, Kp, BM);
-            m.b[p] = make_map(B[p], N, Kp, pair ? BN / 2 : BN);
-        }
-        e.out = C;
-        e.vec = ((uintptr_t)C % 16 == 0) && (N % 2 == 0);
-        launch_gemm(c, m, 2, 0, 0, (int)M, (int)N, (int)Kp, BN, m_fastest, 16, pair, e, algo_flops);
-        return;
-    }
-    double* T = c.arena.dalloc((size_t)(S * M * N));
-    ensure_side_streams(c, S);
-    ADC_CUDA(cudaEventRecord(c.side_fork, c.stream));
-    for (int sl = 0; sl < S; ++sl) {
-        const long long k0 = sl * ks, kn = std::min(ks, Kp - k0);
-        Maps m{};
-        for (int p = 0; p < 2; ++p) {
-            m.a[p] = make_map_ld((const __nv_bfloat16*)A[p] + k0, M, kn, Kp, BM);
-            m.b[p] = make_map_ld((const __nv_bfloat16*)B[p] + k0, N, kn, Kp, pair ? BN / 2 : BN);
-        }
-        e.out = T + sl * M * N;
-        e.vec = ((uintptr_t)e.out % 16 == 0) && (N % 2 == 0);
-        ADC_CUDA(cudaStreamWaitEvent(c.side[sl], c.side_fork, 0));
-        launch_gemm(c, m, 2, 0, 0, (int)M, (int)N, (int)kn, BN, m_fastest, 16, pair, e, algo_flops * kn / Kp, c.side[sl]);
-        ADC_CUDA(cudaEventRecord(c.side_join[sl], c.side[sl]));
-    }
-    for (int sl = 0; sl < S; ++sl) ADC_CUDA(cudaStreamWaitEvent(c.stream, c.side_join[sl], 0));
-    sum_slices(c, S, M * N, T, C);
+    return tc_gemm_bn(c, A, B, M, N, Kp, algo_flops, BN, S);
 }
 
 }  // namespace adc

@@ -30,14 +30,30 @@ void ladder_tc_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, doubl
 // factors share naux; e.g. the alpha and beta virtual blocks of an open-shell reference)
 void ladder_tc_apply_pair(LadderTC& Ll, LadderTC& Lr, Ctx& c, const double* X, long long nmat, double* out,
                           const LadderMode& md);
+// The pair-adapted integrals V+-_{ab,cd} = (ac|bd) +- (ad|bc), as two BF16 planes and, where there
+// is room (third), a third one: prepare forms them from B^Q_vv (false, holding nothing, if the
+// device has no room; a bounded wait that gives up raises c.d_err), and ladder_tc_apply then
+// contracts with them in sigma's arithmetic (epoch1 == 0) and, with the third plane, in three-plane
+// arithmetic (raising c.d_err likewise, without reading it back).  bytes: what two planes take for
+// nvir virtuals; drop releases all of them, drop_third the third.
+size_t ladder_pairs_bytes(int nvir);
+bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv);
+bool ladder_pairs_third(const LadderTC* L);
+void ladder_pairs_drop_third(LadderTC& L, Ctx& c);
+void ladder_pairs_drop(LadderTC& L, Ctx& c);
+// A call that may use L's integrals (L may be NULL): while one is in progress they stay, except
+// that, with own, an allocation of the same host thread that fails may release them (the ladder
+// then takes the two-GEMM form).
+struct PairsPin {
+    LadderTC* L;
+    void* before = nullptr;
+    PairsPin(LadderTC* L, Ctx& c, bool own);
+    ~PairsPin();
+    PairsPin(const PairsPin&) = delete;
+};
 bool ladder_tc_apply_scratch(LadderTC& L, Ctx& c, const double* X, long long nmat, double* out, const LadderMode& md,
                              void* scratch, size_t bytes);
 
-// Generic contraction on the same kernel: C[M][N] (FP64 row-major, overwritten)
-// = sum_k A[m][k] B[n][k] for two-plane split-BF16 K-major operands A[p]
-// [M][Kp], B[p] [N][Kp] (Kp a multiple of 8, zeros beyond K), FP32 partial
-// sums promoted every 16 K blocks (64 deep).  A bounded device wait that gives
-// up raises c.d_err.
 // Tile autotuner: measured tile choices (GEMM2 tile width and auxiliary chunk of the
 // ladder, tile width of the generic contractions) kept per problem in a text file;
 // one instance per path, shared by the process's handles (Ctx::tuner).
@@ -46,7 +62,12 @@ TuneCache* tune_cache_open(const char* path);
 
 // the shape fits the kernel's 32-bit tile coordinates and K >= 64 (one K block)
 bool tc_gemm_fits(long long M, long long N, long long K);
-void tc_gemm(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp, double algo_flops,
-             double* C);
+// Generic contraction on the same kernel: C[M][N] = sum_k A[m][k] B[n][k] for two-plane
+// split-BF16 K-major operands A[p] [M][Kp], B[p] [N][Kp] (Kp a multiple of 8, zeros beyond K),
+// FP32 partial sums promoted every 16 K blocks (64 deep).  Returns S FP32 results [S][M][N] in
+// c.arena, one per K slice, whose FP64 sum is C (few-tile shapes take several slices).  A bounded
+// device wait that gives up raises c.d_err.
+float* tc_gemm(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp, double algo_flops,
+               int& S);
 
 }  // namespace adc
