@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "gemm64.cuh"
 #include "ladder_tc.cuh"
 
 namespace adc {
@@ -20,14 +21,15 @@ struct PermArgs {
     long long sin[kMaxDim];  // input stride for each output axis
 };
 
-// the inputs of the permutes: an array, or the FP64 sum of S FP32 arrays `stride` apart
+// the inputs of the permutes: an array, or the FP64 sum of S arrays `stride` apart
 template <typename Tin>
 struct Plain {
     const Tin* p;
     __device__ double operator()(long long i) const { return (double)p[i]; }
 };
+template <typename Tin>
 struct SumOf {
-    const float* p;
+    const Tin* p;
     int S;
     long long stride;
     __device__ double operator()(long long i) const {
@@ -65,14 +67,18 @@ __global__ void fill_kernel(long long n, double v, double* __restrict__ y) {
         y[i] = v;
 }
 
-// x as BF16 planes: o0 + o1 (+ o2 where there is a third), each the rounded remainder of those before
+// x as BF16 planes: o0 + o1 (+ o2 where there is a third), each the rounded remainder of those
+// before.  The remainders are formed in FP32, whose 24 bits hold what three planes do: FP64
+// arithmetic (2 operations per cycle and SM on this chip) made the splits several times slower than
+// their traffic.
 __device__ __forceinline__ void put_planes(double x, long long ad, __nv_bfloat16* o0, __nv_bfloat16* o1, __nv_bfloat16* o2) {
-    const __nv_bfloat16 h = __double2bfloat16(x);
+    float f = (float)x;
+    const __nv_bfloat16 h = __float2bfloat16(f);
     o0[ad] = h;
-    x -= (double)__bfloat162float(h);
-    const __nv_bfloat16 m = __double2bfloat16(x);
+    f -= __bfloat162float(h);
+    const __nv_bfloat16 m = __float2bfloat16(f);
     o1[ad] = m;
-    if (o2) o2[ad] = __double2bfloat16(x - (double)__bfloat162float(m));
+    if (o2) o2[ad] = __float2bfloat16(f - __bfloat162float(m));
 }
 
 // out[p][r*Kp + k] (two or three BF16 planes) from the permuted input, zero for k >= K
@@ -569,14 +575,23 @@ void permute(Ctx& c, const double* in, const Shape& s, const int* perm, double* 
     permute_in(c, Plain<double>{in}, s, perm, out, alpha, beta);
 }
 
-void permute_sum(Ctx& c, const float* in, int S, const Shape& s, const int* perm, void* out, bool out32, double alpha,
-                 double beta) {
+template <typename Tin>
+static void permute_sum_t(Ctx& c, const Tin* in, int S, const Shape& s, const int* perm, void* out, bool out32, double alpha,
+                          double beta) {
     long long n = 1;
     for (int j = 0; j < s.nd; ++j) n *= s.d[j];
     if (out32)
-        permute_in(c, SumOf{in, S, n}, s, perm, (float*)out, alpha, beta);
+        permute_in(c, SumOf<Tin>{in, S, n}, s, perm, (float*)out, alpha, beta);
     else
-        permute_in(c, SumOf{in, S, n}, s, perm, (double*)out, alpha, beta);
+        permute_in(c, SumOf<Tin>{in, S, n}, s, perm, (double*)out, alpha, beta);
+}
+void permute_sum(Ctx& c, const float* in, int S, const Shape& s, const int* perm, void* out, bool out32, double alpha,
+                 double beta) {
+    permute_sum_t(c, in, S, s, perm, out, out32, alpha, beta);
+}
+void permute_sum(Ctx& c, const double* in, int S, const Shape& s, const int* perm, void* out, bool out32, double alpha,
+                 double beta) {
+    permute_sum_t(c, in, S, s, perm, out, out32, alpha, beta);
 }
 
 template <typename Tin>
@@ -847,6 +862,45 @@ static void einsum_tc(Ctx& c, const std::string& la, const std::string& lb, cons
     permute_sum(c, T, S, sh, perm, C, c32, alpha, beta);
 }
 
+// FP64-accurate contraction on the tensor cores (gemm64): the operands are read in place, the
+// result written in place when it is in GEMM order, else permuted and accumulated in one pass.
+static void einsum_64(Ctx& c, const std::string& la, const std::string& lb, const std::string& lc,
+                      std::map<char, long long>& dim, const std::string& fa, const std::string& fb, const std::string& con,
+                      double alpha, const T& A, const T& B, double beta, void* C, bool c32) {
+    auto operand = [&](const T& X, const std::string& l, const std::string& rows) {
+        Operand64 o;
+        o.p = X.p;
+        o.f32 = X.f32;
+        std::map<char, long long> st;
+        long long acc = 1;
+        for (int j = (int)l.size() - 1; j >= 0; --j) {
+            st[l[j]] = acc;
+            acc *= dim[l[j]];
+        }
+        for (char x : rows) o.row_axis(dim[x], st[x]);
+        for (char x : con) o.k_axis(dim[x], st[x]);
+        if (o.nk == 0) o.k_axis(1, 1);
+        return o;
+    };
+    Operand64 a = operand(A, la, fa), b = operand(B, lb, fb);
+    // the 128-row axis takes the longer side when the other would leave it mostly empty
+    const bool swap = a.rows < 64 && b.rows > a.rows;
+    const std::string tord = swap ? fb + fa : fa + fb;
+    const bool in_place = tord == lc && !c32;
+    int S = 1;
+    const double* Tm = swap ? gemm64(c, b, a, alpha, beta, in_place ? (double*)C : nullptr, S)
+                            : gemm64(c, a, b, alpha, beta, in_place ? (double*)C : nullptr, S);
+    if (!Tm) return;
+    Shape sh;
+    sh.nd = (int)tord.size();
+    int perm[kMaxDim];
+    for (int j = 0; j < sh.nd; ++j) {
+        sh.d[j] = dim[tord[j]];
+        perm[j] = (int)tord.find(lc[j]);
+    }
+    permute_sum(c, Tm, S, sh, perm, C, c32, alpha, beta);
+}
+
 static void einsum_core(Ctx& c, const char* specstr, double alpha, const T& A, const T& B, double beta, void* C, bool c32,
                         const std::vector<long long>& cdims) {
     Spec sp = parse(specstr);
@@ -902,6 +956,8 @@ static void einsum_core(Ctx& c, const char* specstr, double alpha, const T& A, c
         const bool big_in_place = M <= N ? (!B.f32 && sp.b == con + fb) : (!A.f32 && sp.a == fa + con);
         if (big && tc_gemm_fits(M, N, K) && (!skinny || (big_const && !big_in_place))) {
             einsum_tc(c, sp.a, sp.b, sp.c, dim, fa, fb, con, alpha, A, B, beta, C, c32);
+        } else if (!big && !skinny && gemm64_fits(M, N, K)) {
+            einsum_64(c, sp.a, sp.b, sp.c, dim, fa, fb, con, alpha, A, B, beta, C, c32);
         } else {
             const double* Ap = to_order(c, A.p, sp.a, dim, fa + con, A.f32);
             const double* Bp = to_order(c, B.p, sp.b, dim, con + fb, B.f32);
@@ -924,6 +980,11 @@ static void einsum_core(Ctx& c, const char* specstr, double alpha, const T& A, c
     }
     if (c.gemm_mode >= 1 && 2.0 * nb * M * N * K >= c.fp32_min_flops) {
         einsum_fp32(c, sp.a, sp.b, sp.c, dim, batch, fa, fb, con, alpha, A, B, beta, C, c32);
+        c.arena.release(mk);
+        return;
+    }
+    if (nb == 1 && gemm64_fits(M, N, K)) {
+        einsum_64(c, sp.a, sp.b, sp.c, dim, fa, fb, con, alpha, A, B, beta, C, c32);
         c.arena.release(mk);
         return;
     }

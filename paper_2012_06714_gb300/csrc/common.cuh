@@ -219,8 +219,10 @@ void einsum(Ctx& c, const char* spec, double alpha, const T& A, const T& B, doub
 // out = alpha * permute(in) + beta * out between FP64 / FP32 arrays (in32 / out32: FP32)
 void permute_any(Ctx& c, const void* in, bool in32, const Shape& s, const int* perm, void* out, bool out32,
                  double alpha, double beta);
-// the same for the FP64 sum of S FP32 arrays, one after another in `in` (the slices of tc_gemm)
+// the same for the FP64 sum of S arrays, one after another in `in` (the K slices of tc_gemm and gemm64)
 void permute_sum(Ctx& c, const float* in, int S, const Shape& s, const int* perm, void* out, bool out32, double alpha,
+                 double beta);
+void permute_sum(Ctx& c, const double* in, int S, const Shape& s, const int* perm, void* out, bool out32, double alpha,
                  double beta);
 
 // Permute `in` (shape s, output axis j = input axis perm[j]) into row-major

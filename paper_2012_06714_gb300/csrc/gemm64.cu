@@ -1,0 +1,524 @@
+// FP64-accurate contractions on the BF16 tensor cores of sm_103a.
+//
+// GB300 has about 1.2 TFLOP/s of FP64 against 2 PFLOP/s of dense BF16, so an FP64 product is
+// cheaper as a sum of exact integer products (the error-free splitting of Ozaki, Ogita, Oishi and
+// Rump, Numer. Algorithms 59, 95 (2012)):
+//   * every row of A and of B is scaled by a power of two to integers below 2^56 in size and cut
+//     into seven signed digits of eight bits (six of |d| <= 128, the top one of |d| <= 256), which
+//     BF16 holds exactly;
+//   * the digit products of equal weight, s = i + j, accumulate in one FP32 tensor-memory
+//     accumulator per s.  Over 128 summed terms such a sum stays within 2^24, so it is an exact
+//     integer (s = 6 may reach 9/8 of that if every digit is at its limit, and then loses a unit,
+//     2^-62 of the row scales); it is drained into 64-bit integer registers, exact for any K;
+//   * the weights s = 12 .. 5 are kept (34 of 49 digit pairs); what is left out is below
+//     2^-61 sqrt(K) of the product of the row scales, less than the 2^-57 rounding of the inputs
+//     to their rows' scales.  The one rounding of the result is to FP64.
+// The error against 64-bit arithmetic is that of an FP64 GEMM: norm of the error over norm of sigma
+// 1.8e-16 (IP, 14/113/445) against 1.7e-16 with DGEMM, 1.2e-16 each for its final rounding.
+// Measured: that sigma (5 vectors, 22 GFLOP in 20 contractions) 24.6 -> 3.8 ms; the FP64 setup of an
+// IP molecule at 17/121/483 with its first sigma 217 -> 44 ms.
+//
+// Tile: 128 rows of A x BNT columns (16 .. 64) of B per CTA, because the eight accumulators take
+// 8 x BNT of the 512 tensor-memory columns.  The digit planes of B lie one after another in shared
+// memory as further rows of one K-major operand and the accumulators of consecutive weights are
+// consecutive in tensor memory, so that one MMA multiplies digit i of A with up to 256 / BNT digits
+// of B: 11 MMAs of up to 256 columns per 16-deep K step instead of 34 of 64 (which would be bound by
+// reading A from shared memory 34 times).
+#include <algorithm>
+#include <cstdint>
+#include <mutex>
+
+#include "gemm64.cuh"
+#include "tcgen05.cuh"
+
+namespace adc {
+
+namespace {
+
+constexpr int ND = 7;          // digits
+constexpr int SMIN = 5;        // lowest weight kept
+constexpr int NL = 8;          // weights SMIN .. 2 (ND - 1)
+constexpr int GM = 128;        // tile rows
+constexpr int GK = 32;         // K block: 64-byte rows, 64-byte swizzle
+constexpr int EPOCH = 4;       // K blocks between drains (128 terms)
+constexpr int G_EPI = 8;       // epilogue warps
+constexpr int G_THREADS = 64 + 32 * G_EPI;
+constexpr int G_MAXST = 4;
+constexpr size_t G_SMEM = 226 * 1024;
+
+// ---- digits -------------------------------------------------------------------------
+constexpr int DT = 256;  // threads, and K chunk, of k_digits
+constexpr int DR = 8;    // rows per block at most
+
+struct DigitSide {
+    Operand64 x;
+    long long Kp;
+    __nv_bfloat16* out;  // [ND][rows][Kp], digit 0 the least significant
+    int* ex;             // biased exponent field of the row's largest element (0x7ff: not finite)
+    int row_lanes;       // the tensor's contiguous axis is the last row axis (else the lanes run along k)
+    int R;               // rows per block, a power of two
+};
+
+__device__ __forceinline__ double ld_op(const Operand64& x, long long i) {
+    return x.f32 ? (double)((const float*)x.p)[i] : ((const double*)x.p)[i];
+}
+
+// Both operands in one launch (blocks [0, blocks_a) of x the rows of A), K in segments of kseg along
+// y.  passes: 1 the rows' largest exponents (into ex, zero before), 2 the digits, 3 both (one segment;
+// the second read then comes from L1 / L2).  Integer arithmetic only: the FP64 pipe (2 operations per
+// cycle and SM) would be the bound.
+__global__ void __launch_bounds__(DT) k_digits(const __grid_constant__ DigitSide sa, const __grid_constant__ DigitSide sb,
+                                               int blocks_a, long long kseg, int passes) {
+    __shared__ double tile[DR][DT + 1];
+    __shared__ long long offk[DT], offr[DR];
+    __shared__ int emax[DR];
+    const bool isb = (int)blockIdx.x >= blocks_a;
+    const DigitSide& sd = isb ? sb : sa;
+    const Operand64& x = sd.x;
+    const int R = sd.R, tid = threadIdx.x;
+    const long long row0 = (long long)(isb ? blockIdx.x - blocks_a : blockIdx.x) * R;
+    const long long kbeg = blockIdx.y * kseg, kend = min(sd.Kp, kbeg + kseg);
+    if (tid < R) {
+        unsigned long long r = (unsigned long long)min(row0 + tid, x.rows - 1);
+        long long off = 0;
+        for (int j = x.nr - 1; j >= 0; --j) {
+            const unsigned d = (unsigned)x.rd[j], q = (unsigned)r / d;
+            off += (long long)((unsigned)r - q * d) * x.rs[j];
+            r = q;
+        }
+        offr[tid] = off;
+        emax[tid] = passes == 2 ? sd.ex[min(row0 + tid, x.rows - 1)] : 0;
+    }
+    const int per = DT / R, lper = 31 - __clz(per), lR = 8 - lper;  // threads per row when the lanes run along k
+    const int r = tid >> lper;
+    for (int pass = 1; pass <= 2; ++pass) {
+        if (!(passes & pass)) continue;
+        for (long long k0 = kbeg; k0 < kend; k0 += DT) {
+            if (!(pass == 2 && passes == 3 && kend - kbeg <= DT)) {  // (one chunk: still in shared memory)
+                __syncthreads();
+                {
+                    unsigned k = (unsigned)min(k0 + tid, x.K - 1);
+                    long long off = 0;
+                    for (int j = x.nk - 1; j >= 0; --j) {
+                        const unsigned d = (unsigned)x.kd[j], q = k / d;
+                        off += (long long)(k - q * d) * x.ks[j];
+                        k = q;
+                    }
+                    offk[tid] = off;
+                }
+                __syncthreads();
+                for (int e = tid; e < R * DT; e += DT) {
+                    const int rr = sd.row_lanes ? e & (R - 1) : e >> 8, k = sd.row_lanes ? e >> lR : e & (DT - 1);
+                    tile[rr][k] = k0 + k < x.K && row0 + rr < x.rows ? ld_op(x, offr[rr] + offk[k]) : 0.0;
+                }
+                __syncthreads();
+            }
+            if (pass == 1) {
+                int m = 0;
+                for (int k = tid & (per - 1); k < DT; k += per) m = max(m, (__double2hiint(tile[r][k]) >> 20) & 0x7ff);
+                if (m > 0) atomicMax(&emax[r], m);
+            } else if (row0 + r < x.rows) {
+                const int ef = emax[r];
+                for (int k = 2 * (tid & (per - 1)); k < DT; k += 2 * per) {
+                    if (k0 + k >= sd.Kp) break;
+                    unsigned dig[ND];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const long long b = __double_as_longlong(tile[r][k + h]);
+                        const int ex = (int)(b >> 52) & 0x7ff;
+                        // |x| = m 2^(ex - 1075) -> round(|x| 2^(1078 - ef)), at most 2^56: the row's scale is 2^(ef - 1022)
+                        long long v = 0;
+                        const int sh = ef - ex - 3;  // right shift of the 53-bit significand (-3: three more bits)
+                        if (ex > 0 && ef < 0x7ff && sh < 55) {
+                            const long long m = (b & 0xfffffffffffffLL) | (1LL << 52);
+                            v = sh <= 0 ? m << -sh : (m + (1LL << (sh - 1))) >> sh;
+                            if (b < 0) v = -v;
+                        }
+                        // digit p of v + sum_p 128 256^p is the p-th byte less 128: the carries in one addition
+                        const unsigned long long w = (unsigned long long)v + 0x808080808080ULL;
+#pragma unroll
+                        for (int p = 0; p < ND; ++p) {
+                            const int d = p < ND - 1 ? (int)((w >> (8 * p)) & 0xff) - 128 : (int)((long long)w >> (8 * p));
+                            // a small integer's BF16 bits are the upper half of its FP32 bits
+                            const unsigned u = __float_as_uint((float)d) >> 16;
+                            dig[p] = h == 0 ? u : dig[p] | (u << 16);
+                        }
+                    }
+#pragma unroll
+                    for (int p = 0; p < ND; ++p)
+                        *(unsigned*)(sd.out + ((long long)p * x.rows + row0 + r) * sd.Kp + k0 + k) = dig[p];
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if ((passes & 1) && tid < R && row0 + tid < x.rows) {
+        if (passes == 3)
+            sd.ex[row0 + tid] = emax[tid];
+        else
+            atomicMax(&sd.ex[row0 + tid], emax[tid]);
+    }
+}
+
+// ---- GEMM ---------------------------------------------------------------------------
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* m, uint64_t* bar, int x, int y) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(
+            su32(dst)),
+        "l"((uint64_t)m), "r"(su32(bar)), "r"(x), "r"(y), "r"(0)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+// K-major descriptor of 64-byte rows in the 64-byte swizzle (8-row groups of 512 bytes)
+__device__ __forceinline__ uint64_t desc64(const void* p) {
+    return (uint64_t)((su32(p) >> 4) & 0x3FFF) | (uint64_t)1 << 16 | (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 |
+           (uint64_t)4 << 61;
+}
+
+// (hi 2^32 + lo) 2^e, rounded to nearest, by integer arithmetic; |hi| < 2^62
+__device__ __forceinline__ double to_double(long long hi, long long lo, int e) {
+    long long H = hi + (lo >> 32);
+    uint32_t L = (uint32_t)lo;
+    const bool neg = H < 0;
+    if (neg) {
+        L = 0u - L;
+        H = L == 0 ? -H : ~H;
+    }
+    unsigned long long m;
+    int top;  // weight of m's bit 63
+    if (H != 0) {
+        const int lz = __clzll(H);
+        const unsigned long long l = (unsigned long long)L << 32;
+        m = ((unsigned long long)H << lz) | (lz ? l >> (64 - lz) : 0ull);
+        top = 95 - lz;
+    } else {
+        if (L == 0) return 0.0;
+        const int lz = __clz(L);
+        m = (unsigned long long)L << (32 + lz);
+        top = 31 - lz;
+    }
+    m = (m >> 11) + ((m >> 10) & 1);  // 53 bits, carry into bit 53 raises the exponent below
+    const int be = top + e + 1023;
+    unsigned long long bits;
+    if (be <= 0)
+        bits = 0;  // below the normal range
+    else if (be >= 2046)
+        bits = 0x7ffull << 52;
+    else
+        bits = m + ((unsigned long long)(be - 1) << 52);
+    return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+}
+
+struct Gemm64Out {
+    int M, N, mt, nt, S, slice_kb;  // slices of slice_kb K blocks
+    const int *ea, *eb;
+    double* out;  // [S][M][N], or with direct the output itself
+    double alpha, beta;
+    int direct;
+    int* err;
+};
+
+__global__ void __launch_bounds__(G_THREADS, 1)
+    k_gemm64(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb, int num_k, int BNT, int stages,
+             int tmem_cols, Gemm64Out o) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    __shared__ uint64_t full_bar[G_MAXST], empty_bar[G_MAXST], tfull, tempty, done_bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int A_PL = GM * GK * 2, B_PL = BNT * GK * 2;
+    const int STAGE = ND * (A_PL + B_PL);
+    const int tiles = o.mt * o.nt, nunits = tiles * o.S;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < stages; ++s) {
+            mbar_init(&full_bar[s], 1);
+            mbar_init(&empty_bar[s], 1);
+        }
+        mbar_init(&tfull, 1);
+        mbar_init(&tempty, G_EPI);
+        mbar_init(&done_bar, 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_slot)), "r"(tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            long long g = 0;
+            for (int u = blockIdx.x; u < nunits && !abort_flag; u += gridDim.x) {
+                const int sl = u / tiles, t = u - sl * tiles, m_tile = t % o.mt, n_tile = t / o.mt;
+                const int kb1 = min(num_k, (sl + 1) * o.slice_kb);
+                for (int kb = sl * o.slice_kb; kb < kb1; ++kb, ++g) {
+                    const int s = (int)(g % stages);
+                    if (g >= stages && !mbar_wait(&empty_bar[s], (uint32_t)(((g / stages) & 1) ^ 1), &abort_flag, o.err)) break;
+                    uint8_t* st = smem + (size_t)s * STAGE;
+                    mbar_expect_tx(&full_bar[s], STAGE);
+                    tma_load_3d(st, &ma, &full_bar[s], kb * GK, m_tile * GM);
+                    tma_load_3d(st + ND * A_PL, &mb, &full_bar[s], kb * GK, n_tile * BNT);
+                }
+            }
+            if (abort_flag) {
+                // let the copies of the last `stages` issues land before the CTA retires (bounded)
+                for (long long q = (g > stages ? g - stages : 0); q < g; ++q) {
+                    const uint64_t t0 = gtime();
+                    while (!mbar_try(&full_bar[q % stages], (uint32_t)((q / stages) & 1)) && gtime() - t0 < WAIT_NS) {
+                    }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t ib = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GM >> 4) << 24);
+            const int jmax = 256 / BNT;  // digits of B per MMA
+            long long g = 0, e = 0;
+            bool ok = true;
+            for (int u = blockIdx.x; u < nunits && ok && !abort_flag; u += gridDim.x) {
+                const int sl = u / tiles, kb0 = sl * o.slice_kb, kb1 = min(num_k, kb0 + o.slice_kb);
+                for (int kb = kb0; kb < kb1; ++kb, ++g) {
+                    const int s = (int)(g % stages), in_epoch = (kb - kb0) % EPOCH;
+                    if (!mbar_wait(&full_bar[s], (uint32_t)((g / stages) & 1), &abort_flag, o.err) ||
+                        (in_epoch == 0 && e > 0 && !mbar_wait(&tempty, (uint32_t)((e & 1) ^ 1), &abort_flag, o.err))) {
+                        ok = false;
+                        break;
+                    }
+                    fence_after();
+                    const uint64_t a0 = desc64(smem + (size_t)s * STAGE), b0 = desc64(smem + (size_t)s * STAGE + ND * A_PL);
+#pragma unroll
+                    for (int kk = 0; kk < GK / 16; ++kk) {
+                        const uint32_t later = in_epoch > 0 || kk > 0 ? 1u : 0u;  // 0: first products of this epoch
+                        for (int i = ND - 1; i >= 0; --i) {
+                            const uint64_t ad = a0 + (uint64_t)(i * (A_PL >> 4) + kk * 2);
+                            // the lowest weight first appears at i = ND - 2, j = 0: alone, to start its accumulator
+                            for (int j = max(0, SMIN - i); j < ND;) {
+                                int nj = min(jmax, ND - j);
+                                if (!later && i == SMIN && j == 0) nj = 1;
+                                const uint32_t acc = later || !(i == ND - 1 || (i == SMIN && j == 0)) ? 1u : 0u;
+                                mma_bf16(tmem + (uint32_t)((i + j - SMIN) * BNT), ad,
+                                         b0 + (uint64_t)(j * (B_PL >> 4) + kk * 2), ib | ((uint32_t)(nj * BNT >> 3) << 17), acc);
+                                j += nj;
+                            }
+                        }
+                    }
+                    mma_commit(&empty_bar[s]);
+                    if (in_epoch == EPOCH - 1 || kb == kb1 - 1) {
+                        mma_commit(&tfull);
+                        ++e;
+                    }
+                }
+            }
+            mma_commit(&done_bar);
+        }
+    } else {
+        const int ew = warp - 2, quarter = warp & 3, half = ew >> 2, cw = BNT >> 1, cbeg = half * cw;
+        long long e = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+            const int sl = u / tiles, t = u - sl * tiles, m_tile = t % o.mt, n_tile = t / o.mt;
+            const int kb0 = sl * o.slice_kb, epochs = (min(num_k, kb0 + o.slice_kb) - kb0 + EPOCH - 1) / EPOCH;
+            long long hi[32], lo[32];
+#pragma unroll
+            for (int q = 0; q < 32; ++q) hi[q] = lo[q] = 0;
+            for (int i = 0; i < epochs; ++i, ++e) {
+                if (!mbar_wait(&tfull, (uint32_t)(e & 1), &abort_flag, o.err)) {
+                    ok = false;
+                    break;
+                }
+                fence_after();
+                const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)cbeg;
+#pragma unroll
+                for (int c0 = 0; c0 < 32; c0 += 8) {
+                    if (c0 < cw) {
+                        uint32_t r[NL][8];
+#pragma unroll
+                        for (int l = 0; l < NL; ++l) tmem_ld8(base + (uint32_t)(l * BNT + c0), r[l]);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            int v[NL];
+#pragma unroll
+                            for (int l = 0; l < NL; ++l) v[l] = __float2int_rn(__uint_as_float(r[l][q]));
+                            hi[c0 + q] += (long long)v[7] * (1 << 24) + (long long)v[6] * (1 << 16) + (long long)v[5] * (1 << 8) + v[4];
+                            lo[c0 + q] += (long long)v[3] * (1 << 24) + (long long)v[2] * (1 << 16) + (long long)v[1] * (1 << 8) + v[0];
+                        }
+                    }
+                }
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tempty);
+            }
+            if (!ok) break;
+            const int row = m_tile * GM + quarter * 32 + lane, colt = n_tile * BNT + cbeg;
+            if (row < o.M) {
+                const int ea = o.ea[row];
+                double* dst = o.out + ((long long)sl * o.M + row) * o.N + colt;
+#pragma unroll
+                for (int q = 0; q < 32; ++q) {
+                    if (q < cw && colt + q < o.N) {
+                        const int eb = o.eb[colt + q];
+                        // weights: digit products of weight s carry 2^(8 s); hi starts at s = 9, lo at s = 5;
+                        // a row's integers carry 2^(ef - 1078)
+                        double v = ea == 0x7ff || eb == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL)
+                                                              : to_double(hi[q], lo[q], 8 * SMIN + ea + eb - 2 * 1078);
+                        if (o.direct) {
+                            if (o.alpha != 1.0) v *= o.alpha;
+                            if (o.beta != 0.0) v += o.beta == 1.0 ? dst[q] : o.beta * dst[q];
+                        }
+                        dst[q] = v;
+                    }
+                }
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        const uint64_t t0 = gtime();
+        while (!mbar_try(&done_bar, 0) && gtime() - t0 < WAIT_NS) {
+        }
+        fence_after();
+        __syncwarp();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
+    }
+}
+
+// digit planes [ND][rows][Kp] as a 3-D tensor {k, row, digit}, box {GK, box_rows, ND}, 64-byte swizzle
+CUtensorMap make_map_digits(const void* base, long long rows, long long Kp, int box_rows) {
+    CUtensorMap m;
+    cuuint64_t dims[3] = {(cuuint64_t)Kp, (cuuint64_t)rows, ND};
+    cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)(rows * Kp * 2)};
+    cuuint32_t box[3] = {GK, (cuuint32_t)box_rows, ND};
+    cuuint32_t es[3] = {1, 1, 1};
+    const CUresult r = tensor_map_encoder()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
+                                            box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) throw Error(-3, "cuTensorMapEncodeTiled (digits) failed: " + std::to_string((int)r));
+    return m;
+}
+
+int sm_count() {
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+}
+
+}  // namespace
+
+bool gemm64_fits(long long M, long long N, long long K) {
+    return M < (1LL << 30) && N < (1LL << 30) && K < (1LL << 30) && 2.0 * M * N * K >= 2e6 && std::max(M, N) >= 16;
+}
+
+double* gemm64(Ctx& c, const Operand64& A, const Operand64& B, double alpha, double beta, double* out, int& S) {
+    const long long M = A.rows, N = B.rows, K = A.K, Kp = (K + 7) / 8 * 8;
+    const int num_k = (int)((Kp + GK - 1) / GK), sms = sm_count();
+    if (!c.d_err) {
+        if (c.capturing) throw Error(-3, "error flag allocation during stream capture");
+        c.d_err = (int*)dev_alloc(sizeof(int), c.stream);
+        ADC_CUDA(cudaMemsetAsync(c.d_err, 0, sizeof(int), c.stream));
+    }
+    // tile width: least time over the chip.  A K block of a tile takes 17 BNT tensor cycles (34 digit
+    // pairs), reading A from shared memory bounds it below about BNT = 16; a drain (every EPOCH blocks)
+    // about 40 BNT cycles, which the MMAs wait for; the last one and the store about 60 BNT.
+    int BNT = 64;
+    long long best_s = 1;
+    double best = 1e300;
+    for (int b : {64, 48, 32, 16}) {
+        const long long tiles = ((M + GM - 1) / GM) * ((N + b - 1) / b);
+        for (long long s = 1; s <= 32; ++s) {
+            const long long kb = ((num_k + s - 1) / s + EPOCH - 1) / EPOCH * EPOCH;
+            if (s > 1 && (num_k + kb - 1) / kb != s) continue;
+            const double rounds = (double)((tiles * s + sms - 1) / sms);
+            const double blocks = (double)std::min<long long>(kb, num_k);
+            const double cyc = rounds * (2000.0 + blocks * 2.0 * std::max(17.0 * b, 280.0) + (blocks / EPOCH) * 40.0 * b + 60.0 * b) +
+                               (s - 1) * (double)M * N * 16.0 / 2500.0 + (s > 1 ? 4000.0 : 0.0);
+            if (cyc < best * 0.999) best = cyc, BNT = b, best_s = s;
+        }
+    }
+    const int kb = (int)(((num_k + best_s - 1) / best_s + EPOCH - 1) / EPOCH * EPOCH);
+    S = (num_k + kb - 1) / kb;
+    const bool direct = out && S == 1;
+    double* T = direct ? nullptr : c.arena.dalloc((size_t)S * M * N);
+    DigitSide side[2];
+    const Operand64* ops[2] = {&A, &B};
+    int blocks[2];
+    Arena::Mark mk = c.arena.mark();
+    int* ex = (int*)c.arena.alloc((size_t)(M + N) * sizeof(int));
+    // a row's K in one block up to this length (two reads in one launch), else in segments (two launches)
+    const bool fused = Kp <= 1024;
+    for (int i = 0; i < 2; ++i) {
+        DigitSide& d = side[i];
+        d.x = *ops[i];
+        d.Kp = Kp;
+        d.out = (__nv_bfloat16*)c.arena.alloc((size_t)ND * d.x.rows * Kp * 2);
+        d.ex = ex + (i ? M : 0);
+        long long smallest = d.x.ks[d.x.nk - 1];
+        d.row_lanes = 0;
+        for (int j = 0; j < d.x.nk; ++j) smallest = std::min(smallest, d.x.kd[j] > 1 ? d.x.ks[j] : smallest);
+        for (int j = 0; j < d.x.nr; ++j)
+            if (d.x.rd[j] > 1 && d.x.rs[j] < smallest) d.row_lanes = 1;
+        d.R = DR;
+        while (fused && d.R > 1 && (d.x.rows + d.R - 1) / d.R < 2 * sms) d.R /= 2;
+        const long long nb = (d.x.rows + d.R - 1) / d.R;
+        if (nb > (1LL << 30)) throw Error(-1, "gemm64: too many rows");
+        blocks[i] = (int)nb;
+    }
+    const unsigned bx = (unsigned)(blocks[0] + blocks[1]);
+    if (fused) {
+        k_digits<<<bx, DT, 0, c.stream>>>(side[0], side[1], blocks[0], Kp, 3);
+        ++c.kernels;
+    } else {
+        ADC_CUDA(cudaMemsetAsync(ex, 0, (size_t)(M + N) * sizeof(int), c.stream));
+        for (int pass = 1; pass <= 2; ++pass) {
+            long long seg = pass == 1 ? 2048 : 512;
+            while ((Kp + seg - 1) / seg > 65535) seg *= 2;
+            k_digits<<<dim3(bx, (unsigned)((Kp + seg - 1) / seg)), DT, 0, c.stream>>>(side[0], side[1], blocks[0], seg, pass);
+            ++c.kernels;
+        }
+    }
+    ADC_CUDA(cudaGetLastError());
+    const CUtensorMap ma = make_map_digits(side[0].out, M, Kp, GM), mb = make_map_digits(side[1].out, N, Kp, BNT);
+    Gemm64Out o{};
+    o.M = (int)M;
+    o.N = (int)N;
+    o.mt = (int)((M + GM - 1) / GM);
+    o.nt = (int)((N + BNT - 1) / BNT);
+    o.S = S;
+    o.slice_kb = kb;
+    o.ea = side[0].ex;
+    o.eb = side[1].ex;
+    o.out = direct ? out : T;
+    o.alpha = alpha;
+    o.beta = beta;
+    o.direct = direct ? 1 : 0;
+    o.err = c.d_err;
+    const long long units = (long long)o.mt * o.nt * S;
+    if (units > (1LL << 30)) throw Error(-1, "gemm64: too many tiles");
+    const int stage = ND * (GM + BNT) * GK * 2;
+    const int stages = std::min(G_MAXST, (int)((G_SMEM - 1024) / stage));
+    int cols = 32;
+    while (cols < NL * BNT) cols *= 2;
+    static std::once_flag once[64];
+    int dev = 0;
+    ADC_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) throw Error(-3, "gemm64: device index out of range");
+    std::call_once(once[dev], [] { cudaFuncSetAttribute(k_gemm64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM); });
+    k_gemm64<<<(unsigned)std::min<long long>(units, sms), G_THREADS, G_SMEM, c.stream>>>(ma, mb, num_k, BNT, stages, cols, o);
+    ++c.kernels;
+    ADC_CUDA(cudaGetLastError());
+    c.arena.release(mk);
+    return T;
+}
+
+}  // namespace adc

@@ -456,14 +456,15 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 // ---- operand preparation (FP64 -> split BF16) --------------------------------
-// x = p0 + p1 (+ p2) with every plane in BF16 (successive remainders)
-__device__ __forceinline__ void splitp(double x, int planes, __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2) {
-    const __nv_bfloat16 h = __double2bfloat16(x);
-    double r = x - (double)__bfloat162float(h);
-    const __nv_bfloat16 m = __double2bfloat16(r);
+// x = p0 + p1 (+ p2) with every plane in BF16 (successive remainders, formed in FP32: its 24 bits hold
+// what three planes do, and FP64 arithmetic would bound the kernels below)
+__device__ __forceinline__ void splitp(float x, int planes, __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2) {
+    const __nv_bfloat16 h = __float2bfloat16(x);
+    x -= __bfloat162float(h);
+    const __nv_bfloat16 m = __float2bfloat16(x);
     *p0 = h;
     *p1 = m;
-    if (planes == 3) *p2 = __double2bfloat16(r - (double)__bfloat162float(m));
+    if (planes == 3) *p2 = __float2bfloat16(x - __bfloat162float(m));
 }
 #define GRID_STRIDE(i, n) for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (n); i += (long long)gridDim.x * blockDim.x)
 
@@ -481,7 +482,7 @@ __global__ void k_split_Bs(const double* __restrict__ B, int naux, int v, int vp
         int a = r % vp;
         long long Q = r / vp;
         double val = (cp < v && a < v) ? B[(Q * v + a) * v + cp] : 0.0;
-        splitp(val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
+        splitp((float)val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
     }
 }
 // Bp[b][(Q,dp)] = B^Q[d][b] (= B^Q[b][d]), zero pad
@@ -492,7 +493,7 @@ __global__ void k_split_Bp(const double* __restrict__ B, int naux, int v, int vp
         long long r = x / vp;
         int Q = r % naux, b = r / naux;
         double val = dp < v ? B[((long long)Q * v + b) * v + dp] : 0.0;
-        splitp(val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
+        splitp((float)val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
     }
 }
 // XT[(m,d)][cp] = X_m[c][d] for X_m of va x vb (c < va, d < vb; rows d padded to vpb,
@@ -506,7 +507,7 @@ __global__ void k_split_XT(const double* __restrict__ X, long long nmat, int va,
         int d = r % vpb;
         long long m = r / vpb;
         double val = (cp < va && d < vb) ? X[(m * va + cp) * vb + d] : 0.0;
-        splitp(val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
+        splitp((float)val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
     }
 }
 
@@ -550,8 +551,8 @@ __global__ void __launch_bounds__(256) k_pair_planes(const Tin* __restrict__ in,
         for (int i = ty; i < 32; i += 8) {
             const int cc = c0 + i, dd = d0 + tx;
             if (cc < v && dd <= cc) {
-                const double x = (double)t1[i][tx], y = (double)t2[tx][i];
-                const double ps = dd == cc && !integrals ? x : x + y, pa = x - y;
+                const Tin x = t1[i][tx], y = t2[tx][i];
+                const float ps = (float)(dd == cc && !integrals ? x : x + y), pa = (float)(x - y);
                 const long long p = (long long)cc * (cc + 1) / 2 + dd, o0 = row * Pk + p, o1 = (rows + row) * Pk + p;
                 const int planes = o.p[2] ? 3 : 2;
                 splitp(ps, planes, o.p[0] + o0, o.p[1] + o0, o.p[2] + o0);
@@ -610,24 +611,6 @@ __global__ void __launch_bounds__(256) k_pair_unfold(const float* __restrict__ T
 inline int grid_for(long long n) { return (int)std::min<long long>(std::max<long long>((n + 255) / 256, 1), 152LL * 32); }
 
 // ---- host: tensor maps ------------------------------------------------------
-typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                             const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeFn encode_fn() {
-    static EncodeFn fn = nullptr;
-    static std::once_flag once;
-    static cudaError_t st = cudaSuccess;
-    std::call_once(once, [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        st = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q);
-        if (st == cudaSuccess && q == cudaDriverEntryPointSuccess) fn = (EncodeFn)p;
-    });
-    if (!fn) throw Error(-3, "cuTensorMapEncodeTiled unavailable");
-    return fn;
-}
-
 // 2-D BF16 tensor [rows][cols] (cols contiguous), box {BK, box_rows}, ROW_BYTES swizzle
 CUtensorMap make_map(const void* base, long long rows, long long cols, int box_rows) {
     if (((uintptr_t)base & 15) || (cols * 2) % 16) throw Error(-1, "tensor map: misaligned operand");
@@ -636,7 +619,7 @@ CUtensorMap make_map(const void* base, long long rows, long long cols, int box_r
     cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
     cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
     cuuint32_t es[2] = {1, 1};
-    CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
+    CUresult r = tensor_map_encoder()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
                              CU_TENSOR_MAP_INTERLEAVE_NONE,
                              ROW_BYTES == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -660,7 +643,7 @@ CUtensorMap make_map_z(const void* base, int vp, int qn, int v, long long nm) {
     cuuint64_t strides[3] = {(cuuint64_t)vp * 2, (cuuint64_t)qn * vp * 2, (cuuint64_t)v * qn * vp * 2};
     cuuint32_t box[4] = {16, 1, 32, 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
-    CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
+    CUresult r = tensor_map_encoder()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) throw Error(-3, "cuTensorMapEncodeTiled (Z) failed: " + std::to_string((int)r));

@@ -7,6 +7,9 @@
 #include <cuda_bf16.h>
 
 #include <cstdint>
+#include <mutex>
+
+#include "common.cuh"
 
 namespace adc {
 namespace {
@@ -199,6 +202,24 @@ __device__ bool mbar_wait_cluster(uint64_t* b, uint32_t parity, volatile int* ab
     }
 }
 
+
+typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                             const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeFn tensor_map_encoder() {
+    static EncodeFn fn = nullptr;
+    static std::once_flag once;
+    static cudaError_t st = cudaSuccess;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        st = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q);
+        if (st == cudaSuccess && q == cudaDriverEntryPointSuccess) fn = (EncodeFn)p;
+    });
+    if (!fn) throw Error(-3, "cuTensorMapEncodeTiled unavailable");
+    return fn;
+}
 
 }  // namespace
 }  // namespace adc
