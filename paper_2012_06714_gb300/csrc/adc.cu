@@ -27,6 +27,7 @@
 #include "common.cuh"
 #include "ladder_tc.cuh"
 #include "mlp.cuh"
+#include "pairs64.cuh"
 #include "subspace.cuh"
 
 using namespace adc;
@@ -57,6 +58,7 @@ struct adc_handle {
     int* pair_idx = nullptr;  // [3][npairs] (i, a, b) for EA, (i, j, a) for IP
     LadderTC* tc = nullptr;  // tensor-core ladder state (BF16x3 operands of B^Q_vv; open shells: the alpha block)
     LadderTC* tc_b = nullptr;  // open shells: the beta virtual block's ladder state
+    Pairs64 pairs64;           // FP64 handles: the ladder's pair integrals, where they fit
     size_t pairs_limit = 0;    // device bytes the ladder's pair integrals may take (0: not held)
     int nva = 0;               // open shells: alpha virtual spin orbitals (the first nva of the v)
     // tensor-core ladder arithmetic: Davidson sigma, the setup ladder of t, and
@@ -106,6 +108,7 @@ struct adc_handle {
         return kind == ADC_EA ? (long long)v + (long long)o * v * v : (long long)o + (long long)o * o * v;
     }
     int n1() const { return kind == ADC_EA ? v : o; }
+    Reclaimable* held_for_speed() { return tc ? ladder_pairs_store(tc) : &pairs64.store; }
     double* dmalloc(size_t n) {
         void* p = dev_alloc(std::max<size_t>(n, 1) * sizeof(double), ctx.stream);
         owned.push_back(p);
@@ -441,6 +444,10 @@ static void ladder(adc_handle* h, const double* X, long long nmat, double* out, 
     }
     if (h->opt.precision != ADC_PREC_FP64 && h->tc) {
         ladder_tc_apply(*h->tc, c, X, nmat, out, md);
+        return;
+    }
+    if (h->pairs64.store.mem[0]) {
+        pairs64_apply(h->pairs64, c, X, nmat, out);
         return;
     }
     Scope sc(c.arena);
@@ -1093,7 +1100,7 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
     }
     tick(2);
     Scope setup_scope(c.arena);
-    PairsPin setup_pin(h->tc, c, true);
+    ReclaimPin setup_pin(h->held_for_speed(), c.stream, true);
     double* XL = nullptr;  // EA: the ladder term of the 1p-1p block, formed while the ladder of t is alive
     if (h->order >= 3) {
         const T T4 = op_t(h, false);
@@ -1102,6 +1109,10 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
         // 4 naux o^2 v^3 each without: they are made when that does not cost the setup more.
         const bool pairs = h->tc && (double)v * (Q + 2.0 * o * o) < 8.0 * Q * o * o &&
                            ladder_pairs_bytes((int)v) <= h->pairs_limit && ladder_pairs_prepare(*h->tc, c, h->Bvv);
+        // FP64: forming them and the ladder over them run on the tensor cores at some 20 times the rate
+        // of the FP64 units that the ladder over the auxiliary index takes
+        const bool p64 = h->opt.precision == ADC_PREC_FP64 && (double)v * (Q + o * o) < 80.0 * Q * o * o &&
+                         pairs64_bytes((int)v) <= h->pairs_limit && pairs64_prepare(h->pairs64, c, h->Bvv, (int)Q, (int)v);
         // three-plane pairs: partial sums promoted every K block, where the small products come first
         // and only four MMAs truncate at full size; no extrapolation
         const bool three = pairs && ladder_pairs_third(h->tc);
@@ -1169,6 +1180,10 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
                 ladder_pairs_drop(*h->tc, c);
             else
                 ladder_pairs_drop_third(*h->tc, c);
+        }
+        if (p64) {
+            check_flag(h, "setup");
+            if (h->kind != ADC_EA) h->pairs64.store.drop(c.stream);
         }
         tick(3);
         double* N = Lt;  // t2(2) numerator, formed in the ladder's buffer unless the ladder is kept
@@ -3026,7 +3041,7 @@ int adc_mlp_samples(adc_handle* h, int nroots, const int* iters, int n_iters, lo
             return ADC_ERR_ARG;
         }
     GUARD(h, {
-        PairsPin pin(h->tc, h->ctx, true);
+        ReclaimPin pin(h->held_for_speed(), h->ctx.stream, true);
         mlp_samples(h, nroots, iters, n_iters, per_vector, seed, exact_tol, d, blk, r, t);
         return ADC_OK;
     })
@@ -3108,7 +3123,7 @@ static int setup_one(const double* eps, const double* Bq, int nocc, int nvir, in
             ADC_CUDA(cudaMemGetInfo(&fr, &tot));
             lean = plain_bytes > 0.9 * (double)fr;
         }
-        if (h->opt.precision != ADC_PREC_FP64) {
+        {
             // the pair integrals of the ladder: at most a third of the free memory, and what the
             // plain layout's setup leaves (plain_bytes)
             size_t fr = 0, tot = 0;
@@ -3289,7 +3304,7 @@ int adc_sigma(adc_handle* h, const double* X, double* S, int nvec, int on_device
     }
     GUARD(h, {
         Ctx& c = h->ctx;
-        PairsPin pin(h->tc, c, true);
+        ReclaimPin pin(h->held_for_speed(), c.stream, true);
         const long long dim = h->dim();
         if (on_device) {
             sigma_device(h, X, S, nvec);
@@ -3314,7 +3329,7 @@ int adc_davidson(adc_handle* h, int nroots, double tol, const double* guess, dou
         return ADC_ERR_ARG;
     }
     GUARD(h, {
-        PairsPin pin(h->tc, h->ctx, !h->opt.cuda_graphs);  // (captured sigmas hold the integrals' address)
+        ReclaimPin pin(h->held_for_speed(), h->ctx.stream, !h->opt.cuda_graphs);  // (captured sigmas hold the integrals' address)
         int st = davidson(h, nroots, tol, guess, energies, specfac, vectors, stats);
         if (st == ADC_ERR_NOT_CONVERGED) h->err = "adc_davidson: not converged within max_iter";
         // the solver's scratch (subspace, residuals, sigma intermediates) goes back to the device:

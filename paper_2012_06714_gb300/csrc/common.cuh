@@ -35,8 +35,26 @@ struct Error : std::runtime_error {
                                std::string(#x) + ": cublas status " + std::to_string((int)s_));       \
     } while (0)
 
-// Releases device memory that handles without a call in progress hold for speed only (pair
-// integrals of the ladder, ladder_tc.cu) on the current device; false if there was none.
+// Device memory that a handle holds for speed only (the ladder's pair integrals).  It goes back to
+// the device when an allocation of any handle fails: that of handles with no call in progress
+// (no pins), and that of the failing call itself where it has said so (ReclaimPin::own).
+struct Reclaimable {
+    void* mem[2] = {};
+    int device = 0, pins = 0;
+    void hold(void* a, void* b);  // takes over stream-ordered allocations of the current device
+    void drop(cudaStream_t s);    // releases them, ordered on s
+    ~Reclaimable();
+};
+// A call that may use r (or NULL): while one is in progress r stays, except that, with own, a failing
+// allocation of the same host thread may release it after waiting for the stream.
+struct ReclaimPin {
+    Reclaimable *r, *before = nullptr;
+    cudaStream_t before_stream = nullptr;
+    ReclaimPin(Reclaimable* r, cudaStream_t s, bool own);
+    ~ReclaimPin();
+    ReclaimPin(const ReclaimPin&) = delete;
+};
+// Releases what can be released on the current device; false if there was nothing.
 bool device_memory_reclaim();
 
 // cudaMallocAsync that reclaims such memory once before it gives up

@@ -53,7 +53,8 @@ constexpr int DR = 8;    // rows per block at most
 struct DigitSide {
     Operand64 x;
     long long Kp;
-    __nv_bfloat16* out;  // [ND][rows][Kp], digit 0 the least significant
+    __nv_bfloat16* out;  // [ND] planes, `plane` apart, of [rows][Kp]; digit 0 the least significant
+    long long plane;
     int* ex;             // biased exponent field of the row's largest element (0x7ff: not finite)
     int row_lanes;       // the tensor's contiguous axis is the last row axis (else the lanes run along k)
     int R;               // rows per block, a power of two
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(DT) k_digits(const __grid_constant__ DigitSide
                     }
 #pragma unroll
                     for (int p = 0; p < ND; ++p)
-                        *(unsigned*)(sd.out + ((long long)p * x.rows + row0 + r) * sd.Kp + k0 + k) = dig[p];
+                        *(unsigned*)(sd.out + p * sd.plane + (row0 + r) * sd.Kp + k0 + k) = dig[p];
                 }
             }
         }
@@ -394,15 +395,15 @@ __global__ void __launch_bounds__(G_THREADS, 1)
     }
 }
 
-// digit planes [ND][rows][Kp] as a 3-D tensor {k, row, digit}, box {GK, box_rows, ND}, 64-byte swizzle
-CUtensorMap make_map_digits(const void* base, long long rows, long long Kp, int box_rows) {
+// digit planes as a 3-D tensor {k, row, digit}, box {GK, box_rows, ND}, 64-byte swizzle
+CUtensorMap make_map_digits(const Digits64& d, int box_rows) {
+    const long long rows = d.rows, Kp = d.Kp;
     CUtensorMap m;
     cuuint64_t dims[3] = {(cuuint64_t)Kp, (cuuint64_t)rows, ND};
-    cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)(rows * Kp * 2)};
+    cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)(d.plane * 2)};
     cuuint32_t box[3] = {GK, (cuuint32_t)box_rows, ND};
     cuuint32_t es[3] = {1, 1, 1};
-    const CUresult r = tensor_map_encoder()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
-                                            box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+    const CUresult r = tensor_map_encoder()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, d.d, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
                                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) throw Error(-3, "cuTensorMapEncodeTiled (digits) failed: " + std::to_string((int)r));
     return m;
@@ -414,25 +415,16 @@ int sm_count() {
     return n;
 }
 
-}  // namespace
+struct Gemm64Plan {
+    int BNT, S, kb;  // tile width, K slices, K blocks per slice
+};
 
-bool gemm64_fits(long long M, long long N, long long K) {
-    return M < (1LL << 30) && N < (1LL << 30) && K < (1LL << 30) && 2.0 * M * N * K >= 2e6 && std::max(M, N) >= 16;
-}
-
-double* gemm64(Ctx& c, const Operand64& A, const Operand64& B, double alpha, double beta, double* out, int& S) {
-    const long long M = A.rows, N = B.rows, K = A.K, Kp = (K + 7) / 8 * 8;
+// Tile width and K slices: least time over the chip.  A K block of a tile takes 17 BNT tensor cycles
+// twice (34 digit pairs), reading A from shared memory bounds it below about BNT = 16; a drain (every
+// EPOCH blocks) about 40 BNT cycles, which the MMAs wait for; the last one and the store about 60 BNT.
+Gemm64Plan plan64(long long M, long long N, long long Kp) {
     const int num_k = (int)((Kp + GK - 1) / GK), sms = sm_count();
-    if (!c.d_err) {
-        if (c.capturing) throw Error(-3, "error flag allocation during stream capture");
-        c.d_err = (int*)dev_alloc(sizeof(int), c.stream);
-        ADC_CUDA(cudaMemsetAsync(c.d_err, 0, sizeof(int), c.stream));
-    }
-    // tile width: least time over the chip.  A K block of a tile takes 17 BNT tensor cycles (34 digit
-    // pairs), reading A from shared memory bounds it below about BNT = 16; a drain (every EPOCH blocks)
-    // about 40 BNT cycles, which the MMAs wait for; the last one and the store about 60 BNT.
-    int BNT = 64;
-    long long best_s = 1;
+    Gemm64Plan p{64, 1, num_k};
     double best = 1e300;
     for (int b : {64, 48, 32, 16}) {
         const long long tiles = ((M + GM - 1) / GM) * ((N + b - 1) / b);
@@ -443,26 +435,75 @@ double* gemm64(Ctx& c, const Operand64& A, const Operand64& B, double alpha, dou
             const double blocks = (double)std::min<long long>(kb, num_k);
             const double cyc = rounds * (2000.0 + blocks * 2.0 * std::max(17.0 * b, 280.0) + (blocks / EPOCH) * 40.0 * b + 60.0 * b) +
                                (s - 1) * (double)M * N * 16.0 / 2500.0 + (s > 1 ? 4000.0 : 0.0);
-            if (cyc < best * 0.999) best = cyc, BNT = b, best_s = s;
+            if (cyc < best * 0.999) best = cyc, p = Gemm64Plan{b, (int)s, (int)kb};
         }
     }
-    const int kb = (int)(((num_k + best_s - 1) / best_s + EPOCH - 1) / EPOCH * EPOCH);
-    S = (num_k + kb - 1) / kb;
-    const bool direct = out && S == 1;
-    double* T = direct ? nullptr : c.arena.dalloc((size_t)S * M * N);
+    p.S = (num_k + p.kb - 1) / p.kb;
+    return p;
+}
+
+void launch64(Ctx& c, const Digits64& A, const Digits64& B, const Gemm64Plan& p, double* out, bool direct, double alpha,
+              double beta) {
+    if (!c.d_err) {
+        if (c.capturing) throw Error(-3, "error flag allocation during stream capture");
+        c.d_err = (int*)dev_alloc(sizeof(int), c.stream);
+        ADC_CUDA(cudaMemsetAsync(c.d_err, 0, sizeof(int), c.stream));
+    }
+    const int sms = sm_count(), num_k = (int)((A.Kp + GK - 1) / GK);
+    const CUtensorMap ma = make_map_digits(A, GM), mb = make_map_digits(B, p.BNT);
+    Gemm64Out o{};
+    o.M = (int)A.rows;
+    o.N = (int)B.rows;
+    o.mt = (int)((A.rows + GM - 1) / GM);
+    o.nt = (int)((B.rows + p.BNT - 1) / p.BNT);
+    o.S = p.S;
+    o.slice_kb = p.kb;
+    o.ea = A.ex;
+    o.eb = B.ex;
+    o.out = out;
+    o.alpha = alpha;
+    o.beta = beta;
+    o.direct = direct ? 1 : 0;
+    o.err = c.d_err;
+    const long long units = (long long)o.mt * o.nt * p.S;
+    if (units > (1LL << 30)) throw Error(-1, "gemm64: too many tiles");
+    const int stage = ND * (GM + p.BNT) * GK * 2;
+    const int stages = std::min(G_MAXST, (int)((G_SMEM - 1024) / stage));
+    int cols = 32;
+    while (cols < NL * p.BNT) cols *= 2;
+    static std::once_flag once[64];
+    int dev = 0;
+    ADC_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) throw Error(-3, "gemm64: device index out of range");
+    std::call_once(once[dev], [] { cudaFuncSetAttribute(k_gemm64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM); });
+    k_gemm64<<<(unsigned)std::min<long long>(units, sms), G_THREADS, G_SMEM, c.stream>>>(ma, mb, num_k, p.BNT, stages, cols, o);
+    ++c.kernels;
+    ADC_CUDA(cudaGetLastError());
+}
+
+}  // namespace
+
+bool gemm64_fits(long long M, long long N, long long K) {
+    return M < (1LL << 30) && N < (1LL << 30) && K < (1LL << 30) && 2.0 * M * N * K >= 2e6 && std::max(M, N) >= 16;
+}
+
+size_t digits64_bytes(long long rows, long long K) { return (size_t)ND * rows * ((K + 7) / 8 * 8) * 2; }
+
+void digitise64(Ctx& c, const Operand64* x, Digits64* out, int n) {
     DigitSide side[2];
-    const Operand64* ops[2] = {&A, &B};
-    int blocks[2];
-    Arena::Mark mk = c.arena.mark();
-    int* ex = (int*)c.arena.alloc((size_t)(M + N) * sizeof(int));
+    int blocks[2] = {0, 0};
+    const int sms = sm_count();
+    const long long Kp = out[0].Kp;
     // a row's K in one block up to this length (two reads in one launch), else in segments (two launches)
     const bool fused = Kp <= 1024;
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < n; ++i) {
         DigitSide& d = side[i];
-        d.x = *ops[i];
+        d.x = x[i];
         d.Kp = Kp;
-        d.out = (__nv_bfloat16*)c.arena.alloc((size_t)ND * d.x.rows * Kp * 2);
-        d.ex = ex + (i ? M : 0);
+        d.out = out[i].d;
+        d.plane = out[i].plane;
+        d.ex = out[i].ex;
+        if (x[i].K > Kp || out[i].Kp != Kp) throw Error(-1, "digitise64: shape mismatch");
         long long smallest = d.x.ks[d.x.nk - 1];
         d.row_lanes = 0;
         for (int j = 0; j < d.x.nk; ++j) smallest = std::min(smallest, d.x.kd[j] > 1 ? d.x.ks[j] : smallest);
@@ -474,12 +515,14 @@ double* gemm64(Ctx& c, const Operand64& A, const Operand64& B, double alpha, dou
         if (nb > (1LL << 30)) throw Error(-1, "gemm64: too many rows");
         blocks[i] = (int)nb;
     }
+    if (n < 2) side[1] = side[0];
     const unsigned bx = (unsigned)(blocks[0] + blocks[1]);
     if (fused) {
         k_digits<<<bx, DT, 0, c.stream>>>(side[0], side[1], blocks[0], Kp, 3);
         ++c.kernels;
     } else {
-        ADC_CUDA(cudaMemsetAsync(ex, 0, (size_t)(M + N) * sizeof(int), c.stream));
+        for (int i = 0; i < n; ++i)
+            ADC_CUDA(cudaMemsetAsync(side[i].ex, 0, (size_t)side[i].x.rows * sizeof(int), c.stream));
         for (int pass = 1; pass <= 2; ++pass) {
             long long seg = pass == 1 ? 2048 : 512;
             while ((Kp + seg - 1) / seg > 65535) seg *= 2;
@@ -488,36 +531,35 @@ double* gemm64(Ctx& c, const Operand64& A, const Operand64& B, double alpha, dou
         }
     }
     ADC_CUDA(cudaGetLastError());
-    const CUtensorMap ma = make_map_digits(side[0].out, M, Kp, GM), mb = make_map_digits(side[1].out, N, Kp, BNT);
-    Gemm64Out o{};
-    o.M = (int)M;
-    o.N = (int)N;
-    o.mt = (int)((M + GM - 1) / GM);
-    o.nt = (int)((N + BNT - 1) / BNT);
-    o.S = S;
-    o.slice_kb = kb;
-    o.ea = side[0].ex;
-    o.eb = side[1].ex;
-    o.out = direct ? out : T;
-    o.alpha = alpha;
-    o.beta = beta;
-    o.direct = direct ? 1 : 0;
-    o.err = c.d_err;
-    const long long units = (long long)o.mt * o.nt * S;
-    if (units > (1LL << 30)) throw Error(-1, "gemm64: too many tiles");
-    const int stage = ND * (GM + BNT) * GK * 2;
-    const int stages = std::min(G_MAXST, (int)((G_SMEM - 1024) / stage));
-    int cols = 32;
-    while (cols < NL * BNT) cols *= 2;
-    static std::once_flag once[64];
-    int dev = 0;
-    ADC_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) throw Error(-3, "gemm64: device index out of range");
-    std::call_once(once[dev], [] { cudaFuncSetAttribute(k_gemm64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM); });
-    k_gemm64<<<(unsigned)std::min<long long>(units, sms), G_THREADS, G_SMEM, c.stream>>>(ma, mb, num_k, BNT, stages, cols, o);
-    ++c.kernels;
-    ADC_CUDA(cudaGetLastError());
+}
+
+double* gemm64(Ctx& c, const Operand64& A, const Operand64& B, double alpha, double beta, double* out, int& S) {
+    const long long K = A.K, Kp = (K + 7) / 8 * 8;
+    const Operand64 ops[2] = {A, B};
+    Digits64 d[2];
+    // (the result is allocated first: it outlives the digits)
+    Gemm64Plan plan = plan64(A.rows, B.rows, Kp);
+    S = plan.S;
+    double* T = out && S == 1 ? nullptr : c.arena.dalloc((size_t)S * A.rows * B.rows);
+    Arena::Mark mk = c.arena.mark();
+    for (int i = 0; i < 2; ++i) {
+        d[i].rows = ops[i].rows;
+        d[i].Kp = Kp;
+        d[i].plane = ops[i].rows * Kp;
+        d[i].d = (__nv_bfloat16*)c.arena.alloc(digits64_bytes(ops[i].rows, K));
+        d[i].ex = (int*)c.arena.alloc((size_t)ops[i].rows * sizeof(int));
+    }
+    digitise64(c, ops, d, 2);
+    launch64(c, d[0], d[1], plan, T ? T : out, T == nullptr, alpha, beta);
     c.arena.release(mk);
+    return T;
+}
+
+double* gemm64_digits(Ctx& c, const Digits64& A, const Digits64& B, int& S) {
+    Gemm64Plan plan = plan64(A.rows, B.rows, A.Kp);
+    S = plan.S;
+    double* T = c.arena.dalloc((size_t)S * A.rows * B.rows);
+    launch64(c, A, B, plan, T, false, 1.0, 0.0);
     return T;
 }
 

@@ -1,5 +1,7 @@
 // FP64-accurate contractions on the BF16 tensor cores of sm_103a (gemm64.cu).
 #pragma once
+#include <cuda_bf16.h>
+
 #include "common.cuh"
 
 namespace adc {
@@ -26,5 +28,18 @@ bool gemm64_fits(long long M, long long N, long long K);
 // c.arena whose FP64 sum is C (without alpha and beta).  A bounded device wait that gives up raises
 // c.d_err.
 double* gemm64(Ctx& c, const Operand64& A, const Operand64& B, double alpha, double beta, double* out, int& S);
+
+// A matrix already in digits: planes (one per digit, `plane` elements apart) of [rows][Kp] (Kp a
+// multiple of 8, zeros beyond K) and the rows' exponents.
+struct Digits64 {
+    __nv_bfloat16* d = nullptr;
+    int* ex = nullptr;
+    long long rows = 0, Kp = 0, plane = 0;
+};
+size_t digits64_bytes(long long rows, long long K);  // of all planes
+// one or two operands (of one Kp) into the caller's planes
+void digitise64(Ctx& c, const Operand64* x, Digits64* out, int n);
+// gemm64 of such matrices, never in place
+double* gemm64_digits(Ctx& c, const Digits64& A, const Digits64& B, int& S);
 
 }  // namespace adc

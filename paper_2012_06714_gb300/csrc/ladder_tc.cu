@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "ladder_tc.cuh"
+#include "pairs.cuh"
 #include "tcgen05.cuh"
 
 namespace adc {
@@ -456,6 +457,9 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 // ---- operand preparation (FP64 -> split BF16) --------------------------------
+struct Planes {
+    __nv_bfloat16* p[3];
+};
 // x = p0 + p1 (+ p2) with every plane in BF16 (successive remainders, formed in FP32: its 24 bits hold
 // what three planes do, and FP64 arithmetic would bound the kernels below)
 __device__ __forceinline__ void splitp(float x, int planes, __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2) {
@@ -466,11 +470,24 @@ __device__ __forceinline__ void splitp(float x, int planes, __nv_bfloat16* p0, _
     *p1 = m;
     if (planes == 3) *p2 = __float2bfloat16(x - __bfloat162float(m));
 }
+// pairs split into two or three (o.p[2] not NULL) BF16 planes o.p[plane][(half * rows + row) * Pk + p],
+// zeros for P <= p < Pk
+struct PutPlanes {
+    Planes o;
+    long long rows, P, Pk, row0;
+    __device__ void operator()(int half, long long row, long long p, double x) const { (*this)(half, row, p, (float)x); }
+    __device__ void operator()(int half, long long row, long long p, float x) const {
+        const long long ad = (half * rows + row) * Pk + p;
+        splitp(x, o.p[2] ? 3 : 2, o.p[0] + ad, o.p[1] + ad, o.p[2] + ad);
+    }
+    __device__ void pad(long long row, int i) const {
+        if (i >= Pk - P) return;
+        for (int k = 0; k < 3; ++k)
+            if (o.p[k]) o.p[k][row * Pk + P + i] = o.p[k][(rows + row) * Pk + P + i] = __float2bfloat16(0.0f);
+    }
+};
 #define GRID_STRIDE(i, n) for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (n); i += (long long)gridDim.x * blockDim.x)
 
-struct Planes {
-    __nv_bfloat16* p[3];
-};
 
 // Bs[(Q,a')][c'] = B^Q[a][c] (a, c < v), zero pad: a' and c' both run over vp,
 // so that GEMM1's 32-row warp slices never straddle two auxiliary functions
@@ -508,103 +525,6 @@ __global__ void k_split_XT(const double* __restrict__ X, long long nmat, int va,
         long long m = r / vpb;
         double val = (cp < va && d < vb) ? X[(m * va + cp) * vb + d] : 0.0;
         splitp((float)val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
-    }
-}
-
-// ---- pair-adapted ladder: operands and result ---------------------------------------
-// A v x v matrix x as its pairs c >= d, p = c (c + 1) / 2 + d: half 0 x_cd + x_dc, half 1
-// x_cd - x_dc, each split into two or three (o.p[2] not NULL) BF16 planes
-// o.p[plane][(half * rows + row) * Pk + p] (zeros for P <= p < Pk).  Matrix m of the input: element (r, s) at in[base(m) + r * rs + s].
-//   integrals (Tin float): m -> a = a0 + m / nb, b = m % nb (b <= a, others skipped), the matrix
-//     (ac|bd) over (c, d), row a (a + 1) / 2 + b of the planes; the diagonal c = d holds 2 (ac|bc)
-//   vectors (Tin double): matrix m is row m; the diagonal holds x_cc
-// Bound by HBM: every element is read once (32 x 32 tiles, the mirrored tile through shared
-// memory) and written as four or six 2-byte values.
-template <typename Tin>
-__global__ void __launch_bounds__(256) k_pair_planes(const Tin* __restrict__ in, int v, long long nmat, long long ms,
-                                                     long long rs, int integrals, int a0, int nb, long long rows,
-                                                     long long P, long long Pk, Planes o) {
-    __shared__ Tin t1[32][33], t2[32][33];
-    const int nt = (v + 31) / 32;
-    const long long ntri = (long long)nt * (nt + 1) / 2;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    for (long long u = blockIdx.x; u < nmat * ntri; u += gridDim.x) {
-        const long long m = u / ntri;
-        int r = (int)(u - m * ntri), ct = (int)((sqrtf(8.0f * r + 1.0f) - 1.0f) * 0.5f);
-        while ((ct + 1) * (ct + 2) / 2 <= r) ++ct;
-        while (ct * (ct + 1) / 2 > r) --ct;
-        const int dt = r - ct * (ct + 1) / 2, c0 = ct * 32, d0 = dt * 32;
-        long long row = m, base = m * ms;
-        if (integrals) {
-            const long long a = m / nb, b = m - a * nb;
-            if (b > a0 + a) continue;  // uniform over the block
-            row = (a0 + a) * (a0 + a + 1) / 2 + b;
-            base = a * v * rs + b * v;
-        }
-        for (int i = ty; i < 32; i += 8) {
-            const int cc = c0 + i, dd = d0 + tx;
-            t1[i][tx] = cc < v && dd < v ? in[base + (long long)cc * rs + dd] : (Tin)0;
-            const int c2 = d0 + i, d2 = c0 + tx;  // the mirrored tile: rows d, columns c
-            t2[i][tx] = c2 < v && d2 < v ? in[base + (long long)c2 * rs + d2] : (Tin)0;
-        }
-        __syncthreads();
-        for (int i = ty; i < 32; i += 8) {
-            const int cc = c0 + i, dd = d0 + tx;
-            if (cc < v && dd <= cc) {
-                const Tin x = t1[i][tx], y = t2[tx][i];
-                const float ps = (float)(dd == cc && !integrals ? x : x + y), pa = (float)(x - y);
-                const long long p = (long long)cc * (cc + 1) / 2 + dd, o0 = row * Pk + p, o1 = (rows + row) * Pk + p;
-                const int planes = o.p[2] ? 3 : 2;
-                splitp(ps, planes, o.p[0] + o0, o.p[1] + o0, o.p[2] + o0);
-                splitp(pa, planes, o.p[0] + o1, o.p[1] + o1, o.p[2] + o1);
-            }
-        }
-        if (ct == nt - 1 && dt == nt - 1 && ty == 0 && tx < Pk - P) {
-            for (int p = 0; p < 3; ++p)
-                if (o.p[p]) o.p[p][row * Pk + P + tx] = o.p[p][(rows + row) * Pk + P + tx] = __float2bfloat16(0.0f);
-        }
-        __syncthreads();
-    }
-}
-
-// out[m][a][b] += (S + A) / 2 and out[m][b][a] += (S - A) / 2 for the pairs a >= b, with S and A
-// the FP64 sums over the K slices of T[half][slice][p][m] (p = a (a + 1) / 2 + b, halves 0 and 1).
-// 16 x 16 pair tiles x 8 matrices through shared memory: T is read in whole sectors along m, out
-// updated along its rows in both orientations.
-__global__ void __launch_bounds__(256) k_pair_unfold(const float* __restrict__ T, int slices, long long P, int nm, int v,
-                                                     double* __restrict__ out) {
-    __shared__ double u[8][16][17], w[8][16][17];
-    const int nt = (v + 15) / 16, nmt = (nm + 7) / 8;
-    const long long ntri = (long long)nt * (nt + 1) / 2, part = P * nm;
-    for (long long blk = blockIdx.x; blk < ntri * nmt; blk += gridDim.x) {
-        const int r = (int)(blk / nmt), m0 = (int)(blk % nmt) * 8;
-        int at = (int)((sqrtf(8.0f * r + 1.0f) - 1.0f) * 0.5f);
-        while ((at + 1) * (at + 2) / 2 <= r) ++at;
-        while (at * (at + 1) / 2 > r) --at;
-        const int bt = r - at * (at + 1) / 2, a0 = at * 16, b0 = bt * 16;
-        const int mi = threadIdx.x & 7, m = m0 + mi;
-        for (int e = threadIdx.x >> 3; e < 256; e += 32) {
-            const int a = a0 + e / 16, b = b0 + e % 16;
-            if (a < v && b <= a && m < nm) {
-                const float* t = T + ((long long)a * (a + 1) / 2 + b) * nm + m;
-                double S = 0.0, A = 0.0;
-                for (int k = 0; k < slices; ++k) {
-                    S += (double)t[k * part];
-                    A += (double)t[(slices + k) * part];
-                }
-                u[mi][e / 16][e % 16] = 0.5 * (S + A);
-                w[mi][e / 16][e % 16] = 0.5 * (S - A);
-            }
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < 8 * 256; e += 256) {
-            const int k = e / 256, i = (e / 16) % 16, j = e % 16, mm = m0 + k;
-            if (mm >= nm) continue;
-            if (a0 + i < v && b0 + j <= a0 + i) out[((long long)mm * v + a0 + i) * v + b0 + j] += u[k][i][j];
-            // the mirrored tile: rows b, columns a > b
-            if (b0 + i < v && a0 + j < v && b0 + i < a0 + j) out[((long long)mm * v + b0 + i) * v + a0 + j] += w[k][j][i];
-        }
-        __syncthreads();
     }
 }
 
@@ -771,8 +691,6 @@ void launch_gemm(Ctx& c, const Maps& maps, int planes, int a_row0, int b_x0, int
 
 }  // namespace
 
-static void ladder_pairs_forget(LadderTC* L);
-
 struct LadderTC {
     int naux = 0, v = 0, vp = 0, chunk = 0;
     int bn2[4] = {256, 256, 256, 256};  // GEMM2 tile width by plane count (2 or 3)
@@ -781,14 +699,15 @@ struct LadderTC {
     __nv_bfloat16 *Bs[3] = {}, *Bp[3] = {};  // BF16 planes of B^Q in the GEMM1-A and GEMM2-B layouts
     CUtensorMap mBs[3];                       // GEMM1-A maps
     int* d_err = nullptr;
-    // pair-adapted integrals (ladder_pairs_prepare): planes [2 halves][P][Pk], NULL when not held
-    __nv_bfloat16* pairs[3] = {};  // (the third plane has an allocation of its own, held during setup)
+    // pair-adapted integrals (ladder_pairs_prepare): planes [2 halves][P][Pk], NULL when not held (the
+    // third plane has an allocation of its own, held during setup)
+    Reclaimable store;
     long long P = 0, Pk = 0;
-    int device = 0, pins = 0;  // pins: calls in progress that may read the pairs (g_pairs_mu)
+    __nv_bfloat16* pair_plane(int p) const {
+        if (p == 2 || !store.mem[0]) return p == 2 ? (__nv_bfloat16*)store.mem[1] : nullptr;
+        return (__nv_bfloat16*)store.mem[0] + p * 2 * P * Pk;
+    }
     ~LadderTC() {
-        ladder_pairs_forget(this);
-        cudaFree(pairs[0]);
-        cudaFree(pairs[2]);
         for (int p = 0; p < 3; ++p) {
             cudaFree(Bs[p]);
             cudaFree(Bp[p]);
@@ -999,81 +918,25 @@ TuneCache* tune_cache_open(const char* path) {
 // ---- the ladder over pair-adapted integrals ----------------------------------------
 // With x+-_cd = x_cd +- x_dc, the symmetric and antisymmetric parts of the ladder are
 //   out_ab +- out_ba = sum_{c>=d} V+-_{ab,cd} x+-_cd,  V+-_{ab,cd} = (ac|bd) +- (ad|bc)
-// (diagonal weights in k_pair_planes): nmat v^4 flops for nmat matrices instead of the
+// (diagonal weights in k_pair_pack): nmat v^4 flops for nmat matrices instead of the
 // 4 naux v^3 nmat of the two-GEMM form over the auxiliary index, i.e. 4 naux / v times fewer (13
 // at 180 virtuals and 600 auxiliary functions, 14 at 400 / 1400).  The integrals cost naux v^4
 // flops once per handle and 4 v^4 bytes (two BF16 planes of both halves: 4.2 GB at v = 180, 51 GB
 // at 400), so they are held where that fits the device and the two-GEMM form stays for the rest.
 // Measured, a sigma of 4 vectors at 20/180/600: 7.9 -> 4.0 ms; at 40/400/1400: 159 -> 36 ms.
 //
-// The integrals are a convenience and go back to the device when an allocation of any handle
-// fails (device_memory_reclaim): those of handles with no call in progress (pins == 0), and those
-// of the call that fails itself, outside a ladder and outside a solve that replays CUDA graphs.
+// The integrals are a convenience (Reclaimable): they go back to the device when an allocation fails.
 namespace {
-std::mutex g_pairs_mu;
-std::vector<LadderTC*> g_pairs;  // holders of pair integrals
-// the handle whose call runs on this host thread, if that call may give its own integrals up
-thread_local LadderTC* tl_own = nullptr;
-thread_local cudaStream_t tl_own_stream = nullptr;
-
 constexpr long long kPairSliceK = 16384;  // FP32 register sums of at most this many terms, FP64 beyond
 }  // namespace
 
-static void ladder_pairs_forget(LadderTC* L) {
-    std::lock_guard<std::mutex> lk(g_pairs_mu);
-    g_pairs.erase(std::remove(g_pairs.begin(), g_pairs.end(), L), g_pairs.end());
-}
+Reclaimable* ladder_pairs_store(LadderTC* L) { return L ? &L->store : nullptr; }
 
-PairsPin::PairsPin(LadderTC* l, Ctx& c, bool own) : L(l) {
-    if (!L) return;
-    std::lock_guard<std::mutex> lk(g_pairs_mu);
-    ++L->pins;
-    before = tl_own;
-    tl_own = own ? L : nullptr;
-    tl_own_stream = c.stream;
-}
-PairsPin::~PairsPin() {
-    if (!L) return;
-    std::lock_guard<std::mutex> lk(g_pairs_mu);
-    --L->pins;
-    tl_own = (LadderTC*)before;
-}
-
-void ladder_pairs_drop(LadderTC& L, Ctx& c) {
-    if (!L.pairs[0]) return;
-    ladder_pairs_forget(&L);
-    cudaFreeAsync(L.pairs[0], c.stream);
-    L.pairs[0] = L.pairs[1] = nullptr;
-    ladder_pairs_drop_third(L, c);
-}
+void ladder_pairs_drop(LadderTC& L, Ctx& c) { L.store.drop(c.stream); }
 
 void ladder_pairs_drop_third(LadderTC& L, Ctx& c) {
-    if (L.pairs[2]) cudaFreeAsync(L.pairs[2], c.stream);
-    L.pairs[2] = nullptr;
-}
-
-bool device_memory_reclaim() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    std::lock_guard<std::mutex> lk(g_pairs_mu);
-    bool any = false;
-    for (size_t i = 0; i < g_pairs.size();) {
-        LadderTC* L = g_pairs[i];
-        const bool own = L == tl_own && L->pins == 1;
-        if (L->device != dev || (L->pins > 0 && !own)) {
-            ++i;
-            continue;
-        }
-        // a handle with no call in progress has no work in flight (every call returns after its
-        // work has completed); this thread's own call waits for what it has issued so far
-        if (own && cudaStreamSynchronize(tl_own_stream) != cudaSuccess) return any;
-        cudaFree(L->pairs[0]);
-        cudaFree(L->pairs[2]);
-        L->pairs[0] = L->pairs[1] = L->pairs[2] = nullptr;
-        g_pairs.erase(g_pairs.begin() + i);
-        any = true;
-    }
-    return any;
+    if (L.store.mem[1]) cudaFreeAsync(L.store.mem[1], c.stream);
+    L.store.mem[1] = nullptr;
 }
 
 size_t ladder_pairs_bytes(int v) {
@@ -1096,15 +959,8 @@ bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv) {
     }
     L.P = P;
     L.Pk = Pk;
-    L.pairs[2] = (__nv_bfloat16*)third;
-    L.pairs[0] = (__nv_bfloat16*)base;
-    L.pairs[1] = L.pairs[0] + 2 * P * Pk;
-    ADC_CUDA(cudaGetDevice(&L.device));
-    {
-        std::lock_guard<std::mutex> lk(g_pairs_mu);
-        g_pairs.push_back(&L);
-    }
-    PairsPin pin(&L, c, false);  // its own allocations may not take them away again
+    L.store.hold(base, third);
+    ReclaimPin pin(&L.store, c.stream, false);  // its own allocations may not take them away again
     Arena::Mark mk = c.arena.mark();
     // K-major planes of B^Q as [(p, q)][Q]: both operands of (ac|bd) = sum_Q B^Q_ac B^Q_bd
     // in three planes (the six products of order <= 2): with two, the dropped lo * lo products of the
@@ -1138,8 +994,8 @@ bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv) {
         // partial sums promoted every K block: the integrals enter the setup ladder too
         launch_gemm(c, m, 3, (int)(a0 * v), 0, e.M, e.N, (int)Qp, BN1[3], 1, 1, e, 2.0 * na * v * nb * v * Q);
         const long long nt = (v + 31) / 32, tiles = na * nb * nt * (nt + 1) / 2;
-        k_pair_planes<float><<<(unsigned)std::min<long long>(tiles, 152LL * 16), dim3(32, 8), 0, c.stream>>>(
-            G, (int)v, na * nb, 0, nb * v, 1, (int)a0, (int)nb, P, P, Pk, Planes{{L.pairs[0], L.pairs[1], L.pairs[2]}});
+        k_pair_pack<float, PutPlanes><<<(unsigned)std::min<long long>(tiles, 152LL * 16), dim3(32, 8), 0, c.stream>>>(
+            G, (int)v, na * nb, 0, nb * v, 1, (int)a0, (int)nb, PutPlanes{Planes{{L.pair_plane(0), L.pair_plane(1), L.pair_plane(2)}}, P, P, Pk, 0});
         ++c.kernels;
         ADC_CUDA(cudaGetLastError());
         c.arena.release(m2);
@@ -1149,7 +1005,7 @@ bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv) {
     return true;
 }
 
-bool ladder_pairs_third(const LadderTC* L) { return L && L->pairs[2]; }
+bool ladder_pairs_third(const LadderTC* L) { return L && L->store.mem[1]; }
 
 namespace {
 
@@ -1176,7 +1032,7 @@ float* pairs_gemm(LadderTC& L, Ctx& c, const Planes& x, int planes, long long nm
     float* T = (float*)c.arena.alloc((size_t)(2 * S * P * nm) * sizeof(float));
     Maps m{};
     for (int p = 0; p < planes; ++p) {
-        m.a[p] = make_map(L.pairs[p], 2 * P, Pk, BM);
+        m.a[p] = make_map(L.pair_plane(p), 2 * P, Pk, BM);
         m.b[p] = make_map(x.p[p], 2 * nm, Pk, bn / 2);
     }
     Epi e{};
@@ -1204,7 +1060,7 @@ void pairs_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* o
     // groups of matrices whose split vectors (8 or 12 P bytes each) and FP32 results stay within ~4 GiB
     const long long smin = (Pk + kPairSliceK - 1) / kPairSliceK;
     const long long mg = std::max<long long>(1, std::min<long long>(nmat, (4LL << 30) / (4 * planes * Pk + 8 * P * (smin + 2))));
-    PairsPin pin(&L, c, false);  // its own allocations may not take the integrals away
+    ReclaimPin pin(&L.store, c.stream, false);  // its own allocations may not take the integrals away
     for (long long m0 = 0; m0 < nmat; m0 += mg) {
         const long long nm = std::min(mg, nmat - m0);
         Arena::Mark mk = c.arena.mark();
@@ -1212,8 +1068,8 @@ void pairs_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* o
         x.p[0] = (__nv_bfloat16*)c.arena.alloc(planes * 2 * nm * Pk * 2);
         for (int p = 1; p < planes; ++p) x.p[p] = x.p[p - 1] + 2 * nm * Pk;
         const long long nt = (v + 31) / 32, tiles = nm * nt * (nt + 1) / 2;
-        k_pair_planes<double><<<(unsigned)std::min<long long>(tiles, 152LL * 16), dim3(32, 8), 0, c.stream>>>(
-            X + m0 * v * v, (int)v, nm, v * v, v, 0, 0, 1, nm, P, Pk, x);
+        k_pair_pack<double, PutPlanes><<<(unsigned)std::min<long long>(tiles, 152LL * 16), dim3(32, 8), 0, c.stream>>>(
+            X + m0 * v * v, (int)v, nm, v * v, v, 0, 0, 1, PutPlanes{x, nm, P, Pk, 0});
         ++c.kernels;
         ADC_CUDA(cudaGetLastError());
         int bn = pick_bn((int)nm, maxbn), S = 1;
@@ -1240,8 +1096,8 @@ void pairs_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* o
         }
         const float* T = pairs_gemm(L, c, x, planes, nm, bn, md.epoch2, S);
         const long long ut = (v + 15) / 16, blocks = ut * (ut + 1) / 2 * ((nm + 7) / 8);
-        k_pair_unfold<<<(unsigned)std::min<long long>(blocks, 152LL * 32), 256, 0, c.stream>>>(T, S, P, (int)nm, (int)v,
-                                                                                           out + m0 * v * v);
+        k_pair_unfold<float><<<(unsigned)std::min<long long>(blocks, 152LL * 32), 256, 0, c.stream>>>(
+            T, T + (long long)S * P * nm, S, P, (int)nm, (int)v, out + m0 * v * v);
         ++c.kernels;
         ADC_CUDA(cudaGetLastError());
         c.arena.release(mk);
@@ -1260,8 +1116,8 @@ void ladder_tc_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, doubl
     // sigma's only (its error there is no larger: 5.2e-7 against 6.0e-7 at 20/180/600); the setup
     // ladder takes three (md.planes == 3) and the refinement the two-GEMM form.
     const double v = L.v;
-    const bool accurate = md.planes == 3 && L.pairs[2];
-    const bool pairs = L.pairs[0] && (accurate || (md.planes == 2 && md.epoch1 == 0)) && (accurate || nmat * (double)L.naux >= 65.0 * v || 4.0 * v * v * v * v < 9e7);
+    const bool accurate = md.planes == 3 && L.store.mem[1];
+    const bool pairs = L.store.mem[0] && (accurate || (md.planes == 2 && md.epoch1 == 0)) && (accurate || nmat * (double)L.naux >= 65.0 * v || 4.0 * v * v * v * v < 9e7);
     if (pairs)
         pairs_apply(L, c, X, nmat, out, md);
     else

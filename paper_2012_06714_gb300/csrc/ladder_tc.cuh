@@ -41,16 +41,7 @@ bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv);
 bool ladder_pairs_third(const LadderTC* L);
 void ladder_pairs_drop_third(LadderTC& L, Ctx& c);
 void ladder_pairs_drop(LadderTC& L, Ctx& c);
-// A call that may use L's integrals (L may be NULL): while one is in progress they stay, except
-// that, with own, an allocation of the same host thread that fails may release them (the ladder
-// then takes the two-GEMM form).
-struct PairsPin {
-    LadderTC* L;
-    void* before = nullptr;
-    PairsPin(LadderTC* L, Ctx& c, bool own);
-    ~PairsPin();
-    PairsPin(const PairsPin&) = delete;
-};
+Reclaimable* ladder_pairs_store(LadderTC* L);  // (NULL for NULL)
 bool ladder_tc_apply_scratch(LadderTC& L, Ctx& c, const double* X, long long nmat, double* out, const LadderMode& md,
                              void* scratch, size_t bytes);
 
