@@ -223,17 +223,47 @@ struct Gemm64Out {
     int* err;
 };
 
+// The digit products of one 16-deep K step: every MMA multiplies digit i of A with nj digits of B.
+// Unrolled at compile time: one thread issues them all, and address arithmetic between them would
+// cost it more than the MMAs take.  kFirst: first step of an epoch (accumulators are started).
+template <int BNT, bool kFirst>
+__device__ __forceinline__ void digit_products(uint32_t tmem, uint64_t a, uint64_t b) {
+    constexpr uint32_t ib = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GM >> 4) << 24);
+    constexpr int jmax = 256 / BNT;  // digits of B per MMA
+#pragma unroll
+    for (int i = ND - 1; i >= 0; --i) {
+        int j = SMIN - i > 0 ? SMIN - i : 0;
+        // the lowest weight first appears at i = SMIN, j = 0: alone, to start its accumulator
+        if (kFirst && i == SMIN && j == 0) {
+            mma_bf16(tmem, a + (uint64_t)(i * (GM * GK * 2 >> 4)), b, ib | ((uint32_t)(BNT >> 3) << 17), 0u);
+            j = 1;
+        }
+        const int parts = (ND - j + jmax - 1) / jmax, nj = (ND - j + parts - 1) / parts;  // nearly equal widths
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q < parts) {
+                const int j0 = j + q * nj, n = nj < ND - j0 ? nj : ND - j0;
+                mma_bf16(tmem + (uint32_t)((i + j0 - SMIN) * BNT), a + (uint64_t)(i * (GM * GK * 2 >> 4)),
+                         b + (uint64_t)(j0 * (BNT * GK * 2 >> 4)), ib | ((uint32_t)(n * BNT >> 3) << 17),
+                         kFirst && i == ND - 1 ? 0u : 1u);
+            }
+        }
+    }
+}
+
+template <int BNT>
 __global__ void __launch_bounds__(G_THREADS, 1)
-    k_gemm64(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb, int num_k, int BNT, int stages,
-             int tmem_cols, Gemm64Out o) {
+    k_gemm64(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb, int num_k, int stages,
+             Gemm64Out o) {
+    constexpr int tmem_cols = BNT <= 16 ? 128 : BNT <= 32 ? 256 : 512;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ uint64_t full_bar[G_MAXST], empty_bar[G_MAXST], tfull, tempty, done_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int A_PL = GM * GK * 2, B_PL = BNT * GK * 2;
-    const int STAGE = ND * (A_PL + B_PL);
+    constexpr int A_PL = GM * GK * 2, B_PL = BNT * GK * 2;
+    constexpr int STAGE = ND * (A_PL + B_PL);
     const int tiles = o.mt * o.nt, nunits = tiles * o.S;
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
@@ -282,8 +312,6 @@ __global__ void __launch_bounds__(G_THREADS, 1)
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t ib = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GM >> 4) << 24);
-            const int jmax = 256 / BNT;  // digits of B per MMA
             long long g = 0, e = 0;
             bool ok = true;
             for (int u = blockIdx.x; u < nunits && ok && !abort_flag; u += gridDim.x) {
@@ -297,22 +325,11 @@ __global__ void __launch_bounds__(G_THREADS, 1)
                     }
                     fence_after();
                     const uint64_t a0 = desc64(smem + (size_t)s * STAGE), b0 = desc64(smem + (size_t)s * STAGE + ND * A_PL);
-#pragma unroll
-                    for (int kk = 0; kk < GK / 16; ++kk) {
-                        const uint32_t later = in_epoch > 0 || kk > 0 ? 1u : 0u;  // 0: first products of this epoch
-                        for (int i = ND - 1; i >= 0; --i) {
-                            const uint64_t ad = a0 + (uint64_t)(i * (A_PL >> 4) + kk * 2);
-                            // the lowest weight first appears at i = ND - 2, j = 0: alone, to start its accumulator
-                            for (int j = max(0, SMIN - i); j < ND;) {
-                                int nj = min(jmax, ND - j);
-                                if (!later && i == SMIN && j == 0) nj = 1;
-                                const uint32_t acc = later || !(i == ND - 1 || (i == SMIN && j == 0)) ? 1u : 0u;
-                                mma_bf16(tmem + (uint32_t)((i + j - SMIN) * BNT), ad,
-                                         b0 + (uint64_t)(j * (B_PL >> 4) + kk * 2), ib | ((uint32_t)(nj * BNT >> 3) << 17), acc);
-                                j += nj;
-                            }
-                        }
-                    }
+                    if (in_epoch == 0)
+                        digit_products<BNT, true>(tmem, a0, b0);
+                    else
+                        digit_products<BNT, false>(tmem, a0, b0);
+                    digit_products<BNT, false>(tmem, a0 + 2, b0 + 2);  // 16 BF16 = 32 bytes along K
                     mma_commit(&empty_bar[s]);
                     if (in_epoch == EPOCH - 1 || kb == kb1 - 1) {
                         mma_commit(&tfull);
@@ -323,15 +340,19 @@ __global__ void __launch_bounds__(G_THREADS, 1)
             mma_commit(&done_bar);
         }
     } else {
-        const int ew = warp - 2, quarter = warp & 3, half = ew >> 2, cw = BNT >> 1, cbeg = half * cw;
+        const int ew = warp - 2, quarter = warp & 3, half = ew >> 2;
+        constexpr int cw = BNT / 2;
+        const int cbeg = half * cw;
+        // staging of the results (after the pipeline stages): a row of 8 results per lane, padded
+        double* stg = (double*)(smem + (size_t)stages * STAGE) + ew * 32 * 9;
         long long e = 0;
         bool ok = true;
         for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
             const int sl = u / tiles, t = u - sl * tiles, m_tile = t % o.mt, n_tile = t / o.mt;
             const int kb0 = sl * o.slice_kb, epochs = (min(num_k, kb0 + o.slice_kb) - kb0 + EPOCH - 1) / EPOCH;
-            long long hi[32], lo[32];
+            long long hi[cw], lo[cw];
 #pragma unroll
-            for (int q = 0; q < 32; ++q) hi[q] = lo[q] = 0;
+            for (int q = 0; q < cw; ++q) hi[q] = lo[q] = 0;
             for (int i = 0; i < epochs; ++i, ++e) {
                 if (!mbar_wait(&tfull, (uint32_t)(e & 1), &abort_flag, o.err)) {
                     ok = false;
@@ -340,20 +361,18 @@ __global__ void __launch_bounds__(G_THREADS, 1)
                 fence_after();
                 const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)cbeg;
 #pragma unroll
-                for (int c0 = 0; c0 < 32; c0 += 8) {
-                    if (c0 < cw) {
-                        uint32_t r[NL][8];
+                for (int c0 = 0; c0 < cw; c0 += 8) {
+                    uint32_t r[NL][8];
 #pragma unroll
-                        for (int l = 0; l < NL; ++l) tmem_ld8(base + (uint32_t)(l * BNT + c0), r[l]);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    for (int l = 0; l < NL; ++l) tmem_ld8(base + (uint32_t)(l * BNT + c0), r[l]);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            int v[NL];
+                    for (int q = 0; q < 8; ++q) {
+                        int v[NL];
 #pragma unroll
-                            for (int l = 0; l < NL; ++l) v[l] = __float2int_rn(__uint_as_float(r[l][q]));
-                            hi[c0 + q] += (long long)v[7] * (1 << 24) + (long long)v[6] * (1 << 16) + (long long)v[5] * (1 << 8) + v[4];
-                            lo[c0 + q] += (long long)v[3] * (1 << 24) + (long long)v[2] * (1 << 16) + (long long)v[1] * (1 << 8) + v[0];
-                        }
+                        for (int l = 0; l < NL; ++l) v[l] = __float2int_rn(__uint_as_float(r[l][q]));
+                        hi[c0 + q] += (long long)v[7] * (1 << 24) + (long long)v[6] * (1 << 16) + (long long)v[5] * (1 << 8) + v[4];
+                        lo[c0 + q] += (long long)v[3] * (1 << 24) + (long long)v[2] * (1 << 16) + (long long)v[1] * (1 << 8) + v[0];
                     }
                 }
                 fence_before();
@@ -361,25 +380,37 @@ __global__ void __launch_bounds__(G_THREADS, 1)
                 if (lane == 0) mbar_arrive(&tempty);
             }
             if (!ok) break;
-            const int row = m_tile * GM + quarter * 32 + lane, colt = n_tile * BNT + cbeg;
-            if (row < o.M) {
-                const int ea = o.ea[row];
-                double* dst = o.out + ((long long)sl * o.M + row) * o.N + colt;
+            const int row0 = m_tile * GM + quarter * 32, row = row0 + lane, colt = n_tile * BNT + cbeg;
+            if (row0 >= o.M || colt >= o.N) continue;  // uniform over the warp
+            const int ea = row < o.M ? o.ea[row] : 0;
 #pragma unroll
-                for (int q = 0; q < 32; ++q) {
-                    if (q < cw && colt + q < o.N) {
-                        const int eb = o.eb[colt + q];
-                        // weights: digit products of weight s carry 2^(8 s); hi starts at s = 9, lo at s = 5;
-                        // a row's integers carry 2^(ef - 1078)
-                        double v = ea == 0x7ff || eb == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL)
-                                                              : to_double(hi[q], lo[q], 8 * SMIN + ea + eb - 2 * 1078);
+            for (int c0 = 0; c0 < cw; c0 += 8) {
+                // 32 rows x 8 columns through shared memory: whole sectors of the output rows
+                const int ebl = colt + c0 + (lane & 7) < o.N ? o.eb[colt + c0 + (lane & 7)] : 0;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int eb = __shfl_sync(0xffffffffu, ebl, q);
+                    // weights: digit products of weight s carry 2^(8 s); hi starts at s = 9, lo at s = 5;
+                    // a row's integers carry 2^(ef - 1078)
+                    stg[lane * 9 + q] = ea == 0x7ff || eb == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL)
+                                                                  : to_double(hi[c0 + q], lo[c0 + q], 8 * SMIN + ea + eb - 2 * 1078);
+                }
+                __syncwarp();
+                const int col = colt + c0 + (lane & 7);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int rr = i * 4 + (lane >> 3);
+                    if (row0 + rr < o.M && col < o.N) {
+                        double v = stg[rr * 9 + (lane & 7)];
+                        double* dst = o.out + ((long long)sl * o.M + row0 + rr) * o.N + col;
                         if (o.direct) {
                             if (o.alpha != 1.0) v *= o.alpha;
-                            if (o.beta != 0.0) v += o.beta == 1.0 ? dst[q] : o.beta * dst[q];
+                            if (o.beta != 0.0) v += o.beta == 1.0 ? *dst : o.beta * *dst;
                         }
-                        dst[q] = v;
+                        *dst = v;
                     }
                 }
+                __syncwarp();
             }
         }
     }
@@ -468,15 +499,17 @@ void launch64(Ctx& c, const Digits64& A, const Digits64& B, const Gemm64Plan& p,
     const long long units = (long long)o.mt * o.nt * p.S;
     if (units > (1LL << 30)) throw Error(-1, "gemm64: too many tiles");
     const int stage = ND * (GM + p.BNT) * GK * 2;
-    const int stages = std::min(G_MAXST, (int)((G_SMEM - 1024) / stage));
-    int cols = 32;
-    while (cols < NL * p.BNT) cols *= 2;
+    const int stages = std::min(G_MAXST, (int)((G_SMEM - 1024 - G_EPI * 32 * 9 * sizeof(double)) / stage));
     static std::once_flag once[64];
     int dev = 0;
     ADC_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) throw Error(-3, "gemm64: device index out of range");
-    std::call_once(once[dev], [] { cudaFuncSetAttribute(k_gemm64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM); });
-    k_gemm64<<<(unsigned)std::min<long long>(units, sms), G_THREADS, G_SMEM, c.stream>>>(ma, mb, num_k, p.BNT, stages, cols, o);
+    std::call_once(once[dev], [] {
+        for (auto k : {k_gemm64<16>, k_gemm64<32>, k_gemm64<48>, k_gemm64<64>})
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G_SMEM);
+    });
+    const auto kern = p.BNT == 16 ? k_gemm64<16> : p.BNT == 32 ? k_gemm64<32> : p.BNT == 48 ? k_gemm64<48> : k_gemm64<64>;
+    kern<<<(unsigned)std::min<long long>(units, sms), G_THREADS, G_SMEM, c.stream>>>(ma, mb, num_k, stages, o);
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
 }
@@ -524,7 +557,7 @@ void digitise64(Ctx& c, const Operand64* x, Digits64* out, int n) {
         for (int i = 0; i < n; ++i)
             ADC_CUDA(cudaMemsetAsync(side[i].ex, 0, (size_t)side[i].x.rows * sizeof(int), c.stream));
         for (int pass = 1; pass <= 2; ++pass) {
-            long long seg = pass == 1 ? 2048 : 512;
+            long long seg = 512;
             while ((Kp + seg - 1) / seg > 65535) seg *= 2;
             k_digits<<<dim3(bx, (unsigned)((Kp + seg - 1) / seg)), DT, 0, c.stream>>>(side[0], side[1], blocks[0], seg, pass);
             ++c.kernels;
