@@ -3130,6 +3130,8 @@ static int setup_one(const double* eps, const double* Bq, int nocc, int nvir, in
             ADC_CUDA(cudaMemGetInfo(&fr, &tot));
             const double left = 0.9 * (double)fr - plain_bytes;
             h->pairs_limit = (size_t)std::max(0.0, std::min((double)fr / 3.0, left));
+            // digits of constant operands of FP64 contractions (not on a lean handle)
+            if (!lean) h->ctx.cache64_bytes = std::min<size_t>(h->pairs_limit / 8, size_t(4) << 30);
         }
         if (lean) {
             h->lean = true;

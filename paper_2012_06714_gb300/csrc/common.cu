@@ -4,7 +4,6 @@
 #include <cstring>
 #include <map>
 #include <mutex>
-#include <type_traits>
 
 #include <cuda_bf16.h>
 
@@ -263,11 +262,10 @@ inline int grid_for(long long n) {
     return (int)std::min<long long>(std::max<long long>(g, 1), 152LL * 32);
 }
 
-// ---- own GEMM kernels for the small and skinny contractions of sigma ------------
-// Row-major A [M][K] (lda), B [K][N] (ldb).  F32: FP64 operands rounded to FP32 in
-// registers, FP32 products summed in FP32 over at most 64 terms, those partial sums
-// accumulated in FP64 (the FP32-accurate class); else FP64 throughout.  Each kernel
-// writes its K slice's partial result P[slice][m][n]; k_reduce_slices finishes
+// ---- own GEMM kernels for the skinny contractions of the mixed sigma ----------------
+// Row-major A [M][K] (lda), B [K][N] (ldb): FP64 operands rounded to FP32 in registers, FP32 products
+// summed in FP32 over at most 64 terms, those partial sums accumulated in FP64 (the FP32-accurate
+// class).  Each kernel writes its K slice's partial result P[slice][m][n]; k_reduce_slices finishes
 // C = alpha sum_slices P + beta C.
 
 constexpr int SK_THREADS = 256;
@@ -275,14 +273,12 @@ constexpr int SK_CHUNK = 64;  // FP32 partial-sum length
 
 // M <= MM rows of A (a few trial vectors): one thread per column n of B, the A values of
 // the current 256-deep K chunk in shared memory; reads B once, coalesced along n.
-template <int MM, bool F32>
+template <int MM>
 __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, long long K, long long kslice,
                                                          const double* __restrict__ A, long long lda,
                                                          const double* __restrict__ B, long long ldb,
                                                          double* __restrict__ P) {
-    // the A chunk in shared memory, already rounded to FP32 for the FP32-product form
-    using AT = typename std::conditional<F32, float, double>::type;
-    __shared__ AT As[MM][SK_THREADS];
+    __shared__ float As[MM][SK_THREADS];  // the A chunk, already rounded to FP32
     const long long n = blockIdx.x * (long long)SK_THREADS + threadIdx.x;
     const long long k0 = blockIdx.y * kslice, k1 = min(K, k0 + kslice);
     double acc[MM];
@@ -293,41 +289,29 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, lon
         __syncthreads();
         if (threadIdx.x < kn)
 #pragma unroll
-            for (int m = 0; m < MM; ++m) As[m][threadIdx.x] = (AT)(m < M ? A[m * lda + kc + threadIdx.x] : 0.0);
+            for (int m = 0; m < MM; ++m) As[m][threadIdx.x] = (float)(m < M ? A[m * lda + kc + threadIdx.x] : 0.0);
         __syncthreads();
         if (n >= N) continue;
         const double* b = B + kc * ldb + n;
         // U independent loads in flight per thread before their FMAs (the loop is bound by
         // memory latency otherwise)
         constexpr int U = 8;
-        if (F32) {
-            for (int k2 = 0; k2 < kn; k2 += SK_CHUNK) {
-                float part[MM];
+        for (int k2 = 0; k2 < kn; k2 += SK_CHUNK) {
+            float part[MM];
 #pragma unroll
-                for (int m = 0; m < MM; ++m) part[m] = 0.f;
-                const int ke = min(kn, k2 + SK_CHUNK);
-                for (int kk = k2; kk < ke; kk += U) {
-                    float bv[U];
+            for (int m = 0; m < MM; ++m) part[m] = 0.f;
+            const int ke = min(kn, k2 + SK_CHUNK);
+            for (int kk = k2; kk < ke; kk += U) {
+                float bv[U];
 #pragma unroll
-                    for (int u = 0; u < U; ++u) bv[u] = kk + u < ke ? (float)b[(long long)(kk + u) * ldb] : 0.f;
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-#pragma unroll
-                        for (int m = 0; m < MM; ++m) part[m] = fmaf(kk + u < ke ? (float)As[m][kk + u] : 0.f, bv[u], part[m]);
-                }
-#pragma unroll
-                for (int m = 0; m < MM; ++m) acc[m] += (double)part[m];
-            }
-        } else {
-            for (int kk = 0; kk < kn; kk += U) {
-                double bv[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) bv[u] = kk + u < kn ? b[(long long)(kk + u) * ldb] : 0.0;
+                for (int u = 0; u < U; ++u) bv[u] = kk + u < ke ? (float)b[(long long)(kk + u) * ldb] : 0.f;
 #pragma unroll
                 for (int u = 0; u < U; ++u)
 #pragma unroll
-                    for (int m = 0; m < MM; ++m) acc[m] = fma(kk + u < kn ? As[m][kk + u] : 0.0, bv[u], acc[m]);
+                    for (int m = 0; m < MM; ++m) part[m] = fmaf(kk + u < ke ? As[m][kk + u] : 0.f, bv[u], part[m]);
             }
+#pragma unroll
+            for (int m = 0; m < MM; ++m) acc[m] += (double)part[m];
         }
     }
     if (n < N)
@@ -338,7 +322,7 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, lon
 
 // N <= NN columns of B: one block per row m of A and K slice; threads stride over k
 // (A read coalesced), then a warp-shuffle and shared-memory reduction of the NN sums.
-template <int NN, bool F32>
+template <int NN>
 __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, long long K, long long kslice,
                                                          const double* __restrict__ A, long long lda,
                                                          const double* __restrict__ B, long long ldb,
@@ -350,45 +334,28 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, lon
 #pragma unroll
     for (int j = 0; j < NN; ++j) acc[j] = 0.0;
     const double* a = A + m * lda;
-    if (F32) {
-        // each thread takes up to SK_CHUNK of its strided terms per FP32 partial sum
-        for (long long kb = k0; kb < k1; kb += (long long)SK_THREADS * SK_CHUNK) {
-            float part[NN];
+    // each thread takes up to SK_CHUNK of its strided terms per FP32 partial sum
+    for (long long kb = k0; kb < k1; kb += (long long)SK_THREADS * SK_CHUNK) {
+        float part[NN];
 #pragma unroll
-            for (int j = 0; j < NN; ++j) part[j] = 0.f;
-            const long long ke = min(k1, kb + (long long)SK_THREADS * SK_CHUNK);
-            constexpr int U = 4;
-            for (long long k = kb + threadIdx.x; k < ke; k += (long long)U * SK_THREADS) {
-                double av[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) av[u] = k + u * SK_THREADS < ke ? a[k + u * SK_THREADS] : 0.0;
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const long long ku = k + u * SK_THREADS;
-                    if (ku < ke)
-#pragma unroll
-                        for (int j = 0; j < NN; ++j)
-                            if (j < N) part[j] = fmaf((float)av[u], (float)B[ku * ldb + j], part[j]);
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < NN; ++j) acc[j] += (double)part[j];
-        }
-    } else {
+        for (int j = 0; j < NN; ++j) part[j] = 0.f;
+        const long long ke = min(k1, kb + (long long)SK_THREADS * SK_CHUNK);
         constexpr int U = 4;
-        for (long long k = k0 + threadIdx.x; k < k1; k += (long long)U * SK_THREADS) {
+        for (long long k = kb + threadIdx.x; k < ke; k += (long long)U * SK_THREADS) {
             double av[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) av[u] = k + u * SK_THREADS < k1 ? a[k + u * SK_THREADS] : 0.0;
+            for (int u = 0; u < U; ++u) av[u] = k + u * SK_THREADS < ke ? a[k + u * SK_THREADS] : 0.0;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const long long ku = k + u * SK_THREADS;
-                if (ku < k1)
+                if (ku < ke)
 #pragma unroll
                     for (int j = 0; j < NN; ++j)
-                        if (j < N) acc[j] = fma(av[u], B[ku * ldb + j], acc[j]);
+                        if (j < N) part[j] = fmaf((float)av[u], (float)B[ku * ldb + j], part[j]);
             }
         }
+#pragma unroll
+        for (int j = 0; j < NN; ++j) acc[j] += (double)part[j];
     }
 #pragma unroll
     for (int j = 0; j < NN; ++j) {
@@ -402,49 +369,6 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, lon
         for (int w = 0; w < SK_THREADS / 32; ++w) x += red[w][threadIdx.x];
         P[((long long)blockIdx.y * M + m) * N + threadIdx.x] = x;
     }
-}
-
-// General small contraction in FP64: 64 x 64 output tiles, 16-deep K steps through
-// shared memory, 4 x 4 outputs per thread.
-__global__ void __launch_bounds__(256) k_tile_f64(long long M, long long N, long long K, const double* __restrict__ A,
-                                                  long long lda, const double* __restrict__ B, long long ldb,
-                                                  double* __restrict__ P) {
-    __shared__ double As[16][64 + 1];
-    __shared__ double Bs[16][64];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const long long m0 = blockIdx.y * 64LL, n0 = blockIdx.x * 64LL;
-    double acc[4][4] = {};
-    for (long long k0 = 0; k0 < K; k0 += 16) {
-        for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-            const int r = e / 16, kk = e % 16;
-            const long long gm = m0 + r, gk = k0 + kk;
-            As[kk][r] = (gm < M && gk < K) ? A[gm * lda + gk] : 0.0;
-            const int kb = e / 64, cn = e % 64;
-            const long long gn = n0 + cn, gk2 = k0 + kb;
-            Bs[kb][cn] = (gn < N && gk2 < K) ? B[gk2 * ldb + gn] : 0.0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) av[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const long long gm = m0 + ty * 4 + i, gn = n0 + tx * 4 + j;
-            if (gm < M && gn < N) P[gm * N + gn] = acc[i][j];
-        }
 }
 
 // As k_reduce_slices for many slices: one warp per output element, lanes over slices,
@@ -479,21 +403,21 @@ __global__ void k_reduce_slices(int S, long long M, long long N, const double* _
     }
 }
 
-template <int MM, bool F32>
+template <int MM>
 void launch_skinny_m(dim3 g, cudaStream_t st, int M, long long N, long long K, long long ks, const double* A, long long lda,
                      const double* B, long long ldb, double* P) {
-    k_skinny_m<MM, F32><<<g, SK_THREADS, 0, st>>>(M, N, K, ks, A, lda, B, ldb, P);
+    k_skinny_m<MM><<<g, SK_THREADS, 0, st>>>(M, N, K, ks, A, lda, B, ldb, P);
 }
-template <int NN, bool F32>
+template <int NN>
 void launch_skinny_n(dim3 g, cudaStream_t st, long long M, int N, long long K, long long ks, const double* A, long long lda,
                      const double* B, long long ldb, double* P) {
-    k_skinny_n<NN, F32><<<g, SK_THREADS, 0, st>>>(M, N, K, ks, A, lda, B, ldb, P);
+    k_skinny_n<NN><<<g, SK_THREADS, 0, st>>>(M, N, K, ks, A, lda, B, ldb, P);
 }
 
 }  // namespace
 
 void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const double* A, long long lda, const double* B,
-              long long ldb, double beta, double* C, long long ldc, bool f32) {
+              long long ldb, double beta, double* C, long long ldc) {
     if (M <= 0 || N <= 0) return;
     if (K <= 0) {
         for (long long m = 0; m < M; ++m) {
@@ -520,7 +444,7 @@ void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const
         switch ((int)M) {
 #define SKM(X)                                                              \
     case X:                                                                 \
-        if (f32) go(launch_skinny_m<X, true>); else go(launch_skinny_m<X, false>); \
+        go(launch_skinny_m<X>);                                             \
         break;
             SKM(1) SKM(2) SKM(3) SKM(4) SKM(5) SKM(6) SKM(7) SKM(8)
 #undef SKM
@@ -537,16 +461,13 @@ void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const
         switch ((int)N) {
 #define SKN(X)                                                              \
     case X:                                                                 \
-        if (f32) go(launch_skinny_n<X, true>); else go(launch_skinny_n<X, false>); \
+        go(launch_skinny_n<X>);                                             \
         break;
             SKN(1) SKN(2) SKN(3) SKN(4) SKN(5) SKN(6) SKN(7) SKN(8)
 #undef SKN
         }
     } else {
-        if ((M + 63) / 64 > 65535) throw Error(-1, "own_gemm: too many row tiles");
-        P = c.arena.dalloc((size_t)M * N);
-        dim3 g((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
-        k_tile_f64<<<g, 256, 0, c.stream>>>(M, N, K, A, lda, B, ldb, P);
+        throw Error(-1, "own_gemm: neither side is skinny");
     }
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
@@ -935,35 +856,73 @@ static void einsum_tc(Ctx& c, const std::string& la, const std::string& lb, cons
     permute_sum(c, T, S, sh, perm, C, c32, alpha, beta);
 }
 
-// FP64-accurate contraction on the tensor cores (gemm64): the operands are read in place, the
-// result written in place when it is in GEMM order, else permuted and accumulated in one pass.
+// FP64 contraction (gemm64 on the tensor cores, small64 below its sizes): the operands are read and
+// the result is written through their strides; K slices are summed by the permute that puts them in
+// place.
 static void einsum_64(Ctx& c, const std::string& la, const std::string& lb, const std::string& lc,
                       std::map<char, long long>& dim, const std::string& fa, const std::string& fb, const std::string& con,
                       double alpha, const T& A, const T& B, double beta, void* C, bool c32) {
-    auto operand = [&](const T& X, const std::string& l, const std::string& rows) {
-        Operand64 o;
-        o.p = X.p;
-        o.f32 = X.f32;
+    auto strides = [&](const std::string& l) {
         std::map<char, long long> st;
         long long acc = 1;
         for (int j = (int)l.size() - 1; j >= 0; --j) {
             st[l[j]] = acc;
             acc *= dim[l[j]];
         }
-        for (char x : rows) o.row_axis(dim[x], st[x]);
-        for (char x : con) o.k_axis(dim[x], st[x]);
+        return st;
+    };
+    auto operand = [&](const T& X, const std::string& l, const std::string& rows) {
+        Operand64 o;
+        o.p = X.p;
+        o.f32 = X.f32;
+        const auto st = strides(l);
+        for (char x : rows) o.row_axis(dim[x], st.at(x));
+        for (char x : con) o.k_axis(dim[x], st.at(x));
         if (o.nk == 0) o.k_axis(1, 1);
         return o;
     };
     Operand64 a = operand(A, la, fa), b = operand(B, lb, fb);
+    const bool tensor = gemm64_fits(a.rows, b.rows, a.K);
     // the 128-row axis takes the longer side when the other would leave it mostly empty
-    const bool swap = a.rows < 64 && b.rows > a.rows;
-    const std::string tord = swap ? fb + fa : fa + fb;
-    const bool in_place = tord == lc && !c32;
+    // (small64: the longer side on the grid's x axis)
+    const bool swap = tensor ? a.rows < 64 && b.rows > a.rows : a.rows > b.rows;
+    // digits of a constant operand, kept while there is room
+    Digits64 da, db;
+    auto kept = [&](const T& X, const Operand64& o, const std::string& l, const std::string& rows, Digits64& d) {
+        if (!tensor || !X.constant || c.cache64_bytes == 0) return false;
+        const size_t bytes = digits64_bytes(o.rows, o.K);
+        std::string key = l + ">" + rows + "," + con;
+        for (char x : l) key += ":" + std::to_string(dim[x]);
+        auto it = c.cache64.find({X.p, key});
+        if (it == c.cache64.end()) {
+            if (bytes > c.cache64_bytes || c.capturing) return false;
+            void* buf = dev_alloc(bytes, c.stream);
+            c.cache64_bytes -= bytes;
+            it = c.cache64.emplace(std::make_pair((const void*)X.p, key), buf).first;
+            d = digits64_in(buf, o.rows, o.K);
+            digitise64(c, &o, &d, 1);
+            return true;
+        }
+        d = digits64_in(it->second, o.rows, o.K);
+        return true;
+    };
+    const bool ka = kept(A, a, la, fa, da), kb = kept(B, b, lb, fb, db);
+    const std::string rows = swap ? fb : fa, cols = swap ? fa : fb;
+    Out64 out;
+    if (!c32) {
+        out.p = (double*)C;
+        out.alpha = alpha;
+        out.beta = beta;
+        const auto st = strides(lc);
+        for (char x : rows) out.row_axis(dim[x], st.at(x));
+        for (char x : cols) out.col_axis(dim[x], st.at(x));
+    }
     int S = 1;
-    const double* Tm = swap ? gemm64(c, b, a, alpha, beta, in_place ? (double*)C : nullptr, S)
-                            : gemm64(c, a, b, alpha, beta, in_place ? (double*)C : nullptr, S);
+    const double* Tm = !tensor ? (swap ? small64(c, b, a, out, S) : small64(c, a, b, out, S))
+                       : swap  ? gemm64(c, b, kb ? &db : nullptr, a, ka ? &da : nullptr, out, S)
+                               : gemm64(c, a, ka ? &da : nullptr, b, kb ? &db : nullptr, out, S);
     if (!Tm) return;
+    const std::string tord = rows + cols;
     Shape sh;
     sh.nd = (int)tord.size();
     int perm[kMaxDim];
@@ -1029,17 +988,17 @@ static void einsum_core(Ctx& c, const char* specstr, double alpha, const T& A, c
         const bool big_in_place = M <= N ? (!B.f32 && sp.b == con + fb) : (!A.f32 && sp.a == fa + con);
         if (big && tc_gemm_fits(M, N, K) && (!skinny || (big_const && !big_in_place))) {
             einsum_tc(c, sp.a, sp.b, sp.c, dim, fa, fb, con, alpha, A, B, beta, C, c32);
-        } else if (!big && !skinny && gemm64_fits(M, N, K)) {
+        } else if (!big || !skinny) {
             einsum_64(c, sp.a, sp.b, sp.c, dim, fa, fb, con, alpha, A, B, beta, C, c32);
         } else {
             const double* Ap = to_order(c, A.p, sp.a, dim, fa + con, A.f32);
             const double* Bp = to_order(c, B.p, sp.b, dim, con + fb, B.f32);
             const std::string tord = fa + fb;
             if (tord == sp.c && !c32) {
-                own_gemm(c, M, N, K, alpha, Ap, K, Bp, N, beta, (double*)C, N, big);
+                own_gemm(c, M, N, K, alpha, Ap, K, Bp, N, beta, (double*)C, N);
             } else {
                 double* Tm = c.arena.dalloc((size_t)(M * N));
-                own_gemm(c, M, N, K, 1.0, Ap, K, Bp, N, 0.0, Tm, N, big);
+                own_gemm(c, M, N, K, 1.0, Ap, K, Bp, N, 0.0, Tm, N);
                 Shape sh;
                 sh.nd = (int)tord.size();
                 for (int j = 0; j < sh.nd; ++j) sh.d[j] = dim[tord[j]];
@@ -1056,7 +1015,7 @@ static void einsum_core(Ctx& c, const char* specstr, double alpha, const T& A, c
         c.arena.release(mk);
         return;
     }
-    if (nb == 1 && gemm64_fits(M, N, K)) {
+    if (nb == 1 && K > 0 && (gemm64_fits(M, N, K) || (std::min(M, N) < 500000 && std::max(M, N) < (1LL << 31) && K < (1LL << 30)))) {
         einsum_64(c, sp.a, sp.b, sp.c, dim, fa, fb, con, alpha, A, B, beta, C, c32);
         c.arena.release(mk);
         return;

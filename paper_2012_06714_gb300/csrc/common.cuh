@@ -192,6 +192,9 @@ struct Ctx {
     std::map<std::pair<const void*, std::string>, float*> f32cache;
     // split BF16 planes (K-major GEMM operand order) of operands marked constant
     std::map<std::pair<const void*, std::string>, void*> bf16cache;
+    // digits of constant operands of FP64 contractions (gemm64), up to cache64_bytes in all
+    std::map<std::pair<const void*, std::string>, void*> cache64;
+    size_t cache64_bytes = 0;
     // constant operands are cached in these forms only if the copy is at most this size
     // (larger ones are converted per call into scratch)
     size_t cache_max_bytes = ~size_t(0);
@@ -203,6 +206,7 @@ struct Ctx {
     ~Ctx() {
         for (auto& kv : f32cache) cudaFree(kv.second);
         for (auto& kv : bf16cache) cudaFree(kv.second);
+        for (auto& kv : cache64) cudaFree(kv.second);
         if (d_err) cudaFree(d_err);
         for (auto e : ev_start) cudaEventDestroy(e);
         for (auto e : ev_stop) cudaEventDestroy(e);
@@ -249,13 +253,12 @@ void permute_sum(Ctx& c, const double* in, int S, const Shape& s, const int* per
 void split_planes(Ctx& c, const double* in, const Shape& s, const int* perm, long long rows, long long K, long long Kp,
                   void* const* out, bool in32 = false, int planes = 2);
 
-// The library's own kernels for small and skinny contractions (row-major A [M][K],
-// B [K][N], C [M][N] with leading dimensions): C = alpha A B + beta C.  M <= 8 or
-// N <= 8 take bandwidth kernels that read the large operand once (K split over
-// blocks, deterministic slice reduction); others a 64 x 64 tiled FP64 kernel.
-// f32: FP32 products and partial sums of <= 64 terms, accumulated in FP64.
+// The library's own kernels for skinny contractions (row-major A [M][K], B [K][N], C [M][N] with
+// leading dimensions; M <= 8 or N <= 8): C = alpha A B + beta C, the large operand read once (K split
+// over blocks, deterministic slice reduction), FP32 products and partial sums of <= 64 terms,
+// accumulated in FP64.
 void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const double* A, long long lda, const double* B,
-              long long ldb, double beta, double* C, long long ldc, bool f32);
+              long long ldb, double beta, double* C, long long ldc);
 
 // Row-major GEMM: C[MxN] = alpha op(A) op(B) + beta C, batched with strides.
 void gemm(Ctx& c, bool ta, bool tb, long long M, long long N, long long K, double alpha, const double* A, long long lda,

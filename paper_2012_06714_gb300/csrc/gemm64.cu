@@ -217,11 +217,26 @@ __device__ __forceinline__ double to_double(long long hi, long long lo, int e) {
 struct Gemm64Out {
     int M, N, mt, nt, S, slice_kb;  // slices of slice_kb K blocks
     const int *ea, *eb;
-    double* out;  // [S][M][N], or with direct the output itself
-    double alpha, beta;
-    int direct;
+    double* T;  // [S][M][N], or NULL: o
+    Out64 o;
     int* err;
 };
+
+__device__ __forceinline__ long long axes_offset(int n, const long long* d, const long long* st, unsigned x) {
+    long long off = 0;
+    for (int j = n - 1; j >= 0; --j) {
+        const unsigned dj = (unsigned)d[j], q = x / dj;
+        off += (long long)(x - q * dj) * st[j];
+        x = q;
+    }
+    return off;
+}
+// out = alpha v + beta out
+__device__ __forceinline__ void put64(const Out64& o, long long at, double v) {
+    if (o.alpha != 1.0) v *= o.alpha;
+    if (o.beta != 0.0) v += o.beta == 1.0 ? o.p[at] : o.beta * o.p[at];
+    o.p[at] = v;
+}
 
 // The digit products of one 16-deep K step: every MMA multiplies digit i of A with nj digits of B.
 // Unrolled at compile time: one thread issues them all, and address arithmetic between them would
@@ -254,7 +269,7 @@ __device__ __forceinline__ void digit_products(uint32_t tmem, uint64_t a, uint64
 template <int BNT>
 __global__ void __launch_bounds__(G_THREADS, 1)
     k_gemm64(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb, int num_k, int stages,
-             Gemm64Out o) {
+             const __grid_constant__ Gemm64Out o) {
     constexpr int tmem_cols = BNT <= 16 ? 128 : BNT <= 32 ? 256 : 512;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -383,6 +398,7 @@ __global__ void __launch_bounds__(G_THREADS, 1)
             const int row0 = m_tile * GM + quarter * 32, row = row0 + lane, colt = n_tile * BNT + cbeg;
             if (row0 >= o.M || colt >= o.N) continue;  // uniform over the warp
             const int ea = row < o.M ? o.ea[row] : 0;
+            const long long orow = o.T ? ((long long)sl * o.M + row) * o.N : axes_offset(o.o.nr, o.o.rd, o.o.rs, (unsigned)row);
 #pragma unroll
             for (int c0 = 0; c0 < cw; c0 += 8) {
                 // 32 rows x 8 columns through shared memory: whole sectors of the output rows
@@ -397,17 +413,16 @@ __global__ void __launch_bounds__(G_THREADS, 1)
                 }
                 __syncwarp();
                 const int col = colt + c0 + (lane & 7);
+                const long long ocol = o.T ? col : axes_offset(o.o.nc, o.o.cd, o.o.cs, (unsigned)col);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int rr = i * 4 + (lane >> 3);
+                    const long long at = __shfl_sync(0xffffffffu, orow, rr) + ocol;
                     if (row0 + rr < o.M && col < o.N) {
-                        double v = stg[rr * 9 + (lane & 7)];
-                        double* dst = o.out + ((long long)sl * o.M + row0 + rr) * o.N + col;
-                        if (o.direct) {
-                            if (o.alpha != 1.0) v *= o.alpha;
-                            if (o.beta != 0.0) v += o.beta == 1.0 ? *dst : o.beta * *dst;
-                        }
-                        *dst = v;
+                        if (o.T)
+                            o.T[at] = stg[rr * 9 + (lane & 7)];
+                        else
+                            put64(o.o, at, stg[rr * 9 + (lane & 7)]);
                     }
                 }
                 __syncwarp();
@@ -473,8 +488,7 @@ Gemm64Plan plan64(long long M, long long N, long long Kp) {
     return p;
 }
 
-void launch64(Ctx& c, const Digits64& A, const Digits64& B, const Gemm64Plan& p, double* out, bool direct, double alpha,
-              double beta) {
+void launch64(Ctx& c, const Digits64& A, const Digits64& B, const Gemm64Plan& p, double* T, const Out64& out) {
     if (!c.d_err) {
         if (c.capturing) throw Error(-3, "error flag allocation during stream capture");
         c.d_err = (int*)dev_alloc(sizeof(int), c.stream);
@@ -491,10 +505,8 @@ void launch64(Ctx& c, const Digits64& A, const Digits64& B, const Gemm64Plan& p,
     o.slice_kb = p.kb;
     o.ea = A.ex;
     o.eb = B.ex;
-    o.out = out;
-    o.alpha = alpha;
-    o.beta = beta;
-    o.direct = direct ? 1 : 0;
+    o.T = T;
+    o.o = out;
     o.err = c.d_err;
     const long long units = (long long)o.mt * o.nt * p.S;
     if (units > (1LL << 30)) throw Error(-1, "gemm64: too many tiles");
@@ -517,10 +529,21 @@ void launch64(Ctx& c, const Digits64& A, const Digits64& B, const Gemm64Plan& p,
 }  // namespace
 
 bool gemm64_fits(long long M, long long N, long long K) {
-    return M < (1LL << 30) && N < (1LL << 30) && K < (1LL << 30) && 2.0 * M * N * K >= 2e6 && std::max(M, N) >= 16;
+    return M < (1LL << 30) && N < (1LL << 30) && K < (1LL << 30) && 2.0 * M * N * K >= 4e6;
 }
 
-size_t digits64_bytes(long long rows, long long K) { return (size_t)ND * rows * ((K + 7) / 8 * 8) * 2; }
+size_t digits64_bytes(long long rows, long long K) {
+    return (size_t)ND * rows * ((K + 7) / 8 * 8) * 2 + ((size_t)rows * sizeof(int) + 255) / 256 * 256;
+}
+Digits64 digits64_in(void* buffer, long long rows, long long K) {
+    Digits64 d;
+    d.rows = rows;
+    d.Kp = (K + 7) / 8 * 8;
+    d.plane = rows * d.Kp;
+    d.d = (__nv_bfloat16*)buffer;
+    d.ex = (int*)(d.d + ND * d.plane);
+    return d;
+}
 
 void digitise64(Ctx& c, const Operand64* x, Digits64* out, int n) {
     DigitSide side[2];
@@ -566,33 +589,87 @@ void digitise64(Ctx& c, const Operand64* x, Digits64* out, int n) {
     ADC_CUDA(cudaGetLastError());
 }
 
-double* gemm64(Ctx& c, const Operand64& A, const Operand64& B, double alpha, double beta, double* out, int& S) {
-    const long long K = A.K, Kp = (K + 7) / 8 * 8;
-    const Operand64 ops[2] = {A, B};
-    Digits64 d[2];
-    // (the result is allocated first: it outlives the digits)
-    Gemm64Plan plan = plan64(A.rows, B.rows, Kp);
+double* gemm64(Ctx& c, const Operand64& A, const Digits64* da, const Operand64& B, const Digits64* db, const Out64& out,
+               int& S) {
+    const long long M = da ? da->rows : A.rows, N = db ? db->rows : B.rows, Kp = da ? da->Kp : (A.K + 7) / 8 * 8;
+    const Gemm64Plan plan = plan64(M, N, Kp);
     S = plan.S;
-    double* T = out && S == 1 ? nullptr : c.arena.dalloc((size_t)S * A.rows * B.rows);
+    // (the result is allocated first: it outlives the digits)
+    double* T = out.p && S == 1 ? nullptr : c.arena.dalloc((size_t)S * M * N);
     Arena::Mark mk = c.arena.mark();
+    Digits64 d[2], todo[2];
+    Operand64 x[2];
+    int n = 0;
     for (int i = 0; i < 2; ++i) {
-        d[i].rows = ops[i].rows;
-        d[i].Kp = Kp;
-        d[i].plane = ops[i].rows * Kp;
-        d[i].d = (__nv_bfloat16*)c.arena.alloc(digits64_bytes(ops[i].rows, K));
-        d[i].ex = (int*)c.arena.alloc((size_t)ops[i].rows * sizeof(int));
+        const Digits64* have = i ? db : da;
+        const Operand64& op = i ? B : A;
+        d[i] = have ? *have : digits64_in(c.arena.alloc(digits64_bytes(op.rows, op.K)), op.rows, op.K);
+        if (!have) x[n] = op, todo[n++] = d[i];
     }
-    digitise64(c, ops, d, 2);
-    launch64(c, d[0], d[1], plan, T ? T : out, T == nullptr, alpha, beta);
+    if (n) digitise64(c, x, todo, n);
+    launch64(c, d[0], d[1], plan, T, out);
     c.arena.release(mk);
     return T;
 }
 
-double* gemm64_digits(Ctx& c, const Digits64& A, const Digits64& B, int& S) {
-    Gemm64Plan plan = plan64(A.rows, B.rows, A.Kp);
-    S = plan.S;
-    double* T = c.arena.dalloc((size_t)S * A.rows * B.rows);
-    launch64(c, A, B, plan, T, false, 1.0, 0.0);
+// ---- the smallest contractions, in FP64 arithmetic ---------------------------------------------
+// 8 x 8 outputs per block of 64 threads: at two FP64 FMAs per cycle and SM, work of this size is only
+// quick when it is spread over all SMs.  Operands and output are reached through their strides, so a
+// contraction is one launch (with K slices: and the permute that sums them).
+namespace {
+constexpr int ST = 8, SK = 32;
+
+__global__ void __launch_bounds__(ST * ST) k_small64(const __grid_constant__ Operand64 A, const __grid_constant__ Operand64 B,
+                                                     long long kslice, double* __restrict__ T, const __grid_constant__ Out64 o) {
+    __shared__ double as[ST][SK + 1], bs[ST][SK + 1];
+    __shared__ long long ra[ST], rb[ST], ka[SK], kb[SK];
+    const int t = threadIdx.x, ti = t / ST, tj = t % ST;
+    const long long m0 = blockIdx.y * (long long)ST, n0 = blockIdx.x * (long long)ST;
+    if (t < ST) ra[t] = axes_offset(A.nr, A.rd, A.rs, (unsigned)min(m0 + t, A.rows - 1));
+    if (t >= 32 && t < 32 + ST) rb[t - 32] = axes_offset(B.nr, B.rd, B.rs, (unsigned)min(n0 + t - 32, B.rows - 1));
+    const long long k0 = blockIdx.z * kslice, k1 = min(A.K, k0 + kslice);
+    double acc = 0.0;
+    for (long long kc = k0; kc < k1; kc += SK) {
+        __syncthreads();
+        const unsigned k = (unsigned)min(kc + (t & 31), A.K - 1);
+        if (t < 32)
+            ka[t] = axes_offset(A.nk, A.kd, A.ks, k);
+        else
+            kb[t - 32] = axes_offset(B.nk, B.kd, B.ks, k);
+        __syncthreads();
+#pragma unroll
+        for (int e = t; e < ST * SK; e += ST * ST) {
+            const int r = e / SK, q = e % SK;
+            as[r][q] = kc + q < k1 ? ld_op(A, ra[r] + ka[q]) : 0.0;
+            bs[r][q] = kc + q < k1 ? ld_op(B, rb[r] + kb[q]) : 0.0;
+        }
+        __syncthreads();
+        const int kn = (int)min((long long)SK, k1 - kc);
+        for (int q = 0; q < kn; ++q) acc = fma(as[ti][q], bs[tj][q], acc);
+    }
+    const long long m = m0 + ti, n = n0 + tj;
+    if (m < A.rows && n < B.rows) {
+        if (T)
+            T[(blockIdx.z * A.rows + m) * B.rows + n] = acc;
+        else
+            put64(o, axes_offset(o.nr, o.rd, o.rs, (unsigned)m) + axes_offset(o.nc, o.cd, o.cs, (unsigned)n), acc);
+    }
+}
+}  // namespace
+
+double* small64(Ctx& c, const Operand64& A, const Operand64& B, const Out64& out, int& S) {
+    const long long mt = (A.rows + ST - 1) / ST, nt = (B.rows + ST - 1) / ST;
+    if (mt > 65535 || nt > 0x7fffffffLL || A.K >= (1LL << 30)) throw Error(-1, "small64: too many rows");
+    // K slices while the blocks leave SMs idle, of at least 64 terms (a sum of slices is another launch)
+    S = 1;
+    if (A.K >= 256 && mt * nt < 2 * sm_count())
+        S = (int)std::max<long long>(1, std::min<long long>({A.K / 64, 4LL * sm_count() / (mt * nt), 64}));
+    long long ks = (A.K + S - 1) / S;
+    S = (int)((A.K + ks - 1) / ks);
+    double* T = out.p && S == 1 ? nullptr : c.arena.dalloc((size_t)S * A.rows * B.rows);
+    k_small64<<<dim3((unsigned)nt, (unsigned)mt, (unsigned)S), ST * ST, 0, c.stream>>>(A, B, ks, T, out);
+    ++c.kernels;
+    ADC_CUDA(cudaGetLastError());
     return T;
 }
 

@@ -34,13 +34,10 @@ Operand64 rows_of(const double* p, long long rows, long long K) {
 
 // digits of one half of L, rows [row0, row0 + rows)
 Digits64 half_of(const Pairs64& L, int half, long long row0, long long rows) {
-    Digits64 d;
-    const size_t planes = digits64_bytes(L.P, L.P);
+    Digits64 d = digits64_in((char*)L.store.mem[0] + half * digits64_bytes(L.P, L.P), L.P, L.P);
     d.rows = rows;
-    d.Kp = L.Pk;
-    d.plane = L.P * L.Pk;
-    d.d = (__nv_bfloat16*)((char*)L.store.mem[0] + half * planes) + row0 * L.Pk;
-    d.ex = (int*)((char*)L.store.mem[0] + 2 * planes) + half * L.P + row0;
+    d.d += row0 * L.Pk;
+    d.ex += row0;
     return d;
 }
 
@@ -48,7 +45,7 @@ Digits64 half_of(const Pairs64& L, int half, long long row0, long long rows) {
 
 size_t pairs64_bytes(int v) {
     const long long P = (long long)v * (v + 1) / 2;
-    return 2 * digits64_bytes(P, P) + 2 * P * sizeof(int);
+    return 2 * digits64_bytes(P, P);
 }
 
 bool pairs64_prepare(Pairs64& L, Ctx& c, const double* Bvv, int naux, int nvir) {
@@ -82,7 +79,11 @@ bool pairs64_prepare(Pairs64& L, Ctx& c, const double* Bvv, int naux, int nvir) 
         B.k_axis(Q, v * v);
         double* G = c.arena.dalloc((size_t)(na * v * nb * v));
         int S = 1;
-        double* T = gemm64(c, A, B, 1.0, 0.0, G, S);
+        Out64 go;
+        go.p = G;
+        go.row_axis(na * v, nb * v);
+        go.col_axis(nb * v, 1);
+        const double* T = gemm64(c, A, nullptr, B, nullptr, go, S);
         if (T) {
             Shape sh{1, {na * v * nb * v}};
             const int id[1] = {0};
@@ -119,17 +120,13 @@ void pairs64_apply(Pairs64& L, Ctx& c, const double* X, long long nmat, double* 
         ADC_CUDA(cudaGetLastError());
         const Operand64 x[2] = {rows_of(XP, nm, P), rows_of(XP + nm * P, nm, P)};
         Digits64 d[2];
-        for (int h = 0; h < 2; ++h) {
-            d[h].rows = nm;
-            d[h].Kp = L.Pk;
-            d[h].plane = nm * L.Pk;
-            d[h].d = (__nv_bfloat16*)c.arena.alloc(digits64_bytes(nm, P));
-            d[h].ex = (int*)c.arena.alloc((size_t)nm * sizeof(int));
-        }
+        for (int h = 0; h < 2; ++h) d[h] = digits64_in(c.arena.alloc(digits64_bytes(nm, P)), nm, P);
         digitise64(c, x, d, 2);
         int S = 1;
-        const double* T0 = gemm64_digits(c, half_of(L, 0, 0, P), d[0], S);
-        const double* T1 = gemm64_digits(c, half_of(L, 1, 0, P), d[1], S);
+        const Operand64 none{};
+        const Digits64 V0 = half_of(L, 0, 0, P), V1 = half_of(L, 1, 0, P);
+        const double* T0 = gemm64(c, none, &V0, none, &d[0], Out64(), S);
+        const double* T1 = gemm64(c, none, &V1, none, &d[1], Out64(), S);
         const long long ut = (v + 15) / 16, blocks = ut * (ut + 1) / 2 * ((nm + 7) / 8);
         k_pair_unfold<double><<<(unsigned)std::min<long long>(blocks, 152LL * 32), 256, 0, c.stream>>>(
             T0, T1, S, P, (int)nm, (int)v, out + m0 * v * v);

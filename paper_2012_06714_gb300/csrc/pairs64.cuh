@@ -8,7 +8,7 @@ namespace adc {
 struct Pairs64 {
     int v = 0;
     long long P = 0, Pk = 0;
-    Reclaimable store;  // digits of both halves, then the rows' exponents
+    Reclaimable store;  // digits of both halves
 };
 
 size_t pairs64_bytes(int nvir);
