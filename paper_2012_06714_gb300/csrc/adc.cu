@@ -380,6 +380,11 @@ void ein(Ctx& c, const char* spec, double alpha, const T& A, const T& B, double 
     else
         einsum(c, spec, alpha, A, B, beta, (double*)C.p, d);
 }
+// Whether an intermediate of M x N x K products may be held in FP32: the mixed sigma, where the product
+// is one of the split-BF16 contractions (FP32 sums) and its result only enters further ones.
+bool f32_product(const Ctx& c, long long M, long long N, long long K) {
+    return c.gemm_mode == 2 && std::min(M, N) > 8 && 2.0 * M * N * K >= c.fp32_min_flops && tc_gemm_fits(M, N, K);
+}
 // C = alpha * permute(X) + beta * C (output axis j = input axis perm[j])
 void perm_into(Ctx& c, const T& X, std::initializer_list<int> perm, const Buf& C, double alpha, double beta) {
     Shape s{(int)X.dims.size(), {}};
@@ -1338,18 +1343,19 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
         double* P = c.arena.dalloc(n * Q * o);
         einsum(c, "Qjm,nlmj->nQl", 1.0, tc(h->Boo, {Q, o, o}), tn(Z, {n, o, o, o}), 0.0, P, {n, Q, o});
         //  sum (ad|em)(2 t_jm^ce - t_jm^ec) Y~_jcd  (a lean handle holds no tau: two contractions with t)
-        double* V = c.arena.dalloc(n * o * v * v);
+        // (the n o v^2 intermediates V and q, in the order in which the GEMMs write them)
+        const Buf V = scratch(c.arena, n * o * v * v, f32_product(c, o * v, n * v, o * v));
         if (h->tau) {
-            einsum(c, "jmce,njcd->nmed", 1.0, tc(h->tau, {o, o, v, v}), tn(Yt, {n, o, v, v}), 0.0, V, {n, o, v, v});
+            ein(c, "jmce,njcd->mend", 1.0, tc(h->tau, {o, o, v, v}), tn(Yt, {n, o, v, v}), 0.0, V, {o, v, n, v});
         } else {
-            einsum(c, "jmce,njcd->nmed", 2.0, T4, tn(Yt, {n, o, v, v}), 0.0, V, {n, o, v, v});
-            einsum(c, "jmec,njcd->nmed", -1.0, T4, tn(Yt, {n, o, v, v}), 1.0, V, {n, o, v, v});
+            ein(c, "jmce,njcd->mend", 2.0, T4, tn(Yt, {n, o, v, v}), 0.0, V, {o, v, n, v});
+            ein(c, "jmec,njcd->mend", -1.0, T4, tn(Yt, {n, o, v, v}), 1.0, V, {o, v, n, v});
         }
-        einsum(c, "nmed,Qme->nQd", 1.0, tn(V, {n, o, v, v}), tc(h->Bov, {Q, o, v}), 1.0, Wq, {n, Q, v});
+        einsum(c, "mend,Qme->nQd", 1.0, V.as({o, v, n, v}), tc(h->Bov, {Q, o, v}), 1.0, Wq, {n, Q, v});
         //  - sum (am|ed) [t_jm^ce Y~_jcd + t_jm^ed Y~_jdc]   (the two exchange-type terms)
-        einsum(c, "jmce,njcd->nmed", 1.0, T4, tn(Yt, {n, o, v, v}), 0.0, V, {n, o, v, v});
-        einsum(c, "jmec,njdc->nmed", 1.0, T4, tn(Yt, {n, o, v, v}), 1.0, V, {n, o, v, v});
-        einsum(c, "nmed,Qed->nQm", -1.0, tn(V, {n, o, v, v}), tc(h->Bvv, {Q, v, v}), 1.0, P, {n, Q, o});
+        ein(c, "jmce,njcd->mend", 1.0, T4, tn(Yt, {n, o, v, v}), 0.0, V, {o, v, n, v});
+        ein(c, "jmec,njdc->mend", 1.0, T4, tn(Yt, {n, o, v, v}), 1.0, V, {o, v, n, v});
+        einsum(c, "mend,Qed->nQm", -1.0, V.as({o, v, n, v}), tc(h->Bvv, {Q, v, v}), 1.0, P, {n, Q, o});
         einsum(c, "nQl,Qla->na", 1.0, tn(P, {n, Q, o}), tc(h->Bov, {Q, o, v}), 1.0, s1, {n, v});
         // 2p1h column, second order:
         //  sum_lm (cl|im) t_lm^ba Y_c
@@ -1359,18 +1365,18 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
         einsum(c, "nQl,Qim->nlim", 1.0, tn(p, {n, Q, o}), tc(h->Boo, {Q, o, o}), 0.0, Pl, {n, o, o, o});
         einsum(c, "nlim,lmba->niab", 1.0, tn(Pl, {n, o, o, o}), T4, 1.0, S2, {n, o, v, v});
         //  sum_me (cb|em)(2 t_im^ae - t_im^ea) Y_c
-        double* q = c.arena.dalloc(n * o * v * v);
-        einsum(c, "nQb,Qme->nbme", 1.0, tn(hq, {n, Q, v}), tc(h->Bov, {Q, o, v}), 0.0, q, {n, v, o, v});
+        const Buf q = scratch(c.arena, n * o * v * v, f32_product(c, n * v, o * v, Q) && f32_product(c, n * o, v * v, Q));
+        ein(c, "nQb,Qme->nbme", 1.0, tn(hq, {n, Q, v}), tc(h->Bov, {Q, o, v}), 0.0, q, {n, v, o, v});
         if (h->tau) {
-            einsum(c, "nbme,imae->niab", 1.0, tn(q, {n, v, o, v}), tc(h->tau, {o, o, v, v}), 1.0, S2, {n, o, v, v});
+            einsum(c, "nbme,imae->niab", 1.0, q.as({n, v, o, v}), tc(h->tau, {o, o, v, v}), 1.0, S2, {n, o, v, v});
         } else {
-            einsum(c, "nbme,imae->niab", 2.0, tn(q, {n, v, o, v}), T4, 1.0, S2, {n, o, v, v});
-            einsum(c, "nbme,imea->niab", -1.0, tn(q, {n, v, o, v}), T4, 1.0, S2, {n, o, v, v});
+            einsum(c, "nbme,imae->niab", 2.0, q.as({n, v, o, v}), T4, 1.0, S2, {n, o, v, v});
+            einsum(c, "nbme,imea->niab", -1.0, q.as({n, v, o, v}), T4, 1.0, S2, {n, o, v, v});
         }
         //  - sum_me (cm|eb) t_im^ae Y_c - sum_me (cm|ea) t_im^eb Y_c
-        einsum(c, "nQm,Qeb->nmeb", 1.0, tn(p, {n, Q, o}), tc(h->Bvv, {Q, v, v}), 0.0, q, {n, o, v, v});
-        einsum(c, "nmeb,imae->niab", -1.0, tn(q, {n, o, v, v}), T4, 1.0, S2, {n, o, v, v});
-        einsum(c, "nmea,imeb->niab", -1.0, tn(q, {n, o, v, v}), T4, 1.0, S2, {n, o, v, v});
+        ein(c, "nQm,Qeb->nmeb", 1.0, tn(p, {n, Q, o}), tc(h->Bvv, {Q, v, v}), 0.0, q, {n, o, v, v});
+        einsum(c, "nmeb,imae->niab", -1.0, q.as({n, o, v, v}), T4, 1.0, S2, {n, o, v, v});
+        einsum(c, "nmea,imeb->niab", -1.0, q.as({n, o, v, v}), T4, 1.0, S2, {n, o, v, v});
         // 2p1h block, first order: ladder sum_cd (ac|bd) Y_icd (vvvv never stored)
         ladder(h, Y2, n * o, S2, h->refining ? h->lm_refine : h->lm_sigma);
         //  - (ac|ji) Y_jcb + 2 (ai|jc) Y_jcb - (ai|jc) Y_jbc - (bd|ji) Y_jad  (the first two as one
@@ -1423,10 +1429,11 @@ static void sigma_ip(adc_handle* h, const double* Xin, double* Sout, long long n
         const double *t = h->t, *tau = h->tau;
         // coupling row, second order
         //  - sum (ad|ie) t_jk^de Y~_jka
-        double* Z = c.arena.dalloc(n * v * v * v);
-        einsum(c, "jkde,njka->ndea", 1.0, tc(t, {o, o, v, v}), tn(Yt, {n, o, o, v}), 0.0, Z, {n, v, v, v});
+        // (the n v^3 intermediates Z and w, in the order in which the GEMMs write them)
+        const Buf Z = scratch(c.arena, n * v * v * v, f32_product(c, v * v, n * v, o * o));
+        ein(c, "jkde,njka->dena", 1.0, tc(t, {o, o, v, v}), tn(Yt, {n, o, o, v}), 0.0, Z, {v, v, n, v});
         double* Hq = c.arena.dalloc(n * Q * v);
-        einsum(c, "ndea,Qad->nQe", 1.0, tn(Z, {n, v, v, v}), tc(h->Bvv, {Q, v, v}), 0.0, Hq, {n, Q, v});
+        einsum(c, "dena,Qad->nQe", 1.0, Z.as({v, v, n, v}), tc(h->Bvv, {Q, v, v}), 0.0, Hq, {n, Q, v});
         einsum(c, "nQe,Qie->ni", -1.0, tn(Hq, {n, Q, v}), tc(h->Bov, {Q, o, v}), 1.0, s1, {n, o});
         //  - sum (ik|lc)(2 t_jl^ac - t_jl^ca) Y~_jka + sum (ic|lk) t_jl^ac Y~_jka + sum (ic|lj) t_kl^ca Y~_jka
         double* G2 = c.arena.dalloc(n * o * o * v);
@@ -1439,9 +1446,9 @@ static void sigma_ip(adc_handle* h, const double* Xin, double* Sout, long long n
         // 2h1p column, second order (same tensor, applied to Y_i)
         double* bq = c.arena.dalloc(n * Q * v);
         einsum(c, "ni,Qie->nQe", 1.0, tn(y1, {n, o}), tc(h->Bov, {Q, o, v}), 0.0, bq, {n, Q, v});
-        double* w = c.arena.dalloc(n * v * v * v);
-        einsum(c, "nQe,Qad->nead", 1.0, tn(bq, {n, Q, v}), tc(h->Bvv, {Q, v, v}), 0.0, w, {n, v, v, v});
-        einsum(c, "nead,jkde->njka", -1.0, tn(w, {n, v, v, v}), tc(t, {o, o, v, v}), 1.0, S2, {n, o, o, v});
+        const Buf w = scratch(c.arena, n * v * v * v, f32_product(c, n * v, v * v, Q));
+        ein(c, "nQe,Qad->nead", 1.0, tn(bq, {n, Q, v}), tc(h->Bvv, {Q, v, v}), 0.0, w, {n, v, v, v});
+        einsum(c, "nead,jkde->njka", -1.0, w.as({n, v, v, v}), tc(t, {o, o, v, v}), 1.0, S2, {n, o, o, v});
         double* m = c.arena.dalloc(n * o * o * v);
         einsum(c, "ni,iklc->nklc", 1.0, tn(y1, {n, o}), tc(h->ooov, {o, o, o, v}), 0.0, m, {n, o, o, v});
         einsum(c, "nklc,jlac->njka", -1.0, tn(m, {n, o, o, v}), tc(tau, {o, o, v, v}), 1.0, S2, {n, o, o, v});

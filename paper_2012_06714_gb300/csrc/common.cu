@@ -97,7 +97,7 @@ struct PermArgs {
 template <typename Tin>
 struct Plain {
     const Tin* p;
-    __device__ double operator()(long long i) const { return (double)p[i]; }
+    __device__ Tin operator()(long long i) const { return p[i]; }
 };
 template <typename Tin>
 struct SumOf {
@@ -124,7 +124,7 @@ __global__ void permute_kernel(In in, Tout* __restrict__ out, PermArgs a, long l
             off += (r - q * d) * (I)a.sin[j];
             r = q;
         }
-        const double v = alpha * in(off);
+        const double v = alpha * (double)in(off);
         out[idx] = (Tout)((beta == 0.0) ? v : v + beta * (double)out[idx]);
     }
 }
@@ -143,8 +143,7 @@ __global__ void fill_kernel(long long n, double v, double* __restrict__ y) {
 // before.  The remainders are formed in FP32, whose 24 bits hold what three planes do: FP64
 // arithmetic (2 operations per cycle and SM on this chip) made the splits several times slower than
 // their traffic.
-__device__ __forceinline__ void put_planes(double x, long long ad, __nv_bfloat16* o0, __nv_bfloat16* o1, __nv_bfloat16* o2) {
-    float f = (float)x;
+__device__ __forceinline__ void put_planes(float f, long long ad, __nv_bfloat16* o0, __nv_bfloat16* o1, __nv_bfloat16* o2) {
     const __nv_bfloat16 h = __float2bfloat16(f);
     o0[ad] = h;
     f -= __bfloat162float(h);
@@ -173,7 +172,7 @@ __global__ void permute_split_kernel(const Tin* __restrict__ in, __nv_bfloat16* 
             }
             x = (double)in[off];
         }
-        put_planes(x, idx, o0, o1, o2);
+        put_planes((float)x, idx, o0, o1, o2);
     }
 }
 
@@ -197,7 +196,37 @@ struct OpPlanes {
         const long long r = lin / K;
         return r * Kp + (lin - r * K);
     }
-    __device__ void put(long long ad, double x) const { put_planes(x, ad, o0, o1, o2); }
+    template <typename V>
+    __device__ void put(long long ad, V x) const {
+        put_planes((float)x, ad, o0, o1, o2);
+    }
+    template <int V, typename X>
+    __device__ void put_n(long long ad, const X (&x)[V]) const {
+        if constexpr (V == 4) {
+            uint2 w[3];
+            float f[4] = {(float)x[0], (float)x[1], (float)x[2], (float)x[3]};
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                const __nv_bfloat162 l = __floats2bfloat162_rn(f[0], f[1]), h = __floats2bfloat162_rn(f[2], f[3]);
+                w[p] = make_uint2(*(const unsigned*)&l, *(const unsigned*)&h);
+                f[0] -= __uint_as_float(w[p].x << 16);
+                f[1] -= __uint_as_float(w[p].x & 0xffff0000u);
+                f[2] -= __uint_as_float(w[p].y << 16);
+                f[3] -= __uint_as_float(w[p].y & 0xffff0000u);
+            }
+            *(uint2*)(o0 + ad) = w[0];
+            *(uint2*)(o1 + ad) = w[1];
+            if (o2) *(uint2*)(o2 + ad) = w[2];
+        } else {
+#pragma unroll
+            for (int e = 0; e < V; ++e) put(ad + e, x[e]);
+        }
+    }
+    // after the line of `len` elements from lin (at address ad): the row's padding, if it ends there
+    __device__ void finish(long long lin, long long len, long long ad, int i, int step) const {
+        if (Kp == K || (lin + len) % K) return;
+        for (long long k = i; k < Kp - K; k += step) put_planes(0.0f, ad + len + k, o0, o1, o2);
+    }
 };
 // out = alpha x + beta out
 template <typename Tout>
@@ -205,15 +234,69 @@ struct OpAxpby {
     Tout* out;
     double alpha, beta;
     __device__ long long addr(long long lin) const { return lin; }
-    __device__ void put(long long ad, double x) const {
-        const double v = alpha * x;
-        out[ad] = (Tout)(beta == 0.0 ? v : v + beta * (double)out[ad]);
+    template <typename V>
+    __device__ void put(long long ad, V x) const {
+        if (alpha == 1.0 && beta == 0.0) {
+            out[ad] = (Tout)x;
+            return;
+        }
+        const double v = alpha == 1.0 ? (double)x : alpha * (double)x;
+        out[ad] = (Tout)(beta == 0.0 ? v : beta == 1.0 ? v + (double)out[ad] : v + beta * (double)out[ad]);
     }
+    template <int V, typename X>
+    __device__ void put_n(long long ad, const X (&x)[V]) const {
+#pragma unroll
+        for (int e = 0; e < V; ++e) put(ad + e, x[e]);
+    }
+    __device__ void finish(long long, long long, long long, int, int) const {}
 };
+
+// ---- permutes along lines -----------------------------------------------------------
+// When the output's fastest axis is contiguous in the input too, a group of tpl threads copies a
+// whole line of it: one coordinate computation per line instead of one per element (the element-wise
+// kernels spend most of their time on integer divisions), four loads in flight per thread.
+struct LineArgs {
+    int nd;  // axes above the line
+    long long dout[kMaxDim], sin[kMaxDim];
+    long long len, nlines, seg;  // lines are cut into segments of seg elements (a multiple of 4)
+    int nseg, tpl;               // segments per line, threads per segment
+};
+// V elements per thread at a time (4 when the lines' lengths are multiples of it: 8-byte stores of the
+// BF16 planes, which 2-byte ones would bound)
+template <int V, typename In, typename Op>
+__global__ void __launch_bounds__(256) k_permute_lines(In in, const __grid_constant__ LineArgs a, Op op) {
+    const int per = 256 / a.tpl, lane = threadIdx.x % a.tpl;
+    const long long units = a.nlines * a.nseg;
+    for (long long u = blockIdx.x * (long long)per + threadIdx.x / a.tpl; u < units; u += (long long)gridDim.x * per) {
+        // (32-bit division where it suffices)
+        const long long line = a.nseg == 1 ? u : u <= 0xffffffffLL ? (long long)((unsigned)u / (unsigned)a.nseg) : u / a.nseg;
+        const long long x0 = (u - line * a.nseg) * a.seg, x1 = min(a.len, x0 + a.seg);
+        long long r = line, off = 0;
+        for (int j = a.nd - 1; j >= 0; --j) {
+            const long long d = a.dout[j], q = r <= 0xffffffffLL ? (long long)((unsigned)r / (unsigned)d) : r / d;
+            off += (r - q * d) * a.sin[j];
+            r = q;
+        }
+        const long long ad = op.addr(line * a.len);
+        constexpr int U = V == 4 ? 2 : 4;
+        for (long long x = x0 + V * lane; x < x1; x += U * V * a.tpl) {
+            decltype(in(0)) v[U][V];
+#pragma unroll
+            for (int w = 0; w < U; ++w)
+                if (x + w * V * a.tpl < x1)
+#pragma unroll
+                    for (int e = 0; e < V; ++e) v[w][e] = in(off + x + w * V * a.tpl + e);
+#pragma unroll
+            for (int w = 0; w < U; ++w)
+                if (x + w * V * a.tpl < x1) op.template put_n<V>(ad + x + w * V * a.tpl, v[w]);
+        }
+        if (x1 == a.len) op.finish(line * a.len, a.len, ad, lane, a.tpl);
+    }
+}
 
 template <typename In, typename Op>
 __global__ void __launch_bounds__(256) k_permute_tiled(In in, TileArgs a, Op op) {
-    __shared__ double tile[32][33];
+    __shared__ decltype(in(0)) tile[32][33];
     for (long long b = blockIdx.x; b < a.nblocks; b += gridDim.x) {
         long long t = b;
         const long long tx = t % a.ntx;
@@ -373,14 +456,15 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, lon
 
 // As k_reduce_slices for many slices: one warp per output element, lanes over slices,
 // then a shuffle reduction.
-__global__ void k_reduce_slices_warp(int S, long long M, long long N, const double* __restrict__ P, double alpha,
+template <typename Tp>
+__global__ void k_reduce_slices_warp(int S, long long M, long long N, const Tp* __restrict__ P, double alpha,
                                      double beta, double* __restrict__ C, long long ldc) {
     const long long total = M * N;
     const int lane = threadIdx.x & 31;
     const long long warps = (long long)gridDim.x * blockDim.x / 32;
     for (long long x = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32; x < total; x += warps) {
         double a = 0.0;
-        for (int s2 = lane; s2 < S; s2 += 32) a += P[s2 * total + x];
+        for (int s2 = lane; s2 < S; s2 += 32) a += (double)P[s2 * total + x];
         for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
         if (lane == 0) {
             const long long m = x / N, n = x - m * N;
@@ -472,7 +556,7 @@ void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
     if (S >= 16)
-        k_reduce_slices_warp<<<grid_for(32 * M * N), 256, 0, c.stream>>>(S, M, N, P, alpha, beta, C, ldc);
+        k_reduce_slices_warp<double><<<grid_for(32 * M * N), 256, 0, c.stream>>>(S, M, N, P, alpha, beta, C, ldc);
     else
         k_reduce_slices<<<grid_for(M * N), 256, 0, c.stream>>>(S, M, N, P, alpha, beta, C, ldc);
     ++c.kernels;
@@ -547,6 +631,51 @@ static PermArgs perm_args(const Shape& s, const int* perm, long long& total) {
     return a;
 }
 
+// The line form applies when the output's fastest axis is contiguous in the input (axes that are
+// neighbours on both sides are merged first, within a row of `unit` elements if it is not 0) and at
+// least 8 long.
+static bool line_args(const PermArgs& p, long long unit, LineArgs& t) {
+    long long d[kMaxDim], si[kMaxDim];
+    int nd = 0;
+    for (int j = 0; j < p.nd; ++j)
+        if (p.dout[j] > 1) {
+            d[nd] = p.dout[j];
+            si[nd] = p.sin[j];
+            ++nd;
+        }
+    if (nd == 0 || si[nd - 1] != 1) return false;
+    t.len = d[--nd];
+    while (nd > 0 && si[nd - 1] == t.len && (unit == 0 || unit % (t.len * d[nd - 1]) == 0)) t.len *= d[--nd];
+    if (t.len < 8 || (unit && unit % t.len)) return false;
+    t.nd = nd;
+    t.nlines = 1;
+    for (int j = 0; j < nd; ++j) {
+        t.dout[j] = d[j];
+        t.sin[j] = si[j];
+        t.nlines *= d[j];
+    }
+    // segments of at most 1024 elements, of 256 when that still leaves the chip idle
+    t.seg = std::min<long long>(1024, (t.len + 3) / 4 * 4);
+    if (t.nlines * ((t.len + t.seg - 1) / t.seg) < 2048) t.seg = std::min<long long>(t.seg, 256);
+    const long long ns = (t.len + t.seg - 1) / t.seg;
+    if (ns > 0x7fffffffLL) return false;
+    t.nseg = (int)ns;
+    t.tpl = 8;
+    while (t.tpl < 256 && t.tpl * 8 < t.seg) t.tpl *= 2;
+    return true;
+}
+
+template <typename In, typename Op>
+static void launch_lines(Ctx& c, const In& in, const LineArgs& t, const Op& op) {
+    const long long per = 256 / t.tpl, g = std::min<long long>((t.nlines * t.nseg + per - 1) / per, 152LL * 32);
+    if (t.len % 4 == 0)
+        k_permute_lines<4, In, Op><<<(unsigned)g, 256, 0, c.stream>>>(in, t, op);
+    else
+        k_permute_lines<1, In, Op><<<(unsigned)g, 256, 0, c.stream>>>(in, t, op);
+    ++c.kernels;
+    ADC_CUDA(cudaGetLastError());
+}
+
 template <typename In, typename Tout>
 static void permute_in(Ctx& c, const In& in, const Shape& s, const int* perm, Tout* out, double alpha, double beta) {
     long long total;
@@ -555,6 +684,11 @@ static void permute_in(Ctx& c, const In& in, const Shape& s, const int* perm, To
     TileArgs t;
     if (tiled_args(a, t)) {
         launch_tiled(c, in, t, OpAxpby<Tout>{out, alpha, beta});
+        return;
+    }
+    LineArgs ln;
+    if (line_args(a, 0, ln)) {
+        launch_lines(c, in, ln, OpAxpby<Tout>{out, alpha, beta});
         return;
     }
     if (total <= 0xffffffffLL)  // every offset is below total
@@ -574,6 +708,24 @@ static void permute_sum_t(Ctx& c, const Tin* in, int S, const Shape& s, const in
                           double beta) {
     long long n = 1;
     for (int j = 0; j < s.nd; ++j) n *= s.d[j];
+    if (S == 1) {
+        if (out32)
+            permute_in(c, Plain<Tin>{in}, s, perm, (float*)out, alpha, beta);
+        else
+            permute_in(c, Plain<Tin>{in}, s, perm, (double*)out, alpha, beta);
+        return;
+    }
+    Arena::Mark mk = c.arena.mark();
+    if (S >= 16) {
+        // many slices are summed by a warp per element first
+        double* sum = c.arena.dalloc((size_t)n);
+        k_reduce_slices_warp<Tin><<<grid_for(32 * n), 256, 0, c.stream>>>(S, 1, n, in, 1.0, 0.0, sum, n);
+        ++c.kernels;
+        ADC_CUDA(cudaGetLastError());
+        permute_sum_t(c, (const double*)sum, 1, s, perm, out, out32, alpha, beta);
+        c.arena.release(mk);
+        return;
+    }
     if (out32)
         permute_in(c, SumOf<Tin>{in, S, n}, s, perm, (float*)out, alpha, beta);
     else
@@ -601,6 +753,11 @@ static void split_planes_t(Ctx& c, const Tin* in, const PermArgs& a, long long r
             ++c.kernels;
             ADC_CUDA(cudaGetLastError());
         }
+        return;
+    }
+    LineArgs ln;
+    if (line_args(a, K, ln)) {
+        launch_lines(c, Plain<Tin>{in}, ln, OpPlanes{o0, o1, o2, K, Kp});
         return;
     }
     // 32-bit coordinates when the output index fits (every input offset is below rows * K)
@@ -846,8 +1003,11 @@ static void einsum_tc(Ctx& c, const std::string& la, const std::string& lb, cons
     const void* A2[2] = {pa, (const char*)pa + M * Kp * 2};
     const void* B2[2] = {pb, (const char*)pb + N * Kp * 2};
     int S = 1;
-    const float* T = tc_gemm(c, A2, B2, M, N, Kp, 2.0 * M * N * K, S);
-    std::string tord = fa + fb;
+    const std::string tord = fa + fb;
+    // an FP32 output in the GEMM's order takes the one slice's result itself
+    float* direct = c32 && tord == lc && alpha == 1.0 && beta == 0.0 ? (float*)C : nullptr;
+    const float* T = tc_gemm(c, A2, B2, M, N, Kp, 2.0 * M * N * K, S, direct);
+    if (T == direct) return;
     Shape sh;
     sh.nd = (int)tord.size();
     for (int j = 0; j < sh.nd; ++j) sh.d[j] = dim[tord[j]];

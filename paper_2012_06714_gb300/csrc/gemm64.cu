@@ -474,7 +474,7 @@ Gemm64Plan plan64(long long M, long long N, long long Kp) {
     double best = 1e300;
     for (int b : {64, 48, 32, 16}) {
         const long long tiles = ((M + GM - 1) / GM) * ((N + b - 1) / b);
-        for (long long s = 1; s <= 32; ++s) {
+        for (long long s = 1; s <= std::max(1LL, std::min<long long>(160, 2 * sms / tiles)) || s <= 32; ++s) {
             const long long kb = ((num_k + s - 1) / s + EPOCH - 1) / EPOCH * EPOCH;
             if (s > 1 && (num_k + kb - 1) / kb != s) continue;
             const double rounds = (double)((tiles * s + sms - 1) / sms);

@@ -1268,10 +1268,10 @@ int pick_slices(long long M, long long N, long long Kp, int bn, int pairs) {
 }
 
 float* tc_gemm_bn(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp,
-                  double algo_flops, int BN, int& S) {
+                  double algo_flops, int BN, int& S, float* direct) {
     S = pick_slices(M, N, Kp, BN, dev_info().max_pairs);
     const long long nkb = (Kp + BK - 1) / BK, kb = (nkb + S - 1) / S;
-    float* T = (float*)c.arena.alloc((size_t)S * M * N * sizeof(float));
+    float* T = S == 1 && direct ? direct : (float*)c.arena.alloc((size_t)S * M * N * sizeof(float));
     Epi e{};
     e.mode = 2;
     e.M = (int)M;
@@ -1280,7 +1280,7 @@ float* tc_gemm_bn(Ctx& c, const void* const* A, const void* const* B, long long 
     e.err = c.d_err;
     e.out32 = T;
     e.zout = M * N;
-    e.vec = N % 4 == 0;  // (arena blocks are 256-byte aligned)
+    e.vec = N % 4 == 0 && (uintptr_t)T % 16 == 0;
     const int m_fastest = M <= N ? 1 : 0;  // consecutive tiles share the B tile when A is the smaller operand
     Maps m{};
     for (int p = 0; p < 2; ++p) {
@@ -1297,7 +1297,7 @@ float* tc_gemm_bn(Ctx& c, const void* const* A, const void* const* B, long long 
 }  // namespace
 
 float* tc_gemm(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp, double algo_flops,
-               int& S) {
+               int& S, float* direct) {
     if (!c.d_err) throw Error(-1, "tc_gemm: no device error flag");
     const int n = (int)std::min<long long>(N, 1 << 20);
     int BN = pick_bn(n, 256);
@@ -1314,7 +1314,7 @@ float* tc_gemm(Ctx& c, const void* const* A, const void* const* B, long long M, 
             int bb = BN;
             for (int b : bn_candidates(n, 256, {256, 128})) {
                 Arena::Mark mk = c.arena.mark();
-                const float ms = time_on_stream(c, [&] { tc_gemm_bn(c, A, B, M, N, Kp, algo_flops, b, S); });
+                const float ms = time_on_stream(c, [&] { tc_gemm_bn(c, A, B, M, N, Kp, algo_flops, b, S, nullptr); });
                 c.arena.release(mk);
                 if (ms < best) best = ms, bb = b;
             }
@@ -1322,7 +1322,7 @@ float* tc_gemm(Ctx& c, const void* const* A, const void* const* B, long long M, 
             BN = bb;
         }
     }
-    return tc_gemm_bn(c, A, B, M, N, Kp, algo_flops, BN, S);
+    return tc_gemm_bn(c, A, B, M, N, Kp, algo_flops, BN, S, direct);
 }
 
 }  // namespace adc

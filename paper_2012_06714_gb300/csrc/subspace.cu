@@ -137,9 +137,10 @@ void multidot(Ctx& c, int na, const double* A, long long lda, int nb, const doub
     const int TJ = nb >= 4 ? 4 : nb > 2 ? 4 : nb;          // 1, 2 or 4 (TJ <= TI)
     const int ti = (na + TI - 1) / TI, tj = (nb + TJ - 1) / TJ, tiles = ti * tj;
     if ((long long)tiles > (1LL << 30)) throw Error(-1, "multidot: too many vectors");
-    // about four resident CTAs per SM in total; each slice at least 4096 elements
+    // about four resident CTAs per SM in total; each slice at least 512 elements (two per thread: the
+    // kernel is bound by the SM's two FP64 FMAs per cycle, so short vectors are spread too)
     long long S = std::max(1LL, (long long)(4 * sm_count()) / tiles);
-    S = std::min(S, std::max(1LL, n / 4096));
+    S = std::min(S, std::max(1LL, n / 512));
     S = std::min(S, 65535LL);
     const long long chunk = (n + S - 1) / S;
     S = (n + chunk - 1) / chunk;
