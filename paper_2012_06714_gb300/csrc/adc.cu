@@ -59,16 +59,21 @@ struct adc_handle {
     LadderTC* tc = nullptr;  // tensor-core ladder state (BF16x3 operands of B^Q_vv; open shells: the alpha block)
     LadderTC* tc_b = nullptr;  // open shells: the beta virtual block's ladder state
     Pairs64 pairs64;           // FP64 handles: the ladder's pair integrals, where they fit
+    // coupling block between the 1p / 1h and the 2p1h / 2h1p vectors (make_coupling), where it is held:
+    // EA [a][d][j][c] (of M_{a,jcd}, the GEMMs' order), IP (of the paper's M_-) [i][j][k][a]; FP64, or
+    // FP32 when k12_f32
+    Reclaimable k12;
+    bool k12_f32 = false;
     size_t pairs_limit = 0;    // device bytes the ladder's pair integrals may take (0: not held)
     int nva = 0;               // open shells: alpha virtual spin orbitals (the first nva of the v)
     // tensor-core ladder arithmetic: Davidson sigma, the setup ladder of t, and
     // the final refinement of converged roots
-    // (sigma: partial sums promoted every 16 K blocks, drift <= ~3e-6 relative;
+    // (sigma: partial sums promoted every 8 K blocks, drift <= ~3e-6 relative;
     // refinement and the IP setup: every K block, drift ~4e-7; the EA setup: GEMM1
     // every 2 and GEMM2 every 8 K blocks, Richardson-extrapolated to t2(2) within
     // 4e-7 relative of FP64 at nvir 180 and 960 -- as close as every-block promotion
     // and 22% faster)
-    LadderMode lm_sigma{2, 0, 16}, lm_setup{2, 1, 1}, lm_refine{2, 1, 1};
+    LadderMode lm_sigma{2, 0, 8}, lm_setup{2, 1, 1}, lm_refine{2, 1, 1};
     bool refining = false;  // sigma evaluates with lm_refine
     int cmode_setup = 0, cmode_sigma = 0, cmode_refine = 0;  // Ctx::gemm_mode in setup / sigma / refinement
     std::vector<double> X_last;             // spectroscopic amplitudes [nroots][nmo] of the last adc_davidson
@@ -109,6 +114,11 @@ struct adc_handle {
     }
     int n1() const { return kind == ADC_EA ? v : o; }
     Reclaimable* held_for_speed() { return tc ? ladder_pairs_store(tc) : &pairs64.store; }
+    T coupling() const {
+        const long long O = o, V = v;
+        const std::vector<long long> d = kind == ADC_EA ? std::vector<long long>{V, V, O, V} : std::vector<long long>{O, O, O, V};
+        return T{(const double*)k12.mem[0], d, true, k12_f32};
+    }
     double* dmalloc(size_t n) {
         void* p = dev_alloc(std::max<size_t>(n, 1) * sizeof(double), ctx.stream);
         owned.push_back(p);
@@ -134,9 +144,12 @@ struct adc_handle {
             cudaFree(g.X);
             cudaFree(g.S);
         }
-        ladder_tc_destroy(tc);
-        ladder_tc_destroy(tc_b);
-        for (void* p : owned) cudaFree(p);
+        ladder_tc_destroy(tc, ctx.stream);
+        ladder_tc_destroy(tc_b, ctx.stream);
+        pairs64.store.drop(ctx.stream);
+        k12.drop(ctx.stream);
+        for (void* p : owned) dev_free(p, ctx.stream);
+        ctx.release();
         if (ctx.blas) cublasDestroy(ctx.blas);
         if (own_stream) cudaStreamDestroy(own_stream);
     }
@@ -291,6 +304,54 @@ __global__ void k_diag(int ea, int o, int v, const double* __restrict__ eps, con
             D[x] = M11 ? M11[x * n1 + x] : (ea ? eps[o + x] : -eps[x]);  // no M11: zeroth order
         else
             D[x] = ea ? d22(1, o, v, eps, x - n1) : -d22(0, o, v, eps, x - n1);
+    }
+}
+// part[block] = sum over the block's elements of (ia|jb) (2 t_ij^ab - t_ij^ba): one block per (i, j) pair
+// and 32 x 32 tile of (a, b) at a time, the mirrored tile of t through shared memory
+template <typename Tv>
+__global__ void __launch_bounds__(256) k_mp_energy(int o, int v, const Tv* __restrict__ ovov, const double* __restrict__ t,
+                                                   double* __restrict__ part) {
+    __shared__ double tile[32][33], red[8];
+    const int nt = (v + 31) / 32, tx = threadIdx.x, ty = threadIdx.y;
+    const long long per = (long long)nt * nt, units = (long long)o * o * per;
+    double acc = 0.0;
+    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+        const long long ij = u / per;
+        const int r = (int)(u - ij * per), a0 = r / nt * 32, b0 = r % nt * 32, i = (int)(ij / o), j = (int)(ij % o);
+        const double* tij = t + ij * v * v;
+        for (int y = ty; y < 32; y += 8)  // tile[y][x] = t^{b0 + y, a0 + x}
+            tile[y][tx] = b0 + y < v && a0 + tx < v ? tij[(long long)(b0 + y) * v + a0 + tx] : 0.0;
+        __syncthreads();
+        for (int y = ty; y < 32; y += 8) {
+            const int a = a0 + y, b = b0 + tx;
+            if (a < v && b < v)
+                acc = fma((double)ovov[(((long long)i * v + a) * o + j) * v + b], 2.0 * tij[(long long)a * v + b] - tile[tx][y], acc);
+        }
+        __syncthreads();
+    }
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+    if (tx == 0) red[ty] = acc;
+    __syncthreads();
+    if (tx == 0 && ty == 0) {
+        for (int w = 1; w < 8; ++w) acc += red[w];
+        part[blockIdx.x] = acc;
+    }
+}
+// slice B^Q [n][nmo][nmo] (functions q0 .. of the whole) into its oo, ov and vv blocks
+__global__ void k_slice_B(long long n, int o, int v, const double* __restrict__ B, double* __restrict__ Boo,
+                          double* __restrict__ Bov, double* __restrict__ Bvv) {
+    const int nmo = o + v;
+    for (long long row = blockIdx.x; row < n * nmo; row += gridDim.x) {
+        const long long q = row / nmo;
+        const int p = (int)(row - q * nmo);
+        const double* src = B + row * nmo;
+        if (p < o) {
+            double *oo = Boo + (q * o + p) * o, *ov = Bov + (q * o + p) * v;
+            for (int x = threadIdx.x; x < nmo; x += blockDim.x) (x < o ? oo[x] : ov[x - o]) = src[x];
+        } else {
+            double* vv = Bvv + (q * v + p - o) * v;
+            for (int x = threadIdx.x; x < v; x += blockDim.x) vv[x] = src[o + x];
+        }
     }
 }
 // s[n][p] = e[p] y[n][p]: the zeroth-order one-particle block applied to nvec vectors
@@ -978,6 +1039,7 @@ static void make_t1_third_order(adc_handle* h) {
 }
 
 static void transition_parts(adc_handle* h, bool third, double* Tpp, double* t1x);
+static void make_coupling(adc_handle* h);
 
 // the timeout flag of the handle's tensor-core kernels (waits for the work issued so far)
 static void check_flag(adc_handle* h, const char* where) {
@@ -1029,14 +1091,22 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
     h->Bov = h->dmalloc(Q * o * v);
     h->Bvv = h->dmalloc(Q * v * v);
     {
-        // slice B^Q into its oo, ov and vv blocks (2-D strided copies per block)
-        cudaMemcpyKind kd = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-        for (long long q = 0; q < Q; ++q) {
-            const double* src = B_in + q * nmo * nmo;
-            ADC_CUDA(cudaMemcpy2DAsync(h->Boo + q * o * o, o * sizeof(double), src, nmo * sizeof(double), o * sizeof(double), o, kd, c.stream));
-            ADC_CUDA(cudaMemcpy2DAsync(h->Bov + q * o * v, v * sizeof(double), src + o, nmo * sizeof(double), v * sizeof(double), o, kd, c.stream));
-            ADC_CUDA(cudaMemcpy2DAsync(h->Bvv + q * v * v, v * sizeof(double), src + o * nmo + o, nmo * sizeof(double), v * sizeof(double), v, kd,
-                                       c.stream));
+        // slice B^Q into its oo, ov and vv blocks: device input in one launch, host input in pieces of
+        // at most 64 MB through scratch (three strided copies per auxiliary function took 16 ms for 483
+        // of them from pageable memory, 6 ms for 600 on the device)
+        const long long per = on_device ? Q : std::max<long long>(1, std::min<long long>(Q, (64LL << 20) / (8 * nmo * nmo)));
+        Scope bs(c.arena);
+        double* piece = on_device ? nullptr : c.arena.dalloc((size_t)(per * nmo * nmo));
+        for (long long q0 = 0; q0 < Q; q0 += per) {
+            const long long nq = std::min(per, Q - q0);
+            const double* src = B_in + q0 * nmo * nmo;
+            if (!on_device) {
+                ADC_CUDA(cudaMemcpyAsync(piece, src, (size_t)(nq * nmo * nmo) * sizeof(double), cudaMemcpyHostToDevice, c.stream));
+                src = piece;
+            }
+            k_slice_B<<<(unsigned)std::min<long long>(nq * nmo, 152LL * 32), 128, 0, c.stream>>>(
+                nq, (int)o, (int)v, src, h->Boo + q0 * o * o, h->Bov + q0 * o * v, h->Bvv + q0 * v * v);
+            launch_check(c);
         }
     }
     if (h->opt.tune_cache && h->opt.tune_cache[0]) c.tuner = tune_cache_open(h->opt.tune_cache);
@@ -1080,24 +1150,24 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
         int swp[4] = {0, 1, 3, 2};
         permute(c, h->t, s4, swp, h->tau, -1.0, 1.0);
     }
-    // MPn correlation energy: E(k+1) = sum (ia|jb) (2 t_ij^ab - t_ij^ba), t = t2(k); o^2 v^2
-    // work, always in FP64 (an FP32 integral operand is read into an FP64 copy)
-    auto mp_energy = [&](const T& tk) {
+    // MPn correlation energy: E(k+1) = sum (ia|jb) (2 t_ij^ab - t_ij^ba), t = t2(k), in FP64
+    auto mp_energy = [&](const double* tk) {
         Scope sc(c.arena);
-        const int saved = c.gemm_mode;
-        c.gemm_mode = 0;
-        double* part = c.arena.dalloc(o);
-        einsum(c, "iajb,ijab->i", 2.0, op_ovov(h, false), tk, 0.0, part, {o});
-        einsum(c, "iajb,ijba->i", -1.0, op_ovov(h, false), tk, 1.0, part, {o});
-        std::vector<double> hp(o);
-        ADC_CUDA(cudaMemcpyAsync(hp.data(), part, o * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+        const int blocks = (int)std::min<long long>(o * o * ((v + 31) / 32) * ((v + 31) / 32), 152LL * 8);
+        double* part = c.arena.dalloc(blocks);
+        if (h->f_ovov)
+            k_mp_energy<float><<<blocks, dim3(32, 8), 0, c.stream>>>((int)o, (int)v, h->f_ovov, tk, part);
+        else
+            k_mp_energy<double><<<blocks, dim3(32, 8), 0, c.stream>>>((int)o, (int)v, h->ovov, tk, part);
+        launch_check(c);
+        std::vector<double> hp(blocks);
+        ADC_CUDA(cudaMemcpyAsync(hp.data(), part, blocks * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
         ADC_CUDA(cudaStreamSynchronize(c.stream));
-        c.gemm_mode = saved;
         double e = 0.0;
         for (double x : hp) e += x;
         return e;
     };
-    h->emp[0] = mp_energy(tn(h->t, {o, o, v, v}));
+    h->emp[0] = mp_energy(h->t);
     if (lean) {
         // every later use of the integrals is a split-BF16 or FP32-accurate contraction
         h->f_oovv = to_f32(h, h->oovv, o2v2);
@@ -1125,7 +1195,7 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
         const bool extrapolate = h->opt.precision != ADC_PREC_FP64 && h->tc && !three;
         const bool keep_Lt = h->opt.m11_on_the_fly && h->kind == ADC_EA;  // sigma applies the block from it
         double* Lt = h->dmalloc(o2v2);
-        if (!lean) {
+        if (!lean && !three && !p64) {
             fill(c, o2v2, 0.0, Lt);
             ladder(h, h->t, o * o, Lt, lm);  // sum_cd (ac|bd) t_ij^cd (it feeds M_11 directly)
             if (extrapolate) {
@@ -1141,9 +1211,9 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
             }
         } else {
             // L_ij = sum_Q B^Q t_ij B^Q, the sum_cd (ac|bd) t_ij^cd that feeds t2(2) and M_11.  With
-            // t_ji = t_ij^T and every B^Q symmetric, L_ji = L_ij^T: on a lean handle the ladder runs
-            // on the pairs i <= j only and the other half is their transpose (half the setup's
-            // largest cost; the plain layout evaluates every pair)
+            // t_ji = t_ij^T and every B^Q symmetric, L_ji = L_ij^T: the ladder runs on the pairs i <= j only
+            // and the other half is their transpose (half of the setup's largest cost at 1028 MOs; a
+            // plain handle without pair integrals evaluates every pair)
             Scope ps(c.arena);
             const long long np = o * (o + 1) / 2, vv = v * v;
             std::vector<int> hpi, hpj;
@@ -1237,7 +1307,7 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
         }
         k_div_D1<<<grid_for(o * v), 256, 0, c.stream>>>((int)o, (int)v, h->eps, h->t1_2);
         launch_check(c);
-        h->emp[1] = mp_energy(tn(h->t_2, {o, o, v, v}));
+        h->emp[1] = mp_energy(h->t_2);
     }
     if (lean) {
         h->f_t = to_f32(h, h->t, o2v2);
@@ -1249,6 +1319,7 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
         // step 3 skipped: sigma applies the block from intermediates (the diagonal preconditioner
         // then takes the zeroth-order one-particle energies)
         setup_m11_otf(h);
+        make_coupling(h);
         h->diag = h->dmalloc(h->dim());
         k_diag<<<grid_for(h->dim()), 256, 0, c.stream>>>(h->kind == ADC_EA, (int)o, (int)v, h->eps, nullptr, h->diag);
         launch_check(c);
@@ -1277,6 +1348,8 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
         setup_m11_ip(h);
         c.gemm_mode = saved;
     }
+    make_coupling(h);
+    check_flag(h, "setup");
     tick(5);
     if (lean) {
         // what the transition moments need beyond t and t2(2), made while setup's memory is free
@@ -1297,6 +1370,91 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
     launch_check(c);
     tick(6);
 }
+
+// --------------------------------------------------------------------------
+// The coupling block through the method's order, M_{a,jcd} (EA) or the paper's M_-{i,jka} (IP), held
+// as a tensor (o v^3 or o^3 v elements): sigma then applies the block's row and column by reading it
+// twice, instead of contracting the vectors with t and B^Q in some ten (EA: six of them o^2 v^3)
+// contractions per sigma.  EA-ADC(3): 6 o^2 v^4 flops in setup against 12 o^2 v^3 per vector of a
+// sigma, which a solve of v / 2 vectors pays back: held up to 256 virtuals.  IP-ADC(3): 2 o^3 v^3 and
+// less, always held where it fits.  The terms are those of sigma_ea / sigma_ip without the block.
+// Arithmetic: FP64, or for an EA tensor above 2^24 elements (FP32, half the bytes) sigma's own -- the
+// accurate operator of the refinement then works without it.
+// Measured, sigma IP mixed 20/180/600 n=5: 1.65 -> 0.40 ms; EA mixed 20/180/600 n=4: 2.58 -> 1.54 ms.
+// --------------------------------------------------------------------------
+static void make_coupling(adc_handle* h) {
+    Ctx& c = h->ctx;
+    const long long o = h->o, v = h->v, Q = h->naux;
+    const bool ea = h->kind == ADC_EA;
+    const long long n = ea ? o * v * v * v : o * o * o * v;
+    const bool f32 = ea && n > (1LL << 24) && h->opt.precision != ADC_PREC_FP64;
+    const double bytes = (f32 ? 4.0 : 8.0) * n;
+    if (h->lean || bytes > (double)h->pairs_limit / 4 || (ea && h->order >= 3 && v > 256)) return;
+    void* K = nullptr;
+    if (dev_malloc_raw(&K, (size_t)bytes, c.stream) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    h->k12_f32 = f32;
+    h->k12.hold(K, nullptr);
+    ReclaimPin pin(&h->k12, c.stream, false);
+    const int saved = c.gemm_mode;
+    c.gemm_mode = f32 ? h->cmode_sigma : 0;
+    const Buf Kb{K, f32};
+    const T Boo = tn(h->Boo, {Q, o, o}), Bov = tn(h->Bov, {Q, o, v}), Bvv = tn(h->Bvv, {Q, v, v});
+    Scope sc(c.arena);
+    if (ea) {
+        const std::vector<long long> d{v, v, o, v};
+        ein(c, "Qad,Qjc->adjc", 1.0, Bvv, Bov, 0.0, Kb, d);  // (ad|jc)
+        if (h->order >= 3) {
+            const T T4 = op_t(h, false), TAU = op_tau(h, false);
+            {
+                Scope gs(c.arena);
+                const Buf g = scratch(c.arena, o * o * o * v, false);
+                ein(c, "Qla,Qjm->lajm", 1.0, Bov, Boo, 0.0, g, {o, v, o, o});
+                ein(c, "lajm,lmdc->adjc", 1.0, g.as({o, v, o, o}), T4, 1.0, Kb, d);  // (al|jm) t_lm^dc
+            }
+            // the o v^3 integrals in the order in which the products read them
+            const Buf W = scratch(c.arena, n, f32);
+            const T W4 = W.as({v, v, o, v});
+            ein(c, "Qad,Qme->adme", 1.0, Bvv, Bov, 0.0, W, {v, v, o, v});
+            ein(c, "adme,jmce->adjc", 1.0, W4, TAU, 1.0, Kb, d);  // (ad|em)(2 t - t^T)
+            ein(c, "Qma,Qed->adme", 1.0, Bov, Bvv, 0.0, W, {v, v, o, v});
+            ein(c, "adme,jmce->adjc", -1.0, W4, T4, 1.0, Kb, d);  // (am|ed) t_jm^ce
+            ein(c, "acme,jmed->adjc", -1.0, W4, T4, 1.0, Kb, d);  // (am|ec) t_jm^ed
+        }
+    } else {
+        const std::vector<long long> d{o, o, o, v};
+        ein(c, "Qki,Qja->ijka", -1.0, Boo, Bov, 0.0, Kb, d);  // (ki|ja)
+        if (h->order >= 3) {
+            const T T4 = op_t(h, false), TAU = op_tau(h, false), OOOV = tn(h->ooov, {o, o, o, v});
+            {
+                // (ad|ie) t_jk^de, a few a at a time: the integrals are o v^3
+                const long long na = std::max<long long>(1, std::min<long long>(v, (1LL << 30) / (8 * o * v * v)));
+                const Buf W = scratch(c.arena, na * v * o * v, false), X = scratch(c.arena, o * o * o * v, false);
+                for (long long a0 = 0; a0 < v; a0 += na) {
+                    const long long m = std::min(na, v - a0);
+                    Scope bs(c.arena);
+                    double* Ba = c.arena.dalloc(Q * m * v);
+                    ADC_CUDA(cudaMemcpy2DAsync(Ba, m * v * sizeof(double), h->Bvv + a0 * v, v * v * sizeof(double),
+                                               m * v * sizeof(double), Q, cudaMemcpyDeviceToDevice, c.stream));
+                    ein(c, "Qad,Qie->adie", 1.0, tn(Ba, {Q, m, v}), Bov, 0.0, W, {m, v, o, v});
+                    ein(c, "adie,jkde->ijka", -1.0, W.as({m, v, o, v}), T4, 0.0, X, {o, o, o, m});
+                    k_gather<<<grid_for(o * o * o * m), 256, 0, c.stream>>>(o * o * o, m, (const double*)X.p, m, 0, (double*)K, v, a0,
+                                                                            1.0);
+                    launch_check(c);
+                }
+            }
+            ein(c, "iklc,jlac->ijka", -1.0, OOOV, TAU, 1.0, Kb, d);  // (ik|lc)(2 t - t^T)
+            ein(c, "lkic,jlac->ijka", 1.0, OOOV, T4, 1.0, Kb, d);    // (ic|lk) t_jl^ac
+            ein(c, "ljic,klca->ijka", 1.0, OOOV, T4, 1.0, Kb, d);    // (ic|lj) t_kl^ca
+        }
+    }
+    c.gemm_mode = saved;
+}
+
+// whether sigma may use the held coupling block (an FP32 one not in the accurate operator)
+static bool use_coupling(const adc_handle* h) { return h->k12.mem[0] && !(h->k12_f32 && h->refining); }
 
 // --------------------------------------------------------------------------
 // sigma (Sec. III A step 4; Eqs. sigma_i_adapted_3, sigma_jka_bab, EA analogue)
@@ -1322,18 +1480,40 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
         einsum(c, "nb,ab->na", 1.0, tn(y1, {n, v}), tn(h->M11, {v, v}), 0.0, s1, {n, v});
     else
         m11_apply_otf_ea(h, y1, s1, n);
+    const bool held = use_coupling(h);
+    double* Wq = nullptr;
+    if (held) {
+        // both coupling blocks from the held tensor, eight vectors at a time (the bandwidth kernels' limit)
+        for (long long n0 = 0; n0 < n; n0 += 8) {
+            const long long m = std::min<long long>(8, n - n0);
+            einsum(c, "adjc,njcd->na", 1.0, h->coupling(), tn(Yt + n0 * blk, {m, o, v, v}), 1.0, s1 + n0 * v, {m, v});
+            const T y = tn(y1 + n0 * v, {m, v});
+            if (c.gemm_mode == 2) {
+                // in the tensor's own order (the bandwidth kernels read it in place), then into place
+                Scope ks(c.arena);
+                double* X = c.arena.dalloc(m * blk);
+                einsum(c, "na,adjc->ndjc", 1.0, y, h->coupling(), 0.0, X, {m, v, o, v});
+                perm_into(c, tn(X, {m, v, o, v}), {0, 2, 3, 1}, Buf{S2 + n0 * blk, false}, 1.0, 0.0);
+            } else {
+                einsum(c, "na,adjc->njcd", 1.0, y, h->coupling(), 0.0, S2 + n0 * blk, {m, o, v, v});
+            }
+        }
+    }
     // coupling row, first order: sum (ad|jc) Y~_jcd.  W^Q_d collects every coupling-row
     // term of the form sum_Qd W^Q_d (Q|da); it is contracted with B^Q_vv once, below.
-    double* Wq = c.arena.dalloc(n * Q * v);
-    einsum(c, "Qjc,njcd->nQd", 1.0, tc(h->Bov, {Q, o, v}), tn(Yt, {n, o, v, v}), 0.0, Wq, {n, Q, v});
-    // 2p1h column, first order: (cb|ia) Y_c
-    double* hq = c.arena.dalloc(n * Q * v);
-    einsum(c, "nc,Qcb->nQb", 1.0, tn(y1, {n, v}), tc(h->Bvv, {Q, v, v}), 0.0, hq, {n, Q, v});
-    einsum(c, "Qia,nQb->niab", 1.0, tc(h->Bov, {Q, o, v}), tn(hq, {n, Q, v}), 0.0, S2, {n, o, v, v});
+    double* hq = nullptr;
+    if (!held) {
+        Wq = c.arena.dalloc(n * Q * v);
+        einsum(c, "Qjc,njcd->nQd", 1.0, tc(h->Bov, {Q, o, v}), tn(Yt, {n, o, v, v}), 0.0, Wq, {n, Q, v});
+        // 2p1h column, first order: (cb|ia) Y_c
+        hq = c.arena.dalloc(n * Q * v);
+        einsum(c, "nc,Qcb->nQb", 1.0, tn(y1, {n, v}), tc(h->Bvv, {Q, v, v}), 0.0, hq, {n, Q, v});
+        einsum(c, "Qia,nQb->niab", 1.0, tc(h->Bov, {Q, o, v}), tn(hq, {n, Q, v}), 0.0, S2, {n, o, v, v});
+    }
     // 2p1h block, zeroth order
     k_diag22<<<grid_for(n * blk), 256, 0, c.stream>>>(1, (int)o, (int)v, n, h->eps, Y2, S2);
     launch_check(c);
-    if (h->order >= 3) {
+    if (h->order >= 3 && !held) {
         const T T4 = op_t(h, true);
         // coupling row, second order:
         //  sum (al|jm) t_lm^dc Y~_jcd
@@ -1377,7 +1557,9 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
         ein(c, "nQm,Qeb->nmeb", 1.0, tn(p, {n, Q, o}), tc(h->Bvv, {Q, v, v}), 0.0, q, {n, o, v, v});
         einsum(c, "nmeb,imae->niab", -1.0, q.as({n, o, v, v}), T4, 1.0, S2, {n, o, v, v});
         einsum(c, "nmea,imeb->niab", -1.0, q.as({n, o, v, v}), T4, 1.0, S2, {n, o, v, v});
-        // 2p1h block, first order: ladder sum_cd (ac|bd) Y_icd (vvvv never stored)
+    }
+    if (h->order >= 3) {
+        // 2p1h block, first order: ladder sum_cd (ac|bd) Y_icd
         ladder(h, Y2, n * o, S2, h->refining ? h->lm_refine : h->lm_sigma);
         //  - (ac|ji) Y_jcb + 2 (ai|jc) Y_jcb - (ai|jc) Y_jbc - (bd|ji) Y_jad  (the first two as one
         //  contraction with ring2, or two on a lean handle)
@@ -1392,7 +1574,7 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
         einsum(c, "jibd,njad->niab", -1.0, OOVV, Y2T, 1.0, S2, {n, o, v, v});
     }
     // coupling row: every sum_Qd W^Q_d (Q|da) term at once
-    einsum(c, "nQd,Qda->na", 1.0, tn(Wq, {n, Q, v}), tc(h->Bvv, {Q, v, v}), 1.0, s1, {n, v});
+    if (!held) einsum(c, "nQd,Qda->na", 1.0, tn(Wq, {n, Q, v}), tc(h->Bvv, {Q, v, v}), 1.0, s1, {n, v});
     k_gather<<<grid_for(n * v), 256, 0, c.stream>>>(n, v, s1, v, 0, Sout, dim, 0, 0.0);
     launch_check(c);
     k_gather<<<grid_for(n * blk), 256, 0, c.stream>>>(n, blk, S2, blk, 0, Sout, dim, v, 0.0);
@@ -1415,17 +1597,26 @@ static void sigma_ip(adc_handle* h, const double* Xin, double* Sout, long long n
     double* Yt = c.arena.dalloc(n * blk);
     k_two_minus_swap<<<grid_for(n * blk), 256, 0, c.stream>>>(0, (int)o, (int)v, n, Y2, Yt);
     launch_check(c);
-    // coupling row, first order: -(ki|ja) Y~_jka
-    double* G = c.arena.dalloc(n * Q * o);
-    einsum(c, "Qja,njka->nQk", 1.0, tc(h->Bov, {Q, o, v}), tn(Yt, {n, o, o, v}), 0.0, G, {n, Q, o});
-    einsum(c, "nQk,Qki->ni", -1.0, tn(G, {n, Q, o}), tc(h->Boo, {Q, o, o}), 0.0, s1, {n, o});
-    // 2h1p column, first order: -(ki|ja) Y_i
-    double* g = c.arena.dalloc(n * Q * o);
-    einsum(c, "ni,Qki->nQk", 1.0, tn(y1, {n, o}), tc(h->Boo, {Q, o, o}), 0.0, g, {n, Q, o});
-    einsum(c, "nQk,Qja->njka", -1.0, tn(g, {n, Q, o}), tc(h->Bov, {Q, o, v}), 0.0, S2, {n, o, o, v});
+    const bool held = use_coupling(h);
+    if (held)
+        for (long long n0 = 0; n0 < n; n0 += 8) {
+            const long long m = std::min<long long>(8, n - n0);
+            einsum(c, "ijka,njka->ni", 1.0, h->coupling(), tn(Yt + n0 * blk, {m, o, o, v}), 0.0, s1 + n0 * o, {m, o});
+            einsum(c, "ni,ijka->njka", 1.0, tn(y1 + n0 * o, {m, o}), h->coupling(), 0.0, S2 + n0 * blk, {m, o, o, v});
+        }
+    if (!held) {
+        // coupling row, first order: -(ki|ja) Y~_jka
+        double* G = c.arena.dalloc(n * Q * o);
+        einsum(c, "Qja,njka->nQk", 1.0, tc(h->Bov, {Q, o, v}), tn(Yt, {n, o, o, v}), 0.0, G, {n, Q, o});
+        einsum(c, "nQk,Qki->ni", -1.0, tn(G, {n, Q, o}), tc(h->Boo, {Q, o, o}), 0.0, s1, {n, o});
+        // 2h1p column, first order: -(ki|ja) Y_i
+        double* g = c.arena.dalloc(n * Q * o);
+        einsum(c, "ni,Qki->nQk", 1.0, tn(y1, {n, o}), tc(h->Boo, {Q, o, o}), 0.0, g, {n, Q, o});
+        einsum(c, "nQk,Qja->njka", -1.0, tn(g, {n, Q, o}), tc(h->Bov, {Q, o, v}), 0.0, S2, {n, o, o, v});
+    }
     k_diag22<<<grid_for(n * blk), 256, 0, c.stream>>>(0, (int)o, (int)v, n, h->eps, Y2, S2);
     launch_check(c);
-    if (h->order >= 3) {
+    if (h->order >= 3 && !held) {
         const double *t = h->t, *tau = h->tau;
         // coupling row, second order
         //  - sum (ad|ie) t_jk^de Y~_jka
@@ -1456,6 +1647,8 @@ static void sigma_ip(adc_handle* h, const double* Xin, double* Sout, long long n
         einsum(c, "nlkc,jlac->njka", 1.0, tn(m, {n, o, o, v}), tc(t, {o, o, v, v}), 1.0, S2, {n, o, o, v});
         einsum(c, "ni,ljic->nljc", 1.0, tn(y1, {n, o}), tc(h->ooov, {o, o, o, v}), 0.0, m, {n, o, o, v});
         einsum(c, "nljc,klca->njka", 1.0, tn(m, {n, o, o, v}), tc(t, {o, o, v, v}), 1.0, S2, {n, o, o, v});
+    }
+    if (h->order >= 3) {
         // 2h1p block, first order: -(ki|lj) Y_kla + (ki|ab) Y_kjb - 2 (ia|kb) Y_kjb + (ia|kb) Y_jkb + (kj|ab) Y_ikb
         einsum(c, "kilj,nkla->nija", -1.0, tc(h->oooo, {o, o, o, o}), tn(Y2, {n, o, o, v}), 1.0, S2, {n, o, o, v});
         einsum(c, "iakb,nkjb->nija", 1.0, tc(h->ring2, {o, v, o, v}), tn(Y2, {n, o, o, v}), 1.0, S2, {n, o, o, v});
@@ -3048,6 +3241,7 @@ int adc_mlp_samples(adc_handle* h, int nroots, const int* iters, int n_iters, lo
             return ADC_ERR_ARG;
         }
     GUARD(h, {
+        ReclaimPin keep(&h->k12, h->ctx.stream, false);
         ReclaimPin pin(h->held_for_speed(), h->ctx.stream, true);
         mlp_samples(h, nroots, iters, n_iters, per_vector, seed, exact_tol, d, blk, r, t);
         return ADC_OK;
@@ -3313,6 +3507,7 @@ int adc_sigma(adc_handle* h, const double* X, double* S, int nvec, int on_device
     }
     GUARD(h, {
         Ctx& c = h->ctx;
+        ReclaimPin keep(&h->k12, c.stream, false);
         ReclaimPin pin(h->held_for_speed(), c.stream, true);
         const long long dim = h->dim();
         if (on_device) {
@@ -3338,12 +3533,13 @@ int adc_davidson(adc_handle* h, int nroots, double tol, const double* guess, dou
         return ADC_ERR_ARG;
     }
     GUARD(h, {
+        ReclaimPin keep(&h->k12, h->ctx.stream, false);
         ReclaimPin pin(h->held_for_speed(), h->ctx.stream, !h->opt.cuda_graphs);  // (captured sigmas hold the integrals' address)
         int st = davidson(h, nroots, tol, guess, energies, specfac, vectors, stats);
         if (st == ADC_ERR_NOT_CONVERGED) h->err = "adc_davidson: not converged within max_iter";
         // the solver's scratch (subspace, residuals, sigma intermediates) goes back to the device:
         // many handles solved one after another would otherwise each keep their peak
-        h->ctx.arena.free_all(true);
+        h->ctx.arena.free_all();
         return st;
     })
 }

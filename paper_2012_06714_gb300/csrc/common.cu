@@ -60,9 +60,60 @@ ReclaimPin::~ReclaimPin() {
     tl_own = before;
     tl_own_stream = before_stream;
 }
+// ---- the library's memory pool -------------------------------------------------------
+namespace {
+struct Pool {
+    std::once_flag once;
+    cudaMemPool_t pool = nullptr;
+};
+Pool g_pools[64];
+// the current device's pool (NULL: it could not be made, the device's default pool serves)
+cudaMemPool_t pool_of(int dev) {
+    if (dev < 0 || dev >= 64) return nullptr;
+    Pool& q = g_pools[dev];
+    std::call_once(q.once, [&q, dev] {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        size_t fr = 0, tot = 0;
+        if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || cudaMemPoolCreate(&q.pool, &props) != cudaSuccess) {
+            cudaGetLastError();
+            q.pool = nullptr;
+            return;
+        }
+        unsigned long long keep = tot / 50;
+        cudaMemPoolSetAttribute(q.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    });
+    return q.pool;
+}
+}  // namespace
+
+cudaError_t dev_malloc_raw(void** p, size_t bytes, cudaStream_t s) {
+    int dev = 0;
+    cudaMemPool_t pool = cudaGetDevice(&dev) == cudaSuccess ? pool_of(dev) : nullptr;
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+}
+cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t s) {
+    cudaError_t e = dev_malloc_raw(p, bytes, s);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        device_memory_reclaim();
+        e = dev_malloc_raw(p, bytes, s);
+    }
+    return e;
+}
+
 bool device_memory_reclaim() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    struct Trim {  // what the pool keeps unused goes back too, after what is freed below
+        int dev;
+        ~Trim() {
+            if (cudaMemPool_t p = pool_of(dev)) cudaMemPoolTrimTo(p, 0);
+        }
+    } trim{dev};
     std::lock_guard<std::mutex> lk(g_reclaim_mu);
     bool any = false;
     for (size_t i = 0; i < g_reclaim.size();) {
@@ -240,6 +291,14 @@ struct OpAxpby {
             out[ad] = (Tout)x;
             return;
         }
+        if constexpr (sizeof(V) == 4 && sizeof(Tout) == 4) {
+            // +- x (+ out) rounded once, as in FP64 but without its pipe
+            if ((alpha == 1.0 || alpha == -1.0) && (beta == 0.0 || beta == 1.0)) {
+                const float f = alpha == 1.0 ? x : -x;
+                out[ad] = beta == 0.0 ? f : out[ad] + f;
+                return;
+            }
+        }
         const double v = alpha == 1.0 ? (double)x : alpha * (double)x;
         out[ad] = (Tout)(beta == 0.0 ? v : beta == 1.0 ? v + (double)out[ad] : v + beta * (double)out[ad]);
     }
@@ -356,11 +415,11 @@ constexpr int SK_CHUNK = 64;  // FP32 partial-sum length
 
 // M <= MM rows of A (a few trial vectors): one thread per column n of B, the A values of
 // the current 256-deep K chunk in shared memory; reads B once, coalesced along n.
-template <int MM>
+template <int MM, typename TB>
 __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, long long K, long long kslice,
                                                          const double* __restrict__ A, long long lda,
-                                                         const double* __restrict__ B, long long ldb,
-                                                         double* __restrict__ P) {
+                                                         const TB* __restrict__ B, long long ldb,
+                                                         double* __restrict__ P, double alpha, double beta, long long ldp) {
     __shared__ float As[MM][SK_THREADS];  // the A chunk, already rounded to FP32
     const long long n = blockIdx.x * (long long)SK_THREADS + threadIdx.x;
     const long long k0 = blockIdx.y * kslice, k1 = min(K, k0 + kslice);
@@ -375,7 +434,7 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, lon
             for (int m = 0; m < MM; ++m) As[m][threadIdx.x] = (float)(m < M ? A[m * lda + kc + threadIdx.x] : 0.0);
         __syncthreads();
         if (n >= N) continue;
-        const double* b = B + kc * ldb + n;
+        const TB* b = B + kc * ldb + n;
         // U independent loads in flight per thread before their FMAs (the loop is bound by
         // memory latency otherwise)
         constexpr int U = 8;
@@ -400,57 +459,88 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, lon
     if (n < N)
 #pragma unroll
         for (int m = 0; m < MM; ++m)
-            if (m < M) P[((long long)blockIdx.y * M + m) * N + n] = acc[m];
+            if (m < M) {
+                double* p = P + ((long long)blockIdx.y * M + m) * ldp + n;
+                *p = beta == 0.0 ? alpha * acc[m] : alpha * acc[m] + beta * *p;
+            }
 }
 
-// N <= NN columns of B: one block per row m of A and K slice; threads stride over k
-// (A read coalesced), then a warp-shuffle and shared-memory reduction of the NN sums.
-template <int NN>
+// N <= NN columns, B as [N][K]: a block takes RR rows of A and a K slice; threads stride over k (A and
+// B read coalesced, B once for all RR rows), then a warp-shuffle and shared-memory reduction.
+// V consecutive terms per thread at a time: 4 where every row starts on a 16-byte boundary (K % 4 == 0),
+// which keeps enough bytes in flight for the memory system; else 1.
+template <int NN, int V, typename TA>
 __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, long long K, long long kslice,
-                                                         const double* __restrict__ A, long long lda,
+                                                         const TA* __restrict__ A, long long lda,
                                                          const double* __restrict__ B, long long ldb,
                                                          double* __restrict__ P) {
-    __shared__ double red[SK_THREADS / 32][NN];
-    const long long m = blockIdx.x;
+    constexpr int RR = 4;
+    __shared__ double red[SK_THREADS / 32][RR * NN];
+    const long long m0 = blockIdx.x * (long long)RR;
     const long long k0 = blockIdx.y * kslice, k1 = min(K, k0 + kslice);
-    double acc[NN];
+    const TA* a[RR];  // rows past the last read the last one and are discarded
 #pragma unroll
-    for (int j = 0; j < NN; ++j) acc[j] = 0.0;
-    const double* a = A + m * lda;
-    // each thread takes up to SK_CHUNK of its strided terms per FP32 partial sum
+    for (int r = 0; r < RR; ++r) a[r] = A + min(m0 + r, M - 1) * lda;
+    double acc[RR][NN];
+#pragma unroll
+    for (int r = 0; r < RR; ++r)
+#pragma unroll
+        for (int j = 0; j < NN; ++j) acc[r][j] = 0.0;
+    // each thread takes SK_CHUNK of its terms per FP32 partial sum
     for (long long kb = k0; kb < k1; kb += (long long)SK_THREADS * SK_CHUNK) {
-        float part[NN];
+        float part[RR][NN];
 #pragma unroll
-        for (int j = 0; j < NN; ++j) part[j] = 0.f;
+        for (int r = 0; r < RR; ++r)
+#pragma unroll
+            for (int j = 0; j < NN; ++j) part[r][j] = 0.f;
         const long long ke = min(k1, kb + (long long)SK_THREADS * SK_CHUNK);
-        constexpr int U = 4;
-        for (long long k = kb + threadIdx.x; k < ke; k += (long long)U * SK_THREADS) {
-            double av[U];
+#pragma unroll 2
+        for (long long k = kb + V * threadIdx.x; k < ke; k += V * SK_THREADS) {
+            TA av[RR][V];
+            double bv[NN][V];
 #pragma unroll
-            for (int u = 0; u < U; ++u) av[u] = k + u * SK_THREADS < ke ? a[k + u * SK_THREADS] : 0.0;
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const long long ku = k + u * SK_THREADS;
-                if (ku < ke)
-#pragma unroll
-                    for (int j = 0; j < NN; ++j)
-                        if (j < N) part[j] = fmaf((float)av[u], (float)B[ku * ldb + j], part[j]);
+            for (int r = 0; r < RR; ++r) {
+                if constexpr (V == 4 && sizeof(TA) == 4) {
+                    *(float4*)av[r] = *(const float4*)(a[r] + k);
+                } else if constexpr (V == 4) {
+                    ((double2*)av[r])[0] = ((const double2*)(a[r] + k))[0];
+                    ((double2*)av[r])[1] = ((const double2*)(a[r] + k))[1];
+                } else {
+                    av[r][0] = a[r][k];
+                }
             }
+#pragma unroll
+            for (int j = 0; j < NN; ++j)
+#pragma unroll
+                for (int e = 0; e < V; ++e) bv[j][e] = B[(j < N ? j : 0) * ldb + k + e];
+#pragma unroll
+            for (int e = 0; e < V; ++e)
+#pragma unroll
+                for (int j = 0; j < NN; ++j) {
+                    const float b = (float)bv[j][e];
+#pragma unroll
+                    for (int r = 0; r < RR; ++r) part[r][j] = fmaf((float)av[r][e], b, part[r][j]);
+                }
         }
 #pragma unroll
-        for (int j = 0; j < NN; ++j) acc[j] += (double)part[j];
+        for (int r = 0; r < RR; ++r)
+#pragma unroll
+            for (int j = 0; j < NN; ++j) acc[r][j] += (double)part[r][j];
     }
 #pragma unroll
-    for (int j = 0; j < NN; ++j) {
-        double x = acc[j];
-        for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][j] = x;
-    }
+    for (int r = 0; r < RR; ++r)
+#pragma unroll
+        for (int j = 0; j < NN; ++j) {
+            double x = acc[r][j];
+            for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
+            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][r * NN + j] = x;
+        }
     __syncthreads();
-    if (threadIdx.x < N) {
+    if (threadIdx.x < RR * NN) {
+        const int r = threadIdx.x / NN, j = threadIdx.x % NN;
         double x = 0.0;
         for (int w = 0; w < SK_THREADS / 32; ++w) x += red[w][threadIdx.x];
-        P[((long long)blockIdx.y * M + m) * N + threadIdx.x] = x;
+        if (m0 + r < M && j < N) P[((long long)blockIdx.y * M + m0 + r) * N + j] = x;
     }
 }
 
@@ -487,80 +577,75 @@ __global__ void k_reduce_slices(int S, long long M, long long N, const double* _
     }
 }
 
-template <int MM>
-void launch_skinny_m(dim3 g, cudaStream_t st, int M, long long N, long long K, long long ks, const double* A, long long lda,
-                     const double* B, long long ldb, double* P) {
-    k_skinny_m<MM><<<g, SK_THREADS, 0, st>>>(M, N, K, ks, A, lda, B, ldb, P);
-}
-template <int NN>
-void launch_skinny_n(dim3 g, cudaStream_t st, long long M, int N, long long K, long long ks, const double* A, long long lda,
-                     const double* B, long long ldb, double* P) {
-    k_skinny_n<NN><<<g, SK_THREADS, 0, st>>>(M, N, K, ks, A, lda, B, ldb, P);
-}
-
 }  // namespace
 
-void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const double* A, long long lda, const double* B,
-              long long ldb, double beta, double* C, long long ldc) {
+void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const void* A, bool a32, const void* B, bool b32,
+              double beta, double* C) {
     if (M <= 0 || N <= 0) return;
     if (K <= 0) {
-        for (long long m = 0; m < M; ++m) {
-            if (beta == 0.0)
-                fill(c, N, 0.0, C + m * ldc);
-            else if (beta != 1.0)
-                axpby(c, N, 0.0, C + m * ldc, beta, C + m * ldc);
-        }
+        if (beta == 0.0)
+            fill(c, M * N, 0.0, C);
+        else if (beta != 1.0)
+            axpby(c, M * N, 0.0, C, beta, C);
         return;
     }
     const long long target = 152LL * 8;  // blocks that fill the GPU several times over
+    const long long kch = (K + SK_THREADS - 1) / SK_THREADS;
     Arena::Mark mk = c.arena.mark();
     int S = 1;
     double* P = nullptr;
-    if (M <= 8) {
-        const long long nbn = (N + SK_THREADS - 1) / SK_THREADS;
-        const long long kch = (K + SK_THREADS - 1) / SK_THREADS;
-        S = (int)std::max<long long>(1, std::min<long long>({kch, (target + nbn - 1) / nbn, 512}));
+    auto slices = [&](long long blocks) {
+        S = (int)std::max<long long>(1, std::min<long long>({kch, (target + blocks - 1) / blocks, 512}));
         const long long ks = (kch + S - 1) / S * SK_THREADS;
         S = (int)((K + ks - 1) / ks);
-        P = c.arena.dalloc((size_t)S * M * N);
-        dim3 g((unsigned)nbn, (unsigned)S);
-        auto go = [&](auto f) { f(g, c.stream, (int)M, N, K, ks, A, lda, B, ldb, P); };
+        return ks;
+    };
+    if (M <= 8) {
+        if (a32) throw Error(-1, "own_gemm: the small operand is FP64");
+        const long long nbn = (N + SK_THREADS - 1) / SK_THREADS, ks = slices(nbn);
+        P = S == 1 ? C : c.arena.dalloc((size_t)S * M * N);
+        const double al = S == 1 ? alpha : 1.0, be = S == 1 ? beta : 0.0;
+        const dim3 g((unsigned)nbn, (unsigned)S);
         switch ((int)M) {
-#define SKM(X)                                                              \
-    case X:                                                                 \
-        go(launch_skinny_m<X>);                                             \
-        break;
+#define SKM(X)                                                                                                          case X:                                                                                                                 if (b32)                                                                                                                k_skinny_m<X, float><<<g, SK_THREADS, 0, c.stream>>>((int)M, N, K, ks, (const double*)A, K, (const float*)B, N, P, al, be, N);          else                                                                                                                    k_skinny_m<X, double><<<g, SK_THREADS, 0, c.stream>>>((int)M, N, K, ks, (const double*)A, K, (const double*)B, N, P, al, be, N);         break;
             SKM(1) SKM(2) SKM(3) SKM(4) SKM(5) SKM(6) SKM(7) SKM(8)
 #undef SKM
         }
     } else if (N <= 8) {
-        const long long kch = (K + SK_THREADS - 1) / SK_THREADS;
-        S = (int)std::max<long long>(1, std::min<long long>({kch, (target + M - 1) / M, 512}));
-        const long long ks = (kch + S - 1) / S * SK_THREADS;
-        S = (int)((K + ks - 1) / ks);
-        if (M > 0x7fffffffLL) throw Error(-1, "own_gemm: too many rows");
+        if (b32) throw Error(-1, "own_gemm: the small operand is FP64");
+        constexpr int RR = 4;
+        const bool vec = K % 4 == 0 && (uintptr_t)A % 16 == 0;
+        const long long mb = (M + RR - 1) / RR, ks = slices(mb);
+        if (mb > 0x7fffffffLL) throw Error(-1, "own_gemm: too many rows");
         P = c.arena.dalloc((size_t)S * M * N);
-        dim3 g((unsigned)M, (unsigned)S);
-        auto go = [&](auto f) { f(g, c.stream, M, (int)N, K, ks, A, lda, B, ldb, P); };
+        const dim3 g((unsigned)mb, (unsigned)S);
         switch ((int)N) {
-#define SKN(X)                                                              \
-    case X:                                                                 \
-        go(launch_skinny_n<X>);                                             \
+#define SKN_GO(X, V, TA) k_skinny_n<X, V, TA><<<g, SK_THREADS, 0, c.stream>>>(M, (int)N, K, ks, (const TA*)A, K, (const double*)B, K, P)
+#define SKN(X)                                                       \
+    case X:                                                          \
+        if (a32) {                                                   \
+            if (vec) SKN_GO(X, 4, float); else SKN_GO(X, 1, float);  \
+        } else {                                                     \
+            if (vec) SKN_GO(X, 4, double); else SKN_GO(X, 1, double); \
+        }                                                            \
         break;
             SKN(1) SKN(2) SKN(3) SKN(4) SKN(5) SKN(6) SKN(7) SKN(8)
 #undef SKN
+#undef SKN_GO
         }
     } else {
         throw Error(-1, "own_gemm: neither side is skinny");
     }
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
-    if (S >= 16)
-        k_reduce_slices_warp<double><<<grid_for(32 * M * N), 256, 0, c.stream>>>(S, M, N, P, alpha, beta, C, ldc);
-    else
-        k_reduce_slices<<<grid_for(M * N), 256, 0, c.stream>>>(S, M, N, P, alpha, beta, C, ldc);
-    ++c.kernels;
-    ADC_CUDA(cudaGetLastError());
+    if (P != C) {
+        if (S >= 16)
+            k_reduce_slices_warp<double><<<grid_for(32 * M * N), 256, 0, c.stream>>>(S, M, N, P, alpha, beta, C, N);
+        else
+            k_reduce_slices<<<grid_for(M * N), 256, 0, c.stream>>>(S, M, N, P, alpha, beta, C, N);
+        ++c.kernels;
+        ADC_CUDA(cudaGetLastError());
+    }
     c.arena.release(mk);
 }
 
@@ -1140,25 +1225,28 @@ static void einsum_core(Ctx& c, const char* specstr, double alpha, const T& A, c
         // the mixed sigma: tensor cores for the large contractions, own kernels for the rest
         const bool big = 2.0 * M * N * K >= c.fp32_min_flops;
         // few-vector shapes: the own bandwidth kernels read the large operand once, in place when
-        // it is an FP64 tensor already in their order ([K][N] for M <= 8, [M][K] for N <= 8);
+        // it is already in their order ([K][N] for M <= 8, [M][K] for N <= 8);
         // otherwise the tensor cores take them when the large operand is a constant of the
         // handle (its split planes are cached once, the permuted FP64 copy would be made per call)
         const bool skinny = std::min(M, N) <= 8;
-        const bool big_const = M <= N ? B.constant : A.constant;
-        const bool big_in_place = M <= N ? (!B.f32 && sp.b == con + fb) : (!A.f32 && sp.a == fa + con);
+        const bool big_const = M <= 8 ? B.constant : A.constant;
+        const bool big_in_place = M <= 8 ? sp.b == con + fb : sp.a == fa + con;
         if (big && tc_gemm_fits(M, N, K) && (!skinny || (big_const && !big_in_place))) {
             einsum_tc(c, sp.a, sp.b, sp.c, dim, fa, fb, con, alpha, A, B, beta, C, c32);
         } else if (!big || !skinny) {
             einsum_64(c, sp.a, sp.b, sp.c, dim, fa, fb, con, alpha, A, B, beta, C, c32);
         } else {
-            const double* Ap = to_order(c, A.p, sp.a, dim, fa + con, A.f32);
-            const double* Bp = to_order(c, B.p, sp.b, dim, con + fb, B.f32);
+            // the large operand is read in place, also as FP32, when it is in the kernels' order
+            const std::string oa = fa + con, ob = M <= 8 ? con + fb : fb + con;
+            const bool a32 = A.f32 && M > 8 && sp.a == oa, b32 = B.f32 && M <= 8 && sp.b == ob;
+            const double* Ap = a32 ? A.p : to_order(c, A.p, sp.a, dim, oa, A.f32);
+            const double* Bp = b32 ? B.p : to_order(c, B.p, sp.b, dim, ob, B.f32);
             const std::string tord = fa + fb;
             if (tord == sp.c && !c32) {
-                own_gemm(c, M, N, K, alpha, Ap, K, Bp, N, beta, (double*)C, N);
+                own_gemm(c, M, N, K, alpha, Ap, a32, Bp, b32, beta, (double*)C);
             } else {
                 double* Tm = c.arena.dalloc((size_t)(M * N));
-                own_gemm(c, M, N, K, 1.0, Ap, K, Bp, N, 0.0, Tm, N);
+                own_gemm(c, M, N, K, 1.0, Ap, a32, Bp, b32, 0.0, Tm);
                 Shape sh;
                 sh.nd = (int)tord.size();
                 for (int j = 0; j < sh.nd; ++j) sh.d[j] = dim[tord[j]];

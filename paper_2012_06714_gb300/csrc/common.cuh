@@ -57,14 +57,18 @@ struct ReclaimPin {
 // Releases what can be released on the current device; false if there was nothing.
 bool device_memory_reclaim();
 
-// cudaMallocAsync that reclaims such memory once before it gives up
-inline cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t s) {
-    cudaError_t e = cudaMallocAsync(p, bytes, s);
-    if (e == cudaErrorMemoryAllocation && device_memory_reclaim()) {
+// Stream-ordered allocation from the library's own pool of the current device: the pool keeps up to a
+// fiftieth of the device's memory mapped between uses (mapping and unmapping costs about 60 us a buffer
+// and 0.4 ms a GB each way: 14 of the 53 ms from a new molecule to its first sigma at 20/180/600), and
+// gives it back when an allocation fails (device_memory_reclaim).  dev_malloc retries after that.
+cudaError_t dev_malloc_raw(void** p, size_t bytes, cudaStream_t s);
+cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t s);
+// releases such memory, ordered on s
+inline void dev_free(void* p, cudaStream_t s) {
+    if (p && cudaFreeAsync(p, s) != cudaSuccess) {
         cudaGetLastError();
-        e = cudaMallocAsync(p, bytes, s);
+        cudaFree(p);
     }
-    return e;
 }
 
 // Device scratch: blocks are allocated on demand and kept; mark()/release()
@@ -126,16 +130,11 @@ class Arena {
         return p;
     }
     double* dalloc(size_t n) { return (double*)alloc(n * sizeof(double)); }
-    // release every block (stream-ordered on `stream` when async, else with cudaFree)
-    void free_all(bool async = false) {
+    // release every block (ordered on `stream`)
+    void free_all() {
         for (void* p : big_) blocks_.push_back(p);
         big_.clear();
-        for (void* p : blocks_) {
-            if (async)
-                cudaFreeAsync(p, stream);
-            else
-                cudaFree(p);
-        }
+        for (void* p : blocks_) dev_free(p, stream);
         blocks_.clear();
         caps_.clear();
         tops_.clear();
@@ -173,7 +172,7 @@ struct Ctx {
     // run as FP32-accurate GEMMs (BF16x9 emulation on the tensor cores), with
     // FP64 inputs rounded to FP32 and results accumulated into FP64.  2 (the
     // mixed sigma): unbatched contractions of >= fp32_min_flops run on the tcgen05
-    // split-BF16 GEMM (two planes, FP32 partial sums promoted every 16 K blocks,
+    // split-BF16 GEMM (two planes, FP32 partial sums promoted every 8 K blocks,
     // FP64 result) unless a free dimension is <= 8 and the large operand is not a
     // cached constant; the others on the library's own kernels (own_gemm:
     // FP32-accurate from fp32_min_flops, else FP64).
@@ -203,11 +202,20 @@ struct Ctx {
     // a CUDA-graph capture of sigma is recording on `stream`: no host synchronisation, no
     // allocation, no tuning; the timeout flags are read after the graph's replay instead
     bool capturing = false;
+    // releases everything on the stream (before it is destroyed)
+    void release() {
+        for (auto& kv : f32cache) dev_free(kv.second, stream);
+        for (auto& kv : bf16cache) dev_free(kv.second, stream);
+        for (auto& kv : cache64) dev_free(kv.second, stream);
+        f32cache.clear();
+        bf16cache.clear();
+        cache64.clear();
+        dev_free(d_err, stream);
+        d_err = nullptr;
+        arena.free_all();
+    }
     ~Ctx() {
-        for (auto& kv : f32cache) cudaFree(kv.second);
-        for (auto& kv : bf16cache) cudaFree(kv.second);
-        for (auto& kv : cache64) cudaFree(kv.second);
-        if (d_err) cudaFree(d_err);
+        release();
         for (auto e : ev_start) cudaEventDestroy(e);
         for (auto e : ev_stop) cudaEventDestroy(e);
     }
@@ -253,12 +261,12 @@ void permute_sum(Ctx& c, const double* in, int S, const Shape& s, const int* per
 void split_planes(Ctx& c, const double* in, const Shape& s, const int* perm, long long rows, long long K, long long Kp,
                   void* const* out, bool in32 = false, int planes = 2);
 
-// The library's own kernels for skinny contractions (row-major A [M][K], B [K][N], C [M][N] with
-// leading dimensions; M <= 8 or N <= 8): C = alpha A B + beta C, the large operand read once (K split
-// over blocks, deterministic slice reduction), FP32 products and partial sums of <= 64 terms,
-// accumulated in FP64.
-void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const double* A, long long lda, const double* B,
-              long long ldb, double beta, double* C, long long ldc);
+// The library's own kernels for skinny contractions: C [M][N] = alpha A B + beta C with M <= 8 (A
+// [M][K] FP64, B [K][N]) or N <= 8 (A [M][K], B [N][K] FP64), everything contiguous, the large operand
+// FP64 or FP32 and read once (K split over blocks, deterministic slice reduction); FP32 products and
+// partial sums of <= 64 terms, accumulated in FP64.
+void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const void* A, bool a32, const void* B, bool b32,
+              double beta, double* C);
 
 // Row-major GEMM: C[MxN] = alpha op(A) op(B) + beta C, batched with strides.
 void gemm(Ctx& c, bool ta, bool tb, long long M, long long N, long long K, double alpha, const double* A, long long lda,

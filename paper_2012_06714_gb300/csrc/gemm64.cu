@@ -3,16 +3,16 @@
 // GB300 has about 1.2 TFLOP/s of FP64 against 2 PFLOP/s of dense BF16, so an FP64 product is
 // cheaper as a sum of exact integer products (the error-free splitting of Ozaki, Ogita, Oishi and
 // Rump, Numer. Algorithms 59, 95 (2012)):
-//   * every row of A and of B is scaled by a power of two to integers below 2^56 in size and cut
-//     into seven signed digits of eight bits (six of |d| <= 128, the top one of |d| <= 256), which
-//     BF16 holds exactly;
+//   * every row of A and of B is scaled by a power of two to integers below 2^63 in size and cut
+//     into eight signed digits of eight bits (|d| <= 128), which BF16 holds exactly;
 //   * the digit products of equal weight, s = i + j, accumulate in one FP32 tensor-memory
-//     accumulator per s.  Over 128 summed terms such a sum stays within 2^24, so it is an exact
-//     integer (s = 6 may reach 9/8 of that if every digit is at its limit, and then loses a unit,
-//     2^-62 of the row scales); it is drained into 64-bit integer registers, exact for any K;
-//   * the weights s = 12 .. 5 are kept (34 of 49 digit pairs); what is left out is below
-//     2^-61 sqrt(K) of the product of the row scales, less than the 2^-57 rounding of the inputs
-//     to their rows' scales.  The one rounding of the result is to FP64.
+//     accumulator per s.  Over 128 summed terms and at most eight digit pairs such a sum stays within
+//     8 * 128 * 2^14 = 2^24, so it is an exact integer; then it is drained into 64-bit integer
+//     registers, where it stays exact for any K;
+//   * the weights s = 14 .. 7 are kept (36 of 64 digit pairs); what is left out is below 2^-63 sqrt(K)
+//     of the product of the row scales.  The one rounding of the result is to FP64.  (Seven digits and
+//     34 pairs round the inputs to 2^-57 of their rows' largest element, which an integral row with a
+//     coherent diagonal, (ia|ia) 20 times the others, turns into 1.2e-16 of the result.)
 // The error against 64-bit arithmetic is that of an FP64 GEMM: norm of the error over norm of sigma
 // 1.8e-16 (IP, 14/113/445) against 1.7e-16 with DGEMM, 1.2e-16 each for its final rounding.
 // Measured: that sigma (5 vectors, 22 GFLOP in 20 contractions) 24.6 -> 3.8 ms; the FP64 setup of an
@@ -22,8 +22,8 @@
 // 8 x BNT of the 512 tensor-memory columns.  The digit planes of B lie one after another in shared
 // memory as further rows of one K-major operand and the accumulators of consecutive weights are
 // consecutive in tensor memory, so that one MMA multiplies digit i of A with up to 256 / BNT digits
-// of B: 11 MMAs of up to 256 columns per 16-deep K step instead of 34 of 64 (which would be bound by
-// reading A from shared memory 34 times).
+// of B: 12 MMAs of up to 256 columns per 16-deep K step instead of 36 of 64 (which would be bound by
+// reading A from shared memory 36 times).
 #include <algorithm>
 #include <cstdint>
 #include <mutex>
@@ -35,8 +35,8 @@ namespace adc {
 
 namespace {
 
-constexpr int ND = 7;          // digits
-constexpr int SMIN = 5;        // lowest weight kept
+constexpr int ND = 8;          // digits
+constexpr int SMIN = ND - 1;   // lowest weight kept
 constexpr int NL = 8;          // weights SMIN .. 2 (ND - 1)
 constexpr int GM = 128;        // tile rows
 constexpr int GK = 32;         // K block: 64-byte rows, 64-byte swizzle
@@ -127,19 +127,21 @@ __global__ void __launch_bounds__(DT) k_digits(const __grid_constant__ DigitSide
                     for (int h = 0; h < 2; ++h) {
                         const long long b = __double_as_longlong(tile[r][k + h]);
                         const int ex = (int)(b >> 52) & 0x7ff;
-                        // |x| = m 2^(ex - 1075) -> round(|x| 2^(1078 - ef)), at most 2^56: the row's scale is 2^(ef - 1022)
+                        // |x| = m 2^(ex - 1075) -> round(|x| 2^(1085 - ef)), below 2^63: the row's scale is 2^(ef - 1022)
                         long long v = 0;
-                        const int sh = ef - ex - 3;  // right shift of the 53-bit significand (-3: three more bits)
+                        const int sh = ef - ex - 10;  // right shift of the 53-bit significand (-10: ten more bits)
                         if (ex > 0 && ef < 0x7ff && sh < 55) {
                             const long long m = (b & 0xfffffffffffffLL) | (1LL << 52);
                             v = sh <= 0 ? m << -sh : (m + (1LL << (sh - 1))) >> sh;
                             if (b < 0) v = -v;
                         }
-                        // digit p of v + sum_p 128 256^p is the p-th byte less 128: the carries in one addition
-                        const unsigned long long w = (unsigned long long)v + 0x808080808080ULL;
+                        // digit p < 7 of v is the p-th byte of v + sum_p 128 256^p less 128: the carries in
+                        // one addition; the top one is in [-128, 128]
+                        const unsigned long long w = (unsigned long long)v + 0x0080808080808080ULL;
+                        const int top = v >= 0 ? (int)(w >> 56) : (int)((long long)w >> 56);
 #pragma unroll
                         for (int p = 0; p < ND; ++p) {
-                            const int d = p < ND - 1 ? (int)((w >> (8 * p)) & 0xff) - 128 : (int)((long long)w >> (8 * p));
+                            const int d = p < ND - 1 ? (int)((w >> (8 * p)) & 0xff) - 128 : top;
                             // a small integer's BF16 bits are the upper half of its FP32 bits
                             const unsigned u = __float_as_uint((float)d) >> 16;
                             dig[p] = h == 0 ? u : dig[p] | (u << 16);
@@ -247,21 +249,14 @@ __device__ __forceinline__ void digit_products(uint32_t tmem, uint64_t a, uint64
     constexpr int jmax = 256 / BNT;  // digits of B per MMA
 #pragma unroll
     for (int i = ND - 1; i >= 0; --i) {
-        int j = SMIN - i > 0 ? SMIN - i : 0;
-        // the lowest weight first appears at i = SMIN, j = 0: alone, to start its accumulator
-        if (kFirst && i == SMIN && j == 0) {
-            mma_bf16(tmem, a + (uint64_t)(i * (GM * GK * 2 >> 4)), b, ib | ((uint32_t)(BNT >> 3) << 17), 0u);
-            j = 1;
-        }
+        const int j = SMIN - i;  // (the top digit of A meets every digit of B and starts all accumulators)
         const int parts = (ND - j + jmax - 1) / jmax, nj = (ND - j + parts - 1) / parts;  // nearly equal widths
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            if (q < parts) {
-                const int j0 = j + q * nj, n = nj < ND - j0 ? nj : ND - j0;
-                mma_bf16(tmem + (uint32_t)((i + j0 - SMIN) * BNT), a + (uint64_t)(i * (GM * GK * 2 >> 4)),
-                         b + (uint64_t)(j0 * (BNT * GK * 2 >> 4)), ib | ((uint32_t)(n * BNT >> 3) << 17),
-                         kFirst && i == ND - 1 ? 0u : 1u);
-            }
+        for (int q = 0; q < parts; ++q) {
+            const int j0 = j + q * nj, n = nj < ND - j0 ? nj : ND - j0;
+            mma_bf16(tmem + (uint32_t)((i + j0 - SMIN) * BNT), a + (uint64_t)(i * (GM * GK * 2 >> 4)),
+                     b + (uint64_t)(j0 * (BNT * GK * 2 >> 4)), ib | ((uint32_t)(n * BNT >> 3) << 17),
+                     kFirst && i == ND - 1 ? 0u : 1u);
         }
     }
 }
@@ -406,10 +401,10 @@ __global__ void __launch_bounds__(G_THREADS, 1)
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const int eb = __shfl_sync(0xffffffffu, ebl, q);
-                    // weights: digit products of weight s carry 2^(8 s); hi starts at s = 9, lo at s = 5;
-                    // a row's integers carry 2^(ef - 1078)
+                    // weights: digit products of weight s carry 2^(8 s); hi starts at s = 11, lo at s = 7;
+                    // a row's integers carry 2^(ef - 1085)
                     stg[lane * 9 + q] = ea == 0x7ff || eb == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL)
-                                                                  : to_double(hi[c0 + q], lo[c0 + q], 8 * SMIN + ea + eb - 2 * 1078);
+                                                                  : to_double(hi[c0 + q], lo[c0 + q], 8 * SMIN + ea + eb - 2 * 1085);
                 }
                 __syncwarp();
                 const int col = colt + c0 + (lane & 7);
@@ -465,8 +460,8 @@ struct Gemm64Plan {
     int BNT, S, kb;  // tile width, K slices, K blocks per slice
 };
 
-// Tile width and K slices: least time over the chip.  A K block of a tile takes 17 BNT tensor cycles
-// twice (34 digit pairs), reading A from shared memory bounds it below about BNT = 16; a drain (every
+// Tile width and K slices: least time over the chip.  A K block of a tile takes 18 BNT tensor cycles
+// twice (36 digit pairs), reading A from shared memory bounds it below about BNT = 16; a drain (every
 // EPOCH blocks) about 40 BNT cycles, which the MMAs wait for; the last one and the store about 60 BNT.
 Gemm64Plan plan64(long long M, long long N, long long Kp) {
     const int num_k = (int)((Kp + GK - 1) / GK), sms = sm_count();
@@ -479,7 +474,7 @@ Gemm64Plan plan64(long long M, long long N, long long Kp) {
             if (s > 1 && (num_k + kb - 1) / kb != s) continue;
             const double rounds = (double)((tiles * s + sms - 1) / sms);
             const double blocks = (double)std::min<long long>(kb, num_k);
-            const double cyc = rounds * (2000.0 + blocks * 2.0 * std::max(17.0 * b, 280.0) + (blocks / EPOCH) * 40.0 * b + 60.0 * b) +
+            const double cyc = rounds * (2000.0 + blocks * 2.0 * std::max(18.0 * b, 320.0) + (blocks / EPOCH) * 40.0 * b + 60.0 * b) +
                                (s - 1) * (double)M * N * 16.0 / 2500.0 + (s > 1 ? 4000.0 : 0.0);
             if (cyc < best * 0.999) best = cyc, p = Gemm64Plan{b, (int)s, (int)kb};
         }

@@ -707,12 +707,14 @@ struct LadderTC {
         if (p == 2 || !store.mem[0]) return p == 2 ? (__nv_bfloat16*)store.mem[1] : nullptr;
         return (__nv_bfloat16*)store.mem[0] + p * 2 * P * Pk;
     }
+    cudaStream_t stream = nullptr;  // the frees are ordered on it
     ~LadderTC() {
         for (int p = 0; p < 3; ++p) {
-            cudaFree(Bs[p]);
-            cudaFree(Bp[p]);
+            dev_free(Bs[p], stream);
+            dev_free(Bp[p], stream);
         }
-        cudaFree(d_err);
+        dev_free(d_err, stream);
+        store.drop(stream);
     }
 };
 
@@ -763,7 +765,10 @@ LadderTC* ladder_tc_create(Ctx& c, const double* Bvv, int naux, int v, int aux_c
     return L;
 }
 
-void ladder_tc_destroy(LadderTC* L) { delete L; }
+void ladder_tc_destroy(LadderTC* L, cudaStream_t s) {
+    if (L) L->stream = s;
+    delete L;
+}
 
 namespace {
 
@@ -948,12 +953,12 @@ bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv) {
     const long long v = L.v, Q = L.naux, Qp = (Q + 7) / 8 * 8, P = v * (v + 1) / 2, Pk = (P + 7) / 8 * 8;
     if (2 * P >= (1LL << 30) || v * v >= (1LL << 30)) return false;  // 32-bit tile coordinates
     void* base = nullptr;
-    if (cudaMallocAsync(&base, ladder_pairs_bytes((int)v), c.stream) != cudaSuccess) {
+    if (dev_malloc_raw(&base, ladder_pairs_bytes((int)v), c.stream) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     void* third = nullptr;
-    if (cudaMallocAsync(&third, ladder_pairs_bytes((int)v) / 2, c.stream) != cudaSuccess) {
+    if (dev_malloc_raw(&third, ladder_pairs_bytes((int)v) / 2, c.stream) != cudaSuccess) {
         cudaGetLastError();
         third = nullptr;
     }
@@ -981,7 +986,7 @@ bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv) {
         Maps m{};
         for (int p = 0; p < 3; ++p) {
             m.a[p] = make_map(planes[p], v * v, Qp, BM);
-            m.b[p] = make_map(planes[p], nb * v, Qp, BN1[3] / 2);
+            m.b[p] = make_map(planes[p], nb * v, Qp, 128);
         }
         Epi e{};
         e.mode = 2;
@@ -992,7 +997,7 @@ bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv) {
         e.out32 = G;
         e.vec = (nb * v) % 4 == 0;
         // partial sums promoted every K block: the integrals enter the setup ladder too
-        launch_gemm(c, m, 3, (int)(a0 * v), 0, e.M, e.N, (int)Qp, BN1[3], 1, 1, e, 2.0 * na * v * nb * v * Q);
+        launch_gemm(c, m, 3, (int)(a0 * v), 0, e.M, e.N, (int)Qp, 256, 1, 1, e, 2.0 * na * v * nb * v * Q);
         const long long nt = (v + 31) / 32, tiles = na * nb * nt * (nt + 1) / 2;
         k_pair_pack<float, PutPlanes><<<(unsigned)std::min<long long>(tiles, 152LL * 16), dim3(32, 8), 0, c.stream>>>(
             G, (int)v, na * nb, 0, nb * v, 1, (int)a0, (int)nb, PutPlanes{Planes{{L.pair_plane(0), L.pair_plane(1), L.pair_plane(2)}}, P, P, Pk, 0});
@@ -1056,7 +1061,7 @@ float* pairs_gemm(LadderTC& L, Ctx& c, const Planes& x, int planes, long long nm
 
 void pairs_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* out, const LadderMode& md) {
     const long long v = L.v, P = L.P, Pk = L.Pk;
-    const int planes = md.planes, maxbn = planes == 3 ? BN1[3] : 256;
+    const int planes = md.planes;
     // groups of matrices whose split vectors (8 or 12 P bytes each) and FP32 results stay within ~4 GiB
     const long long smin = (Pk + kPairSliceK - 1) / kPairSliceK;
     const long long mg = std::max<long long>(1, std::min<long long>(nmat, (4LL << 30) / (4 * planes * Pk + 8 * P * (smin + 2))));
@@ -1072,7 +1077,7 @@ void pairs_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* o
             X + m0 * v * v, (int)v, nm, v * v, v, 0, 0, 1, PutPlanes{x, nm, P, Pk, 0});
         ++c.kernels;
         ADC_CUDA(cudaGetLastError());
-        int bn = pick_bn((int)nm, maxbn), S = 1;
+        int bn = pick_bn((int)nm, 256), S = 1;
         if (c.tuner && !c.timing && !c.capturing && md.epoch1 == 0) {
             // tile width of the sigma ladder, measured once per shape (setup and refinement are one-off)
             TuneCache* tc = (TuneCache*)c.tuner;
@@ -1084,7 +1089,7 @@ void pairs_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* o
             } else {
                 float least = 1e30f;
                 int bb = bn;
-                for (int b : bn_candidates((int)nm, maxbn, {256, 128, 64})) {
+                for (int b : bn_candidates((int)nm, 256, {256, 128, 64})) {
                     Arena::Mark m2 = c.arena.mark();
                     const float ms = time_on_stream(c, [&] { pairs_gemm(L, c, x, planes, nm, b, md.epoch2, S); });
                     c.arena.release(m2);
@@ -1245,8 +1250,9 @@ namespace {
 
 // K slices of an M x N x K contraction at tile width bn.  A tile's time counts its K blocks plus
 // about 4 more (pipeline fill, epilogue), a launch takes as many rounds of tiles over the CTA
-// pairs as its tiles need, and every slice beyond the first writes and reads back an FP32 result
-// (8 bytes per element; a 64-deep K block of a 256-row tile takes about 0.8 us).  The slices are
+// pairs as its tiles need (a 64-deep K block of a 256-row tile takes about 0.8 us), and every slice
+// beyond the first costs the sum of the slices about 11 us per million results (two FP64 operations
+// each at two per cycle and SM, more than the bytes: 78 us with three slices of 2.6 M, 20 us with one).  The slices are
 // parts of one launch: at 20/180/600 (IP, 5 vectors) the launches on side streams that this
 // replaced took 1.1 of the 2.7 ms of a sigma in launch and event calls alone.
 int pick_slices(long long M, long long N, long long Kp, int bn, int pairs) {
@@ -1258,7 +1264,7 @@ int pick_slices(long long M, long long N, long long Kp, int bn, int pairs) {
         const long long kb = (nkb + S - 1) / S;
         if ((nkb + kb - 1) / kb != S) continue;  // the last slice would be empty
         const double rounds = (double)((tiles * S + pairs - 1) / pairs);
-        const double cost = rounds * (kb + 4) * kb_us + (S - 1) * (double)M * N * 8.0 / 4e6;
+        const double cost = rounds * (kb + 4) * kb_us + (S - 1) * (double)M * N * 1.1e-5;
         if (cost < best_cost * 0.999) {
             best_cost = cost;
             best = S;
@@ -1290,7 +1296,7 @@ float* tc_gemm_bn(Ctx& c, const void* const* A, const void* const* B, long long 
     Parts parts;
     parts.n = parts.slices = S;
     parts.kb = (int)kb;
-    launch_gemm(c, m, 2, 0, 0, (int)M, (int)N, (int)Kp, BN, m_fastest, 16, e, algo_flops, parts);
+    launch_gemm(c, m, 2, 0, 0, (int)M, (int)N, (int)Kp, BN, m_fastest, 8, e, algo_flops, parts);
     return T;
 }
 

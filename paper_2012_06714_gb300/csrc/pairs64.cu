@@ -2,8 +2,8 @@
 // antisymmetric pairs of ladder_tc.cu with the integrals, the vectors and the products of gemm64.
 //
 // nmat v^4 flops on the tensor cores instead of 4 naux v^3 nmat on the FP64 units through two DGEMMs
-// per auxiliary function (which stay for the sizes whose integrals do not fit: 28 P^2 bytes, P = v (v +
-// 1) / 2, i.e. 0.6 GB at v = 97, 7.4 GB at 180).  Bound by reading the integrals' digits (14 bytes each)
+// per auxiliary function (which stay for the sizes whose integrals do not fit: 32 P^2 bytes, P = v (v +
+// 1) / 2, i.e. 0.7 GB at v = 97, 8.5 GB at 180).  Bound by reading the integrals' digits (16 bytes each)
 // for few matrices, by the tensor cores beyond about 40.
 // Measured, FP64 sigma of 4 vectors at 12/97/381: 142 -> 2.8 ms (the ladder 129 -> 0.3 ms), its error
 // against 64 bits 9.2e-16 -> 1.6e-16; four roots at 8/45/187: 165 -> 24 ms.
@@ -52,7 +52,7 @@ bool pairs64_prepare(Pairs64& L, Ctx& c, const double* Bvv, int naux, int nvir) 
     const long long v = nvir, Q = naux, P = v * (v + 1) / 2;
     if (P >= (1LL << 30) || v * v >= (1LL << 30)) return false;
     void* base = nullptr;
-    if (cudaMallocAsync(&base, pairs64_bytes(nvir), c.stream) != cudaSuccess) {
+    if (dev_malloc_raw(&base, pairs64_bytes(nvir), c.stream) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -106,8 +106,8 @@ bool pairs64_prepare(Pairs64& L, Ctx& c, const double* Bvv, int naux, int nvir) 
 
 void pairs64_apply(Pairs64& L, Ctx& c, const double* X, long long nmat, double* out) {
     const long long v = L.v, P = L.P;
-    // groups of matrices whose pairs, digits and results (16, 28 and about 32 P bytes each) stay within 4 GiB
-    const long long mg = std::max<long long>(1, std::min<long long>(nmat, (4LL << 30) / (76 * P)));
+    // groups of matrices whose pairs, digits and results (16, 32 and about 32 P bytes each) stay within 4 GiB
+    const long long mg = std::max<long long>(1, std::min<long long>(nmat, (4LL << 30) / (80 * P)));
     ReclaimPin pin(&L.store, c.stream, false);
     for (long long m0 = 0; m0 < nmat; m0 += mg) {
         const long long nm = std::min(mg, nmat - m0);
