@@ -230,23 +230,57 @@ __global__ void k_div_D1(int o, int v, const double* __restrict__ eps, double* _
         X[x] /= eps[i] - eps[o + a];
     }
 }
-// Y~ = 2 Y - P Y on the 2p1h (EA: swap last two) or 2h1p (IP: swap first two) part, nvec blocks
-__global__ void k_two_minus_swap(int ea, int o, int v, long long nvec, const double* __restrict__ Y, double* __restrict__ Yt) {
-    long long blk = ea ? (long long)o * v * v : (long long)o * o * v;
-    long long n = nvec * blk;
-    GRID_STRIDE(x, n) {
-        long long r = x % blk, base = x - r;
-        long long s;
-        if (ea) {
-            int b = r % v, a = (r / v) % v;
-            long long i = r / ((long long)v * v);
-            s = (i * v + b) * v + a;
-        } else {
-            int a = r % v, k = (r / v) % o;
-            long long j = r / ((long long)o * v);
-            s = ((long long)k * o + j) * v + a;
+// The 2p1h / 2h1p parts of nvec vectors (rows of ldx, from element off) as contiguous Y2, and Y~ = 2 Y - P Y
+// (P: EA swaps the last two axes, IP the first two).  EA: 32 x 32 tiles of (a, b), the mirrored tile
+// through shared memory.
+__global__ void __launch_bounds__(256) k_take_ea(int o, int v, long long nvec, const double* __restrict__ X, long long ldx,
+                                                 long long off, double* __restrict__ Y2, double* __restrict__ Yt) {
+    __shared__ double tile[32][33];
+    const int nt = (v + 31) / 32, tx = threadIdx.x, ty = threadIdx.y;
+    const long long per = (long long)nt * nt, units = nvec * o * per, vv = (long long)v * v;
+    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+        const long long m = u / per;
+        const int r = (int)(u - m * per), a0 = r / nt * 32, b0 = r % nt * 32;
+        const double* src = X + (m / o) * ldx + off + (m % o) * vv;
+        for (int y = ty; y < 32; y += 8)  // tile[y][x] = Y^{b0 + y, a0 + x}
+            tile[y][tx] = b0 + y < v && a0 + tx < v ? src[(long long)(b0 + y) * v + a0 + tx] : 0.0;
+        __syncthreads();
+        for (int y = ty; y < 32; y += 8) {
+            const int a = a0 + y, b = b0 + tx;
+            if (a < v && b < v) {
+                const double x = src[(long long)a * v + b];
+                const long long at = m * vv + (long long)a * v + b;
+                Y2[at] = x;
+                Yt[at] = 2.0 * x - tile[tx][y];
+            }
         }
-        Yt[x] = 2.0 * Y[x] - Y[base + s];
+        __syncthreads();
+    }
+}
+__global__ void k_take_ip(int o, int v, long long nvec, const double* __restrict__ X, long long ldx, long long off,
+                          double* __restrict__ Y2, double* __restrict__ Yt) {
+    const long long lines = nvec * o * o;  // (n, j, k), a along the threads
+    for (long long l = blockIdx.x; l < lines; l += gridDim.x) {
+        const long long n = l / (o * o);
+        const int jk = (int)(l - n * o * o), j = jk / o, k = jk - j * o;
+        const double *x = X + n * ldx + off + (long long)jk * v, *y = X + n * ldx + off + ((long long)k * o + j) * v;
+        for (int a = threadIdx.x; a < v; a += blockDim.x) {
+            const double z = x[a];
+            Y2[l * v + a] = z;
+            Yt[l * v + a] = 2.0 * z - y[a];
+        }
+    }
+}
+// the vectors of sigma: out[n] = [s1[n], sgn S2[n] + D Y2[n]] with D the zeroth-order 2p1h / 2h1p diagonal
+__global__ void k_put(long long nvec, long long n1, long long blk, double sgn, const double* __restrict__ s1,
+                      const double* __restrict__ S2, const double* __restrict__ Y2, const double* __restrict__ D,
+                      double* __restrict__ out) {
+    const long long dim = n1 + blk;
+    for (long long n = blockIdx.y; n < nvec; n += gridDim.y) {
+        GRID_STRIDE(x, dim) {
+            out[n * dim + x] = x < n1 ? s1[n * n1 + x]
+                                      : fma(D[x], Y2[n * blk + x - n1], sgn > 0 ? S2[n * blk + x - n1] : -S2[n * blk + x - n1]);
+        }
     }
 }
 // full vectors [nvec][dim]: out = S Y (mode 0) or S^-1 Y (mode 1); S = diag(1, 2 - P)
@@ -1183,11 +1217,13 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
         // them is naux v^4 flops, the two passes of the setup ladder o^2 v^4 each with them and
         // 4 naux o^2 v^3 each without: they are made when that does not cost the setup more.
         const bool pairs = h->tc && (double)v * (Q + 2.0 * o * o) < 8.0 * Q * o * o &&
-                           ladder_pairs_bytes((int)v) <= h->pairs_limit && ladder_pairs_prepare(*h->tc, c, h->Bvv);
+                           ladder_pairs_bytes((int)v) <= h->pairs_limit &&
+                           form_if_it_fits(c, *ladder_pairs_store(h->tc), [&] { return ladder_pairs_prepare(*h->tc, c, h->Bvv); });
         // FP64: forming them and the ladder over them run on the tensor cores at some 20 times the rate
         // of the FP64 units that the ladder over the auxiliary index takes
         const bool p64 = h->opt.precision == ADC_PREC_FP64 && (double)v * (Q + o * o) < 80.0 * Q * o * o &&
-                         pairs64_bytes((int)v) <= h->pairs_limit && pairs64_prepare(h->pairs64, c, h->Bvv, (int)Q, (int)v);
+                         pairs64_bytes((int)v) <= h->pairs_limit &&
+                         form_if_it_fits(c, h->pairs64.store, [&] { return pairs64_prepare(h->pairs64, c, h->Bvv, (int)Q, (int)v); });
         // three-plane pairs: partial sums promoted every K block, where the small products come first
         // and only four MMAs truncate at full size; no extrapolation
         const bool three = pairs && ladder_pairs_third(h->tc);
@@ -1371,12 +1407,77 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
     tick(6);
 }
 
+static void coupling_into(adc_handle* h, void* K) {
+    Ctx& c = h->ctx;
+    const long long o = h->o, v = h->v, Q = h->naux;
+    const bool ea = h->kind == ADC_EA, f32 = h->k12_f32;
+    ReclaimPin pin(&h->k12, c.stream, false);
+    const int saved = c.gemm_mode;
+    c.gemm_mode = f32 ? h->cmode_sigma : 0;
+    const T Boo = tn(h->Boo, {Q, o, o}), Bov = tn(h->Bov, {Q, o, v}), Bvv = tn(h->Bvv, {Q, v, v});
+    const T T4 = op_t(h, false);
+    Scope sc(c.arena);
+    // a few a at a time: the integrals with three virtual indices are o v^2 for each (at most 2^28 values)
+    const long long na = std::max<long long>(1, std::min<long long>(v, (1LL << 28) / (o * v * v)));
+    const Buf W = h->order >= 3 ? scratch(c.arena, na * v * o * v, f32) : Buf{};
+    for (long long a0 = 0; a0 < v; a0 += na) {
+        const long long m = std::min(na, v - a0);
+        Scope bs(c.arena);
+        double* ba = c.arena.dalloc(Q * m * v);   // B^Q_ad of these a
+        double* bo = c.arena.dalloc(Q * o * m);   // B^Q_la
+        ADC_CUDA(cudaMemcpy2DAsync(ba, m * v * sizeof(double), h->Bvv + a0 * v, v * v * sizeof(double), m * v * sizeof(double), Q,
+                                   cudaMemcpyDeviceToDevice, c.stream));
+        ADC_CUDA(cudaMemcpy2DAsync(bo, m * sizeof(double), h->Bov + a0, v * sizeof(double), m * sizeof(double), Q * o,
+                                   cudaMemcpyDeviceToDevice, c.stream));
+        const T Ba = tn(ba, {Q, m, v}), Bo = tn(bo, {Q, o, m});
+        if (ea) {
+            const std::vector<long long> d{m, v, o, v};
+            const Buf Ka{f32 ? (void*)((float*)K + a0 * v * o * v) : (void*)((double*)K + a0 * v * o * v), f32};
+            ein(c, "Qad,Qjc->adjc", 1.0, Ba, Bov, 0.0, Ka, d);  // (ad|jc)
+            if (h->order < 3) continue;
+            {
+                Scope gs(c.arena);
+                const Buf g = scratch(c.arena, o * o * o * m, false);
+                ein(c, "Qla,Qjm->lajm", 1.0, Bo, Boo, 0.0, g, {o, m, o, o});
+                ein(c, "lajm,lmdc->adjc", 1.0, g.as({o, m, o, o}), T4, 1.0, Ka, d);  // (al|jm) t_lm^dc
+            }
+            // the integrals in the order in which the products read them
+            const T W4 = W.as({m, v, o, v});
+            ein(c, "Qad,Qme->adme", 1.0, Ba, Bov, 0.0, W, {m, v, o, v});
+            ein(c, "adme,jmce->adjc", 1.0, W4, op_tau(h, false), 1.0, Ka, d);  // (ad|em)(2 t - t^T)
+            ein(c, "Qma,Qed->adme", 1.0, Bo, Bvv, 0.0, W, {m, v, o, v});
+            ein(c, "adme,jmce->adjc", -1.0, W4, T4, 1.0, Ka, d);  // (am|ed) t_jm^ce
+            ein(c, "acme,jmed->adjc", -1.0, W4, T4, 1.0, Ka, d);  // (am|ec) t_jm^ed
+        } else {
+            const Buf X = scratch(c.arena, o * o * o * m, false);
+            const std::vector<long long> d{o, o, o, m};
+            ein(c, "Qki,Qja->ijka", -1.0, Boo, Bo, 0.0, X, d);  // (ki|ja)
+            if (h->order >= 3) {
+                ein(c, "Qad,Qie->adie", 1.0, Ba, Bov, 0.0, W, {m, v, o, v});
+                ein(c, "adie,jkde->ijka", -1.0, W.as({m, v, o, v}), T4, 1.0, X, d);  // (ad|ie) t_jk^de
+            }
+            k_gather<<<grid_for(o * o * o * m), 256, 0, c.stream>>>(o * o * o, m, (const double*)X.p, m, 0, (double*)K, v, a0, 0.0);
+            launch_check(c);
+        }
+    }
+    if (!ea && h->order >= 3) {
+        const std::vector<long long> d{o, o, o, v};
+        const Buf Kb{K, false};
+        const T OOOV = tn(h->ooov, {o, o, o, v});
+        ein(c, "iklc,jlac->ijka", -1.0, OOOV, op_tau(h, false), 1.0, Kb, d);  // (ik|lc)(2 t - t^T)
+        ein(c, "lkic,jlac->ijka", 1.0, OOOV, T4, 1.0, Kb, d);                 // (ic|lk) t_jl^ac
+        ein(c, "ljic,klca->ijka", 1.0, OOOV, T4, 1.0, Kb, d);                 // (ic|lj) t_kl^ca
+    }
+    c.gemm_mode = saved;
+}
+
 // --------------------------------------------------------------------------
 // The coupling block through the method's order, M_{a,jcd} (EA) or the paper's M_-{i,jka} (IP), held
 // as a tensor (o v^3 or o^3 v elements): sigma then applies the block's row and column by reading it
 // twice, instead of contracting the vectors with t and B^Q in some ten (EA: six of them o^2 v^3)
 // contractions per sigma.  EA-ADC(3): 6 o^2 v^4 flops in setup against 12 o^2 v^3 per vector of a
-// sigma, which a solve of v / 2 vectors pays back: held up to 256 virtuals.  IP-ADC(3): 2 o^3 v^3 and
+// sigma, which a solve of v / 2 vectors pays back (226 vectors for four roots at 40/400/1400): held up
+// to 512 virtuals.  IP-ADC(3): 2 o^3 v^3 and
 // less, always held where it fits.  The terms are those of sigma_ea / sigma_ip without the block.
 // Arithmetic: FP64, or for an EA tensor above 2^24 elements (FP32, half the bytes) sigma's own -- the
 // accurate operator of the refinement then works without it.
@@ -1389,7 +1490,13 @@ static void make_coupling(adc_handle* h) {
     const long long n = ea ? o * v * v * v : o * o * o * v;
     const bool f32 = ea && n > (1LL << 24) && h->opt.precision != ADC_PREC_FP64;
     const double bytes = (f32 ? 4.0 : 8.0) * n;
-    if (h->lean || bytes > (double)h->pairs_limit / 4 || (ea && h->order >= 3 && v > 256)) return;
+    if (h->lean || bytes > (double)h->pairs_limit / 4 || (ea && h->order >= 3 && v > 512)) return;
+    {
+        // with the pieces it is made from
+        size_t fr = 0, tot = 0;
+        ADC_CUDA(cudaMemGetInfo(&fr, &tot));
+        if (1.2 * bytes + 8e9 > (double)fr && bytes > 64e6) return;
+    }
     void* K = nullptr;
     if (dev_malloc_raw(&K, (size_t)bytes, c.stream) != cudaSuccess) {
         cudaGetLastError();
@@ -1397,62 +1504,11 @@ static void make_coupling(adc_handle* h) {
     }
     h->k12_f32 = f32;
     h->k12.hold(K, nullptr);
-    ReclaimPin pin(&h->k12, c.stream, false);
-    const int saved = c.gemm_mode;
-    c.gemm_mode = f32 ? h->cmode_sigma : 0;
-    const Buf Kb{K, f32};
-    const T Boo = tn(h->Boo, {Q, o, o}), Bov = tn(h->Bov, {Q, o, v}), Bvv = tn(h->Bvv, {Q, v, v});
-    Scope sc(c.arena);
-    if (ea) {
-        const std::vector<long long> d{v, v, o, v};
-        ein(c, "Qad,Qjc->adjc", 1.0, Bvv, Bov, 0.0, Kb, d);  // (ad|jc)
-        if (h->order >= 3) {
-            const T T4 = op_t(h, false), TAU = op_tau(h, false);
-            {
-                Scope gs(c.arena);
-                const Buf g = scratch(c.arena, o * o * o * v, false);
-                ein(c, "Qla,Qjm->lajm", 1.0, Bov, Boo, 0.0, g, {o, v, o, o});
-                ein(c, "lajm,lmdc->adjc", 1.0, g.as({o, v, o, o}), T4, 1.0, Kb, d);  // (al|jm) t_lm^dc
-            }
-            // the o v^3 integrals in the order in which the products read them
-            const Buf W = scratch(c.arena, n, f32);
-            const T W4 = W.as({v, v, o, v});
-            ein(c, "Qad,Qme->adme", 1.0, Bvv, Bov, 0.0, W, {v, v, o, v});
-            ein(c, "adme,jmce->adjc", 1.0, W4, TAU, 1.0, Kb, d);  // (ad|em)(2 t - t^T)
-            ein(c, "Qma,Qed->adme", 1.0, Bov, Bvv, 0.0, W, {v, v, o, v});
-            ein(c, "adme,jmce->adjc", -1.0, W4, T4, 1.0, Kb, d);  // (am|ed) t_jm^ce
-            ein(c, "acme,jmed->adjc", -1.0, W4, T4, 1.0, Kb, d);  // (am|ec) t_jm^ed
-        }
-    } else {
-        const std::vector<long long> d{o, o, o, v};
-        ein(c, "Qki,Qja->ijka", -1.0, Boo, Bov, 0.0, Kb, d);  // (ki|ja)
-        if (h->order >= 3) {
-            const T T4 = op_t(h, false), TAU = op_tau(h, false), OOOV = tn(h->ooov, {o, o, o, v});
-            {
-                // (ad|ie) t_jk^de, a few a at a time: the integrals are o v^3
-                const long long na = std::max<long long>(1, std::min<long long>(v, (1LL << 30) / (8 * o * v * v)));
-                const Buf W = scratch(c.arena, na * v * o * v, false), X = scratch(c.arena, o * o * o * v, false);
-                for (long long a0 = 0; a0 < v; a0 += na) {
-                    const long long m = std::min(na, v - a0);
-                    Scope bs(c.arena);
-                    double* Ba = c.arena.dalloc(Q * m * v);
-                    ADC_CUDA(cudaMemcpy2DAsync(Ba, m * v * sizeof(double), h->Bvv + a0 * v, v * v * sizeof(double),
-                                               m * v * sizeof(double), Q, cudaMemcpyDeviceToDevice, c.stream));
-                    ein(c, "Qad,Qie->adie", 1.0, tn(Ba, {Q, m, v}), Bov, 0.0, W, {m, v, o, v});
-                    ein(c, "adie,jkde->ijka", -1.0, W.as({m, v, o, v}), T4, 0.0, X, {o, o, o, m});
-                    k_gather<<<grid_for(o * o * o * m), 256, 0, c.stream>>>(o * o * o, m, (const double*)X.p, m, 0, (double*)K, v, a0,
-                                                                            1.0);
-                    launch_check(c);
-                }
-            }
-            ein(c, "iklc,jlac->ijka", -1.0, OOOV, TAU, 1.0, Kb, d);  // (ik|lc)(2 t - t^T)
-            ein(c, "lkic,jlac->ijka", 1.0, OOOV, T4, 1.0, Kb, d);    // (ic|lk) t_jl^ac
-            ein(c, "ljic,klca->ijka", 1.0, OOOV, T4, 1.0, Kb, d);    // (ic|lj) t_kl^ca
-        }
-    }
-    c.gemm_mode = saved;
+    form_if_it_fits(c, h->k12, [&] {
+        coupling_into(h, K);
+        return true;
+    });
 }
-
 // whether sigma may use the held coupling block (an FP32 one not in the accurate operator)
 static bool use_coupling(const adc_handle* h) { return h->k12.mem[0] && !(h->k12_f32 && h->refining); }
 
@@ -1470,11 +1526,13 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
     double* S2 = c.arena.dalloc(n * blk);
     k_gather<<<grid_for(n * v), 256, 0, c.stream>>>(n, v, Xin, dim, 0, y1, v, 0, 0.0);
     launch_check(c);
-    k_gather<<<grid_for(n * blk), 256, 0, c.stream>>>(n, blk, Xin, dim, v, Y2, blk, 0, 0.0);
-    launch_check(c);
     double* Yt = c.arena.dalloc(n * blk);
-    k_two_minus_swap<<<grid_for(n * blk), 256, 0, c.stream>>>(1, (int)o, (int)v, n, Y2, Yt);
-    launch_check(c);
+    {
+        const long long nt = (v + 31) / 32;
+        k_take_ea<<<(unsigned)std::min<long long>(n * o * nt * nt, 152LL * 32), dim3(32, 8), 0, c.stream>>>((int)o, (int)v, n, Xin, dim,
+                                                                                                     v, Y2, Yt);
+        launch_check(c);
+    }
     // 1p row: M_ab Y_b (precomputed block, or on the fly)
     if (h->M11)
         einsum(c, "nb,ab->na", 1.0, tn(y1, {n, v}), tn(h->M11, {v, v}), 0.0, s1, {n, v});
@@ -1510,9 +1568,6 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
         einsum(c, "nc,Qcb->nQb", 1.0, tn(y1, {n, v}), tc(h->Bvv, {Q, v, v}), 0.0, hq, {n, Q, v});
         einsum(c, "Qia,nQb->niab", 1.0, tc(h->Bov, {Q, o, v}), tn(hq, {n, Q, v}), 0.0, S2, {n, o, v, v});
     }
-    // 2p1h block, zeroth order
-    k_diag22<<<grid_for(n * blk), 256, 0, c.stream>>>(1, (int)o, (int)v, n, h->eps, Y2, S2);
-    launch_check(c);
     if (h->order >= 3 && !held) {
         const T T4 = op_t(h, true);
         // coupling row, second order:
@@ -1575,9 +1630,9 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
     }
     // coupling row: every sum_Qd W^Q_d (Q|da) term at once
     if (!held) einsum(c, "nQd,Qda->na", 1.0, tn(Wq, {n, Q, v}), tc(h->Bvv, {Q, v, v}), 1.0, s1, {n, v});
-    k_gather<<<grid_for(n * v), 256, 0, c.stream>>>(n, v, s1, v, 0, Sout, dim, 0, 0.0);
-    launch_check(c);
-    k_gather<<<grid_for(n * blk), 256, 0, c.stream>>>(n, blk, S2, blk, 0, Sout, dim, v, 0.0);
+    // (with the zeroth-order 2p1h diagonal)
+    k_put<<<dim3((unsigned)grid_for(dim), (unsigned)std::min<long long>(n, 64)), 256, 0, c.stream>>>(n, v, blk, 1.0, s1, S2, Y2, h->diag,
+                                                                                             Sout);
     launch_check(c);
 }
 
@@ -1592,10 +1647,8 @@ static void sigma_ip(adc_handle* h, const double* Xin, double* Sout, long long n
     double* S2 = c.arena.dalloc(n * blk);
     k_gather<<<grid_for(n * o), 256, 0, c.stream>>>(n, o, Xin, dim, 0, y1, o, 0, 0.0);
     launch_check(c);
-    k_gather<<<grid_for(n * blk), 256, 0, c.stream>>>(n, blk, Xin, dim, o, Y2, blk, 0, 0.0);
-    launch_check(c);
     double* Yt = c.arena.dalloc(n * blk);
-    k_two_minus_swap<<<grid_for(n * blk), 256, 0, c.stream>>>(0, (int)o, (int)v, n, Y2, Yt);
+    k_take_ip<<<(unsigned)std::min<long long>(n * o * o, 152LL * 32), 128, 0, c.stream>>>((int)o, (int)v, n, Xin, dim, o, Y2, Yt);
     launch_check(c);
     const bool held = use_coupling(h);
     if (held)
@@ -1614,8 +1667,6 @@ static void sigma_ip(adc_handle* h, const double* Xin, double* Sout, long long n
         einsum(c, "ni,Qki->nQk", 1.0, tn(y1, {n, o}), tc(h->Boo, {Q, o, o}), 0.0, g, {n, Q, o});
         einsum(c, "nQk,Qja->njka", -1.0, tn(g, {n, Q, o}), tc(h->Bov, {Q, o, v}), 0.0, S2, {n, o, o, v});
     }
-    k_diag22<<<grid_for(n * blk), 256, 0, c.stream>>>(0, (int)o, (int)v, n, h->eps, Y2, S2);
-    launch_check(c);
     if (h->order >= 3 && !held) {
         const double *t = h->t, *tau = h->tau;
         // coupling row, second order
@@ -1662,10 +1713,9 @@ static void sigma_ip(adc_handle* h, const double* Xin, double* Sout, long long n
         m11_apply_otf_ip(h, y1, s1, n);
         axpby(c, n * o, 0.0, s1, -1.0, s1);
     }
-    k_gather<<<grid_for(n * o), 256, 0, c.stream>>>(n, o, s1, o, 0, Sout, dim, 0, 0.0);
-    launch_check(c);
-    axpby(c, n * blk, 0.0, S2, -1.0, S2);
-    k_gather<<<grid_for(n * blk), 256, 0, c.stream>>>(n, blk, S2, blk, 0, Sout, dim, o, 0.0);
+    // (negated, with the zeroth-order 2h1p diagonal of -M_-)
+    k_put<<<dim3((unsigned)grid_for(dim), (unsigned)std::min<long long>(n, 64)), 256, 0, c.stream>>>(n, o, blk, -1.0, s1, S2, Y2, h->diag,
+                                                                                             Sout);
     launch_check(c);
 }
 
@@ -3325,12 +3375,12 @@ static int setup_one(const double* eps, const double* Bq, int nocc, int nvir, in
             lean = plain_bytes > 0.9 * (double)fr;
         }
         {
-            // the pair integrals of the ladder: at most a third of the free memory, and what the
+            // the pair integrals of the ladder: at most two fifths of the free memory, and what the
             // plain layout's setup leaves (plain_bytes)
             size_t fr = 0, tot = 0;
             ADC_CUDA(cudaMemGetInfo(&fr, &tot));
             const double left = 0.9 * (double)fr - plain_bytes;
-            h->pairs_limit = (size_t)std::max(0.0, std::min((double)fr / 3.0, left));
+            h->pairs_limit = (size_t)std::max(0.0, std::min(0.4 * (double)fr, left));
             // digits of constant operands of FP64 contractions (not on a lean handle)
             if (!lean) h->ctx.cache64_bytes = std::min<size_t>(h->pairs_limit / 8, size_t(4) << 30);
         }

@@ -413,19 +413,22 @@ inline int grid_for(long long n) {
 constexpr int SK_THREADS = 256;
 constexpr int SK_CHUNK = 64;  // FP32 partial-sum length
 
-// M <= MM rows of A (a few trial vectors): one thread per column n of B, the A values of
-// the current 256-deep K chunk in shared memory; reads B once, coalesced along n.
-template <int MM, typename TB>
+// M <= MM rows of A (a few trial vectors): V consecutive columns of B per thread (4 where every row of B
+// starts on a 16-byte boundary, N % 4 == 0: enough bytes in flight for the memory system), the A values
+// of the current K chunk in shared memory; reads B once, coalesced along n.
+template <int MM, int V, typename TB>
 __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, long long K, long long kslice,
                                                          const double* __restrict__ A, long long lda,
                                                          const TB* __restrict__ B, long long ldb,
-                                                         double* __restrict__ P, double alpha, double beta, long long ldp) {
+                                                         double* __restrict__ P, double alpha, double beta) {
     __shared__ float As[MM][SK_THREADS];  // the A chunk, already rounded to FP32
-    const long long n = blockIdx.x * (long long)SK_THREADS + threadIdx.x;
+    const long long n = (blockIdx.x * (long long)SK_THREADS + threadIdx.x) * V;
     const long long k0 = blockIdx.y * kslice, k1 = min(K, k0 + kslice);
-    double acc[MM];
+    double acc[MM][V];
 #pragma unroll
-    for (int m = 0; m < MM; ++m) acc[m] = 0.0;
+    for (int m = 0; m < MM; ++m)
+#pragma unroll
+        for (int e = 0; e < V; ++e) acc[m][e] = 0.0;
     for (long long kc = k0; kc < k1; kc += SK_THREADS) {
         const int kn = (int)min((long long)SK_THREADS, k1 - kc);
         __syncthreads();
@@ -437,32 +440,52 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, lon
         const TB* b = B + kc * ldb + n;
         // U independent loads in flight per thread before their FMAs (the loop is bound by
         // memory latency otherwise)
-        constexpr int U = 8;
+        constexpr int U = V == 4 ? 4 : 8;
         for (int k2 = 0; k2 < kn; k2 += SK_CHUNK) {
-            float part[MM];
+            float part[MM][V];
 #pragma unroll
-            for (int m = 0; m < MM; ++m) part[m] = 0.f;
+            for (int m = 0; m < MM; ++m)
+#pragma unroll
+                for (int e = 0; e < V; ++e) part[m][e] = 0.f;
             const int ke = min(kn, k2 + SK_CHUNK);
             for (int kk = k2; kk < ke; kk += U) {
-                float bv[U];
+                TB bv[U][V];
 #pragma unroll
-                for (int u = 0; u < U; ++u) bv[u] = kk + u < ke ? (float)b[(long long)(kk + u) * ldb] : 0.f;
+                for (int u = 0; u < U; ++u) {
+                    const TB* p = b + (long long)(kk + u < ke ? kk + u : ke - 1) * ldb;
+                    if constexpr (V == 4 && sizeof(TB) == 4) {
+                        *(float4*)bv[u] = *(const float4*)p;
+                    } else if constexpr (V == 4) {
+                        ((double2*)bv[u])[0] = ((const double2*)p)[0];
+                        ((double2*)bv[u])[1] = ((const double2*)p)[1];
+                    } else {
+                        bv[u][0] = *p;
+                    }
+                }
 #pragma unroll
                 for (int u = 0; u < U; ++u)
 #pragma unroll
-                    for (int m = 0; m < MM; ++m) part[m] = fmaf(kk + u < ke ? As[m][kk + u] : 0.f, bv[u], part[m]);
+                    for (int m = 0; m < MM; ++m) {
+                        const float a = kk + u < ke ? As[m][kk + u] : 0.f;
+#pragma unroll
+                        for (int e = 0; e < V; ++e) part[m][e] = fmaf(a, (float)bv[u][e], part[m][e]);
+                    }
             }
 #pragma unroll
-            for (int m = 0; m < MM; ++m) acc[m] += (double)part[m];
+            for (int m = 0; m < MM; ++m)
+#pragma unroll
+                for (int e = 0; e < V; ++e) acc[m][e] += (double)part[m][e];
         }
     }
     if (n < N)
 #pragma unroll
         for (int m = 0; m < MM; ++m)
-            if (m < M) {
-                double* p = P + ((long long)blockIdx.y * M + m) * ldp + n;
-                *p = beta == 0.0 ? alpha * acc[m] : alpha * acc[m] + beta * *p;
-            }
+            if (m < M)
+#pragma unroll
+                for (int e = 0; e < V; ++e) {
+                    double* p = P + ((long long)blockIdx.y * M + m) * N + n + e;
+                    *p = beta == 0.0 ? alpha * acc[m][e] : alpha * acc[m][e] + beta * *p;
+                }
 }
 
 // N <= NN columns, B as [N][K]: a block takes RR rows of A and a K slice; threads stride over k (A and
@@ -472,7 +495,7 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, lon
 template <int NN, int V, typename TA>
 __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, long long K, long long kslice,
                                                          const TA* __restrict__ A, long long lda,
-                                                         const double* __restrict__ B, long long ldb,
+                                                         const float* __restrict__ B, long long ldb,
                                                          double* __restrict__ P) {
     constexpr int RR = 4;
     __shared__ double red[SK_THREADS / 32][RR * NN];
@@ -497,7 +520,7 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, lon
 #pragma unroll 2
         for (long long k = kb + V * threadIdx.x; k < ke; k += V * SK_THREADS) {
             TA av[RR][V];
-            double bv[NN][V];
+            float bv[NN][V];
 #pragma unroll
             for (int r = 0; r < RR; ++r) {
                 if constexpr (V == 4 && sizeof(TA) == 4) {
@@ -511,13 +534,18 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, lon
             }
 #pragma unroll
             for (int j = 0; j < NN; ++j)
-#pragma unroll
-                for (int e = 0; e < V; ++e) bv[j][e] = B[(j < N ? j : 0) * ldb + k + e];
+            {
+                const float* b = B + (j < N ? j : 0) * ldb + k;
+                if constexpr (V == 4)
+                    *(float4*)bv[j] = *(const float4*)b;
+                else
+                    bv[j][0] = *b;
+            }
 #pragma unroll
             for (int e = 0; e < V; ++e)
 #pragma unroll
                 for (int j = 0; j < NN; ++j) {
-                    const float b = (float)bv[j][e];
+                    const float b = bv[j][e];
 #pragma unroll
                     for (int r = 0; r < RR; ++r) part[r][j] = fmaf((float)av[r][e], b, part[r][j]);
                 }
@@ -602,25 +630,35 @@ void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const
     };
     if (M <= 8) {
         if (a32) throw Error(-1, "own_gemm: the small operand is FP64");
-        const long long nbn = (N + SK_THREADS - 1) / SK_THREADS, ks = slices(nbn);
+        const bool vec = N % 4 == 0 && (uintptr_t)B % 16 == 0 && N >= 4096;
+        const long long cols = vec ? 4 * SK_THREADS : SK_THREADS, nbn = (N + cols - 1) / cols, ks = slices(nbn);
         P = S == 1 ? C : c.arena.dalloc((size_t)S * M * N);
         const double al = S == 1 ? alpha : 1.0, be = S == 1 ? beta : 0.0;
         const dim3 g((unsigned)nbn, (unsigned)S);
         switch ((int)M) {
-#define SKM(X)                                                                                                          case X:                                                                                                                 if (b32)                                                                                                                k_skinny_m<X, float><<<g, SK_THREADS, 0, c.stream>>>((int)M, N, K, ks, (const double*)A, K, (const float*)B, N, P, al, be, N);          else                                                                                                                    k_skinny_m<X, double><<<g, SK_THREADS, 0, c.stream>>>((int)M, N, K, ks, (const double*)A, K, (const double*)B, N, P, al, be, N);         break;
+#define SKM_GO(X, V, TB) k_skinny_m<X, V, TB><<<g, SK_THREADS, 0, c.stream>>>((int)M, N, K, ks, (const double*)A, K, (const TB*)B, N, P, al, be)
+#define SKM(X)                                                       \
+    case X:                                                          \
+        if (b32) {                                                   \
+            if (vec) SKM_GO(X, 4, float); else SKM_GO(X, 1, float);  \
+        } else {                                                     \
+            if (vec) SKM_GO(X, 4, double); else SKM_GO(X, 1, double); \
+        }                                                            \
+        break;
             SKM(1) SKM(2) SKM(3) SKM(4) SKM(5) SKM(6) SKM(7) SKM(8)
 #undef SKM
+#undef SKM_GO
         }
     } else if (N <= 8) {
-        if (b32) throw Error(-1, "own_gemm: the small operand is FP64");
+        if (!b32) throw Error(-1, "own_gemm: the small operand is FP32");
         constexpr int RR = 4;
-        const bool vec = K % 4 == 0 && (uintptr_t)A % 16 == 0;
+        const bool vec = K % 4 == 0 && (uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0;
         const long long mb = (M + RR - 1) / RR, ks = slices(mb);
         if (mb > 0x7fffffffLL) throw Error(-1, "own_gemm: too many rows");
         P = c.arena.dalloc((size_t)S * M * N);
         const dim3 g((unsigned)mb, (unsigned)S);
         switch ((int)N) {
-#define SKN_GO(X, V, TA) k_skinny_n<X, V, TA><<<g, SK_THREADS, 0, c.stream>>>(M, (int)N, K, ks, (const TA*)A, K, (const double*)B, K, P)
+#define SKN_GO(X, V, TA) k_skinny_n<X, V, TA><<<g, SK_THREADS, 0, c.stream>>>(M, (int)N, K, ks, (const TA*)A, K, (const float*)B, K, P)
 #define SKN(X)                                                       \
     case X:                                                          \
         if (a32) {                                                   \
@@ -1238,9 +1276,24 @@ static void einsum_core(Ctx& c, const char* specstr, double alpha, const T& A, c
         } else {
             // the large operand is read in place, also as FP32, when it is in the kernels' order
             const std::string oa = fa + con, ob = M <= 8 ? con + fb : fb + con;
-            const bool a32 = A.f32 && M > 8 && sp.a == oa, b32 = B.f32 && M <= 8 && sp.b == ob;
+            const bool a32 = A.f32 && M > 8 && sp.a == oa, b32 = M > 8 || (B.f32 && sp.b == ob);
             const double* Ap = a32 ? A.p : to_order(c, A.p, sp.a, dim, oa, A.f32);
-            const double* Bp = b32 ? B.p : to_order(c, B.p, sp.b, dim, ob, B.f32);
+            const void* Bp;
+            if (M > 8 && !(B.f32 && sp.b == ob)) {
+                // the few columns rounded to FP32 once (the kernel would do it for every four rows)
+                Shape bs;
+                bs.nd = (int)sp.b.size();
+                int bp[kMaxDim];
+                for (int j = 0; j < bs.nd; ++j) {
+                    bs.d[j] = dim[sp.b[j]];
+                    bp[j] = (int)sp.b.find(ob[j]);
+                }
+                float* f = (float*)c.arena.alloc((size_t)(K * N) * sizeof(float));
+                permute_any(c, B.p, B.f32, bs, bp, f, true, 1.0, 0.0);
+                Bp = f;
+            } else {
+                Bp = b32 ? B.p : to_order(c, B.p, sp.b, dim, ob, B.f32);
+            }
             const std::string tord = fa + fb;
             if (tord == sp.c && !c32) {
                 own_gemm(c, M, N, K, alpha, Ap, a32, Bp, b32, beta, (double*)C);

@@ -221,6 +221,25 @@ struct Ctx {
     }
 };
 
+// Forms memory held for speed (r) by f; true if f said so.  f may run out of memory on the way: r and what
+// f took are then given back, and the caller goes on without r.
+template <typename F>
+bool form_if_it_fits(Ctx& c, Reclaimable& r, F f) {
+    const Arena::Mark mk = c.arena.mark();
+    const int saved = c.gemm_mode;
+    try {
+        return f();
+    } catch (const Error& e) {
+        if (e.code != -2) throw;  // (ADC_ERR_OOM)
+    }
+    cudaGetLastError();
+    c.arena.release(mk);
+    c.gemm_mode = saved;
+    r.drop(c.stream);
+    device_memory_reclaim();
+    return false;
+}
+
 constexpr int kMaxDim = 8;
 struct Shape {
     int nd;
@@ -262,7 +281,7 @@ void split_planes(Ctx& c, const double* in, const Shape& s, const int* perm, lon
                   void* const* out, bool in32 = false, int planes = 2);
 
 // The library's own kernels for skinny contractions: C [M][N] = alpha A B + beta C with M <= 8 (A
-// [M][K] FP64, B [K][N]) or N <= 8 (A [M][K], B [N][K] FP64), everything contiguous, the large operand
+// [M][K] FP64, B [K][N]) or N <= 8 (A [M][K], B [N][K] FP32), everything contiguous, the large operand
 // FP64 or FP32 and read once (K split over blocks, deterministic slice reduction); FP32 products and
 // partial sums of <= 64 terms, accumulated in FP64.
 void own_gemm(Ctx& c, long long M, long long N, long long K, double alpha, const void* A, bool a32, const void* B, bool b32,
