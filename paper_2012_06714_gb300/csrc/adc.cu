@@ -405,12 +405,17 @@ __global__ void k_gather(long long nvec, long long len, const double* __restrict
     }
 }
 // Davidson correction: out[r][x] = R[r][x] / (w_r - D[x]) with |w - D| >= 1e-8
-__global__ void k_precond(long long nr, long long dim, const double* __restrict__ R, const double* __restrict__ w,
-                          const double* __restrict__ D, double* __restrict__ out) {
-    long long n = nr * dim;
-    GRID_STRIDE(x, n) {
-        long long r = x / dim, k = x % dim;
-        double den = w[r] - D[k];
+struct Corrections {
+    int root[8], to[8];
+    double w[8];
+};
+__global__ void k_corrections(Corrections q, long long dim, const double* __restrict__ R, const double* __restrict__ D,
+                              double* __restrict__ out) {
+    const double w = q.w[blockIdx.y];
+    R += q.root[blockIdx.y] * dim;
+    out += q.to[blockIdx.y] * dim;
+    GRID_STRIDE(x, dim) {
+        double den = w - D[x];
         if (fabs(den) < 1e-8) den = den < 0 ? -1e-8 : 1e-8;
         out[x] = R[x] / den;
     }
@@ -1485,7 +1490,7 @@ static void coupling_into(adc_handle* h, void* K) {
 // --------------------------------------------------------------------------
 static void make_coupling(adc_handle* h) {
     Ctx& c = h->ctx;
-    const long long o = h->o, v = h->v, Q = h->naux;
+    const long long o = h->o, v = h->v;
     const bool ea = h->kind == ADC_EA;
     const long long n = ea ? o * v * v * v : o * o * o * v;
     const bool f32 = ea && n > (1LL << 24) && h->opt.precision != ADC_PREC_FP64;
@@ -1896,8 +1901,8 @@ struct Davidson {
         Scope gs(c.arena);
         const int kt = k0 + kn;
         double* A = c.arena.dalloc((size_t)kt * kn * 2);
-        multidot(c, kt, SV, dim, kn, W + (long long)k0 * dim, dim, dim, A);            // SV_i . W_{k0+j}
-        multidot(c, kt, W, dim, kn, SV + (long long)k0 * dim, dim, dim, A + kt * kn);  // W_i . SV_{k0+j}
+        // SV_i . W_{k0+j} and W_i . SV_{k0+j}
+        multidot(c, kt, SV, dim, kn, W + (long long)k0 * dim, dim, dim, A, W, SV + (long long)k0 * dim);
         std::vector<double> hA((size_t)kt * kn * 2);
         ADC_CUDA(cudaMemcpyAsync(hA.data(), A, hA.size() * sizeof(double), cudaMemcpyDeviceToHost, h->ctx.stream));
         ADC_CUDA(cudaStreamSynchronize(h->ctx.stream));
@@ -1909,37 +1914,59 @@ struct Davidson {
             }
     }
     // S-orthonormalise rows [first, first+count) of V against rows [0, first) and each other; returns kept count.
-    // Block classical Gram-Schmidt against the basis (two passes), then one new vector at a time.
+    // Block classical Gram-Schmidt against the basis (a second pass only where the first removed more than
+    // 1 - 1/sqrt(2) of a vector's S-norm, the Daniel-Gragg-Kaufman-Stewart criterion), then the Cholesky
+    // factor of the new vectors' overlap where they are well apart, else one new vector at a time.
     int orthonormalise(int first, int count) {
         Ctx& c = h->ctx;
         Scope os(c.arena);
-        double* D = V + (long long)first * dim;
+        double *D = V + (long long)first * dim, *SD = SV + (long long)first * dim;
         double* cf = c.arena.dalloc((size_t)std::max(1, count) * std::max(1, first + count));
-        if (first > 0) {
-            // second pass only where the first removed more than 1 - 1/sqrt(2) of a vector's
-            // S-norm (the Daniel-Gragg-Kaufman-Stewart criterion)
-            double* SD = c.arena.dalloc((size_t)count * dim);
-            double* nn = c.arena.dalloc((size_t)count * count);
-            auto snorms = [&](std::vector<double>& out) {
-                metric(D, SD, count, 0);
-                multidot(c, count, D, dim, count, SD, dim, dim, nn);
-                std::vector<double> m((size_t)count * count);
-                ADC_CUDA(cudaMemcpyAsync(m.data(), nn, m.size() * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-                ADC_CUDA(cudaStreamSynchronize(c.stream));
-                out.resize(count);
-                for (int r = 0; r < count; ++r) out[r] = m[(size_t)r * count + r];
-            };
-            std::vector<double> before, after;
-            snorms(before);
-            for (int pass = 0; pass < 2; ++pass) {
+        double* nn = c.arena.dalloc((size_t)2 * count * count);
+        std::vector<double> g((size_t)2 * count * count);  // overlaps of the new vectors before and after a pass
+        double *before = g.data(), *M = before + count * count;
+        auto overlap = [&](double* out) {
+            metric(D, SD, count, 0);
+            multidot(c, count, D, dim, count, SD, dim, dim, out);
+        };
+        if (first > 0) overlap(nn);
+        for (int pass = 0; pass < 2; ++pass) {
+            if (first > 0) {
                 multidot(c, count, D, dim, first, SV, dim, dim, cf);           // cf[r][i] = D_r . (S V)_i
                 lincomb(c, count, first, cf, V, dim, dim, -1.0, 1.0, D, dim);  // D_r -= sum_i cf[r][i] V_i
-                if (pass == 1) break;
-                snorms(after);
-                bool again = false;
-                for (int r = 0; r < count; ++r) again = again || !(after[r] >= 0.5 * before[r]);
-                if (!again) break;
             }
+            overlap(nn + count * count);
+            ADC_CUDA(cudaMemcpyAsync(first > 0 ? before : M, first > 0 ? nn : nn + count * count,
+                                     (size_t)(first > 0 ? 2 : 1) * count * count * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+            ADC_CUDA(cudaStreamSynchronize(c.stream));
+            bool again = false;
+            for (int r = 0; r < count; ++r) again = again || !(M[r * count + r] >= 0.5 * before[r * count + r]);
+            if (first == 0 || !again) break;
+        }
+        // M = C C^T; the vectors C^-1 D are orthonormal to rounding times the condition of M scaled to
+        // unit diagonal, small where every pivot keeps a quarter of its vector's norm
+        bool apart = count <= kTriangle;
+        std::vector<double> C((size_t)count * count, 0.0), L((size_t)count * count, 0.0);
+        for (int r = 0; apart && r < count; ++r) {
+            for (int j = 0; j <= r; ++j) {
+                double x = 0.5 * (M[r * count + j] + M[j * count + r]);
+                for (int k = 0; k < j; ++k) x -= C[r * count + k] * C[j * count + k];
+                if (j < r) {
+                    C[r * count + j] = x / C[j * count + j];
+                } else {
+                    apart = M[r * count + r] > 1e-20 && std::isfinite(x) && x >= 0.25 * M[r * count + r];
+                    C[r * count + r] = std::sqrt(apart ? x : 1.0);
+                }
+            }
+            for (int j = 0; j <= r; ++j) {  // row r of C^-1
+                double x = j == r ? 1.0 : 0.0;
+                for (int k = j; k < r; ++k) x -= C[r * count + k] * L[k * count + j];
+                L[r * count + j] = x / C[r * count + r];
+            }
+        }
+        if (apart) {
+            triangle(c, count, L.data(), D, SD, dim);
+            return count;
         }
         int kept = 0;
         for (int r = 0; r < count; ++r) {
@@ -2064,7 +2091,7 @@ static int davidson(adc_handle* h, int nroots, double tol, const double* guess, 
     double* AX = c.arena.dalloc((size_t)nroots * dim);
     double* R = c.arena.dalloc((size_t)nroots * dim);
     double* SR = c.arena.dalloc((size_t)nroots * dim);
-    double* Cd = c.arena.dalloc((size_t)cap * nroots);
+    double* Cd = c.arena.dalloc((size_t)(cap + 1) * nroots);
     double* Gd = c.arena.dalloc((size_t)cap * cap);
     double* wd = c.arena.dalloc(nroots);
     // guesses
@@ -2140,12 +2167,9 @@ static int davidson(adc_handle* h, int nroots, double tol, const double* guess, 
         std::vector<double> Ct((size_t)nroots * k);
         for (int r = 0; r < nroots; ++r)
             for (int i = 0; i < k; ++i) Ct[(size_t)r * k + i] = C[(size_t)i * k + r];
+        for (int r = 0; r < nroots; ++r) Ct.push_back(w[r]);
         ADC_CUDA(cudaMemcpyAsync(Cd, Ct.data(), Ct.size() * sizeof(double), cudaMemcpyHostToDevice, c.stream));
-        lincomb(c, nroots, k, Cd, d.V, dim, dim, 1.0, 0.0, X, dim);
-        lincomb(c, nroots, k, Cd, d.W, dim, dim, 1.0, 0.0, AX, dim);
-        // R = AX - w X
-        ADC_CUDA(cudaMemcpyAsync(R, AX, (size_t)nroots * dim * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
-        for (int r = 0; r < nroots; ++r) axpby(c, dim, -w[r], X + (long long)r * dim, 1.0, R + (long long)r * dim);
+        ritz(c, nroots, k, Cd, Cd + (size_t)nroots * k, d.V, d.W, dim, X, R);  // X and R = A X - w X
         d.metric(R, SR, nroots, 0);
         std::vector<double> rr(nroots), rrm((size_t)nroots * nroots);
         multidot(c, nroots, R, dim, nroots, SR, dim, dim, Gd);
@@ -2216,28 +2240,34 @@ static int davidson(adc_handle* h, int nroots, double tol, const double* guess, 
             for (int r = 0; r < nkeep; ++r) d.G[(size_t)r * d.ldg + r] = w[r];
         }
         // corrections for unconverged roots
-        std::vector<double> wt(nnew);
+        Corrections q;
+        int m = 0;
+        auto flush = [&] {  // the diagonal ones, up to eight a launch
+            if (m)
+                k_corrections<<<dim3((unsigned)grid_for(dim), m), 256, 0, c.stream>>>(q, dim, R, h->diag, d.V + (long long)d.k * dim);
+            if (m) launch_check(c);
+            m = 0;
+        };
         for (int j = 0; j < nnew; ++j) {
-            wt[j] = w[todo[j]];
-            ADC_CUDA(cudaMemcpyAsync(SR + (long long)j * dim, R + (long long)todo[j] * dim, dim * sizeof(double),
-                                     cudaMemcpyDeviceToDevice, c.stream));
-        }
-        ADC_CUDA(cudaMemcpyAsync(wd, wt.data(), nnew * sizeof(double), cudaMemcpyHostToDevice, c.stream));
-        for (int j = 0; j < nnew; ++j) {
+            const int r = todo[j];
             double* dst = d.V + (long long)(d.k + j) * dim;
-            if (!diag_only[todo[j]]) {
-                mlp_precondition(c, 1, dim, h->n1(), SR + (long long)j * dim, wd + j, h->diag, h->mlp_w, dst);
+            if (!diag_only[r]) {
+                ADC_CUDA(cudaMemcpyAsync(wd, &w[r], sizeof(double), cudaMemcpyHostToDevice, c.stream));
+                mlp_precondition(c, 1, dim, h->n1(), R + (long long)r * dim, wd, h->diag, h->mlp_w, dst);
                 // a non-finite learned correction (bad weights) falls back to the diagonal one at once
                 double nrm2 = 0.0;
                 multidot(c, 1, dst, dim, 1, dst, dim, dim, Cd);
                 ADC_CUDA(cudaMemcpyAsync(&nrm2, Cd, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
                 ADC_CUDA(cudaStreamSynchronize(c.stream));
                 if (std::isfinite(nrm2)) continue;
-                diag_only[todo[j]] = 1;
+                diag_only[r] = 1;
             }
-            k_precond<<<grid_for(dim), 256, 0, c.stream>>>(1, dim, SR + (long long)j * dim, wd + j, h->diag, dst);
-            launch_check(c);
+            q.root[m] = r;
+            q.to[m] = j;
+            q.w[m] = w[r];
+            if (++m == 8) flush();
         }
+        flush();
         int kept = d.orthonormalise(d.k, nnew);
         if (kept == 0) {
             // no correction survives orthonormalisation while roots are unconverged: the space

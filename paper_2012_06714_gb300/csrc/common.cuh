@@ -202,8 +202,22 @@ struct Ctx {
     // a CUDA-graph capture of sigma is recording on `stream`: no host synchronisation, no
     // allocation, no tuning; the timeout flags are read after the graph's replay instead
     bool capturing = false;
+    // kDone zeros that a kernel may count in, if it leaves them zero (one launch at a time: on `stream`)
+    static constexpr int kDone = 4096;
+    unsigned* done_ = nullptr;
+    unsigned* done_counters() {
+        if (!done_) {
+            void* p = nullptr;
+            ADC_CUDA(dev_malloc(&p, kDone * sizeof(unsigned), stream));
+            done_ = (unsigned*)p;
+            ADC_CUDA(cudaMemsetAsync(done_, 0, kDone * sizeof(unsigned), stream));
+        }
+        return done_;
+    }
     // releases everything on the stream (before it is destroyed)
     void release() {
+        dev_free(done_, stream);
+        done_ = nullptr;
         for (auto& kv : f32cache) dev_free(kv.second, stream);
         for (auto& kv : bf16cache) dev_free(kv.second, stream);
         for (auto& kv : cache64) dev_free(kv.second, stream);
