@@ -24,6 +24,8 @@
 // consecutive in tensor memory, so that one MMA multiplies digit i of A with up to 256 / BNT digits
 // of B: 12 MMAs of up to 256 columns per 16-deep K step instead of 36 of 64 (which would be bound by
 // reading A from shared memory 36 times).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cstdint>
 #include <mutex>
@@ -47,7 +49,7 @@ constexpr int G_MAXST = 4;
 constexpr size_t G_SMEM = 226 * 1024;
 
 // ---- digits -------------------------------------------------------------------------
-constexpr int DT = 256;  // threads, and K chunk, of k_digits
+constexpr int DT = 256;  // threads of the digit kernels
 constexpr int DR = 8;    // rows per block at most
 
 struct DigitSide {
@@ -64,12 +66,114 @@ __device__ __forceinline__ double ld_op(const Operand64& x, long long i) {
     return x.f32 ? (double)((const float*)x.p)[i] : ((const double*)x.p)[i];
 }
 
-// Both operands in one launch (blocks [0, blocks_a) of x the rows of A), K in segments of kseg along
-// y.  passes: 1 the rows' largest exponents (into ex, zero before), 2 the digits, 3 both (one segment;
-// the second read then comes from L1 / L2).  Integer arithmetic only: the FP64 pipe (2 operations per
-// cycle and SM) would be the bound.
+__device__ __forceinline__ long long digit_row(const Operand64& x, unsigned r) {
+    long long off = 0;
+    for (int j = x.nr - 1; j >= 0; --j) {
+        const unsigned d = (unsigned)x.rd[j], q = r / d;
+        off += (long long)(r - q * d) * x.rs[j];
+        r = q;
+    }
+    return off;
+}
+__device__ __forceinline__ long long digit_k(const Operand64& x, unsigned k) {
+    long long off = 0;
+    for (int j = x.nk - 1; j >= 0; --j) {
+        const unsigned d = (unsigned)x.kd[j], q = k / d;
+        off += (long long)(k - q * d) * x.ks[j];
+        k = q;
+    }
+    return off;
+}
+__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// x[0], x[1] of a row of largest exponent field ef -> their digits, at `at` of each plane.  Integer
+// arithmetic only: the FP64 pipe (2 operations per cycle and SM) would be the bound.
+__device__ __forceinline__ void put_digits(const DigitSide& sd, long long at, const double* x, int ef) {
+    unsigned dig[ND];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const long long b = __double_as_longlong(x[h]);
+        const int ex = (int)(b >> 52) & 0x7ff;
+        // |x| = m 2^(ex - 1075) -> round(|x| 2^(1085 - ef)), below 2^63: the row's scale is 2^(ef - 1022)
+        long long v = 0;
+        const int sh = ef - ex - 10;  // right shift of the 53-bit significand (-10: ten more bits)
+        if (ex > 0 && ef < 0x7ff && sh < 55) {
+            const long long m = (b & 0xfffffffffffffLL) | (1LL << 52);
+            v = sh <= 0 ? m << -sh : (m + (1LL << (sh - 1))) >> sh;
+            if (b < 0) v = -v;
+        }
+        // digit p < 7 of v is the p-th byte of v + sum_p 128 256^p less 128: the carries in
+        // one addition; the top one is in [-128, 128]
+        const unsigned long long w = (unsigned long long)v + 0x0080808080808080ULL;
+        const int top = v >= 0 ? (int)(w >> 56) : (int)((long long)w >> 56);
+#pragma unroll
+        for (int p = 0; p < ND; ++p) {
+            const int d = p < ND - 1 ? (int)((w >> (8 * p)) & 0xff) - 128 : top;
+            // a small integer's BF16 bits are the upper half of its FP32 bits
+            const unsigned u = __float_as_uint((float)d) >> 16;
+            dig[p] = h == 0 ? u : dig[p] | (u << 16);
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < ND; ++p) *(unsigned*)(sd.out + p * sd.plane + at) = dig[p];
+}
+
+// Rows of up to 8 DSEG terms: both operands in one launch (blocks [0, blocks_a) of x the rows of A), a
+// row's K over the blocks of a cluster, seg terms each in shared memory.  The rows' largest exponents go
+// around through distributed shared memory, so every element is read once and neither a second launch
+// nor a cleared array is needed (for 70 rows of 1582: 8 us for the pair of launches and the clearing's 2).
+constexpr int DSEG = 512;
 __global__ void __launch_bounds__(DT) k_digits(const __grid_constant__ DigitSide sa, const __grid_constant__ DigitSide sb,
-                                               int blocks_a, long long kseg, int passes) {
+                                               int blocks_a, int seg) {
+    extern __shared__ double tile[];  // [R][seg + 1]
+    __shared__ long long offk[DSEG], offr[DR];
+    __shared__ int emax[DR], eall[DR];
+    const bool isb = (int)blockIdx.x >= blocks_a;
+    const DigitSide& sd = isb ? sb : sa;
+    const Operand64& x = sd.x;
+    const int R = sd.R, tid = threadIdx.x, ld = seg + 1;
+    const long long row0 = (long long)(isb ? blockIdx.x - blocks_a : blockIdx.x) * R, k0 = (long long)blockIdx.y * seg;
+    if (tid < R) {
+        offr[tid] = digit_row(x, (unsigned)min(row0 + tid, x.rows - 1));
+        emax[tid] = 0;
+    }
+    for (int k = tid; k < seg; k += DT) offk[k] = digit_k(x, (unsigned)min(k0 + k, x.K - 1));
+    __syncthreads();
+    const int per = DT / R, lper = 31 - __clz(per), lR = 8 - lper;
+    if (sd.row_lanes) {
+        const int rr = tid & (R - 1);
+#pragma unroll 4
+        for (int k = tid >> lR; k < seg; k += per)
+            tile[rr * ld + k] = k0 + k < x.K && row0 + rr < x.rows ? ld_op(x, offr[rr] + offk[k]) : 0.0;
+    } else {
+        for (int rr = 0; rr < R; ++rr)
+#pragma unroll
+            for (int k = tid; k < seg; k += DT)
+                tile[rr * ld + k] = k0 + k < x.K && row0 + rr < x.rows ? ld_op(x, offr[rr] + offk[k]) : 0.0;
+    }
+    __syncthreads();
+    const int r = tid >> lper, t = tid & (per - 1);  // per threads to a row
+    int m = 0;
+    for (int k = t; k < seg; k += per) m = max(m, exponent_of(tile[r * ld + k]));
+    if (m > 0) atomicMax(&emax[r], m);
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    if (tid < R) {
+        int e = 0;
+        for (unsigned q = 0; q < cl.num_blocks(); ++q) e = max(e, *cl.map_shared_rank(&emax[tid], q));
+        eall[tid] = e;
+        if (blockIdx.y == 0 && row0 + tid < x.rows) sd.ex[row0 + tid] = e;
+    }
+    cl.sync();  // (no block leaves while its maxima are read)
+    if (row0 + r >= x.rows) return;
+    const int ef = eall[r];
+    for (int k = 2 * t; k < seg && k0 + k < sd.Kp; k += 2 * per) put_digits(sd, (row0 + r) * sd.Kp + k0 + k, tile + r * ld + k, ef);
+}
+
+// Longer rows: K in segments of kseg along y and two launches, pass 1 the rows' largest exponents (into
+// ex, zero before), pass 2 the digits.
+__global__ void __launch_bounds__(DT) k_digits_long(const __grid_constant__ DigitSide sa, const __grid_constant__ DigitSide sb,
+                                                    int blocks_a, long long kseg, int pass) {
     __shared__ double tile[DR][DT + 1];
     __shared__ long long offk[DT], offr[DR];
     __shared__ int emax[DR];
@@ -80,87 +184,31 @@ __global__ void __launch_bounds__(DT) k_digits(const __grid_constant__ DigitSide
     const long long row0 = (long long)(isb ? blockIdx.x - blocks_a : blockIdx.x) * R;
     const long long kbeg = blockIdx.y * kseg, kend = min(sd.Kp, kbeg + kseg);
     if (tid < R) {
-        unsigned long long r = (unsigned long long)min(row0 + tid, x.rows - 1);
-        long long off = 0;
-        for (int j = x.nr - 1; j >= 0; --j) {
-            const unsigned d = (unsigned)x.rd[j], q = (unsigned)r / d;
-            off += (long long)((unsigned)r - q * d) * x.rs[j];
-            r = q;
-        }
-        offr[tid] = off;
-        emax[tid] = passes == 2 ? sd.ex[min(row0 + tid, x.rows - 1)] : 0;
+        offr[tid] = digit_row(x, (unsigned)min(row0 + tid, x.rows - 1));
+        emax[tid] = pass == 2 ? sd.ex[min(row0 + tid, x.rows - 1)] : 0;
     }
     const int per = DT / R, lper = 31 - __clz(per), lR = 8 - lper;  // threads per row when the lanes run along k
     const int r = tid >> lper;
-    for (int pass = 1; pass <= 2; ++pass) {
-        if (!(passes & pass)) continue;
-        for (long long k0 = kbeg; k0 < kend; k0 += DT) {
-            if (!(pass == 2 && passes == 3 && kend - kbeg <= DT)) {  // (one chunk: still in shared memory)
-                __syncthreads();
-                {
-                    unsigned k = (unsigned)min(k0 + tid, x.K - 1);
-                    long long off = 0;
-                    for (int j = x.nk - 1; j >= 0; --j) {
-                        const unsigned d = (unsigned)x.kd[j], q = k / d;
-                        off += (long long)(k - q * d) * x.ks[j];
-                        k = q;
-                    }
-                    offk[tid] = off;
-                }
-                __syncthreads();
-                for (int e = tid; e < R * DT; e += DT) {
-                    const int rr = sd.row_lanes ? e & (R - 1) : e >> 8, k = sd.row_lanes ? e >> lR : e & (DT - 1);
-                    tile[rr][k] = k0 + k < x.K && row0 + rr < x.rows ? ld_op(x, offr[rr] + offk[k]) : 0.0;
-                }
-                __syncthreads();
-            }
-            if (pass == 1) {
-                int m = 0;
-                for (int k = tid & (per - 1); k < DT; k += per) m = max(m, (__double2hiint(tile[r][k]) >> 20) & 0x7ff);
-                if (m > 0) atomicMax(&emax[r], m);
-            } else if (row0 + r < x.rows) {
-                const int ef = emax[r];
-                for (int k = 2 * (tid & (per - 1)); k < DT; k += 2 * per) {
-                    if (k0 + k >= sd.Kp) break;
-                    unsigned dig[ND];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const long long b = __double_as_longlong(tile[r][k + h]);
-                        const int ex = (int)(b >> 52) & 0x7ff;
-                        // |x| = m 2^(ex - 1075) -> round(|x| 2^(1085 - ef)), below 2^63: the row's scale is 2^(ef - 1022)
-                        long long v = 0;
-                        const int sh = ef - ex - 10;  // right shift of the 53-bit significand (-10: ten more bits)
-                        if (ex > 0 && ef < 0x7ff && sh < 55) {
-                            const long long m = (b & 0xfffffffffffffLL) | (1LL << 52);
-                            v = sh <= 0 ? m << -sh : (m + (1LL << (sh - 1))) >> sh;
-                            if (b < 0) v = -v;
-                        }
-                        // digit p < 7 of v is the p-th byte of v + sum_p 128 256^p less 128: the carries in
-                        // one addition; the top one is in [-128, 128]
-                        const unsigned long long w = (unsigned long long)v + 0x0080808080808080ULL;
-                        const int top = v >= 0 ? (int)(w >> 56) : (int)((long long)w >> 56);
-#pragma unroll
-                        for (int p = 0; p < ND; ++p) {
-                            const int d = p < ND - 1 ? (int)((w >> (8 * p)) & 0xff) - 128 : top;
-                            // a small integer's BF16 bits are the upper half of its FP32 bits
-                            const unsigned u = __float_as_uint((float)d) >> 16;
-                            dig[p] = h == 0 ? u : dig[p] | (u << 16);
-                        }
-                    }
-#pragma unroll
-                    for (int p = 0; p < ND; ++p)
-                        *(unsigned*)(sd.out + p * sd.plane + (row0 + r) * sd.Kp + k0 + k) = dig[p];
-                }
-            }
+    for (long long k0 = kbeg; k0 < kend; k0 += DT) {
+        __syncthreads();
+        offk[tid] = digit_k(x, (unsigned)min(k0 + tid, x.K - 1));
+        __syncthreads();
+        for (int e = tid; e < R * DT; e += DT) {
+            const int rr = sd.row_lanes ? e & (R - 1) : e >> 8, k = sd.row_lanes ? e >> lR : e & (DT - 1);
+            tile[rr][k] = k0 + k < x.K && row0 + rr < x.rows ? ld_op(x, offr[rr] + offk[k]) : 0.0;
         }
         __syncthreads();
+        if (pass == 1) {
+            int m = 0;
+            for (int k = tid & (per - 1); k < DT; k += per) m = max(m, exponent_of(tile[r][k]));
+            if (m > 0) atomicMax(&emax[r], m);
+        } else if (row0 + r < x.rows) {
+            for (int k = 2 * (tid & (per - 1)); k < DT && k0 + k < sd.Kp; k += 2 * per)
+                put_digits(sd, (row0 + r) * sd.Kp + k0 + k, &tile[r][k], emax[r]);
+        }
     }
-    if ((passes & 1) && tid < R && row0 + tid < x.rows) {
-        if (passes == 3)
-            sd.ex[row0 + tid] = emax[tid];
-        else
-            atomicMax(&sd.ex[row0 + tid], emax[tid]);
-    }
+    __syncthreads();
+    if (pass == 1 && tid < R && row0 + tid < x.rows) atomicMax(&sd.ex[row0 + tid], emax[tid]);
 }
 
 // ---- GEMM ---------------------------------------------------------------------------
@@ -545,8 +593,15 @@ void digitise64(Ctx& c, const Operand64* x, Digits64* out, int n) {
     int blocks[2] = {0, 0};
     const int sms = sm_count();
     const long long Kp = out[0].Kp;
-    // a row's K in one block up to this length (two reads in one launch), else in segments (two launches)
-    const bool fused = Kp <= 1024;
+    // one launch where a cluster's eight blocks hold a row: as few blocks to a row as hold it, more (of at
+    // least 256 terms) while the launch leaves SMs idle
+    const bool once = Kp <= 8 * DSEG;
+    long long rows8 = 0;
+    for (int i = 0; i < n; ++i) rows8 += (x[i].rows + DR - 1) / DR;
+    long long cs = std::max<long long>(1, (Kp + DSEG - 1) / DSEG);
+    while (once && cs < 8 && Kp > 256 * cs && rows8 * cs < 2 * sms) ++cs;
+    const long long seg = once ? ((Kp + cs - 1) / cs + 255) / 256 * 256 : DSEG;
+    cs = (Kp + seg - 1) / seg;
     for (int i = 0; i < n; ++i) {
         DigitSide& d = side[i];
         d.x = x[i];
@@ -561,23 +616,36 @@ void digitise64(Ctx& c, const Operand64* x, Digits64* out, int n) {
         for (int j = 0; j < d.x.nr; ++j)
             if (d.x.rd[j] > 1 && d.x.rs[j] < smallest) d.row_lanes = 1;
         d.R = DR;
-        while (fused && d.R > 1 && (d.x.rows + d.R - 1) / d.R < 2 * sms) d.R /= 2;
+        while (d.R > 1 && (d.x.rows + d.R - 1) / d.R * cs < 2 * sms) d.R /= 2;
         const long long nb = (d.x.rows + d.R - 1) / d.R;
         if (nb > (1LL << 30)) throw Error(-1, "gemm64: too many rows");
         blocks[i] = (int)nb;
     }
     if (n < 2) side[1] = side[0];
     const unsigned bx = (unsigned)(blocks[0] + blocks[1]);
-    if (fused) {
-        k_digits<<<bx, DT, 0, c.stream>>>(side[0], side[1], blocks[0], Kp, 3);
+    if (once) {
+        const int R = std::max(side[0].R, side[1].R);
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute cl[1];
+        cl[0].id = cudaLaunchAttributeClusterDimension;
+        cl[0].val.clusterDim.x = 1;
+        cl[0].val.clusterDim.y = (unsigned)cs;
+        cl[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(bx, (unsigned)cs);
+        cfg.blockDim = dim3(DT);
+        cfg.dynamicSmemBytes = (size_t)R * (seg + 1) * sizeof(double);
+        cfg.stream = c.stream;
+        cfg.attrs = cl;
+        cfg.numAttrs = 1;
+        ADC_CUDA(cudaLaunchKernelEx(&cfg, k_digits, side[0], side[1], blocks[0], (int)seg));
         ++c.kernels;
     } else {
         for (int i = 0; i < n; ++i)
             ADC_CUDA(cudaMemsetAsync(side[i].ex, 0, (size_t)side[i].x.rows * sizeof(int), c.stream));
         for (int pass = 1; pass <= 2; ++pass) {
-            long long seg = 512;
-            while ((Kp + seg - 1) / seg > 65535) seg *= 2;
-            k_digits<<<dim3(bx, (unsigned)((Kp + seg - 1) / seg)), DT, 0, c.stream>>>(side[0], side[1], blocks[0], seg, pass);
+            long long ks = seg;
+            while ((Kp + ks - 1) / ks > 65535) ks *= 2;
+            k_digits_long<<<dim3(bx, (unsigned)((Kp + ks - 1) / ks)), DT, 0, c.stream>>>(side[0], side[1], blocks[0], ks, pass);
             ++c.kernels;
         }
     }
@@ -658,7 +726,7 @@ double* small64(Ctx& c, const Operand64& A, const Operand64& B, const Out64& out
     // K slices while the blocks leave SMs idle, of at least 64 terms (a sum of slices is another launch)
     S = 1;
     if (A.K >= 256 && mt * nt < 2 * sm_count())
-        S = (int)std::max<long long>(1, std::min<long long>({A.K / 64, 4LL * sm_count() / (mt * nt), 64}));
+        S = (int)std::max<long long>(1, std::min<long long>({A.K / 64, 4LL * sm_count() / (mt * nt), 256}));
     long long ks = (A.K + S - 1) / S;
     S = (int)((A.K + ks - 1) / ks);
     double* T = out.p && S == 1 ? nullptr : c.arena.dalloc((size_t)S * A.rows * B.rows);

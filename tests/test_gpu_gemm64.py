@@ -50,3 +50,19 @@ def test_non_finite_rows_stay_apart():
     g.close()
     assert not np.isfinite(S[0, :v]).any() and not np.isfinite(S[2, :v]).any()
     assert np.array_equal(S[1], R[1])
+
+
+@pytest.mark.parametrize("o,v,nvec", [(2, 16, 260), (3, 14, 260), (4, 16, 130), (2, 23, 90), (4, 32, 20), (2, 46, 17)])
+def test_rows_of_a_cluster(o, v, nvec):
+    """Contractions of o v^2 = 512, 588, 1024, 1058, 4096 and 4232 terms (ADC(2): the singles row), the
+    lengths between which rows are cut into digits by one block, by clusters of up to eight, and in two
+    passes.  The bound of the test above."""
+    from paper_2012_06714_gb300 import ADC
+
+    s = make_system(o, v, 60, seed=v)
+    ref = SpinAdaptedADC(s.eps, o, s.B, 2, "ea")
+    g = ADC(s.eps, s.B, o, order=2, kind="ea", precision="fp64")
+    X = np.random.default_rng(v).standard_normal((nvec, g.dim))
+    S, R = g.sigma(X), ref.sigma(X)
+    g.close()
+    assert np.abs(S - R).max() <= 1e-13 * np.abs(R).max()
