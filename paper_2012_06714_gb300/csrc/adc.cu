@@ -1482,11 +1482,12 @@ static void coupling_into(adc_handle* h, void* K) {
 // twice, instead of contracting the vectors with t and B^Q in some ten (EA: six of them o^2 v^3)
 // contractions per sigma.  EA-ADC(3): 6 o^2 v^4 flops in setup against 12 o^2 v^3 per vector of a
 // sigma, which a solve of v / 2 vectors pays back (226 vectors for four roots at 40/400/1400): held up
-// to 512 virtuals.  IP-ADC(3): 2 o^3 v^3 and
-// less, always held where it fits.  The terms are those of sigma_ea / sigma_ip without the block.
+// to 512 virtuals.  IP-ADC(3): 2 o^3 v^3 and less, always held where it fits.  The terms are those of
+// sigma_ea / sigma_ip without the block.
 // Arithmetic: FP64, or for an EA tensor above 2^24 elements (FP32, half the bytes) sigma's own -- the
 // accurate operator of the refinement then works without it.
-// Measured, sigma IP mixed 20/180/600 n=5: 1.65 -> 0.40 ms; EA mixed 20/180/600 n=4: 2.58 -> 1.54 ms.
+// Measured, split-BF16 sigma: IP 20/180/600, 5 vectors 1.65 -> 0.40 ms; EA 20/180/600, 4 vectors 2.58 ->
+// 1.54 ms; EA 40/400/1400, 4 vectors 34.9 -> 21.6 ms for 0.8 s of setup.
 // --------------------------------------------------------------------------
 static void make_coupling(adc_handle* h) {
     Ctx& c = h->ctx;
@@ -3208,6 +3209,28 @@ static void sigma_unrestricted(adc_handle* h, const double* Xin, double* Sout, l
     launch_check(c);
 }
 
+// f() with the handle's memory held for speed pinned; own: the ladder's may go while f runs (it then takes
+// its other form).  If f runs out of memory with some of it held, that is given back and f runs again.
+template <typename F>
+static void with_held_memory(adc_handle* h, bool own, F f) {
+    try {
+        ReclaimPin keep(&h->k12, h->ctx.stream, false);
+        ReclaimPin pin(h->held_for_speed(), h->ctx.stream, own);
+        f();
+        return;
+    } catch (const Error& e) {
+        const Reclaimable* r = h->held_for_speed();
+        if (e.code != ADC_ERR_OOM || !(h->k12.mem[0] || (r && r->mem[0]))) throw;
+    }
+    cudaGetLastError();
+    ADC_CUDA(cudaStreamSynchronize(h->ctx.stream));
+    h->ctx.arena.free_all();
+    h->k12.drop(h->ctx.stream);
+    if (Reclaimable* r = h->held_for_speed()) r->drop(h->ctx.stream);
+    device_memory_reclaim();
+    f();
+}
+
 #define GUARD(h, ...)                                    \
     try {                                                \
         __VA_ARGS__                                      \
@@ -3328,9 +3351,7 @@ int adc_mlp_samples(adc_handle* h, int nroots, const int* iters, int n_iters, lo
             return ADC_ERR_ARG;
         }
     GUARD(h, {
-        ReclaimPin keep(&h->k12, h->ctx.stream, false);
-        ReclaimPin pin(h->held_for_speed(), h->ctx.stream, true);
-        mlp_samples(h, nroots, iters, n_iters, per_vector, seed, exact_tol, d, blk, r, t);
+        with_held_memory(h, true, [&] { mlp_samples(h, nroots, iters, n_iters, per_vector, seed, exact_tol, d, blk, r, t); });
         return ADC_OK;
     })
 }
@@ -3594,19 +3615,19 @@ int adc_sigma(adc_handle* h, const double* X, double* S, int nvec, int on_device
     }
     GUARD(h, {
         Ctx& c = h->ctx;
-        ReclaimPin keep(&h->k12, c.stream, false);
-        ReclaimPin pin(h->held_for_speed(), c.stream, true);
         const long long dim = h->dim();
-        if (on_device) {
-            sigma_device(h, X, S, nvec);
-        } else {
-            Scope sc(c.arena);
-            double* dX = c.arena.dalloc((size_t)nvec * dim);
-            double* dS = c.arena.dalloc((size_t)nvec * dim);
-            ADC_CUDA(cudaMemcpyAsync(dX, X, (size_t)nvec * dim * sizeof(double), cudaMemcpyHostToDevice, c.stream));
-            sigma_device(h, dX, dS, nvec);
-            ADC_CUDA(cudaMemcpyAsync(S, dS, (size_t)nvec * dim * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-        }
+        with_held_memory(h, true, [&] {
+            if (on_device) {
+                sigma_device(h, X, S, nvec);
+            } else {
+                Scope sc(c.arena);
+                double* dX = c.arena.dalloc((size_t)nvec * dim);
+                double* dS = c.arena.dalloc((size_t)nvec * dim);
+                ADC_CUDA(cudaMemcpyAsync(dX, X, (size_t)nvec * dim * sizeof(double), cudaMemcpyHostToDevice, c.stream));
+                sigma_device(h, dX, dS, nvec);
+                ADC_CUDA(cudaMemcpyAsync(S, dS, (size_t)nvec * dim * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+            }
+        });
         ADC_CUDA(cudaStreamSynchronize(c.stream));
         return ADC_OK;
     })
@@ -3620,9 +3641,9 @@ int adc_davidson(adc_handle* h, int nroots, double tol, const double* guess, dou
         return ADC_ERR_ARG;
     }
     GUARD(h, {
-        ReclaimPin keep(&h->k12, h->ctx.stream, false);
-        ReclaimPin pin(h->held_for_speed(), h->ctx.stream, !h->opt.cuda_graphs);  // (captured sigmas hold the integrals' address)
-        int st = davidson(h, nroots, tol, guess, energies, specfac, vectors, stats);
+        int st = ADC_OK;
+        // (captured sigmas hold the integrals' address)
+        with_held_memory(h, !h->opt.cuda_graphs, [&] { st = davidson(h, nroots, tol, guess, energies, specfac, vectors, stats); });
         if (st == ADC_ERR_NOT_CONVERGED) h->err = "adc_davidson: not converged within max_iter";
         // the solver's scratch (subspace, residuals, sigma intermediates) goes back to the device:
         // many handles solved one after another would otherwise each keep their peak

@@ -101,6 +101,7 @@ cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t s) {
         cudaGetLastError();
         device_memory_reclaim();
         e = dev_malloc_raw(p, bytes, s);
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // reported here, not by the next launch's check
     }
     return e;
 }

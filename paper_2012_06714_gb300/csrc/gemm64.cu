@@ -15,8 +15,10 @@
 //     coherent diagonal, (ia|ia) 20 times the others, turns into 1.2e-16 of the result.)
 // The error against 64-bit arithmetic is that of an FP64 GEMM: norm of the error over norm of sigma
 // 1.8e-16 (IP, 14/113/445) against 1.7e-16 with DGEMM, 1.2e-16 each for its final rounding.
-// Measured: that sigma (5 vectors, 22 GFLOP in 20 contractions) 24.6 -> 3.8 ms; the FP64 setup of an
-// IP molecule at 17/121/483 with its first sigma 217 -> 44 ms.
+// Measured: that sigma (5 vectors) 24.6 -> 3.8 ms in 20 contractions, 0.30 ms with the coupling block held
+// (three of 70 x 1582 x 1582 results and terms take 37 us each: 40 MB of cached digits read from L2 by 99
+// tiles; other tile widths, slices and the exchanged sides are all between 34 and 140 us); the FP64 setup of
+// an IP molecule at 17/121/483 with its first sigma 217 -> 18.7 ms, about half of it here.
 //
 // Tile: 128 rows of A x BNT columns (16 .. 64) of B per CTA, because the eight accumulators take
 // 8 x BNT of the 512 tensor-memory columns.  The digit planes of B lie one after another in shared
@@ -120,7 +122,7 @@ __device__ __forceinline__ void put_digits(const DigitSide& sd, long long at, co
 // Rows of up to 8 DSEG terms: both operands in one launch (blocks [0, blocks_a) of x the rows of A), a
 // row's K over the blocks of a cluster, seg terms each in shared memory.  The rows' largest exponents go
 // around through distributed shared memory, so every element is read once and neither a second launch
-// nor a cleared array is needed (for 70 rows of 1582: 8 us for the pair of launches and the clearing's 2).
+// nor a cleared array is needed (70 rows of 1582: 5.8 us, against 8.5 + 9.7 and 1.1 for the clearing).
 constexpr int DSEG = 512;
 __global__ void __launch_bounds__(DT) k_digits(const __grid_constant__ DigitSide sa, const __grid_constant__ DigitSide sb,
                                                int blocks_a, int seg) {

@@ -928,7 +928,8 @@ TuneCache* tune_cache_open(const char* path) {
 // at 180 virtuals and 600 auxiliary functions, 14 at 400 / 1400).  The integrals cost naux v^4
 // flops once per handle and 4 v^4 bytes (two BF16 planes of both halves: 4.2 GB at v = 180, 51 GB
 // at 400), so they are held where that fits the device and the two-GEMM form stays for the rest.
-// Measured, a sigma of 4 vectors at 20/180/600: 7.9 -> 4.0 ms; at 40/400/1400: 159 -> 36 ms.
+// Measured, the ladder of a sigma of 4 vectors: 3.1 -> 0.36 ms at 20/180/600, 126 -> 9.6 ms at 40/400/1400
+// (51 GB of integrals: 5.4 TB/s, 1.3 PFLOP/s of split products).
 //
 // The integrals are a convenience (Reclaimable): they go back to the device when an allocation fails.
 namespace {

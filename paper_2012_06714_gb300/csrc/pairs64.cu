@@ -5,8 +5,9 @@
 // per auxiliary function (which stay for the sizes whose integrals do not fit: 32 P^2 bytes, P = v (v +
 // 1) / 2, i.e. 0.7 GB at v = 97, 8.5 GB at 180).  Bound by reading the integrals' digits (16 bytes each)
 // for few matrices, by the tensor cores beyond about 40.
-// Measured, FP64 sigma of 4 vectors at 12/97/381: 142 -> 2.8 ms (the ladder 129 -> 0.3 ms), its error
-// against 64 bits 9.2e-16 -> 1.6e-16; four roots at 8/45/187: 165 -> 24 ms.
+// Measured, FP64 sigma of 4 vectors at 12/97/381: 142 -> 0.73 ms (the ladder 129 -> 0.25 ms, both halves'
+// 361 MB of digits at 3.5 TB/s), its error against 64 bits 9.2e-16 -> 1.7e-16; four roots at 8/45/187:
+// 165 -> 7.6 ms.
 #include "pairs64.cuh"
 
 #include <algorithm>

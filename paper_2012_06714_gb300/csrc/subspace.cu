@@ -11,7 +11,8 @@ constexpr int kRT = 8;  // output rows of a linear combination per pass
 
 // Sums N (a power of two, <= 32) values per lane over the warp: each step exchanges half of the values
 // that are left, N - 1 additions per lane instead of 5 N (the FP64 units' two a cycle per SM bound the
-// reduction of a 8 x 4 block: 20 of its 32 us at 40 x 4 vectors of 16,245).  v[0] of lane l is value l N / 32.
+// reduction of a 8 x 4 block: 20 -> 14 us a call at some 30 x 4 vectors of 16,245, of which the products'
+// own FP64 is 9).  v[0] of lane l is value l N / 32.
 template <int N>
 __device__ __forceinline__ void warp_fold(double (&v)[N], int lane) {
     int off = 16;

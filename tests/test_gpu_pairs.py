@@ -56,3 +56,27 @@ def test_pair_integrals_are_given_back():
     tol = 3e-5 * np.abs(before).max()
     assert np.abs(after - before).max() <= tol and np.abs(Sb - before).max() <= tol
     a.close()
+
+
+def test_out_of_memory_leaves_the_handle_usable():
+    """A block of vectors too large for the device is refused with ADC_ERR_OOM after the handle gave back what
+    it held for speed, and later calls are right (sigma's split-BF16 bound)."""
+    from paper_2012_06714_gb300 import ADC
+    from paper_2012_06714_gb300._lib import ADCError
+
+    o, v, naux = 6, 160, 200
+    s = make_system(o, v, naux, seed=1)
+    a = ADC(s.eps, s.B, o, order=3, kind="ea", precision="bf16x3")
+    X = np.random.default_rng(2).standard_normal((400, a.dim))  # 0.49 GB, and more than four times that as scratch
+    before = a.sigma(X[:4])
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(free - (200 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(ADCError) as e:
+            a.sigma(X)
+        assert e.value.code == -2
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.abs(a.sigma(X[:4]) - before).max() <= 3e-5 * np.abs(before).max()
+    a.close()
