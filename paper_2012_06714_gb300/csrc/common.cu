@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "warp.cuh"
 #include "gemm64.cuh"
 #include "ladder_tc.cuh"
 
@@ -411,14 +412,21 @@ inline int grid_for(long long n) {
 // class).  Each kernel writes its K slice's partial result P[slice][m][n]; k_reduce_slices finishes
 // C = alpha sum_slices P + beta C.
 
-constexpr int SK_THREADS = 256;
+// Both are bound by reading the large operand, as far as enough of its bytes are in flight: blocks of 128
+// threads waste less of an SM's registers and of the last wave than ones of 256 (one to three resident
+// blocks), and the FP64 adds (two a cycle and SM) are kept to one a result and 64 terms.
+// Measured, the products of a 4-vector EA sigma with the coupling block (blocks of 256 -> 128, wider loads
+// in flight, folded sums): 180 x 648,000 (467 MB) row 162 -> 96 us, column 138 -> 88 us (5 TB/s); 400 x
+// 6,400,000 (10.2 GB) 2.2 -> 1.6 and 2.1 -> 1.5 ms (6.2 and 6.7 TB/s).  64 threads, 16 loads, 8 rows a block
+// and more slices are no faster.
+constexpr int SK_THREADS = 128;
 constexpr int SK_CHUNK = 64;  // FP32 partial-sum length
 
 // M <= MM rows of A (a few trial vectors): V consecutive columns of B per thread (4 where every row of B
 // starts on a 16-byte boundary, N % 4 == 0: enough bytes in flight for the memory system), the A values
 // of the current K chunk in shared memory; reads B once, coalesced along n.
 template <int MM, int V, typename TB>
-__global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, long long K, long long kslice,
+__global__ void __launch_bounds__(SK_THREADS, V == 4 && MM <= 4 && sizeof(TB) == 4 ? 5 : 1) k_skinny_m(int M, long long N, long long K, long long kslice,
                                                          const double* __restrict__ A, long long lda,
                                                          const TB* __restrict__ B, long long ldb,
                                                          double* __restrict__ P, double alpha, double beta) {
@@ -441,7 +449,7 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, lon
         const TB* b = B + kc * ldb + n;
         // U independent loads in flight per thread before their FMAs (the loop is bound by
         // memory latency otherwise)
-        constexpr int U = V == 4 ? 4 : 8;
+        constexpr int U = V == 4 && sizeof(TB) == 8 ? 4 : 8;
         for (int k2 = 0; k2 < kn; k2 += SK_CHUNK) {
             float part[MM][V];
 #pragma unroll
@@ -472,10 +480,18 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, lon
                         for (int e = 0; e < V; ++e) part[m][e] = fmaf(a, (float)bv[u][e], part[m][e]);
                     }
             }
+            const bool first = kc == k0 && k2 == 0;
+            if (first) {
 #pragma unroll
-            for (int m = 0; m < MM; ++m)
+                for (int m = 0; m < MM; ++m)
 #pragma unroll
-                for (int e = 0; e < V; ++e) acc[m][e] += (double)part[m][e];
+                    for (int e = 0; e < V; ++e) acc[m][e] = (double)part[m][e];
+            } else {
+#pragma unroll
+                for (int m = 0; m < MM; ++m)
+#pragma unroll
+                    for (int e = 0; e < V; ++e) acc[m][e] += (double)part[m][e];
+            }
         }
     }
     if (n < N)
@@ -485,7 +501,8 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_m(int M, long long N, lon
 #pragma unroll
                 for (int e = 0; e < V; ++e) {
                     double* p = P + ((long long)blockIdx.y * M + m) * N + n + e;
-                    *p = beta == 0.0 ? alpha * acc[m][e] : alpha * acc[m][e] + beta * *p;
+                    const double x = alpha == 1.0 ? acc[m][e] : alpha * acc[m][e];
+                    *p = beta == 0.0 ? x : x + beta * *p;
                 }
 }
 
@@ -499,7 +516,8 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, lon
                                                          const float* __restrict__ B, long long ldb,
                                                          double* __restrict__ P) {
     constexpr int RR = 4;
-    __shared__ double red[SK_THREADS / 32][RR * NN];
+    constexpr int NV = NN == 1 ? RR : NN == 2 ? 2 * RR : NN <= 4 ? 4 * RR : 8 * RR;  // RR NN to a power of two
+    __shared__ double red[SK_THREADS / 32][NV];
     const long long m0 = blockIdx.x * (long long)RR;
     const long long k0 = blockIdx.y * kslice, k1 = min(K, k0 + kslice);
     const TA* a[RR];  // rows past the last read the last one and are discarded
@@ -556,14 +574,12 @@ __global__ void __launch_bounds__(SK_THREADS) k_skinny_n(long long M, int N, lon
 #pragma unroll
             for (int j = 0; j < NN; ++j) acc[r][j] += (double)part[r][j];
     }
+    double val[NV];
 #pragma unroll
-    for (int r = 0; r < RR; ++r)
-#pragma unroll
-        for (int j = 0; j < NN; ++j) {
-            double x = acc[r][j];
-            for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
-            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][r * NN + j] = x;
-        }
+    for (int x = 0; x < NV; ++x) val[x] = x < RR * NN ? acc[x / NN % RR][x % NN] : 0.0;
+    const int lane = threadIdx.x & 31;
+    warp_fold<NV>(val, lane);
+    if (lane % (32 / NV) == 0) red[threadIdx.x >> 5][lane * NV / 32] = val[0];
     __syncthreads();
     if (threadIdx.x < RR * NN) {
         const int r = threadIdx.x / NN, j = threadIdx.x % NN;
