@@ -752,7 +752,7 @@ def run_ours(args):
     achieved = kt["ladder_algo_flops"] / (kt["ladder_ms"] / 1e3) / 1e12
     traffic = profiled_traffic()
     roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": traffic, "kernel": "k_gemm_pair, DF-ladder GEMMs (GEMM1 + GEMM2, cta_group::2)",
+            "traffic": traffic, "kernel": "k_gemm_pair (tcgen05, cta_group::2), the DF ladder (over held pair integrals where they fit)",
             "peak_note": f"{peak_src} sustained BF16 dense {bf16_peak:.1f} TF/s / 3 split products "
                          f"(burst {bf16_burst:.1f} TF/s: frac {achieved / (bf16_burst / 3.0):.3f})",
             "tensor_pipe_frac": kt["ladder_mma_flops"] / (kt["ladder_ms"] / 1e3) / 1e12 / bf16_peak,

@@ -89,7 +89,7 @@ typedef struct {
     int contractions;        /* non-ladder contractions: -1 follow precision (default:*/
                              /* FP64 -> 0; BF16X3 -> 2 in sigma, 1 in setup and      */
                              /* refinement for EA, 0 in setup and refinement for IP), */
-                             /* 0 FP64 DGEMM, 1 FP32-accurate emulated GEMM, 2 (sigma)*/
+                             /* 0 FP64,      1 FP32-accurate emulated GEMM, 2 (sigma)*/
                              /* unbatched contractions of >= 1e8 flop on the tensor-  */
                              /* core split-BF16 GEMM of the ladder, unless a free     */
                              /* dimension is <= 8 and the large operand is not a      */

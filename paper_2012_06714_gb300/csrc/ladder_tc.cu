@@ -926,7 +926,7 @@ TuneCache* tune_cache_open(const char* path) {
 // (diagonal weights in k_pair_pack): nmat v^4 flops for nmat matrices instead of the
 // 4 naux v^3 nmat of the two-GEMM form over the auxiliary index, i.e. 4 naux / v times fewer (13
 // at 180 virtuals and 600 auxiliary functions, 14 at 400 / 1400).  The integrals cost naux v^4
-// flops once per handle and 4 v^4 bytes (two BF16 planes of both halves: 4.2 GB at v = 180, 51 GB
+// flops once per handle and 2 v^4 bytes (two BF16 planes of both halves: 2.1 GB at v = 180, 51 GB
 // at 400), so they are held where that fits the device and the two-GEMM form stays for the rest.
 // Measured, the ladder of a sigma of 4 vectors: 3.1 -> 0.36 ms at 20/180/600, 126 -> 9.6 ms at 40/400/1400
 // (51 GB of integrals: 5.4 TB/s, 1.3 PFLOP/s of split products).
@@ -1114,7 +1114,7 @@ void pairs_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* o
 
 void ladder_tc_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* out, const LadderMode& md) {
     if (nmat <= 0) return;
-    // Few matrices: the pair form streams 4 v^4 bytes whatever their number (6.5 TB/s), the
+    // Few matrices: the pair form streams 2 v^4 bytes whatever their number (5.4 TB/s), the
     // two-GEMM form computes 4 naux v^3 flops for each (about 420 TF/s), which is faster below
     // nmat = 65 v / naux (about 19 at naux = 3.5 v) -- unless the integrals stay in L2.
     // Precision: a pair integral rounded to two planes (2^-18 relative at most) is not averaged over
