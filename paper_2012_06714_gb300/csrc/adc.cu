@@ -113,6 +113,7 @@ struct adc_handle {
         return kind == ADC_EA ? (long long)v + (long long)o * v * v : (long long)o + (long long)o * o * v;
     }
     int n1() const { return kind == ADC_EA ? v : o; }
+    adc_handle() { k12.call = pairs64.store.call = &ctx.call; }
     Reclaimable* held_for_speed() { return tc ? ladder_pairs_store(tc) : &pairs64.store; }
     T coupling() const {
         const long long O = o, V = v;
@@ -1078,7 +1079,7 @@ static void make_t1_third_order(adc_handle* h) {
 }
 
 static void transition_parts(adc_handle* h, bool third, double* Tpp, double* t1x);
-static void make_coupling(adc_handle* h);
+static void make_coupling(adc_handle* h, const ReclaimPin& call);
 
 // the timeout flag of the handle's tensor-core kernels (waits for the work issued so far)
 static void check_flag(adc_handle* h, const char* where) {
@@ -1090,7 +1091,7 @@ static void check_flag(adc_handle* h, const char* where) {
     if (e) throw Error(ADC_ERR_TIMEOUT, std::string(where) + ": a bounded device wait of the tensor-core GEMM timed out");
 }
 
-static void setup(adc_handle* h, const double* eps_in, const double* B_in, int on_device) {
+static void setup(adc_handle* h, const double* eps_in, const double* B_in, int on_device, ReclaimPin& call) {
     Ctx& c = h->ctx;
     // phase timer: 0 inputs and the ladder's operand planes, 1 integrals, 2 amplitudes and E(2),
     // 3 the ladder of t, 4 the rest of t2(2), t1(2) and E(3), 5 the 1p-1p / 1h-1h block,
@@ -1214,7 +1215,7 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
     }
     tick(2);
     Scope setup_scope(c.arena);
-    ReclaimPin setup_pin(h->held_for_speed(), c.stream, true);
+    call.give(h->held_for_speed());
     double* XL = nullptr;  // EA: the ladder term of the 1p-1p block, formed while the ladder of t is alive
     if (h->order >= 3) {
         const T T4 = op_t(h, false);
@@ -1360,7 +1361,7 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
         // step 3 skipped: sigma applies the block from intermediates (the diagonal preconditioner
         // then takes the zeroth-order one-particle energies)
         setup_m11_otf(h);
-        make_coupling(h);
+        make_coupling(h, call);
         h->diag = h->dmalloc(h->dim());
         k_diag<<<grid_for(h->dim()), 256, 0, c.stream>>>(h->kind == ADC_EA, (int)o, (int)v, h->eps, nullptr, h->diag);
         launch_check(c);
@@ -1389,7 +1390,7 @@ static void setup(adc_handle* h, const double* eps_in, const double* B_in, int o
         setup_m11_ip(h);
         c.gemm_mode = saved;
     }
-    make_coupling(h);
+    make_coupling(h, call);
     check_flag(h, "setup");
     tick(5);
     if (lean) {
@@ -1416,7 +1417,7 @@ static void coupling_into(adc_handle* h, void* K) {
     Ctx& c = h->ctx;
     const long long o = h->o, v = h->v, Q = h->naux;
     const bool ea = h->kind == ADC_EA, f32 = h->k12_f32;
-    ReclaimPin pin(&h->k12, c.stream, false);
+    ReclaimPin pin(h->k12, c.stream);
     const int saved = c.gemm_mode;
     c.gemm_mode = f32 ? h->cmode_sigma : 0;
     const T Boo = tn(h->Boo, {Q, o, o}), Bov = tn(h->Bov, {Q, o, v}), Bvv = tn(h->Bvv, {Q, v, v});
@@ -1489,7 +1490,7 @@ static void coupling_into(adc_handle* h, void* K) {
 // Measured, split-BF16 sigma: IP 20/180/600, 5 vectors 1.65 -> 0.40 ms; EA 20/180/600, 4 vectors 2.58 ->
 // 1.54 ms; EA 40/400/1400, 4 vectors 34.9 -> 21.6 ms for 0.8 s of setup.
 // --------------------------------------------------------------------------
-static void make_coupling(adc_handle* h) {
+static void make_coupling(adc_handle* h, const ReclaimPin& call) {
     Ctx& c = h->ctx;
     const long long o = h->o, v = h->v;
     const bool ea = h->kind == ADC_EA;
@@ -1509,7 +1510,7 @@ static void make_coupling(adc_handle* h) {
         return;
     }
     h->k12_f32 = f32;
-    h->k12.hold(K, nullptr);
+    h->k12.hold(K, nullptr, call);
     form_if_it_fits(c, h->k12, [&] {
         coupling_into(h, K);
         return true;
@@ -3209,26 +3210,30 @@ static void sigma_unrestricted(adc_handle* h, const double* Xin, double* Sout, l
     launch_check(c);
 }
 
-// f() with the handle's memory held for speed pinned; own: the ladder's may go while f runs (it then takes
-// its other form).  If f runs out of memory with some of it held, that is given back and f runs again.
+// f() with the handle's memory held for speed pinned until the work that f issued has completed; own: the
+// ladder's may go while f runs (it then takes its other form).  If f runs out of memory with some of it
+// held, that is given back and f runs again.
 template <typename F>
 static void with_held_memory(adc_handle* h, bool own, F f) {
+    Ctx& c = h->ctx;
     try {
-        ReclaimPin keep(&h->k12, h->ctx.stream, false);
-        ReclaimPin pin(h->held_for_speed(), h->ctx.stream, own);
+        ReclaimPin call(c.call, c.stream);
+        if (own) call.give(h->held_for_speed());
         f();
+        ADC_CUDA(call.wait());
         return;
     } catch (const Error& e) {
-        const Reclaimable* r = h->held_for_speed();
-        if (e.code != ADC_ERR_OOM || !(h->k12.mem[0] || (r && r->mem[0]))) throw;
+        if (e.code != ADC_ERR_OOM || !(h->k12.held() || h->held_for_speed()->held())) throw;
     }
     cudaGetLastError();
-    ADC_CUDA(cudaStreamSynchronize(h->ctx.stream));
-    h->ctx.arena.free_all();
-    h->k12.drop(h->ctx.stream);
-    if (Reclaimable* r = h->held_for_speed()) r->drop(h->ctx.stream);
+    ReclaimPin call(c.call, c.stream);
+    c.arena.free_all();
+    h->k12.drop(c.stream);
+    h->held_for_speed()->drop(c.stream);
+    ADC_CUDA(cudaStreamSynchronize(c.stream));
     device_memory_reclaim();
     f();
+    ADC_CUDA(call.wait());
 }
 
 #define GUARD(h, ...)                                    \
@@ -3447,8 +3452,9 @@ static int setup_one(const double* eps, const double* Bq, int nocc, int nvir, in
             h->ctx.cache_max_bytes = 0;               // operand planes / FP32 copies made per call
             h->ctx.arena.big_bytes = size_t(256) << 20;  // large scratch in blocks of its own
         }
-        setup(h, eps, Bq, on_device);
-        ADC_CUDA(cudaStreamSynchronize(h->ctx.stream));
+        ReclaimPin call(h->ctx.call, h->ctx.stream);
+        setup(h, eps, Bq, on_device, call);
+        ADC_CUDA(call.wait());
         // setup's scratch (ladder Z, o^2 v^2 temporaries) goes back to the device; sigma regrows
         // what it needs (many handles at once would otherwise each keep their setup peak)
         h->ctx.arena.free_all();
@@ -3628,7 +3634,6 @@ int adc_sigma(adc_handle* h, const double* X, double* S, int nvec, int on_device
                 ADC_CUDA(cudaMemcpyAsync(S, dS, (size_t)nvec * dim * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
             }
         });
-        ADC_CUDA(cudaStreamSynchronize(c.stream));
         return ADC_OK;
     })
 }

@@ -12,6 +12,8 @@
 #include <string>
 #include <vector>
 
+#include "memory.cuh"
+
 namespace adc {
 
 struct Error : std::runtime_error {
@@ -34,42 +36,6 @@ struct Error : std::runtime_error {
             throw ::adc::Error(s_ == CUBLAS_STATUS_ALLOC_FAILED ? -2 : -3,                            \
                                std::string(#x) + ": cublas status " + std::to_string((int)s_));       \
     } while (0)
-
-// Device memory that a handle holds for speed only (the ladder's pair integrals).  It goes back to
-// the device when an allocation of any handle fails: that of handles with no call in progress
-// (no pins), and that of the failing call itself where it has said so (ReclaimPin::own).
-struct Reclaimable {
-    void* mem[2] = {};
-    int device = 0, pins = 0;
-    void hold(void* a, void* b);  // takes over stream-ordered allocations of the current device
-    void drop(cudaStream_t s);    // releases them, ordered on s
-    ~Reclaimable();
-};
-// A call that may use r (or NULL): while one is in progress r stays, except that, with own, a failing
-// allocation of the same host thread may release it after waiting for the stream.
-struct ReclaimPin {
-    Reclaimable *r, *before = nullptr;
-    cudaStream_t before_stream = nullptr;
-    ReclaimPin(Reclaimable* r, cudaStream_t s, bool own);
-    ~ReclaimPin();
-    ReclaimPin(const ReclaimPin&) = delete;
-};
-// Releases what can be released on the current device; false if there was nothing.
-bool device_memory_reclaim();
-
-// Stream-ordered allocation from the library's own pool of the current device: the pool keeps up to a
-// fiftieth of the device's memory mapped between uses (mapping and unmapping costs about 60 us a buffer
-// and 0.4 ms a GB each way: 14 of the 53 ms from a new molecule to its first sigma at 20/180/600), and
-// gives it back when an allocation fails (device_memory_reclaim).  dev_malloc retries after that.
-cudaError_t dev_malloc_raw(void** p, size_t bytes, cudaStream_t s);
-cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t s);
-// releases such memory, ordered on s
-inline void dev_free(void* p, cudaStream_t s) {
-    if (p && cudaFreeAsync(p, s) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(p);
-    }
-}
 
 // Device scratch: blocks are allocated on demand and kept; mark()/release()
 // give stack semantics so that repeated calls reuse the same memory.  Blocks
@@ -205,6 +171,8 @@ struct Ctx {
     // kDone zeros that a kernel may count in, if it leaves them zero (one launch at a time: on `stream`)
     static constexpr int kDone = 4096;
     unsigned* done_ = nullptr;
+    // no memory of its own: its pins are the handle's calls in progress, and cover what the handle holds
+    Reclaimable call;
     unsigned* done_counters() {
         if (!done_) {
             void* p = nullptr;

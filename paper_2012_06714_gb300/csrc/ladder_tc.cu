@@ -753,6 +753,7 @@ LadderTC* ladder_tc_create(Ctx& c, const double* Bvv, int naux, int v, int aux_c
         L->vp = (v + 31) / 32 * 32;
         L->chunk = aux_chunk;
         L->Bvv = Bvv;
+        L->store.call = &c.call;
         L->bn2[2] = pick_bn(v, 256);
         L->bn2[3] = pick_bn(v, 128);
         L->d_err = (int*)dev_alloc(sizeof(int), c.stream);
@@ -965,8 +966,8 @@ bool ladder_pairs_prepare(LadderTC& L, Ctx& c, const double* Bvv) {
     }
     L.P = P;
     L.Pk = Pk;
-    L.store.hold(base, third);
-    ReclaimPin pin(&L.store, c.stream, false);  // its own allocations may not take them away again
+    ReclaimPin pin(L.store, c.stream);  // its own allocations may not take them away again
+    L.store.hold(base, third, pin);
     Arena::Mark mk = c.arena.mark();
     // K-major planes of B^Q as [(p, q)][Q]: both operands of (ac|bd) = sum_Q B^Q_ac B^Q_bd
     // in three planes (the six products of order <= 2): with two, the dropped lo * lo products of the
@@ -1066,7 +1067,7 @@ void pairs_apply(LadderTC& L, Ctx& c, const double* X, long long nmat, double* o
     // groups of matrices whose split vectors (8 or 12 P bytes each) and FP32 results stay within ~4 GiB
     const long long smin = (Pk + kPairSliceK - 1) / kPairSliceK;
     const long long mg = std::max<long long>(1, std::min<long long>(nmat, (4LL << 30) / (4 * planes * Pk + 8 * P * (smin + 2))));
-    ReclaimPin pin(&L.store, c.stream, false);  // its own allocations may not take the integrals away
+    ReclaimPin pin(L.store, c.stream);  // its own allocations may not take the integrals away
     for (long long m0 = 0; m0 < nmat; m0 += mg) {
         const long long nm = std::min(mg, nmat - m0);
         Arena::Mark mk = c.arena.mark();

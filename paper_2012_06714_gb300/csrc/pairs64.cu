@@ -60,8 +60,8 @@ bool pairs64_prepare(Pairs64& L, Ctx& c, const double* Bvv, int naux, int nvir) 
     L.v = nvir;
     L.P = P;
     L.Pk = (P + 7) / 8 * 8;
-    L.store.hold(base, nullptr);
-    ReclaimPin pin(&L.store, c.stream, false);  // its own allocations may not take them away again
+    ReclaimPin pin(L.store, c.stream);  // its own allocations may not take them away again
+    L.store.hold(base, nullptr, pin);
     // rows (a, c) of a block of a's against the columns (b, d), b <= the block's last a: at most 1 GB,
     // packed into the pairs' rows a (a + 1) / 2 + b and cut into digits
     for (long long a0 = 0; a0 < v;) {
@@ -109,7 +109,7 @@ void pairs64_apply(Pairs64& L, Ctx& c, const double* X, long long nmat, double* 
     const long long v = L.v, P = L.P;
     // groups of matrices whose pairs, digits and results (16, 32 and about 32 P bytes each) stay within 4 GiB
     const long long mg = std::max<long long>(1, std::min<long long>(nmat, (4LL << 30) / (80 * P)));
-    ReclaimPin pin(&L.store, c.stream, false);
+    ReclaimPin pin(L.store, c.stream);
     for (long long m0 = 0; m0 < nmat; m0 += mg) {
         const long long nm = std::min(mg, nmat - m0);
         Arena::Mark mk = c.arena.mark();

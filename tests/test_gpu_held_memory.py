@@ -1,0 +1,64 @@
+"""Memory held for speed under an exhausted device: two host threads, one making small FP64 handles and using
+their held coupling blocks, the other making a handle whose setup does not fit what is left, so that its
+allocations take back whatever no call keeps.  Every result that is returned is right; running out of memory
+(ADC_ERR_OOM) is an answer too.  Tolerances: 1e-11 of max |sigma| in FP64, the split-BF16 bound 3e-5
+(test_gpu_mixed.py) in mixed precision."""
+import threading
+
+import numpy as np
+import pytest
+
+from adc_inputs import make_system
+from oracle.spinadapted import SpinAdaptedADC
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def test_two_host_threads_on_an_exhausted_device():
+    from paper_2012_06714_gb300 import ADC
+    from paper_2012_06714_gb300._lib import ADCError
+
+    small, big = make_system(4, 18, 60, seed=1), make_system(6, 160, 200, seed=1)
+    Xs = np.random.default_rng(1).standard_normal((3, 4 + 16 * 18))
+    Xb = np.random.default_rng(2).standard_normal((4, 160 + 6 * 160 * 160))
+    Rs = SpinAdaptedADC(small.eps, 4, small.B, 3, "ip").sigma(Xs)
+    g = ADC(big.eps, big.B, 6, order=3, kind="ea", precision="bf16x3")
+    Rb = g.sigma(Xb)
+    g.close()
+    right, wrong = {"small": 0, "big": 0}, []
+
+    def use(name, rounds, sys, nocc, kind, precision, X, R, tol, sigmas):
+        for _ in range(rounds):
+            h = None
+            try:
+                h = ADC(sys.eps, sys.B, nocc, order=3, kind=kind, precision=precision)
+                for _ in range(sigmas):
+                    d = np.abs(h.sigma(X) - R).max()
+                    if d <= tol * np.abs(R).max():
+                        right[name] += 1
+                    else:
+                        wrong.append((name, d))
+            except ADCError as e:
+                if e.code != -2:
+                    wrong.append((name, str(e)))
+            finally:
+                if h is not None:
+                    h.close()
+
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(free - (1300 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        threads = [threading.Thread(target=use, args=("small", 30, small, 4, "ip", "fp64", Xs, Rs, 1e-11, 4)),
+                   threading.Thread(target=use, args=("big", 8, big, 6, "ea", "bf16x3", Xb, Rb, 3e-5, 2))]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert not wrong, wrong[:3]
+    use("small", 1, small, 4, "ip", "fp64", Xs, Rs, 1e-11, 1)
+    use("big", 1, big, 6, "ea", "bf16x3", Xb, Rb, 3e-5, 1)
+    assert not wrong and right["small"] >= 1 and right["big"] >= 1, (right, wrong)
