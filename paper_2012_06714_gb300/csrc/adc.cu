@@ -3210,15 +3210,16 @@ static void sigma_unrestricted(adc_handle* h, const double* Xin, double* Sout, l
     launch_check(c);
 }
 
-// f() with the handle's memory held for speed pinned until the work that f issued has completed; own: the
-// ladder's may go while f runs (it then takes its other form).  If f runs out of memory with some of it
-// held, that is given back and f runs again.
+// f() with the handle's memory held for speed pinned until the work that f issued has completed.  The
+// ladder's may go while f runs (it then takes its other form), unless f solves with CUDA graphs: captured
+// sigmas hold its address.  If f runs out of memory with some of it held, that is given back and f runs
+// again.
 template <typename F>
-static void with_held_memory(adc_handle* h, bool own, F f) {
+static void with_held_memory(adc_handle* h, bool solves, F f) {
     Ctx& c = h->ctx;
     try {
         ReclaimPin call(c.call, c.stream);
-        if (own) call.give(h->held_for_speed());
+        if (!(solves && h->opt.cuda_graphs)) call.give(h->held_for_speed());
         f();
         ADC_CUDA(call.wait());
         return;
@@ -3622,7 +3623,7 @@ int adc_sigma(adc_handle* h, const double* X, double* S, int nvec, int on_device
     GUARD(h, {
         Ctx& c = h->ctx;
         const long long dim = h->dim();
-        with_held_memory(h, true, [&] {
+        with_held_memory(h, false, [&] {
             if (on_device) {
                 sigma_device(h, X, S, nvec);
             } else {
@@ -3647,8 +3648,7 @@ int adc_davidson(adc_handle* h, int nroots, double tol, const double* guess, dou
     }
     GUARD(h, {
         int st = ADC_OK;
-        // (captured sigmas hold the integrals' address)
-        with_held_memory(h, !h->opt.cuda_graphs, [&] { st = davidson(h, nroots, tol, guess, energies, specfac, vectors, stats); });
+        with_held_memory(h, true, [&] { st = davidson(h, nroots, tol, guess, energies, specfac, vectors, stats); });
         if (st == ADC_ERR_NOT_CONVERGED) h->err = "adc_davidson: not converged within max_iter";
         // the solver's scratch (subspace, residuals, sigma intermediates) goes back to the device:
         // many handles solved one after another would otherwise each keep their peak

@@ -62,3 +62,28 @@ def test_two_host_threads_on_an_exhausted_device():
     use("small", 1, small, 4, "ip", "fp64", Xs, Rs, 1e-11, 1)
     use("big", 1, big, 6, "ea", "bf16x3", Xb, Rb, 3e-5, 1)
     assert not wrong and right["small"] >= 1 and right["big"] >= 1, (right, wrong)
+
+
+def test_samples_with_graphs_when_memory_runs_out():
+    """adc_mlp_samples solves like adc_davidson: with cuda_graphs the replayed sigmas hold the pair integrals'
+    address, which no allocation of the same call may then take back.  The same samples as from plain launches
+    (equal kernels, so equal to rounding: 1e-9 of their maximum)."""
+    from paper_2012_06714_gb300 import ADC
+
+    o, v = 3, 40
+    s = make_system(o, v, 120, seed=5)
+    stream = torch.cuda.Stream()
+    got = []
+    for graphs in (0, 1):
+        g = ADC(s.eps, s.B, o, order=3, kind="ea", precision="bf16x3", cuda_graphs=graphs)
+        g.set_stream(stream.cuda_stream)
+        free, _ = torch.cuda.mem_get_info()
+        hold = torch.empty(free - (600 << 20), dtype=torch.uint8, device="cuda")
+        try:
+            got.append(g.mlp_samples(2, iters=(2, 4), per_vector=500, seed=3))
+        finally:
+            del hold
+            torch.cuda.empty_cache()
+        g.close()
+    for a, b in zip(*got):
+        assert np.abs(a.astype(float) - b).max() <= 1e-9 * max(np.abs(a).max(), 1e-300)
