@@ -56,8 +56,7 @@ extern "C" {
                                     /* with the best estimates                */
 #define ADC_ERR_TIMEOUT (-5)        /* a bounded device wait gave up; the     */
                                     /* kernel returned and the handle stays   */
-                                    /* usable (the device flag is cleared at  */
-                                    /* the start of the next call)            */
+                                    /* usable; any results written are void   */
 #define ADC_ERR_NONFINITE (-6)      /* a non-finite value: in a guess vector, */
                                     /* or a Ritz value / residual (non-finite */
                                     /* sigma, e.g. from non-finite inputs)    */

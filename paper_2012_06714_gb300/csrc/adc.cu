@@ -951,6 +951,32 @@ static void m11_apply_otf_ip(adc_handle* h, const double* y1, double* s1, long l
     }
 }
 
+// The timeout flag of the handle's tensor-core kernels (c.d_err).  It is zero when a call begins; a bounded
+// wait that gives up raises it and leaves its results unwritten, so every call that can launch one reads
+// it before it returns (finish_call), and before it keeps a result for later calls.
+static thread_local std::string tl_raise;  // where the next reading finds the flag raised (tests)
+static void check_flag(adc_handle* h, const char* where) {
+    Ctx& c = h->ctx;
+    if (!c.d_err) return;
+    if (!tl_raise.empty() && tl_raise == where) {
+        tl_raise.clear();
+        ADC_CUDA(cudaMemsetAsync(c.d_err, 1, sizeof(int), c.stream));
+    }
+    int e = 0;
+    ADC_CUDA(cudaMemcpyAsync(&e, c.d_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+    ADC_CUDA(cudaStreamSynchronize(c.stream));
+    if (e) throw Error(ADC_ERR_TIMEOUT, std::string(where) + ": a bounded device wait of the tensor-core GEMM timed out");
+}
+// Ends a call: its work has completed and none of its device waits gave up.
+static void finish_call(adc_handle* h, ReclaimPin& call, const char* where) {
+    check_flag(h, where);
+    ADC_CUDA(call.wait());
+}
+// A call that failed leaves the flag as it found it.
+static void clear_flag(adc_handle* h) {
+    if (h->ctx.d_err && cudaMemsetAsync(h->ctx.d_err, 0, sizeof(int), h->ctx.stream) != cudaSuccess) cudaGetLastError();
+}
+
 // --------------------------------------------------------------------------
 // Third-order singles t_i^a(3) (Eq. t_singles at k = 3), spin-integrated.
 // They enter only the ADC(3) transition moments, so they are made on first
@@ -1075,21 +1101,12 @@ static void make_t1_third_order(adc_handle* h) {
         einsum(c, "ijab,jb->ia", 0.5, U4, tn(t1, {o, v}), 1.0, out, {o, v});
     }
     c.gemm_mode = saved;
+    check_flag(h, "t1(3)");
     h->t1_3 = out;
 }
 
 static void transition_parts(adc_handle* h, bool third, double* Tpp, double* t1x);
 static void make_coupling(adc_handle* h, const ReclaimPin& call);
-
-// the timeout flag of the handle's tensor-core kernels (waits for the work issued so far)
-static void check_flag(adc_handle* h, const char* where) {
-    Ctx& c = h->ctx;
-    if (!c.d_err) return;
-    int e = 0;
-    ADC_CUDA(cudaMemcpyAsync(&e, c.d_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
-    ADC_CUDA(cudaStreamSynchronize(c.stream));
-    if (e) throw Error(ADC_ERR_TIMEOUT, std::string(where) + ": a bounded device wait of the tensor-core GEMM timed out");
-}
 
 static void setup(adc_handle* h, const double* eps_in, const double* B_in, int on_device, ReclaimPin& call) {
     Ctx& c = h->ctx;
@@ -1732,8 +1749,6 @@ static void sigma_unrestricted(adc_handle* h, const double* Xin, double* Sout, l
 static void sigma_launch(adc_handle* h, const double* X, double* S, long long nvec) {
     Ctx& c = h->ctx;
     if (!h->refining) c.gemm_mode = h->cmode_sigma;
-    // a timeout of an earlier call left the flag raised; every call starts clean
-    if (c.d_err) ADC_CUDA(cudaMemsetAsync(c.d_err, 0, sizeof(int), c.stream));
     if (h->unrestricted)
         sigma_unrestricted(h, X, S, nvec);
     else if (h->kind == ADC_EA)
@@ -3033,6 +3048,7 @@ static void make_t1_third_order_u(adc_handle* h) {
     launch_check(c);
     ADC_CUDA(cudaMemcpyAsync(out, num, o * v * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
     einsum(c, "ijab,jb->ia", 0.5, T4, t1, 1.0, out, {o, v});
+    check_flag(h, "t1(3)");
     h->t1_3 = out;
 }
 
@@ -3213,28 +3229,34 @@ static void sigma_unrestricted(adc_handle* h, const double* Xin, double* Sout, l
 // f() with the handle's memory held for speed pinned until the work that f issued has completed.  The
 // ladder's may go while f runs (it then takes its other form), unless f solves with CUDA graphs: captured
 // sigmas hold its address.  If f runs out of memory with some of it held, that is given back and f runs
-// again.
+// again.  where: the public call, for finish_call.
 template <typename F>
-static void with_held_memory(adc_handle* h, bool solves, F f) {
+static void with_held_memory(adc_handle* h, const char* where, bool solves, F f) {
     Ctx& c = h->ctx;
-    try {
+    auto run = [&](bool give) {
         ReclaimPin call(c.call, c.stream);
-        if (!(solves && h->opt.cuda_graphs)) call.give(h->held_for_speed());
-        f();
-        ADC_CUDA(call.wait());
+        if (give) call.give(h->held_for_speed());
+        try {
+            f();
+            finish_call(h, call, where);
+        } catch (...) {
+            clear_flag(h);
+            throw;
+        }
+    };
+    try {
+        run(!(solves && h->opt.cuda_graphs));
         return;
     } catch (const Error& e) {
         if (e.code != ADC_ERR_OOM || !(h->k12.held() || h->held_for_speed()->held())) throw;
     }
     cudaGetLastError();
-    ReclaimPin call(c.call, c.stream);
     c.arena.free_all();
     h->k12.drop(c.stream);
     h->held_for_speed()->drop(c.stream);
     ADC_CUDA(cudaStreamSynchronize(c.stream));
     device_memory_reclaim();
-    f();
-    ADC_CUDA(call.wait());
+    run(false);
 }
 
 #define GUARD(h, ...)                                    \
@@ -3357,7 +3379,7 @@ int adc_mlp_samples(adc_handle* h, int nroots, const int* iters, int n_iters, lo
             return ADC_ERR_ARG;
         }
     GUARD(h, {
-        with_held_memory(h, true, [&] { mlp_samples(h, nroots, iters, n_iters, per_vector, seed, exact_tol, d, blk, r, t); });
+        with_held_memory(h, "adc_mlp_samples", true, [&] { mlp_samples(h, nroots, iters, n_iters, per_vector, seed, exact_tol, d, blk, r, t); });
         return ADC_OK;
     })
 }
@@ -3455,7 +3477,7 @@ static int setup_one(const double* eps, const double* Bq, int nocc, int nvir, in
         }
         ReclaimPin call(h->ctx.call, h->ctx.stream);
         setup(h, eps, Bq, on_device, call);
-        ADC_CUDA(call.wait());
+        finish_call(h, call, "adc_setup");
         // setup's scratch (ladder Z, o^2 v^2 temporaries) goes back to the device; sigma regrows
         // what it needs (many handles at once would otherwise each keep their setup peak)
         h->ctx.arena.free_all();
@@ -3574,8 +3596,9 @@ int adc_setup_unrestricted(const double* eps_a, const double* eps_b, const doubl
     adc_default_options(&h->opt);
     if (opt) h->opt = *opt;
     try {
+        ReclaimPin call(h->ctx.call, h->ctx.stream);
         setup_unrestricted(h, eps_so.data(), Bso.data());
-        ADC_CUDA(cudaStreamSynchronize(h->ctx.stream));
+        finish_call(h, call, "adc_setup_unrestricted");
         h->ctx.arena.free_all();
     } catch (const adc::Error& e) {
         g_setup_error = e.what();
@@ -3623,15 +3646,15 @@ int adc_sigma(adc_handle* h, const double* X, double* S, int nvec, int on_device
     GUARD(h, {
         Ctx& c = h->ctx;
         const long long dim = h->dim();
-        with_held_memory(h, false, [&] {
+        with_held_memory(h, "adc_sigma", false, [&] {
             if (on_device) {
-                sigma_device(h, X, S, nvec);
+                sigma_launch(h, X, S, nvec);
             } else {
                 Scope sc(c.arena);
                 double* dX = c.arena.dalloc((size_t)nvec * dim);
                 double* dS = c.arena.dalloc((size_t)nvec * dim);
                 ADC_CUDA(cudaMemcpyAsync(dX, X, (size_t)nvec * dim * sizeof(double), cudaMemcpyHostToDevice, c.stream));
-                sigma_device(h, dX, dS, nvec);
+                sigma_launch(h, dX, dS, nvec);
                 ADC_CUDA(cudaMemcpyAsync(S, dS, (size_t)nvec * dim * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
             }
         });
@@ -3648,7 +3671,7 @@ int adc_davidson(adc_handle* h, int nroots, double tol, const double* guess, dou
     }
     GUARD(h, {
         int st = ADC_OK;
-        with_held_memory(h, true, [&] { st = davidson(h, nroots, tol, guess, energies, specfac, vectors, stats); });
+        with_held_memory(h, "adc_davidson", true, [&] { st = davidson(h, nroots, tol, guess, energies, specfac, vectors, stats); });
         if (st == ADC_ERR_NOT_CONVERGED) h->err = "adc_davidson: not converged within max_iter";
         // the solver's scratch (subspace, residuals, sigma intermediates) goes back to the device:
         // many handles solved one after another would otherwise each keep their peak
@@ -3700,10 +3723,12 @@ int adc_get_tensor(adc_handle* h, const char* name, double* out, long long n) {
             src = h->t1_2;
             cnt = o * v;
         } else if (s == "t1_3") {
-            if (h->unrestricted)
-                make_t1_third_order_u(h);
-            else
-                make_t1_third_order(h);
+            with_held_memory(h, "adc_get_tensor", false, [&] {
+                if (h->unrestricted)
+                    make_t1_third_order_u(h);
+                else
+                    make_t1_third_order(h);
+            });
             src = h->t1_3;
             cnt = o * v;
         } else if (s == "diag") {
@@ -3830,6 +3855,10 @@ long long adc_kernel_launches(adc_handle* h, double* out, long long n) {
     }
     return cnt;
 }
+
+// Not part of the interface: the reading of the timeout flag named `where` (a public call, "t1(3)") that this
+// host thread comes to next finds it raised, as after a bounded device wait that gave up.
+void adc_internal_raise_timeout(const char* where) { tl_raise = where ? where : ""; }
 
 const char* adc_last_error(const adc_handle* h) { return h ? h->err.c_str() : g_setup_error.c_str(); }
 
