@@ -37,6 +37,16 @@
  * Work is issued on the handle's stream (adc_set_stream; default stream 0)
  * and every call returns after its work has completed on that stream.
  *
+ * Memory held for speed: beyond what it needs, a closed-shell handle that is not
+ * lean holds what shortens its sigma, as far as the device has room when it is
+ * set up: the ladder's pair integrals (EA; at most 2/5 of the free memory: 2 nvir^4
+ * bytes in BF16X3, 8 nvir^4 in FP64), the coupling block (at most 1/10; 4 or 8 bytes
+ * for nocc nvir^3 or nocc^3 nvir elements) and digits of constant operands of FP64
+ * contractions (at most 1/20, 4 GB).  It is given back when an allocation of this
+ * library fails, or by adc_release_memory, and the handle then goes on without it,
+ * slower (the digits alone are formed again).  With and without it results agree to
+ * the handle's precision, not bit for bit.
+ *
  * Errors: every int-returning call returns ADC_OK (0) or a negative code; the
  * message of the last failure is available from adc_last_error.  No C++
  * exception crosses the ABI.  A failed handle stays valid for adc_destroy.
@@ -406,8 +416,14 @@ int adc_mlp_samples(adc_handle* h, int nroots, const int* iters, int n_iters, lo
  * when h is NULL).  Never NULL. */
 const char* adc_last_error(const adc_handle* h);
 
-/* Release the handle and all its device memory.  NULL is ignored. */
+/* Release the handle and all its device memory.  NULL is ignored.  While other
+ * handles live on the device, up to a fiftieth of its memory stays mapped for them
+ * in the library's pool; with the last one everything goes back to the device. */
 void adc_destroy(adc_handle* h);
+
+/* Give the current device back what this process's handles hold for speed (those
+ * with no call in progress) and what the library's pool keeps unused.  ADC_OK. */
+int adc_release_memory(void);
 
 #ifdef __cplusplus
 }

@@ -5,7 +5,7 @@ The compute path is the CUDA library ``_build/libadc.so`` (C ABI declared in
 CPU fallback: if the library is missing, importing the binding raises.
 """
 from ._lib import (ADC, ADCBatch, ADCUnrestricted, build_library, library_path, load_library,  # noqa: F401
-                   mlp_loss_grad, mlp_nweights, mlp_train, spectrum)
+                   mlp_loss_grad, mlp_nweights, mlp_train, release_memory, spectrum)
 
 __all__ = ["ADC", "ADCBatch", "ADCUnrestricted", "build_library", "library_path", "load_library", "mlp_loss_grad", "mlp_nweights",
-           "mlp_train", "spectrum"]
+           "mlp_train", "release_memory", "spectrum"]

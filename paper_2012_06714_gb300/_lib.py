@@ -39,6 +39,7 @@ EXPORTED = [
     "adc_ladder_noalloc",
     "adc_last_error",
     "adc_destroy",
+    "adc_release_memory",
 ]
 
 
@@ -115,11 +116,18 @@ def load_library():
     lib.adc_last_error.restype = ctypes.c_char_p
     lib.adc_destroy.argtypes = [P]
     lib.adc_destroy.restype = None
+    lib.adc_release_memory.argtypes = []
     for name in EXPORTED:
         if not hasattr(lib, name):
             raise ImportError(f"libadc.so lacks {name}")
     _lib = lib
     return lib
+
+
+def release_memory():
+    """Give the current device back what idle handles hold for speed and what the library keeps unused
+    (adc_release_memory)."""
+    load_library().adc_release_memory()
 
 
 def spectrum(energies, specfac, omega, eta):

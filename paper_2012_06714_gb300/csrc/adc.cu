@@ -113,7 +113,13 @@ struct adc_handle {
         return kind == ADC_EA ? (long long)v + (long long)o * v * v : (long long)o + (long long)o * o * v;
     }
     int n1() const { return kind == ADC_EA ? v : o; }
-    adc_handle() { k12.call = pairs64.store.call = &ctx.call; }
+    int device = 0;
+    static std::atomic<int> live[64];  // handles by device: the last one's memory goes back to the device
+    adc_handle() {
+        k12.call = pairs64.store.call = &ctx.call;
+        if (cudaGetDevice(&device) != cudaSuccess) cudaGetLastError();
+        if (device >= 0 && device < 64) ++live[device];
+    }
     Reclaimable* held_for_speed() { return tc ? ladder_pairs_store(tc) : &pairs64.store; }
     T coupling() const {
         const long long O = o, V = v;
@@ -152,10 +158,13 @@ struct adc_handle {
         for (void* p : owned) dev_free(p, ctx.stream);
         ctx.release();
         if (ctx.blas) cublasDestroy(ctx.blas);
+        cudaStreamSynchronize(ctx.stream);
         if (own_stream) cudaStreamDestroy(own_stream);
+        if (device >= 0 && device < 64 && --live[device] == 0) device_memory_trim(device);
     }
 };
 
+std::atomic<int> adc_handle::live[64];
 static thread_local std::string g_setup_error = "no error";  // last adc_setup failure of this host thread
 
 // --------------------------------------------------------------------------
@@ -3859,6 +3868,11 @@ long long adc_kernel_launches(adc_handle* h, double* out, long long n) {
 // Not part of the interface: the reading of the timeout flag named `where` (a public call, "t1(3)") that this
 // host thread comes to next finds it raised, as after a bounded device wait that gave up.
 void adc_internal_raise_timeout(const char* where) { tl_raise = where ? where : ""; }
+
+int adc_release_memory(void) {
+    device_memory_reclaim();
+    return ADC_OK;
+}
 
 const char* adc_last_error(const adc_handle* h) { return h ? h->err.c_str() : g_setup_error.c_str(); }
 

@@ -121,14 +121,16 @@ cudaError_t dev_malloc(void** p, size_t bytes, cudaStream_t s) {
     return e;
 }
 
+void device_memory_trim(int device) {
+    if (cudaMemPool_t p = pool_of(device)) cudaMemPoolTrimTo(p, 0);
+}
+
 bool device_memory_reclaim() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     struct Trim {  // what the pool keeps unused goes back too, after what is freed below
         int dev;
-        ~Trim() {
-            if (cudaMemPool_t p = pool_of(dev)) cudaMemPoolTrimTo(p, 0);
-        }
+        ~Trim() { device_memory_trim(dev); }
     } trim{dev};
     std::lock_guard<std::mutex> lk(g_reclaim_mu);
     bool any = false;

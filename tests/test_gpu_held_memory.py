@@ -87,3 +87,44 @@ def test_samples_with_graphs_when_memory_runs_out():
         g.close()
     for a, b in zip(*got):
         assert np.abs(a.astype(float) - b).max() <= 1e-9 * max(np.abs(a).max(), 1e-300)
+
+
+def _free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def test_the_last_handle_gives_everything_back():
+    """adc_destroy releases all of a handle's device memory: with no handle left the device has as much free
+    memory as before the handle was made (8 MB for what the driver itself keeps)."""
+    from paper_2012_06714_gb300 import ADC, release_memory
+
+    s = make_system(6, 160, 200, seed=1)
+
+    def use():
+        g = ADC(s.eps, s.B, 6, order=3, kind="ea", precision="bf16x3")
+        g.sigma(np.ones((2, g.dim)))
+        g.close()
+
+    use()  # (loads the kernels)
+    release_memory()
+    free = _free()
+    use()
+    assert _free() >= free - (8 << 20)
+
+
+def test_release_memory():
+    """adc_release_memory gives back what an idle handle holds for speed, and sigma goes on without it within the
+    split-BF16 bound."""
+    from paper_2012_06714_gb300 import ADC, release_memory
+
+    o, v = 6, 160
+    s = make_system(o, v, 200, seed=1)
+    g = ADC(s.eps, s.B, o, order=3, kind="ea", precision="bf16x3")
+    X = np.random.default_rng(2).standard_normal((4, g.dim))
+    before = g.sigma(X)
+    free = _free()
+    release_memory()
+    assert _free() - free >= 8 * (v * (v + 1) // 2) ** 2 + 4 * o * v**3  # pair integrals, FP32 coupling block
+    assert np.abs(g.sigma(X) - before).max() <= 3e-5 * np.abs(before).max()
+    g.close()
