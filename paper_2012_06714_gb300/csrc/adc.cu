@@ -3257,10 +3257,11 @@ static void with_held_memory(adc_handle* h, const char* where, bool solves, F f)
         run(!(solves && h->opt.cuda_graphs));
         return;
     } catch (const Error& e) {
-        if (e.code != ADC_ERR_OOM || !(h->k12.held() || h->held_for_speed()->held())) throw;
+        if (e.code != ADC_ERR_OOM || !(h->k12.held() || h->held_for_speed()->held() || c.digits_held())) throw;
     }
     cudaGetLastError();
     c.arena.free_all();
+    c.drop_digits();
     h->k12.drop(c.stream);
     h->held_for_speed()->drop(c.stream);
     ADC_CUDA(cudaStreamSynchronize(c.stream));

@@ -1064,21 +1064,31 @@ static void einsum_64(Ctx& c, const std::string& la, const std::string& lb, cons
     // digits of a constant operand, kept while there is room
     Digits64 da, db;
     auto kept = [&](const T& X, const Operand64& o, const std::string& l, const std::string& rows, Digits64& d) {
-        if (!tensor || !X.constant || c.cache64_bytes == 0) return false;
+        if (!tensor || !X.constant || (c.cache64_bytes == 0 && c.cache64.empty())) return false;
         const size_t bytes = digits64_bytes(o.rows, o.K);
         std::string key = l + ">" + rows + "," + con;
         for (char x : l) key += ":" + std::to_string(dim[x]);
         auto it = c.cache64.find({X.p, key});
-        if (it == c.cache64.end()) {
-            if (bytes > c.cache64_bytes || c.capturing) return false;
-            void* buf = dev_alloc(bytes, c.stream);
-            c.cache64_bytes -= bytes;
-            it = c.cache64.emplace(std::make_pair((const void*)X.p, key), buf).first;
+        const bool known = it != c.cache64.end();
+        if (!known || !it->second->mem[0]) {
+            if (c.capturing || (!known && bytes > c.cache64_bytes)) return false;
+            // (no other memory is given up for them: without room they are made in scratch)
+            void* buf = nullptr;
+            if (dev_malloc_raw(&buf, bytes, c.stream) != cudaSuccess) {
+                cudaGetLastError();
+                return false;
+            }
+            if (!known) {
+                c.cache64_bytes -= bytes;
+                it = c.cache64.emplace(std::make_pair((const void*)X.p, key), std::make_unique<Reclaimable>()).first;
+                it->second->call = &c.call;
+            }
+            it->second->hold(buf, nullptr, ReclaimPin(c.call, c.stream));
             d = digits64_in(buf, o.rows, o.K);
             digitise64(c, &o, &d, 1);
             return true;
         }
-        d = digits64_in(it->second, o.rows, o.K);
+        d = digits64_in(it->second->mem[0], o.rows, o.K);
         return true;
     };
     const bool ka = kept(A, a, la, fa, da), kb = kept(B, b, lb, fb, db);

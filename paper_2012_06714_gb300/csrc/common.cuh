@@ -8,6 +8,7 @@
 
 #include <cstdint>
 #include <map>
+#include <memory>
 #include <stdexcept>
 #include <string>
 #include <vector>
@@ -157,8 +158,9 @@ struct Ctx {
     std::map<std::pair<const void*, std::string>, float*> f32cache;
     // split BF16 planes (K-major GEMM operand order) of operands marked constant
     std::map<std::pair<const void*, std::string>, void*> bf16cache;
-    // digits of constant operands of FP64 contractions (gemm64), up to cache64_bytes in all
-    std::map<std::pair<const void*, std::string>, void*> cache64;
+    // digits of constant operands of FP64 contractions (gemm64), up to cache64_bytes in all; held for
+    // speed only (formed again where they were given back and there is room)
+    std::map<std::pair<const void*, std::string>, std::unique_ptr<Reclaimable>> cache64;
     size_t cache64_bytes = 0;
     // constant operands are cached in these forms only if the copy is at most this size
     // (larger ones are converted per call into scratch)
@@ -182,16 +184,25 @@ struct Ctx {
         }
         return done_;
     }
+    bool digits_held() const {
+        for (auto& kv : cache64)
+            if (kv.second->held()) return true;
+        return false;
+    }
+    void drop_digits() {  // and make no more
+        for (auto& kv : cache64) kv.second->drop(stream);
+        cache64.clear();
+        cache64_bytes = 0;
+    }
     // releases everything on the stream (before it is destroyed)
     void release() {
         dev_free(done_, stream);
         done_ = nullptr;
         for (auto& kv : f32cache) dev_free(kv.second, stream);
         for (auto& kv : bf16cache) dev_free(kv.second, stream);
-        for (auto& kv : cache64) dev_free(kv.second, stream);
+        drop_digits();
         f32cache.clear();
         bf16cache.clear();
-        cache64.clear();
         dev_free(d_err, stream);
         d_err = nullptr;
         arena.free_all();
