@@ -490,11 +490,6 @@ void ein(Ctx& c, const char* spec, double alpha, const T& A, const T& B, double 
     else
         einsum(c, spec, alpha, A, B, beta, (double*)C.p, d);
 }
-// Whether an intermediate of M x N x K products may be held in FP32: the mixed sigma, where the product
-// is one of the split-BF16 contractions (FP32 sums) and its result only enters further ones.
-bool f32_product(const Ctx& c, long long M, long long N, long long K) {
-    return c.gemm_mode == 2 && std::min(M, N) > 8 && 2.0 * M * N * K >= c.fp32_min_flops && tc_gemm_fits(M, N, K);
-}
 // C = alpha * permute(X) + beta * C (output axis j = input axis perm[j])
 void perm_into(Ctx& c, const T& X, std::initializer_list<int> perm, const Buf& C, double alpha, double beta) {
     Shape s{(int)X.dims.size(), {}};
@@ -1612,7 +1607,7 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
         einsum(c, "Qjm,nlmj->nQl", 1.0, tc(h->Boo, {Q, o, o}), tn(Z, {n, o, o, o}), 0.0, P, {n, Q, o});
         //  sum (ad|em)(2 t_jm^ce - t_jm^ec) Y~_jcd  (a lean handle holds no tau: two contractions with t)
         // (the n o v^2 intermediates V and q, in the order in which the GEMMs write them)
-        const Buf V = scratch(c.arena, n * o * v * v, f32_product(c, o * v, n * v, o * v));
+        const Buf V = scratch(c.arena, n * o * v * v, false);
         if (h->tau) {
             ein(c, "jmce,njcd->mend", 1.0, tc(h->tau, {o, o, v, v}), tn(Yt, {n, o, v, v}), 0.0, V, {o, v, n, v});
         } else {
@@ -1633,7 +1628,7 @@ static void sigma_ea(adc_handle* h, const double* Xin, double* Sout, long long n
         einsum(c, "nQl,Qim->nlim", 1.0, tn(p, {n, Q, o}), tc(h->Boo, {Q, o, o}), 0.0, Pl, {n, o, o, o});
         einsum(c, "nlim,lmba->niab", 1.0, tn(Pl, {n, o, o, o}), T4, 1.0, S2, {n, o, v, v});
         //  sum_me (cb|em)(2 t_im^ae - t_im^ea) Y_c
-        const Buf q = scratch(c.arena, n * o * v * v, f32_product(c, n * v, o * v, Q) && f32_product(c, n * o, v * v, Q));
+        const Buf q = scratch(c.arena, n * o * v * v, false);
         ein(c, "nQb,Qme->nbme", 1.0, tn(hq, {n, Q, v}), tc(h->Bov, {Q, o, v}), 0.0, q, {n, v, o, v});
         if (h->tau) {
             einsum(c, "nbme,imae->niab", 1.0, q.as({n, v, o, v}), tc(h->tau, {o, o, v, v}), 1.0, S2, {n, o, v, v});
@@ -1705,7 +1700,7 @@ static void sigma_ip(adc_handle* h, const double* Xin, double* Sout, long long n
         // coupling row, second order
         //  - sum (ad|ie) t_jk^de Y~_jka
         // (the n v^3 intermediates Z and w, in the order in which the GEMMs write them)
-        const Buf Z = scratch(c.arena, n * v * v * v, f32_product(c, v * v, n * v, o * o));
+        const Buf Z = scratch(c.arena, n * v * v * v, false);
         ein(c, "jkde,njka->dena", 1.0, tc(t, {o, o, v, v}), tn(Yt, {n, o, o, v}), 0.0, Z, {v, v, n, v});
         double* Hq = c.arena.dalloc(n * Q * v);
         einsum(c, "dena,Qad->nQe", 1.0, Z.as({v, v, n, v}), tc(h->Bvv, {Q, v, v}), 0.0, Hq, {n, Q, v});
@@ -1721,7 +1716,7 @@ static void sigma_ip(adc_handle* h, const double* Xin, double* Sout, long long n
         // 2h1p column, second order (same tensor, applied to Y_i)
         double* bq = c.arena.dalloc(n * Q * v);
         einsum(c, "ni,Qie->nQe", 1.0, tn(y1, {n, o}), tc(h->Bov, {Q, o, v}), 0.0, bq, {n, Q, v});
-        const Buf w = scratch(c.arena, n * v * v * v, f32_product(c, n * v, v * v, Q));
+        const Buf w = scratch(c.arena, n * v * v * v, false);
         ein(c, "nQe,Qad->nead", 1.0, tn(bq, {n, Q, v}), tc(h->Bvv, {Q, v, v}), 0.0, w, {n, v, v, v});
         einsum(c, "nead,jkde->njka", -1.0, w.as({n, v, v, v}), tc(t, {o, o, v, v}), 1.0, S2, {n, o, o, v});
         double* m = c.arena.dalloc(n * o * o * v);
