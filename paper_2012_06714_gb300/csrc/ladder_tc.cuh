@@ -55,7 +55,7 @@ TuneCache* tune_cache_open(const char* path);
 bool tc_gemm_fits(long long M, long long N, long long K);
 // Generic contraction on the same kernel: C[M][N] = sum_k A[m][k] B[n][k] for two-plane
 // split-BF16 K-major operands A[p] [M][Kp], B[p] [N][Kp] (Kp a multiple of 8, zeros beyond K),
-// FP32 partial sums promoted every 8 K blocks (64 deep).  Returns S FP32 results [S][M][N] in
+// FP32 partial sums promoted every 8 K blocks (64 deep) or fewer.  Returns S FP32 results [S][M][N] in
 // c.arena, one per K slice, whose FP64 sum is C (few-tile shapes take several slices).  A bounded
 // device wait that gives up raises c.d_err.  direct: where a single result goes instead (or NULL).
 float* tc_gemm(Ctx& c, const void* const* A, const void* const* B, long long M, long long N, long long Kp, double algo_flops,
