@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "split.cuh"
 #include "warp.cuh"
 #include "gemm64.cuh"
 #include "ladder_tc.cuh"
@@ -67,17 +68,17 @@ __global__ void fill_kernel(long long n, double v, double* __restrict__ y) {
         y[i] = v;
 }
 
-// x as BF16 planes: o0 + o1 (+ o2 where there is a third), each the rounded remainder of those
-// before.  The remainders are formed in FP32, whose 24 bits hold what three planes do: FP64
-// arithmetic (2 operations per cycle and SM on this chip) made the splits several times slower than
-// their traffic.
-__device__ __forceinline__ void put_planes(float f, long long ad, __nv_bfloat16* o0, __nv_bfloat16* o1, __nv_bfloat16* o2) {
-    const __nv_bfloat16 h = __float2bfloat16(f);
+// x as BF16 planes: o0 + o1 (+ o2 where there is a third), each the rounded remainder of those before
+template <typename X>
+__device__ __forceinline__ void put_planes(X x, long long ad, __nv_bfloat16* o0, __nv_bfloat16* o1, __nv_bfloat16* o2) {
+    float f, lo;
+    two_floats(x, f, lo);
+    const __nv_bfloat16 h = __float2bfloat16(odd(f, lo));
     o0[ad] = h;
-    f -= __bfloat162float(h);
+    f = add_keep(f - __bfloat162float(h), lo);
     const __nv_bfloat16 m = __float2bfloat16(f);
     o1[ad] = m;
-    if (o2) o2[ad] = __float2bfloat16(f - __bfloat162float(m));
+    if (o2) o2[ad] = __float2bfloat16((f - __bfloat162float(m)) + lo);
 }
 
 // out[p][r*Kp + k] (two or three BF16 planes) from the permuted input, zero for k >= K
@@ -89,7 +90,7 @@ __global__ void permute_split_kernel(const Tin* __restrict__ in, __nv_bfloat16* 
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
         const I r = (I)(idx / Kp), k = (I)(idx - (long long)r * Kp);
-        double x = 0.0;
+        Tin x = 0;
         if (k < (I)K) {
             I lin = r * (I)K + k, off = 0;
             for (int j = a.nd - 1; j >= 0; --j) {
@@ -98,9 +99,9 @@ __global__ void permute_split_kernel(const Tin* __restrict__ in, __nv_bfloat16* 
                 off += (lin - q * d) * (I)a.sin[j];
                 lin = q;
             }
-            x = (double)in[off];
+            x = in[off];
         }
-        put_planes((float)x, idx, o0, o1, o2);
+        put_planes(x, idx, o0, o1, o2);
     }
 }
 
@@ -126,21 +127,26 @@ struct OpPlanes {
     }
     template <typename V>
     __device__ void put(long long ad, V x) const {
-        put_planes((float)x, ad, o0, o1, o2);
+        put_planes(x, ad, o0, o1, o2);
     }
     template <int V, typename X>
     __device__ void put_n(long long ad, const X (&x)[V]) const {
         if constexpr (V == 4) {
             uint2 w[3];
-            float f[4] = {(float)x[0], (float)x[1], (float)x[2], (float)x[3]};
+            float f[4], lo[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) two_floats(x[i], f[i], lo[i]);
 #pragma unroll
             for (int p = 0; p < 3; ++p) {
-                const __nv_bfloat162 l = __floats2bfloat162_rn(f[0], f[1]), h = __floats2bfloat162_rn(f[2], f[3]);
+                const __nv_bfloat162 l = p ? __floats2bfloat162_rn(f[0], f[1]) : __floats2bfloat162_rn(odd(f[0], lo[0]), odd(f[1], lo[1])),
+                                     h = p ? __floats2bfloat162_rn(f[2], f[3]) : __floats2bfloat162_rn(odd(f[2], lo[2]), odd(f[3], lo[3]));
                 w[p] = make_uint2(*(const unsigned*)&l, *(const unsigned*)&h);
                 f[0] -= __uint_as_float(w[p].x << 16);
                 f[1] -= __uint_as_float(w[p].x & 0xffff0000u);
                 f[2] -= __uint_as_float(w[p].y << 16);
                 f[3] -= __uint_as_float(w[p].y & 0xffff0000u);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) f[i] = add_keep(f[i], lo[i]);
             }
             *(uint2*)(o0 + ad) = w[0];
             *(uint2*)(o1 + ad) = w[1];

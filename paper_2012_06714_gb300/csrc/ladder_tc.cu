@@ -36,6 +36,7 @@
 
 #include "ladder_tc.cuh"
 #include "pairs.cuh"
+#include "split.cuh"
 #include "tcgen05.cuh"
 
 namespace adc {
@@ -460,23 +461,25 @@ __global__ void __launch_bounds__(THREADS, 1)
 struct Planes {
     __nv_bfloat16* p[3];
 };
-// x = p0 + p1 (+ p2) with every plane in BF16 (successive remainders, formed in FP32: its 24 bits hold
-// what three planes do, and FP64 arithmetic would bound the kernels below)
-__device__ __forceinline__ void splitp(float x, int planes, __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2) {
-    const __nv_bfloat16 h = __float2bfloat16(x);
-    x -= __bfloat162float(h);
-    const __nv_bfloat16 m = __float2bfloat16(x);
+// x = p0 + p1 (+ p2) with every plane in BF16 (successive remainders)
+template <typename X>
+__device__ __forceinline__ void splitp(X x, int planes, __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2) {
+    float f, lo;
+    two_floats(x, f, lo);
+    const __nv_bfloat16 h = __float2bfloat16(odd(f, lo));
+    f = add_keep(f - __bfloat162float(h), lo);
+    const __nv_bfloat16 m = __float2bfloat16(f);
     *p0 = h;
     *p1 = m;
-    if (planes == 3) *p2 = __float2bfloat16(x - __bfloat162float(m));
+    if (planes == 3) *p2 = __float2bfloat16((f - __bfloat162float(m)) + lo);
 }
 // pairs split into two or three (o.p[2] not NULL) BF16 planes o.p[plane][(half * rows + row) * Pk + p],
 // zeros for P <= p < Pk
 struct PutPlanes {
     Planes o;
     long long rows, P, Pk, row0;
-    __device__ void operator()(int half, long long row, long long p, double x) const { (*this)(half, row, p, (float)x); }
-    __device__ void operator()(int half, long long row, long long p, float x) const {
+    template <typename X>
+    __device__ void operator()(int half, long long row, long long p, X x) const {
         const long long ad = (half * rows + row) * Pk + p;
         splitp(x, o.p[2] ? 3 : 2, o.p[0] + ad, o.p[1] + ad, o.p[2] + ad);
     }
@@ -499,7 +502,7 @@ __global__ void k_split_Bs(const double* __restrict__ B, int naux, int v, int vp
         int a = r % vp;
         long long Q = r / vp;
         double val = (cp < v && a < v) ? B[(Q * v + a) * v + cp] : 0.0;
-        splitp((float)val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
+        splitp(val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
     }
 }
 // Bp[b][(Q,dp)] = B^Q[d][b] (= B^Q[b][d]), zero pad
@@ -510,7 +513,7 @@ __global__ void k_split_Bp(const double* __restrict__ B, int naux, int v, int vp
         long long r = x / vp;
         int Q = r % naux, b = r / naux;
         double val = dp < v ? B[((long long)Q * v + b) * v + dp] : 0.0;
-        splitp((float)val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
+        splitp(val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
     }
 }
 // XT[(m,d)][cp] = X_m[c][d] for X_m of va x vb (c < va, d < vb; rows d padded to vpb,
@@ -524,7 +527,7 @@ __global__ void k_split_XT(const double* __restrict__ X, long long nmat, int va,
         int d = r % vpb;
         long long m = r / vpb;
         double val = (cp < va && d < vb) ? X[(m * va + cp) * vb + d] : 0.0;
-        splitp((float)val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
+        splitp(val, planes, o.p[0] + x, o.p[1] + x, o.p[2] + x);
     }
 }
 
