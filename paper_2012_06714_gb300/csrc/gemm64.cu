@@ -9,10 +9,15 @@
 //     accumulator per s.  Over 128 summed terms and at most eight digit pairs such a sum stays within
 //     8 * 128 * 2^14 = 2^24, so it is an exact integer; then it is drained into 64-bit integer
 //     registers, where it stays exact for any K;
-//   * the weights s = 14 .. 7 are kept (36 of 64 digit pairs); what is left out is below 2^-63 sqrt(K)
-//     of the product of the row scales.  The one rounding of the result is to FP64.  (Seven digits and
-//     34 pairs round the inputs to 2^-57 of their rows' largest element, which an integral row with a
-//     coherent diagonal, (ia|ia) 20 times the others, turns into 1.2e-16 of the result.)
+//   * the weights s = 14 .. 7 are kept (36 of 64 digit pairs).  What is left out of a sum of K terms is at most
+//     2^-61 K of the product of the row scales (seven pairs of weight 6 to a term, all of one sign at their
+//     largest: constant rows), and for digits of random signs about 2^-63 sqrt(K).  The one rounding of the
+//     result is to FP64.  (Seven digits and 34 pairs round the inputs to 2^-57 of their rows' largest element,
+//     which an integral row with a coherent diagonal, (ia|ia) 20 times the others, turns into 1.2e-16 of the
+//     result.)
+// So a product is fixed point to 63 bits of its rows' largest elements: in norm as accurate as an FP64 GEMM,
+// but an element 2^-63 below its row's largest does not count, where floating point would keep it.  A row
+// with an infinity or a NaN gives NaN.
 // The error against 64-bit arithmetic is that of an FP64 GEMM: norm of the error over norm of sigma
 // 1.8e-16 (IP, 14/113/445) against 1.7e-16 with DGEMM, 1.2e-16 each for its final rounding.
 // Measured: that sigma (5 vectors) 24.6 -> 3.8 ms in 20 contractions, 0.30 ms with the coupling block held
@@ -32,6 +37,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "digits.cuh"
 #include "gemm64.cuh"
 #include "tcgen05.cuh"
 
@@ -39,9 +45,6 @@ namespace adc {
 
 namespace {
 
-constexpr int ND = 8;          // digits
-constexpr int SMIN = ND - 1;   // lowest weight kept
-constexpr int NL = 8;          // weights SMIN .. 2 (ND - 1)
 constexpr int GM = 128;        // tile rows
 constexpr int GK = 32;         // K block: 64-byte rows, 64-byte swizzle
 constexpr int EPOCH = 4;       // K blocks between drains (128 terms)
@@ -86,32 +89,17 @@ __device__ __forceinline__ long long digit_k(const Operand64& x, unsigned k) {
     }
     return off;
 }
-__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-// x[0], x[1] of a row of largest exponent field ef -> their digits, at `at` of each plane.  Integer
-// arithmetic only: the FP64 pipe (2 operations per cycle and SM) would be the bound.
+// x[0], x[1] of a row of largest exponent field ef -> their digits, at `at` of each plane
 __device__ __forceinline__ void put_digits(const DigitSide& sd, long long at, const double* x, int ef) {
     unsigned dig[ND];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const long long b = __double_as_longlong(x[h]);
-        const int ex = (int)(b >> 52) & 0x7ff;
-        // |x| = m 2^(ex - 1075) -> round(|x| 2^(1085 - ef)), below 2^63: the row's scale is 2^(ef - 1022)
-        long long v = 0;
-        const int sh = ef - ex - 10;  // right shift of the 53-bit significand (-10: ten more bits)
-        if (ex > 0 && ef < 0x7ff && sh < 55) {
-            const long long m = (b & 0xfffffffffffffLL) | (1LL << 52);
-            v = sh <= 0 ? m << -sh : (m + (1LL << (sh - 1))) >> sh;
-            if (b < 0) v = -v;
-        }
-        // digit p < 7 of v is the p-th byte of v + sum_p 128 256^p less 128: the carries in
-        // one addition; the top one is in [-128, 128]
-        const unsigned long long w = (unsigned long long)v + 0x0080808080808080ULL;
-        const int top = v >= 0 ? (int)(w >> 56) : (int)((long long)w >> 56);
+        const long long v = scaled_integer((uint64_t)__double_as_longlong(x[h]), ef);
+        const uint64_t w = with_carries(v);
 #pragma unroll
         for (int p = 0; p < ND; ++p) {
-            const int d = p < ND - 1 ? (int)((w >> (8 * p)) & 0xff) - 128 : top;
             // a small integer's BF16 bits are the upper half of its FP32 bits
-            const unsigned u = __float_as_uint((float)d) >> 16;
+            const unsigned u = __float_as_uint((float)digit(v, w, p)) >> 16;
             dig[p] = h == 0 ? u : dig[p] | (u << 16);
         }
     }
@@ -155,7 +143,7 @@ __global__ void __launch_bounds__(DT) k_digits(const __grid_constant__ DigitSide
     __syncthreads();
     const int r = tid >> lper, t = tid & (per - 1);  // per threads to a row
     int m = 0;
-    for (int k = t; k < seg; k += per) m = max(m, exponent_of(tile[r * ld + k]));
+    for (int k = t; k < seg; k += per) m = max(m, exponent_of((uint64_t)__double_as_longlong(tile[r * ld + k])));
     if (m > 0) atomicMax(&emax[r], m);
     namespace cg = cooperative_groups;
     const cg::cluster_group cl = cg::this_cluster();
@@ -202,7 +190,7 @@ __global__ void __launch_bounds__(DT) k_digits_long(const __grid_constant__ Digi
         __syncthreads();
         if (pass == 1) {
             int m = 0;
-            for (int k = tid & (per - 1); k < DT; k += per) m = max(m, exponent_of(tile[r][k]));
+            for (int k = tid & (per - 1); k < DT; k += per) m = max(m, exponent_of((uint64_t)__double_as_longlong(tile[r][k])));
             if (m > 0) atomicMax(&emax[r], m);
         } else if (row0 + r < x.rows) {
             for (int k = 2 * (tid & (per - 1)); k < DT && k0 + k < sd.Kp; k += 2 * per)
@@ -230,40 +218,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 __device__ __forceinline__ uint64_t desc64(const void* p) {
     return (uint64_t)((su32(p) >> 4) & 0x3FFF) | (uint64_t)1 << 16 | (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 |
            (uint64_t)4 << 61;
-}
-
-// (hi 2^32 + lo) 2^e, rounded to nearest, by integer arithmetic; |hi| < 2^62
-__device__ __forceinline__ double to_double(long long hi, long long lo, int e) {
-    long long H = hi + (lo >> 32);
-    uint32_t L = (uint32_t)lo;
-    const bool neg = H < 0;
-    if (neg) {
-        L = 0u - L;
-        H = L == 0 ? -H : ~H;
-    }
-    unsigned long long m;
-    int top;  // weight of m's bit 63
-    if (H != 0) {
-        const int lz = __clzll(H);
-        const unsigned long long l = (unsigned long long)L << 32;
-        m = ((unsigned long long)H << lz) | (lz ? l >> (64 - lz) : 0ull);
-        top = 95 - lz;
-    } else {
-        if (L == 0) return 0.0;
-        const int lz = __clz(L);
-        m = (unsigned long long)L << (32 + lz);
-        top = 31 - lz;
-    }
-    m = (m >> 11) + ((m >> 10) & 1);  // 53 bits, carry into bit 53 raises the exponent below
-    const int be = top + e + 1023;
-    unsigned long long bits;
-    if (be <= 0)
-        bits = 0;  // below the normal range
-    else if (be >= 2046)
-        bits = 0x7ffull << 52;
-    else
-        bits = m + ((unsigned long long)(be - 1) << 52);
-    return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
 }
 
 struct Gemm64Out {

@@ -66,3 +66,19 @@ def test_rows_of_a_cluster(o, v, nvec):
     S, R = g.sigma(X), ref.sigma(X)
     g.close()
     assert np.abs(S - R).max() <= 1e-13 * np.abs(R).max()
+
+
+@pytest.mark.parametrize("p", [-1035, -1000, 960])
+def test_range_of_doubles(p):
+    """Vectors scaled by 2^p, subnormal at -1035: sigma is linear, so it scales with them, to the FP64 bound of
+    the tests above and, where results or intermediates are subnormal, a unit 2^-1074 for each of the up to 1e5
+    terms that a result sums over all its contractions."""
+    from paper_2012_06714_gb300 import ADC
+
+    o, v = 6, 40
+    s = make_system(o, v, 120, seed=3)
+    g = ADC(s.eps, s.B, o, order=3, kind="ip", precision="fp64")
+    X = np.ldexp(np.random.default_rng(5).standard_normal((64, g.dim)), p)
+    S, R = g.sigma(X), g.sigma(np.ldexp(X, -p))
+    g.close()
+    assert np.abs(np.ldexp(S, -p) - R).max() <= 1e-13 * np.abs(R).max() + 1e5 * np.ldexp(1.0, -1074 - p)
