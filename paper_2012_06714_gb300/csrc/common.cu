@@ -1063,6 +1063,7 @@ static void einsum_64(Ctx& c, const std::string& la, const std::string& lb, cons
         return o;
     };
     Operand64 a = operand(A, la, fa), b = operand(B, lb, fb);
+    if (a.rows == 0 || b.rows == 0) return;  // nothing to write
     const bool tensor = gemm64_fits(a.rows, b.rows, a.K);
     // the 128-row axis takes the longer side when the other would leave it mostly empty
     // (small64: the longer side on the grid's x axis)

@@ -8,7 +8,7 @@
 //   * the digit products of equal weight, s = i + j, accumulate in one FP32 tensor-memory
 //     accumulator per s.  Over 128 summed terms and at most eight digit pairs such a sum stays within
 //     8 * 128 * 2^14 = 2^24, so it is an exact integer; then it is drained into 64-bit integer
-//     registers, where it stays exact for any K;
+//     registers, where it stays exact over a slice of up to 2^23 terms (longer K is cut into slices);
 //   * the weights s = 14 .. 7 are kept (36 of 64 digit pairs).  What is left out of a sum of K terms is at most
 //     2^-61 K of the product of the row scales (seven pairs of weight 6 to a term, all of one sign at their
 //     largest: constant rows), and for digits of random signs about 2^-63 sqrt(K).  The one rounding of the
@@ -39,15 +39,13 @@
 
 #include "digits.cuh"
 #include "gemm64.cuh"
+#include "plan64.cuh"
 #include "tcgen05.cuh"
 
 namespace adc {
 
 namespace {
 
-constexpr int GM = 128;        // tile rows
-constexpr int GK = 32;         // K block: 64-byte rows, 64-byte swizzle
-constexpr int EPOCH = 4;       // K blocks between drains (128 terms)
 constexpr int G_EPI = 8;       // epilogue warps
 constexpr int G_THREADS = 64 + 32 * G_EPI;
 constexpr int G_MAXST = 4;
@@ -460,33 +458,6 @@ int sm_count() {
     return n;
 }
 
-struct Gemm64Plan {
-    int BNT, S, kb;  // tile width, K slices, K blocks per slice
-};
-
-// Tile width and K slices: least time over the chip.  A K block of a tile takes 18 BNT tensor cycles
-// twice (36 digit pairs), reading A from shared memory bounds it below about BNT = 16; a drain (every
-// EPOCH blocks) about 40 BNT cycles, which the MMAs wait for; the last one and the store about 60 BNT.
-Gemm64Plan plan64(long long M, long long N, long long Kp) {
-    const int num_k = (int)((Kp + GK - 1) / GK), sms = sm_count();
-    Gemm64Plan p{64, 1, num_k};
-    double best = 1e300;
-    for (int b : {64, 48, 32, 16}) {
-        const long long tiles = ((M + GM - 1) / GM) * ((N + b - 1) / b);
-        for (long long s = 1; s <= std::max(1LL, std::min<long long>(160, 2 * sms / tiles)) || s <= 32; ++s) {
-            const long long kb = ((num_k + s - 1) / s + EPOCH - 1) / EPOCH * EPOCH;
-            if (s > 1 && (num_k + kb - 1) / kb != s) continue;
-            const double rounds = (double)((tiles * s + sms - 1) / sms);
-            const double blocks = (double)std::min<long long>(kb, num_k);
-            const double cyc = rounds * (2000.0 + blocks * 2.0 * std::max(18.0 * b, 320.0) + (blocks / EPOCH) * 40.0 * b + 60.0 * b) +
-                               (s - 1) * (double)M * N * 16.0 / 2500.0 + (s > 1 ? 4000.0 : 0.0);
-            if (cyc < best * 0.999) best = cyc, p = Gemm64Plan{b, (int)s, (int)kb};
-        }
-    }
-    p.S = (num_k + p.kb - 1) / p.kb;
-    return p;
-}
-
 void launch64(Ctx& c, const Digits64& A, const Digits64& B, const Gemm64Plan& p, double* T, const Out64& out) {
     if (!c.d_err) {
         if (c.capturing) throw Error(-3, "error flag allocation during stream capture");
@@ -566,7 +537,7 @@ void digitise64(Ctx& c, const Operand64* x, Digits64* out, int n) {
         d.plane = out[i].plane;
         d.ex = out[i].ex;
         if (x[i].K > Kp || out[i].Kp != Kp) throw Error(-1, "digitise64: shape mismatch");
-        long long smallest = d.x.ks[d.x.nk - 1];
+        long long smallest = d.x.nk > 0 ? d.x.ks[d.x.nk - 1] : 1;
         d.row_lanes = 0;
         for (int j = 0; j < d.x.nk; ++j) smallest = std::min(smallest, d.x.kd[j] > 1 ? d.x.ks[j] : smallest);
         for (int j = 0; j < d.x.nr; ++j)
@@ -611,7 +582,7 @@ void digitise64(Ctx& c, const Operand64* x, Digits64* out, int n) {
 double* gemm64(Ctx& c, const Operand64& A, const Digits64* da, const Operand64& B, const Digits64* db, const Out64& out,
                int& S) {
     const long long M = da ? da->rows : A.rows, N = db ? db->rows : B.rows, Kp = da ? da->Kp : (A.K + 7) / 8 * 8;
-    const Gemm64Plan plan = plan64(M, N, Kp);
+    const Gemm64Plan plan = plan64(M, N, Kp, sm_count());
     S = plan.S;
     // (the result is allocated first: it outlives the digits)
     double* T = out.p && S == 1 ? nullptr : c.arena.dalloc((size_t)S * M * N);
@@ -679,14 +650,10 @@ __global__ void __launch_bounds__(ST * ST) k_small64(const __grid_constant__ Ope
 double* small64(Ctx& c, const Operand64& A, const Operand64& B, const Out64& out, int& S) {
     const long long mt = (A.rows + ST - 1) / ST, nt = (B.rows + ST - 1) / ST;
     if (mt > 65535 || nt > 0x7fffffffLL || A.K >= (1LL << 30)) throw Error(-1, "small64: too many rows");
-    // K slices while the blocks leave SMs idle, of at least 64 terms (a sum of slices is another launch)
-    S = 1;
-    if (A.K >= 256 && mt * nt < 2 * sm_count())
-        S = (int)std::max<long long>(1, std::min<long long>({A.K / 64, 4LL * sm_count() / (mt * nt), 256}));
-    long long ks = (A.K + S - 1) / S;
-    S = (int)((A.K + ks - 1) / ks);
+    const Small64Plan plan = plan_small64(mt * nt, A.K, sm_count());
+    S = plan.S;
     double* T = out.p && S == 1 ? nullptr : c.arena.dalloc((size_t)S * A.rows * B.rows);
-    k_small64<<<dim3((unsigned)nt, (unsigned)mt, (unsigned)S), ST * ST, 0, c.stream>>>(A, B, ks, T, out);
+    k_small64<<<dim3((unsigned)nt, (unsigned)mt, (unsigned)S), ST * ST, 0, c.stream>>>(A, B, plan.terms, T, out);
     ++c.kernels;
     ADC_CUDA(cudaGetLastError());
     return T;

@@ -1,6 +1,5 @@
-// The integer arithmetic of gemm64.cu (digits.cuh): digit products of rows over the whole range of doubles
-// against long double sums.
-#include <algorithm>
+// The host side of gemm64.cu's arithmetic (digits.cuh, plan64.cuh): digit products of rows over the whole range
+// of doubles against long double sums, the 64-bit sums at the longest slice, and launch plans at their ends.
 #include <cfloat>
 #include <cmath>
 #include <cstdio>
@@ -8,6 +7,7 @@
 #include <vector>
 
 #include "digits.cuh"
+#include "plan64.cuh"
 
 using namespace adc;
 
@@ -78,6 +78,19 @@ int main() {
         const long double allowed = fabsl(exact) * 0x1p-53L + K * 4 * ma * mb * 0x1.1p-61L + 0x1p-1074L;
         CHECK(fabsl((long double)r - exact) <= allowed, "K %d, 2^%d 2^%d: %a, exact %La", K, pa, pb, r, exact);
     }
+    // a slice of constant rows at their largest: the leading part within 62 bits, the sum exact
+    {
+        const long long terms = (long long)kExactBlocks * GK, v = 0x7ffffffffffffc00LL;
+        const uint64_t w = with_carries(v);
+        __int128 hi = 0, lo = 0;
+        for (int i = 0; i < ND; ++i)
+            for (int j = SMIN - i; j < ND; ++j) {
+                const __int128 d = (__int128)digit(v, w, i) * digit(v, w, j) * terms;
+                (i + j >= 11 ? hi : lo) += d << (8 * (i + j >= 11 ? i + j - 11 : i + j - SMIN));
+            }
+        const __int128 lim = (__int128)1 << 62;
+        CHECK(hi < lim && hi > -lim && lo < lim && lo > -lim, "%d terms", (int)terms);
+    }
     // the ends of the range of results
     CHECK(to_double((1LL << 53) - 1, 0, 971 - 32) == DBL_MAX, "%a", to_double((1LL << 53) - 1, 0, 971 - 32));
     CHECK(to_double(0, 3, 1022) == 0x1.8p+1023, "%a", to_double(0, 3, 1022));
@@ -86,6 +99,19 @@ int main() {
     CHECK(to_double(0, 5, -1073) == 0xap-1074, " ");
     CHECK(to_double(0, 1, -1076) == 0.0, " ");
     CHECK(to_double(0, 0, 0) == 0.0, " ");
+    // plans: every K block in one slice, no empty slice, no slice beyond the exact sums
+    for (int i = 0; i < 20000; ++i) {
+        auto size = [&](int top) { return (long long)std::exp2(std::uniform_real_distribution<double>(0, top)(g)); };
+        const long long M = i < 8 ? i % 2 : size(24), N = i < 8 ? i / 2 % 2 : size(24);
+        const long long Kp = i < 8 ? i / 4 * 8 : (size(27) + 7) / 8 * 8 << (i % 5 == 0 ? 2 : 0);
+        const Gemm64Plan p = plan64(M, N, Kp, 152);
+        const long long num_k = (Kp + GK - 1) / GK;
+        CHECK(p.S >= 1 && (long long)p.S * p.kb >= num_k && (p.S == 1 || (p.S - 1LL) * p.kb < num_k), "%lld %lld %lld", M, N, Kp);
+        CHECK(p.kb <= kExactBlocks && (p.S == 1 || p.kb % EPOCH == 0), "%lld: %d slices of %d", Kp, p.S, p.kb);
+        const long long tiles = i < 8 ? i % 2 : size(20), K = i < 8 ? i / 2 : size(22);
+        const Small64Plan q = plan_small64(tiles, K, 152);
+        CHECK(q.S >= 1 && q.S * q.terms >= K && (q.S == 1 || (q.S - 1) * q.terms < K), "%lld %lld", tiles, K);
+    }
     if (bad) std::printf("%d wrong\n", bad);
     return bad ? 1 : 0;
 }
