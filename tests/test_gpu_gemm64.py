@@ -82,3 +82,22 @@ def test_range_of_doubles(p):
     S, R = g.sigma(X), g.sigma(np.ldexp(X, -p))
     g.close()
     assert np.abs(np.ldexp(S, -p) - R).max() <= 1e-13 * np.abs(R).max() + 1e5 * np.ldexp(1.0, -1074 - p)
+
+
+@pytest.mark.parametrize("o,v,naux,nvec", [(8, 64, 100, 3), (9, 57, 100, 3), (16, 64, 60, 3), (25, 41, 60, 3), (32, 128, 30, 2), (17, 241, 20, 2)])
+def test_digits_of_long_rows(o, v, naux, nvec):
+    """Rows of o v = 512, 513, 1024, 1025, 4096 and 4097 terms, between which they are cut into digits by one block,
+    by clusters of up to eight, and in two passes: the product Qjc,njcd->nQd of an ADC(2) sigma without the held
+    coupling block, of more than the 4e6 flop from which digits are made.  The bound of the tests above."""
+    from paper_2012_06714_gb300 import ADC, release_memory
+
+    assert 2 * naux * nvec * v * o * v >= 4e6
+    s = make_system(o, v, naux, seed=v)
+    ref = SpinAdaptedADC(s.eps, o, s.B, 2, "ea")
+    g = ADC(s.eps, s.B, o, order=2, kind="ea", precision="fp64")
+    release_memory()  # the coupling block
+    X = np.random.default_rng(v).standard_normal((nvec, g.dim))
+    S, R = g.sigma(X), ref.sigma(X)
+    g.close()
+    assert np.abs(S[:, :v] - R[:, :v]).max() <= 1e-13 * np.abs(R[:, :v]).max()
+    assert np.abs(S - R).max() <= 1e-13 * np.abs(R).max()
