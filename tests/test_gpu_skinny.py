@@ -28,3 +28,23 @@ def test_every_number_of_vectors_vs_oracle(o, v, naux):
         for part in (slice(0, v), slice(v, None)):
             assert np.abs(S[:, part] - R[:n, part]).max() <= 3e-5 * np.abs(R[:n]).max(), n
     g.close()
+
+
+@pytest.mark.parametrize("o,v,naux", [(5, 216, 40), (5, 217, 40)])
+def test_one_and_two_vectors_vs_oracle(o, v, naux):
+    """One and two vectors at sizes whose coupling products reach the bandwidth kernels (1e8 flop for one vector;
+    at the sizes above they are smaller and taken in FP64)."""
+    from paper_2012_06714_gb300 import ADC
+
+    s = make_system(o, v, naux, seed=v)
+    ref = SpinAdaptedADC(s.eps, o, s.B, 3, "ea")
+    g = ADC(s.eps, s.B, o, order=3, kind="ea", precision="bf16x3")
+    X = np.random.default_rng(v).standard_normal((2, g.dim))
+    X[:, v:] /= np.sqrt(v)
+    R = ref.sigma(X)
+    for n in (1, 2):
+        assert 2.0 * n * o * v**3 >= 1e8
+        S = g.sigma(X[:n])
+        for part in (slice(0, v), slice(v, None)):
+            assert np.abs(S[:, part] - R[:n, part]).max() <= 3e-5 * np.abs(R[:n]).max(), n
+    g.close()
