@@ -28,3 +28,21 @@ def test_coupling_block_vs_oracle(kind, precision, o, v, naux, nvec, tol):
     g.close()
     for part in (slice(0, n1), slice(n1, None)):
         assert np.abs(S[:, part] - R[:, part]).max() <= tol * np.abs(R).max()
+
+
+@pytest.mark.parametrize("precision,tol", [("bf16x3", 3e-5), ("fp64", 1e-11)])
+def test_ea_coupling_block_in_slices_vs_oracle(precision, tol):
+    """An EA block formed in two slices of the virtual index, 445 and 3 of 448 (o v^3 > 2^28)."""
+    from paper_2012_06714_gb300 import ADC
+
+    o, v = 3, 448
+    assert o * v**3 > 2**28
+    s = make_system(o, v, 24, seed=v)
+    ref = SpinAdaptedADC(s.eps, o, s.B, 3, "ea")
+    g = ADC(s.eps, s.B, o, order=3, kind="ea", precision=precision)
+    X = np.random.default_rng(v).standard_normal((2, g.dim))
+    X[:, v:] /= np.sqrt(v)
+    S, R = g.sigma(X), ref.sigma(X)
+    g.close()
+    for part in (slice(0, v), slice(v, None)):
+        assert np.abs(S[:, part] - R[:, part]).max() <= tol * np.abs(R).max()

@@ -80,3 +80,22 @@ def test_out_of_memory_leaves_the_handle_usable():
         torch.cuda.empty_cache()
     assert np.abs(a.sigma(X[:4]) - before).max() <= 3e-5 * np.abs(before).max()
     a.close()
+
+
+@pytest.mark.parametrize("precision,nvec,tol", [("bf16x3", 826, 3e-5), ("fp64", 331, 1e-11)])
+def test_matrices_in_groups(precision, nvec, tol):
+    """More matrices than one group of the pair ladder takes (at 180 virtuals 8240 in mixed precision and 3295 in
+    FP64): the first, the middle and the last vectors of the block against the same vectors by themselves."""
+    from paper_2012_06714_gb300 import ADC
+
+    o, v, naux = 10, 180, 300
+    s = make_system(o, v, naux, seed=1)
+    g = ADC(s.eps, s.B, o, order=3, kind="ea", precision=precision)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(7)
+    X = torch.randn(nvec, g.dim, dtype=torch.float64, device="cuda", generator=gen)
+    S = g.sigma(X)
+    pick = [0, 1, nvec // 2, nvec - 3, nvec - 2, nvec - 1]
+    R = g.sigma(X[pick].contiguous())
+    assert float((S[pick] - R).abs().max()) <= tol * float(R.abs().max())
+    g.close()
