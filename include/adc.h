@@ -74,7 +74,11 @@ extern "C" {
 #define ADC_EA 1
 #define ADC_IP (-1)
 
-#define ADC_PREC_FP64 0   /* every contraction in FP64                              */
+#define ADC_PREC_FP64 0   /* every contraction to FP64 accuracy: large ones as exact */
+                          /* digit products on the tensor cores, fixed point to 63   */
+                          /* bits of the largest element of each operand row (in     */
+                          /* norm as accurate as an FP64 GEMM; a row with an infinity */
+                          /* or a NaN gives NaN), small ones in FP64 arithmetic      */
 #define ADC_PREC_BF16X3 1 /* DF ladder on tcgen05 tensor cores with hi/lo BF16       */
                           /* operands (3 products), FP32 accumulation (partial sums */
                           /* promoted to round-to-nearest FP32 registers) within an */

@@ -1,6 +1,7 @@
 // Shared device helpers of the ADC library: error handling, a device scratch
-// arena, an N-d permute kernel and a two-operand tensor contraction executor
-// (permute to GEMM form + cuBLAS strided-batched DGEMM + permute back).
+// arena, N-d permutes and a two-operand tensor contraction executor (einsum),
+// which takes each contraction to one of the library's GEMM kernels (Ctx::gemm_mode)
+// or, batched and FP32-accurate ones, to cuBLAS.
 #pragma once
 
 #include <cublas_v2.h>
@@ -135,11 +136,12 @@ struct Ctx {
     cublasHandle_t blas = nullptr;
     Arena arena;
     long long kernels = 0;  // own kernel launches issued (for reporting)
-    // 0: every contraction in FP64 (DGEMM).  1: contractions of >= fp32_min_flops
+    // 0: every contraction to FP64 accuracy (gemm64 and small64 on operands in place; cuBLAS
+    // DGEMM for batched ones and beyond their sizes).  1: contractions of >= fp32_min_flops
     // run as FP32-accurate GEMMs (BF16x9 emulation on the tensor cores), with
     // FP64 inputs rounded to FP32 and results accumulated into FP64.  2 (the
     // mixed sigma): unbatched contractions of >= fp32_min_flops run on the tcgen05
-    // split-BF16 GEMM (two planes, FP32 partial sums promoted every 8 K blocks,
+    // split-BF16 GEMM (two planes, FP32 partial sums promoted every 8 K blocks or fewer,
     // FP64 result) unless a free dimension is <= 8 and the large operand is not a
     // cached constant; the others on the library's own kernels (own_gemm:
     // FP32-accurate from fp32_min_flops, else FP64).

@@ -18,12 +18,13 @@
 // So a product is fixed point to 63 bits of its rows' largest elements: in norm as accurate as an FP64 GEMM,
 // but an element 2^-63 below its row's largest does not count, where floating point would keep it.  A row
 // with an infinity or a NaN gives NaN.
-// The error against 64-bit arithmetic is that of an FP64 GEMM: norm of the error over norm of sigma
-// 1.8e-16 (IP, 14/113/445) against 1.7e-16 with DGEMM, 1.2e-16 each for its final rounding.
-// Measured: that sigma (5 vectors) 24.6 -> 3.8 ms in 20 contractions, 0.30 ms with the coupling block held
+// Norm of the error over norm of an FP64 sigma of 5 vectors, against long double: 7.4e-17 (IP 8/48/180) and
+// 7.9e-17 (EA 6/40/150), with DGEMM 1.5e-16 and 5.9e-16.
+// Measured, the IP sigma of 5 vectors at 14/113/445: 24.6 -> 3.8 ms in 20 contractions, 0.30 ms with the coupling block held
 // (three of 70 x 1582 x 1582 results and terms take 37 us each: 40 MB of cached digits read from L2 by 99
 // tiles; other tile widths, slices and the exchanged sides are all between 34 and 140 us); the FP64 setup of
-// an IP molecule at 17/121/483 with its first sigma 217 -> 18.7 ms, about half of it here.
+// an IP molecule at 17/121/483 with its first sigma 217 -> 18.7 ms, about half of it here (23.2 ms with the mapping
+// of its memory, where no other handle lives: memory.cuh).
 //
 // Tile: 128 rows of A x BNT columns (16 .. 64) of B per CTA, because the eight accumulators take
 // 8 x BNT of the 512 tensor-memory columns.  The digit planes of B lie one after another in shared

@@ -742,7 +742,6 @@ void split_B(LadderTC& L, Ctx& c, int planes) {
     ADC_CUDA(cudaGetLastError());
     for (int p = 0; p < planes; ++p) {
         L.mBs[p] = make_map(L.Bs[p], (long long)L.naux * L.vp, L.vp, BM);
-        // GEMM2-B boxes: one CTA's half of the tile in pair mode
     }
     L.nplanes = planes;
 }
