@@ -1785,6 +1785,16 @@ static void sigma_run(adc_handle* h, const double* X, double* S, long long n) {
         if (e.n == n) g = &e;
     if (!g) {
         adc_handle::SigmaGraph e;
+        struct Buffers {  // the graph's, or given back where there will be none (also when memory runs out below)
+            adc_handle::SigmaGraph& e;
+            cudaStream_t s;
+            bool kept = false;
+            ~Buffers() {
+                if (kept) return;
+                dev_free(e.X, s);
+                dev_free(e.S, s);
+            }
+        } buffers{e, c.stream};
         e.n = n;
         e.X = (double*)dev_alloc((size_t)n * dim * sizeof(double), c.stream);
         e.S = (double*)dev_alloc((size_t)n * dim * sizeof(double), c.stream);
@@ -1807,6 +1817,7 @@ static void sigma_run(adc_handle* h, const double* X, double* S, long long n) {
         if (ok && ec == cudaSuccess && graph && cudaGraphInstantiate(&e.exec, graph, 0) == cudaSuccess) {
             cudaGraphDestroy(graph);
             h->graphs.push_back(e);
+            buffers.kept = true;
             ADC_CUDA(cudaMemcpyAsync(S, e.S, (size_t)n * dim * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
             return;  // the ordinary evaluation above computed this call's result
         }
@@ -1814,9 +1825,6 @@ static void sigma_run(adc_handle* h, const double* X, double* S, long long n) {
         cudaGetLastError();
         h->graphs_failed = true;
         ADC_CUDA(cudaMemcpyAsync(S, e.S, (size_t)n * dim * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
-        ADC_CUDA(cudaStreamSynchronize(c.stream));
-        cudaFree(e.X);
-        cudaFree(e.S);
         return;
     }
     ADC_CUDA(cudaMemcpyAsync(g->X, X, (size_t)n * dim * sizeof(double), cudaMemcpyDeviceToDevice, c.stream));

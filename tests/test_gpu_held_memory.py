@@ -147,3 +147,38 @@ def test_digits_of_constants_are_given_back():
         release_memory()
         assert _free() - free >= 2 * 16 * (10 * 120) ** 2
     g.close()
+
+
+def test_solves_with_graphs_that_run_out_of_memory_leave_nothing():
+    """A solve with cuda_graphs that runs out of memory somewhere on its way to a captured sigma gives back that
+    sigma's buffers (2 x 7 MB at these sizes): with no handle left the device has as much free memory as before,
+    up to 8 MB."""
+    from paper_2012_06714_gb300 import ADC, release_memory
+    from paper_2012_06714_gb300._lib import ADCError
+
+    o, v = 6, 160
+    s = make_system(o, v, 40, seed=1)
+    stream = torch.cuda.Stream()
+
+    def solve(leave):
+        g = ADC(s.eps, s.B, o, order=3, kind="ea", precision="bf16x3", cuda_graphs=1, max_iter=3)
+        g.set_stream(stream.cuda_stream)
+        release_memory()
+        hold = torch.empty(_free() - leave, dtype=torch.uint8, device="cuda") if leave else None
+        try:
+            g.davidson(4, tol=1e-6)
+            return True
+        except ADCError as e:
+            assert e.code == -2
+            return False
+        finally:
+            del hold
+            torch.cuda.empty_cache()
+            g.close()
+
+    assert solve(0)
+    release_memory()
+    free = _free()
+    done = [solve(m << 20) for m in range(100, 2000, 100)]
+    assert not all(done) and any(done)
+    assert _free() >= free - (8 << 20)
